@@ -317,7 +317,7 @@ int vg_set_depth(vg_ctx *ctx, const double *depth_v);
  * face); a step clamped by dt_max does not depend on the state.  The state at
  * every checkpoint_every-th step is kept on the device, and vg_adj_backward
  * recomputes each segment of checkpoint_every steps once, recording it (about
- * r = 192 bytes per cell and step with a fixed dt, 216 with CFL steps, against
+ * r = 192 bytes per cell and step with a fixed dt, 224 with CFL steps, against
  * 24 per checkpoint).  0 picks the segment length that minimises device memory,
  * round(sqrt(24 n_steps / r)): recordings and checkpoints then take about equal
  * shares, 2 sqrt(24 r n_steps) bytes per cell in all (about 6.1 KB per cell for

@@ -662,17 +662,22 @@ __global__ void adj_stage1_rev_kernel(int nc, double dt, double hthr, const doub
 }
 
 // Gauge functional J = sum weights * (H + z) at the gauge cells: its adjoint.
-__global__ void adj_gauge_kernel(int n_gauges, const int32_t *cells, const double *weights, int nc, double *wb,
-                                 double *zb)
+// Two gauges may share a cell: the first gauge of a cell adds all of that cell's
+// weights, in gauge order (one thread per gauge; one thread walking all gauges
+// was a chain of dependent loads, 18 us for 16 gauges).
+__global__ void adj_gauge_kernel(int n_gauges, const int32_t *cells, const double *weights, double *wb, double *zb)
 {
-    // serial over gauges: two gauges may share a cell
-    if (blockIdx.x == 0 && threadIdx.x == 0)
-        for (int g = 0; g < n_gauges; g++) {
-            int c = cells[g];
-            wb[c] += weights[g];
-            zb[c] += weights[g];
-        }
-    (void)nc;
+    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < n_gauges; g += gridDim.x * blockDim.x) {
+        const int c = cells[g];
+        bool first = true;
+        for (int h = 0; h < g && first; h++) first = cells[h] != c;
+        if (!first) continue;
+        double bw = wb[c], bz = zb[c];
+        for (int h = g; h < n_gauges; h++)
+            if (cells[h] == c) { bw += weights[h]; bz += weights[h]; }
+        wb[c] = bw;
+        zb[c] = bz;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -760,73 +765,81 @@ __device__ FaceIn face_in(const AdjMesh &m, const double *FV, int K, int f)
     return r;
 }
 
-// max_f l_f a_f of cell K (forward order, a tie keeping the earlier face) and its face.
-__device__ double cell_speed(const AdjMesh &m, const double *FV, int K, int &fmax_out)
-{
-    double am = 0.0;
-    fmax_out = -1;
-    for (int f = 0; f < 3; f++) {
-        FaceIn q = face_in(m, FV, K, f);
-        double la = q.l * face_speed(m, q.HfL, q.HufL, q.HvfL, q.zL, q.HfR, q.HufR, q.HvfR, q.zR, q.nx, q.ny, q.wall,
-                                     q.bnd);
-        if (gt_nn(la, am)) { am = la; fmax_out = f; }
-    }
-    return am;
-}
-
 __device__ __forceinline__ bool cfl_less(double b1, int o1, double b2, int o2)
 {
     return b1 < b2 || (b1 == b2 && o1 < o2);
 }
 
-// Per CTA: the cell of smallest bound |K| / (3 max_f l_f a_f) (ties: lowest
-// original id) -> part_b, part_o, part_k [gridDim].
-__global__ void adj_cfl_part_kernel(AdjMesh m, const double *FV, const int32_t *orig, double *part_b, int *part_o,
-                                    int *part_k)
+// Per CTA: the cell of smallest CFL bound |K| / (3 max_f l_f a_f) (ties: lowest
+// original id) -> part_b, part_o, part_k [gridDim].  The bounds are those that the
+// forward stage-1 kernel recorded (recomputing every face's speed here took as
+// long as the reconstruction VJP).
+constexpr int kRedThreads = 256;
+__device__ __forceinline__ void cta_argmin(double &b, int &o, int &k)
 {
-    __shared__ double sb[256];
-    __shared__ int so[256], sk[256];
-    const int nc = m.nc, tid = threadIdx.x;
-    double bb = INFINITY;
-    int bo = 0x7fffffff, bk = -1;
-    for (int K = blockIdx.x * blockDim.x + tid; K < nc; K += gridDim.x * blockDim.x) {
-        int f;
-        double am = cell_speed(m, FV, K, f);
-        if (!is_pos(am)) continue;
-        double b = G(m, GEO_AREA, K) / (3.0 * am);
-        if (cfl_less(b, orig[K], bb, bo)) { bb = b; bo = orig[K]; bk = K; }
+    __shared__ double sb[kRedThreads / 32];
+    __shared__ int so[kRedThreads / 32], sk[kRedThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int s = 16; s > 0; s >>= 1) {
+        const double b2 = __shfl_down_sync(0xffffffffu, b, s);
+        const int o2 = __shfl_down_sync(0xffffffffu, o, s), k2 = __shfl_down_sync(0xffffffffu, k, s);
+        if (cfl_less(b2, o2, b, o)) { b = b2; o = o2; k = k2; }
     }
-    sb[tid] = bb; so[tid] = bo; sk[tid] = bk;
+    if (lane == 0) { sb[warp] = b; so[warp] = o; sk[warp] = k; }
     __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (tid < s && cfl_less(sb[tid + s], so[tid + s], sb[tid], so[tid])) {
-            sb[tid] = sb[tid + s]; so[tid] = so[tid + s]; sk[tid] = sk[tid + s];
-        }
-        __syncthreads();
-    }
-    if (tid == 0) { part_b[blockIdx.x] = sb[0]; part_o[blockIdx.x] = so[0]; part_k[blockIdx.x] = sk[0]; }
+    if (threadIdx.x == 0)
+        for (int w = 1; w < kRedThreads / 32; w++)
+            if (cfl_less(sb[w], so[w], b, o)) { b = sb[w]; o = so[w]; k = sk[w]; }
 }
 
-// dt-bar's face: one thread reduces the parts, finds the face f* of the chosen
-// cell and adds the wave-speed adjoint's contribution to both sides' face slots.
-__global__ void adj_cfl_face_kernel(AdjMesh m, const double *FV, int nparts, const double *part_b,
-                                    const int *part_o, const int *part_k, const double *dtbar, double cfl,
-                                    double dt_max, double *FVb, double *zfb)
+__global__ void __launch_bounds__(kRedThreads) adj_cfl_part_kernel(int nc, const double *bound, const int32_t *orig,
+                                                                   double *part_b, int *part_o, int *part_k)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+    double bb = INFINITY;
+    int bo = 0x7fffffff, bk = -1;
+    for (int K = blockIdx.x * blockDim.x + threadIdx.x; K < nc; K += gridDim.x * blockDim.x) {
+        const double b = bound[K];                       // +inf where nothing moves
+        if (b <= bb && b < INFINITY && cfl_less(b, orig[K], bb, bo)) { bb = b; bo = orig[K]; bk = K; }
+    }
+    cta_argmin(bb, bo, bk);
+    if (threadIdx.x == 0) { part_b[blockIdx.x] = bb; part_o[blockIdx.x] = bo; part_k[blockIdx.x] = bk; }
+}
+
+// dt-bar's face: one CTA reduces the parts, three threads form the speeds of the
+// chosen cell's faces, one finds f* (the first of largest l_f a_f) and adds the
+// wave-speed adjoint's contribution to both sides' face slots.  (One thread
+// walking the parts and the faces took 99 us.)
+__global__ void __launch_bounds__(kRedThreads) adj_cfl_face_kernel(AdjMesh m, const double *FV, int nparts,
+                                    const double *part_b, const int *part_o, const int *part_k, const double *dtbar,
+                                    double cfl, double dt_max, double *FVb, double *zfb)
+{
+    __shared__ double s_a[3], s_la[3];
+    __shared__ int s_k;
     double bb = INFINITY;
     int bo = 0x7fffffff, K = -1;
-    for (int q = 0; q < nparts; q++)
+    for (int q = threadIdx.x; q < nparts; q += blockDim.x)
         if (part_k[q] >= 0 && cfl_less(part_b[q], part_o[q], bb, bo)) { bb = part_b[q]; bo = part_o[q]; K = part_k[q]; }
+    cta_argmin(bb, bo, K);
+    if (threadIdx.x == 0) s_k = K;
+    __syncthreads();
+    K = s_k;
     if (K < 0) return;                                   // nothing moves: dt = dt_max or 0
+    if (threadIdx.x < 3) {
+        const FaceIn q = face_in(m, FV, K, threadIdx.x);
+        const double a = face_speed(m, q.HfL, q.HufL, q.HvfL, q.zL, q.HfR, q.HufR, q.HvfR, q.zR, q.nx, q.ny, q.wall,
+                                    q.bnd);
+        s_a[threadIdx.x] = a;
+        s_la[threadIdx.x] = q.l * a;
+    }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
     const double dtc = cfl * bb;
     if (dt_max > 0.0 && dt_max < dtc) return;            // clamped by dt_max: no dependence
-    int f;
-    cell_speed(m, FV, K, f);
+    int f = 0;
+    for (int k = 1; k < 3; k++)
+        if (gt_nn(s_la[k], s_la[f])) f = k;
     const FaceIn q = face_in(m, FV, K, f);
-    const double a = face_speed(m, q.HfL, q.HufL, q.HvfL, q.zL, q.HfR, q.HufR, q.HvfR, q.zR, q.nx, q.ny, q.wall,
-                                q.bnd);
-    const double ab = -(*dtbar) * dtc / a;
+    const double ab = -(*dtbar) * dtc / s_a[f];
     const double P0[3] = {0.0, 0.0, 0.0};
     double bL[4], bR[4];
     flux_vjp(m, q.HfL, q.HufL, q.HvfL, q.zL, q.HfR, q.HufR, q.HvfR, q.zR, q.nx, q.ny, q.wall, P0, 0.0, 0.0, bL, bR, ab,
@@ -840,30 +853,36 @@ __global__ void adj_cfl_face_kernel(AdjMesh m, const double *FV, int nparts, con
     }
 }
 
-// Deterministic dot product: per-CTA partial sums, then one thread adds them in
-// order, times scale, into *acc (reset: replaces it).
-__global__ void adj_dot_part_kernel(int64_t n, const double *a, const double *b, double *part)
+// Deterministic dot product: per-CTA partial sums, then one CTA adds them, times
+// scale, into *acc (reset: replaces it).  Both sums have a fixed order: a warp's
+// shuffle tree, then the warps in turn.  (One thread adding 1024 partial sums
+// was 58 us of dependent FP64 adds.)
+__device__ __forceinline__ double cta_sum(double s)
 {
-    __shared__ double sh[256];
-    const int tid = threadIdx.x;
-    double s = 0.0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + tid; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        s += a[i] * b[i];
-    sh[tid] = s;
+    __shared__ double sh[kRedThreads / 32];
+    for (int k = 16; k > 0; k >>= 1) s += __shfl_down_sync(0xffffffffu, s, k);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
     __syncthreads();
-    for (int k = blockDim.x / 2; k > 0; k >>= 1) {
-        if (tid < k) sh[tid] += sh[tid + k];
-        __syncthreads();
-    }
-    if (tid == 0) part[blockIdx.x] = sh[0];
+    if (threadIdx.x == 0)
+        for (int w = 1; w < kRedThreads / 32; w++) s += sh[w];
+    return s;                                            // thread 0's is the sum
 }
 
-__global__ void adj_dot_final_kernel(int nparts, const double *part, double scale, double *acc, int reset)
+__global__ void __launch_bounds__(kRedThreads) adj_dot_part_kernel(int64_t n, const double *a, const double *b, double *part)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
     double s = 0.0;
-    for (int q = 0; q < nparts; q++) s += part[q];
-    *acc = reset ? s * scale : *acc + s * scale;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        s += a[i] * b[i];
+    s = cta_sum(s);
+    if (threadIdx.x == 0) part[blockIdx.x] = s;
+}
+
+__global__ void __launch_bounds__(kRedThreads) adj_dot_final_kernel(int nparts, const double *part, double scale, double *acc, int reset)
+{
+    double s = 0.0;
+    for (int q = threadIdx.x; q < nparts; q += blockDim.x) s += part[q];
+    s = cta_sum(s);
+    if (threadIdx.x == 0) *acc = reset ? s * scale : *acc + s * scale;
 }
 
 // ---------------------------------------------------------------------------
@@ -877,14 +896,12 @@ __global__ void adj_dot_final_kernel(int nparts, const double *part, double scal
 //   t-bar_n = sum_v s_v uplift_v R'      (R' = dR/dt = 1 / rise inside the ramp),
 // the last summed per CTA into part (adaptive steps carry it to every earlier dt).
 // ---------------------------------------------------------------------------
-__global__ void adj_bed_vertex_kernel(int nv, int ncs, const int32_t *vptr, const int32_t *vcell, const double *zs,
+__global__ void __launch_bounds__(kRedThreads) adj_bed_vertex_kernel(int nv, int ncs, const int32_t *vptr, const int32_t *vcell, const double *zs,
                                       const double *uplift, const double *onset, double rise, double t, double *gU,
                                       double *gOn, double *part)
 {
-    __shared__ double sh[256];
-    const int tid = threadIdx.x;
     double tb = 0.0;
-    for (int v = blockIdx.x * blockDim.x + tid; v < nv; v += gridDim.x * blockDim.x) {
+    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < nv; v += gridDim.x * blockDim.x) {
         double sv = 0.0;
         for (int k = vptr[v]; k < vptr[v + 1]; k++) {
             const int K = vcell[k] >> 2, j = vcell[k] & 3;
@@ -904,13 +921,8 @@ __global__ void adj_bed_vertex_kernel(int nv, int ncs, const int32_t *vptr, cons
         gOn[v] -= q;
         tb += q;
     }
-    sh[tid] = tb;
-    __syncthreads();
-    for (int k = blockDim.x / 2; k > 0; k >>= 1) {
-        if (tid < k) sh[tid] += sh[tid + k];
-        __syncthreads();
-    }
-    if (tid == 0) part[blockIdx.x] = sh[0];
+    tb = cta_sum(tb);
+    if (threadIdx.x == 0) part[blockIdx.x] = tb;
 }
 
 __global__ void adj_axpy_kernel(int64_t n, const double *x, double *y)
@@ -924,6 +936,13 @@ __global__ void adj_scalar_add_kernel(double *y, const double *x)
     if (threadIdx.x == 0 && blockIdx.x == 0) *y += *x;
 }
 
+// CTAs of a reduction over n values: at least four values a thread, at most
+// kAdjCflParts parts.
+int grid_red(int64_t n)
+{
+    const int64_t g = (n + 4 * kRedThreads - 1) / (4 * kRedThreads);
+    return (int)(g < 1 ? 1 : g < kAdjCflParts ? g : kAdjCflParts);
+}
 int grid_of(int n) { return (n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096; }
 // The two heavy reverse kernels run 128-thread CTAs: at 110 / 146 registers a
 // thread that fits 4 / 3 CTAs per SM (16 / 12 warps) where 256-thread CTAs fit
@@ -968,8 +987,10 @@ int adjoint_residual_vjp(const DevPtrs &d, const StepParams &p, const double *w,
     if (!m.faces) return (int)cudaErrorInvalidValue;     // the face list is built by vg_adj_backward
     adj_flux_vjp_kernel<<<grid_vjp(m.nfaces), kVjpThreads, 0, s>>>(m, FV, Rb, FVb, zfb);
     if (cfl) {
-        adj_cfl_part_kernel<<<kAdjCflParts, 256, 0, s>>>(m, FV, cfl->orig, cfl->part_b, cfl->part_o, cfl->part_k);
-        adj_cfl_face_kernel<<<1, 32, 0, s>>>(m, FV, kAdjCflParts, cfl->part_b, cfl->part_o, cfl->part_k, cfl->dtbar,
+        const int parts = grid_red(m.nc);
+        adj_cfl_part_kernel<<<parts, kRedThreads, 0, s>>>(m.nc, cfl->bound, cfl->orig, cfl->part_b, cfl->part_o,
+                                                          cfl->part_k);
+        adj_cfl_face_kernel<<<1, kRedThreads, 0, s>>>(m, FV, parts, cfl->part_b, cfl->part_o, cfl->part_k, cfl->dtbar,
                                              cfl->cfl, cfl->dt_max, FVb, zfb);
     }
     adj_recon_vjp_kernel<<<grid_vjp(m.nc), kVjpThreads, 0, s>>>(m, w, Rb, FVb, zfb, own, send);
@@ -1004,8 +1025,9 @@ int adjoint_dot(int64_t n, const double *a, const double *b, double scale, doubl
                 void *stream)
 {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    adj_dot_part_kernel<<<kAdjCflParts, 256, 0, s>>>(n, a, b, part);
-    adj_dot_final_kernel<<<1, 32, 0, s>>>(kAdjCflParts, part, scale, acc, reset ? 1 : 0);
+    const int parts = grid_red(n);
+    adj_dot_part_kernel<<<parts, kRedThreads, 0, s>>>(n, a, b, part);
+    adj_dot_final_kernel<<<1, kRedThreads, 0, s>>>(parts, part, scale, acc, reset ? 1 : 0);
     return (int)cudaGetLastError();
 }
 
@@ -1014,8 +1036,9 @@ int adjoint_bed_flush(int nc, int nv, const int32_t *vptr, const int32_t *vcell,
                       double *tsum, double *part, void *stream)
 {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    adj_bed_vertex_kernel<<<kAdjCflParts, 256, 0, s>>>(nv, nc, vptr, vcell, zs, uplift, onset, rise, t, gU, gOn, part);
-    adj_dot_final_kernel<<<1, 32, 0, s>>>(kAdjCflParts, part, 1.0, tsum, 0);
+    const int parts = grid_red(nv);
+    adj_bed_vertex_kernel<<<parts, kRedThreads, 0, s>>>(nv, nc, vptr, vcell, zs, uplift, onset, rise, t, gU, gOn, part);
+    adj_dot_final_kernel<<<1, kRedThreads, 0, s>>>(parts, part, 1.0, tsum, 0);
     adj_axpy_kernel<<<grid_of(4 * nc), 256, 0, s>>>(4 * (int64_t)nc, zs, zb_total);
     return (int)cudaGetLastError();
 }
@@ -1026,10 +1049,9 @@ int adjoint_scalar_add(double *y, const double *x, void *stream)
     return (int)cudaGetLastError();
 }
 
-int adjoint_gauge(int n_gauges, const int32_t *cells, const double *weights, int nc, double *wb, double *zb,
-                  void *stream)
+int adjoint_gauge(int n_gauges, const int32_t *cells, const double *weights, double *wb, double *zb, void *stream)
 {
-    adj_gauge_kernel<<<1, 32, 0, static_cast<cudaStream_t>(stream)>>>(n_gauges, cells, weights, nc, wb, zb);
+    adj_gauge_kernel<<<(n_gauges + 63) / 64, 64, 0, static_cast<cudaStream_t>(stream)>>>(n_gauges, cells, weights, wb, zb);
     return (int)cudaGetLastError();
 }
 

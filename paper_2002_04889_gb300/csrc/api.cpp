@@ -1262,7 +1262,7 @@ int vg_adj_forward(vg_ctx *c, int64_t n_steps, double dt, int64_t checkpoint_eve
     // worth of recordings (per cell: face values of both stages, the segment state,
     // R0, R1 with CFL steps, flag bits) plus n_steps / C checkpoints of 24 bytes
     // each; every segment is recomputed once whatever C is
-    const double rec_bytes = 8.0 * (18 + 3 + 3 + (dt > 0.0 ? 0 : 3)) + 3.0 / 8.0, ckpt_bytes = 24.0;
+    const double rec_bytes = 8.0 * (18 + 3 + 3 + (dt > 0.0 ? 0 : 4)) + 3.0 / 8.0, ckpt_bytes = 24.0;
     int64_t C = checkpoint_every ? checkpoint_every
                                  : std::max<int64_t>(1, std::llround(std::sqrt((double)n_steps * ckpt_bytes / rec_bytes)));
     int64_t nck = (n_steps + C - 1) / C;
@@ -1397,7 +1397,8 @@ int vg_adj_backward(vg_ctx *c, const double *dJ_deta, double *dJ_dH0, double *dJ
     double *recraw;  // reconstruction flags of both stages of every recorded step [RC][2][nc] (bytes)
     double *FVseg;   // face values of both stages of every step of the segment [C][2][9][nc]
     const bool adaptive = !(c->adj_dt > 0.0);
-    double *R1seg = nullptr, *cflscr = nullptr;   // adaptive steps: stage-2 residuals; dt-bar and reduction scratch
+    double *R1seg = nullptr, *cflscr = nullptr, *bndseg = nullptr;   // adaptive steps: stage-2 residuals; dt-bar and
+                                                                     // reduction scratch; the cells' CFL bounds
     int rc = 0;
     if ((rc = alloc((size_t)(N + 1) * G, &W)) || (rc = alloc(w3, &wb)) || (rc = alloc(w3, &wbn)) ||
         (rc = alloc(w3, &wb1)) || (rc = alloc(4 * (size_t)nc, &zb)) || (rc = alloc(w3, &Rb)) || (rc = alloc(w3, &wlast)) ||
@@ -1407,7 +1408,8 @@ int vg_adj_backward(vg_ctx *c, const double *dJ_deta, double *dJ_dH0, double *dJ
         (rc = alloc(w3 * (size_t)(binomial ? 2 + c->adj_slots : C), &seg)) ||
         (rc = alloc(w3 * (size_t)RC, &R0seg)) || (rc = alloc(((size_t)nc * RC + 7) / 8, &m2raw)) ||
         (rc = alloc((2 * (size_t)nc * RC + 7) / 8, &recraw)) ||
-        (adaptive && ((rc = alloc(w3 * (size_t)RC, &R1seg)) || (rc = alloc(8 + 3 * (size_t)kAdjCflParts, &cflscr))))) {
+        (adaptive && ((rc = alloc(w3 * (size_t)RC, &R1seg)) || (rc = alloc((size_t)nc * RC, &bndseg)) ||
+                      (rc = alloc(8 + 3 * (size_t)kAdjCflParts, &cflscr))))) {
         for (void *q : bufs) cudaFree(q);
         return rc;
     }
@@ -1505,7 +1507,7 @@ int vg_adj_backward(vg_ctx *c, const double *dJ_deta, double *dJ_dH0, double *dJ
         VG_CUDA(c, cudaMemsetAsync(zb, 0, 8 * 4 * (size_t)nc, c->stream));
         zacc = bed ? zstep : zb;
         if (bed) VG_CUDA(c, cudaMemsetAsync(zstep, 0, 8 * 4 * (size_t)nc, c->stream));
-        ADJ_CHECK(adjoint_gauge(G, c->gauge_cells, W + (size_t)N * G, nc, wb, zacc, st));
+        ADJ_CHECK(adjoint_gauge(G, c->gauge_cells, W + (size_t)N * G, wb, zacc, st));
         if (bed)
             ADJ_CHECK(adjoint_bed_flush(nc, nv, vptr, vcell, zstep, c->bed_uplift, c->bed_onset, c->bed_rise, tn[N],
                                         gU, gOn, zb, tsum, bedpart, st));
@@ -1522,6 +1524,7 @@ int vg_adj_backward(vg_ctx *c, const double *dJ_deta, double *dJ_dH0, double *dJ
             pn.dt_fixed = c->adj_dts[n];        // the step the forward run took
             int e;
             if (bed && (e = launch_bed_update(d, p, nullptr, 64, false, tn[n], st))) return e;   // bed of step n
+            if (adaptive) dd.bound_out = bndseg + (size_t)r * nc;
             if ((e = launch_stage1_f64(dd, pn, win, lc1, st))) return e;
             dd.fv_out = FVseg + ((size_t)r * 18 + 9) * nc;
             dd.rec_out = recseg + ((size_t)r * 2 + 1) * nc;
@@ -1563,10 +1566,11 @@ int vg_adj_backward(vg_ctx *c, const double *dJ_deta, double *dJ_dH0, double *dJ
             if (adaptive && (e = adjoint_dot((int64_t)w3, Rb, R0, 1.0 / dtn, dtbar, false, dotpart, st))) return e;
             // a moving bed: every later bed depends on this dt through the time
             if (adaptive && bed && (e = adjoint_scalar_add(dtbar, tsum, st))) return e;
+            cfl.bound = adaptive ? bndseg + (size_t)r * nc : nullptr;
             if ((e = adjoint_residual_vjp(d, p, w, rec0, Rb, wbn, zacc, FV0, true, FVb, zfb, own, send, st,
                                           adaptive ? &cfl : nullptr)))
                 return e;
-            if ((e = adjoint_gauge(G, c->gauge_cells, W + (size_t)n * G, nc, wbn, zacc, st))) return e;
+            if ((e = adjoint_gauge(G, c->gauge_cells, W + (size_t)n * G, wbn, zacc, st))) return e;
             if (bed && (e = adjoint_bed_flush(nc, nv, vptr, vcell, zstep, c->bed_uplift, c->bed_onset, c->bed_rise,
                                               tn[n], gU, gOn, zb, tsum, bedpart, st)))
                 return e;

@@ -77,6 +77,7 @@ struct KArgs {
     real *fv_out;           // optional [3 vars][3 faces][nc]: face values of the block cells
     real *r1_out;           // optional [3][nc]: the stage-2 residual L(w1) (stage 2)
     uint8_t *rec_out;       // optional [nc]: 1 where the block cell reconstructed (FP64)
+    double *bound_out;      // optional [nc]: the stage-1 CFL bound of each cell, +inf where nothing moves (FP64)
     DevScalars *sc;
     real g, half_g, hthr;
     double cfl, dt_fixed, dt_max, t_end;
@@ -520,7 +521,10 @@ __device__ __forceinline__ void finish_cell(const KArgs<real> &a, int gid, const
         a.R0[gid] = RH;
         a.R0[nc + gid] = RHu;
         a.R0[2 * nc + gid] = RHv;
-        if (is_pos(am)) my_min = smin(my_min, area / (real(3) * am));
+        const real bnd = is_pos(am) ? area / (real(3) * am) : real_inf<real>();
+        my_min = smin(my_min, bnd);
+        if constexpr (!ETA)
+            if (a.bound_out) a.bound_out[gid] = bnd;
     } else {
         if (a.r1_out) {
             a.r1_out[gid] = RH;
@@ -1322,6 +1326,7 @@ KArgs<real> make_args(const DevPtrs &d, const StepParams &p, const void *w_in, v
     a.fv_out = static_cast<real *>(d.fv_out);
     a.r1_out = static_cast<real *>(d.r1_out);
     a.rec_out = d.rec_out;
+    a.bound_out = d.bound_out;
     a.sc = d.sc;
     a.g = (real)p.g;
     a.half_g = (real)(0.5 * p.g);

@@ -127,6 +127,7 @@ struct DevPtrs {
     uint8_t *mask2;         // optional [nc]: stage-2 dry-fix branch per cell (adjoint)
     void *fv_out;           // optional [9][nc]: face values written by the stage kernels (adjoint)
     void *r1_out;           // optional [3][nc]: stage-2 residual written by the stage-2 kernel (adjoint)
+    double *bound_out;      // optional [nc]: each cell's CFL bound written by the FP64 stage-1 kernel (adjoint)
     uint8_t *rec_out;       // optional [nc]: 1 where a cell reconstructed (its face values stand on
                             // the face beds), written by the stage kernels (adjoint)
     DevScalars *sc;
@@ -194,11 +195,13 @@ int launch_batch_step_f64(const void *table, int n_mesh, int n_items, int n_entr
 
 // Discrete adjoint (adjoint_f64.cu, FP64 contexts).
 // The CFL time step's dependence on the state (adaptive steps): orig = original
-// cell ids [nc] (argmin ties), *dtbar = the step's dt adjoint, cfl / dt_max as in
-// the forward run, part_* scratch of kAdjCflParts entries.
+// cell ids [nc] (argmin ties), bound = the CFL bound of every cell [nc] recorded by
+// the forward stage-1 kernel, *dtbar = the step's dt adjoint, cfl / dt_max as in the
+// forward run, part_* scratch of kAdjCflParts entries.
 constexpr int kAdjCflParts = 1024;
 struct AdjCfl {
     const int32_t *orig;
+    const double *bound;
     const double *dtbar;
     double cfl, dt_max;
     double *part_b;
@@ -232,8 +235,7 @@ int adjoint_stage2_rev(int nc, double dt, const uint8_t *mask2, const double *wb
                        double *Rb, void *stream);
 int adjoint_stage1_rev(int nc, double dt, double hthr, const double *H1pre, const double *wb1, double *wbn,
                        double *Rb, void *stream);
-int adjoint_gauge(int n_gauges, const int32_t *cells, const double *weights, int nc, double *wb, double *zb,
-                  void *stream);
+int adjoint_gauge(int n_gauges, const int32_t *cells, const double *weights, double *wb, double *zb, void *stream);
 
 // Utility kernels (util_kernels.cu).
 int launch_post_step(const DevPtrs &d, const StepParams &p, const void *w, int precision, void *stream);

@@ -1,0 +1,40 @@
+"""Kernels at the sizes where their split of the work can go wrong, against the
+oracle or against the same call split differently."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_2002_04889_gb300 import inputs as I
+from paper_2002_04889_gb300 import volna
+
+pytestmark = pytest.mark.gpu
+
+
+def _moving_basin(n, half_width=1.0):
+    m = I.thacker_mesh(n=n, half_width=half_width)
+    s = I.thacker_initial_state(m)
+    p = m.cell_points()
+    deep = s.H > 2e-2
+    return m, (s.H, s.Hu + 1e-3 * np.sin(3 * p[:, 0]) * deep, s.Hv + 1e-3 * np.cos(2 * p[:, 1]) * deep)
+
+
+@pytest.mark.parametrize("n,n_gauges", [(7, 1), (16, 64), (16, 65), (33, 70)])
+def test_adjoint_reductions_and_shared_gauge_cells(n, n_gauges):
+    """CFL steps (argmin of the recorded bounds over one and several CTAs, the dot
+    products of dt-bar) and gauges that share cells, one to two CTAs of gauges,
+    against the oracle's taped adjoint.  FP64 sums in another order: 1e-10."""
+    m, st = _moving_basin(n)
+    pts = np.array([[0.0, 0.0], [0.31, -0.12], [-0.2, 0.23]])[np.arange(n_gauges) % 3]
+    cells = O.OracleMesh.from_mesh(m).locate(pts)
+    W = np.random.default_rng(n).normal(size=(7, n_gauges))
+    with volna.Solver(64) as sv:
+        sv.set_params(h_threshold=1e-5, cfl=0.9)
+        sv.upload_mesh(m)
+        sv.set_gauges(pts)
+        sv.set_state(*st, 0.0)
+        sv.adj_forward(6, 0.0)
+        g = sv.adj_backward(W, m.nv)
+    ad = O.ad_gauge_gradient(m, st, 0.0, 6, cells, W, h_threshold=1e-5, cfl=0.9)
+    for k in ("H0", "Hu0", "Hv0", "depth"):
+        b = ad["d" + k]
+        assert np.linalg.norm(g[k] - b) <= 1e-10 * np.linalg.norm(b), k
