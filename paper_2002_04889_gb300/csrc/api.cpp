@@ -42,6 +42,7 @@ struct vg_ctx {
     void *geo = nullptr, *z = nullptr, *w[2] = {nullptr, nullptr}, *R0 = nullptr;
     void *zf = nullptr;               // face beds (layout: DevPtrs::zf)
     void *rk_w1 = nullptr, *rk_R1 = nullptr;   // [3][nc] each: w1 and R(w1) of the unfused RK stages
+    double *rarea = nullptr;          // FP64: 1 / area of every cell
     double *z64 = nullptr;
     float *z_orig = nullptr;          // FP32: the bed in the original cell order (state import/export)
     double *z64_orig = nullptr;
@@ -151,7 +152,7 @@ void free_mesh(vg_ctx *c)
     free_adjoint(c);
     if (c->graph2) { cudaGraphExecDestroy(c->graph2); c->graph2 = nullptr; }
     if (c->z64 == c->z) c->z64 = nullptr;
-    dfree(c->geo); dfree(c->z); dfree(c->zf); dfree(c->z64); dfree(c->w[0]); dfree(c->w[1]); dfree(c->R0);
+    dfree(c->geo); dfree(c->rarea); dfree(c->z); dfree(c->zf); dfree(c->z64); dfree(c->w[0]); dfree(c->w[1]); dfree(c->R0);
     dfree(c->rk_w1); dfree(c->rk_R1);
     dfree(c->z_orig); dfree(c->z64_orig); c->zorig_ok = false;
     dfree(c->nbr); dfree(c->halo_ptr); dfree(c->halo_n1); dfree(c->halo_ids); dfree(c->ring1_nbr);
@@ -192,6 +193,7 @@ DevPtrs dev_ptrs(const vg_ctx *c)
     d.n_gauges = c->n_gauges;
     d.ring_cap = kRingCap;
     d.geo = c->geo;
+    d.rarea = c->rarea;
     d.z = c->z;
     d.zf = c->zf;
     d.z64 = c->z64;
@@ -354,6 +356,12 @@ int upload_mesh_arrays(vg_ctx *c)
             }
         }
         VG_CUDA(c, cudaMemcpy(c->geo, r.data(), 4 * r.size(), cudaMemcpyHostToDevice));
+    }
+    if (c->precision == 64) {
+        std::vector<double> ra(m.nc);
+        for (int64_t k = 0; k < m.nc; k++) ra[k] = 1.0 / m.geo[(size_t)GEO_AREA * m.nc + k];
+        if ((rc = dmalloc(c, (void **)&c->rarea, 8 * m.nc))) return rc;
+        VG_CUDA(c, cudaMemcpy(c->rarea, ra.data(), 8 * m.nc, cudaMemcpyHostToDevice));
     }
     if ((rc = upload_real(c, c->z, m.z.data(), m.z.size()))) return rc;
     if ((rc = upload_face_beds(c))) return rc;

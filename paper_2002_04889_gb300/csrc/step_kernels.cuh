@@ -34,9 +34,9 @@
 //    one (FAST = false, step_f64.cu, no multiply-add contraction) evaluates every
 //    formula as written, in the same order as any plain implementation of the
 //    scheme; the fast one (FAST = true, step_f64_fast.cu, contraction allowed)
-//    divides once where the literal form divides several times by the same value
-//    (face velocities, the HLL star flux, the residual's 1/|K|) and finds the
-//    limiter's smallest ratio by cross products with one division.
+//    multiplies by one reciprocal where the literal form forms several correctly
+//    rounded quotients by the same value (face velocities, the HLL star flux, the
+//    residual's 1/|K|).
 //  * FP32 ("deviation"): the state is (eta, Hu, Hv) with eta = H + z, and the
 //    momentum flux through each face is carried relative to the hydrostatic
 //    pressure g (eta_K - z_{K,f})^2 / 2 of the cell's own free surface over the
@@ -51,6 +51,7 @@
 #include <cuda_runtime.h>
 #include <math_constants.h>
 
+#include "exact_div.cuh"
 #include "vg_internal.h"
 
 namespace vg {
@@ -60,6 +61,7 @@ struct KArgs {
     int64_t nc;
     int block, nblocks, max_halo, max_ring1, order;
     const real *geo;        // [GEO_ROWS][nc]
+    const double *rarea;    // [nc] 1 / area (FP64)
     const real *z;          // [nc]
     const real *zf;         // face beds: FP64 [3][nc]; FP32 [nc][2] z_f - z_K of faces 0, 1
     const int32_t *nbr;     // [3][nc]
@@ -177,8 +179,10 @@ __device__ __forceinline__ void hll_normal(real g, real half_g, real HL, real un
         sL = unL - cL;
         sR = unL + real(2) * cL;
     } else {
-        real us = real(0.5) * (unL + unR) + (cL - cR);
-        real cs = real(0.5) * (cL + cR) - real(0.25) * (unR - unL);
+        // u* = (u_L + u_R) / 2 + (c_L - c_R), c* = (c_L + c_R) / 2 - (u_R - u_L) / 4
+        // (halving commutes with rounding: each difference is rounded once as written)
+        real us = half_of(unL + unR) + (cL - cR);
+        real cs = half_of((cL + cR) - half_of(unR - unL));
         sL = smin(unL - cL, us - cs);
         sR = smax(us + cs, unR + cR);
     }
@@ -190,15 +194,15 @@ __device__ __forceinline__ void hll_normal(real g, real half_g, real HL, real un
     } else if (!is_neg(sR)) {
         real den = sR - sL;
         real sLR = sL * sR;
+        const Recip rd = recip(den);
+        const real N0 = (sR * FL0 - sL * FR0) + sLR * (HR - HL);
+        const real N1 = (sR * FL1 - sL * FR1) + sLR * (qR - qL);
+        const real N2 = (sR * FL2 - sL * FR2) + sLR * (HR * utR - HL * utL);
         if constexpr (FAST) {
-            const real rd = real(1) / den;
-            F[0] = ((sR * FL0 - sL * FR0) + sLR * (HR - HL)) * rd;
-            F[1] = ((sR * FL1 - sL * FR1) + sLR * (qR - qL)) * rd;
-            F[2] = ((sR * FL2 - sL * FR2) + sLR * (HR * utR - HL * utL)) * rd;
+            const real r = inverse(rd);
+            F[0] = N0 * r; F[1] = N1 * r; F[2] = N2 * r;
         } else {
-            F[0] = ((sR * FL0 - sL * FR0) + sLR * (HR - HL)) / den;
-            F[1] = ((sR * FL1 - sL * FR1) + sLR * (qR - qL)) / den;
-            F[2] = ((sR * FL2 - sL * FR2) + sLR * (HR * utR - HL * utL)) / den;
+            F[0] = quot(N0, rd); F[1] = quot(N1, rd); F[2] = quot(N2, rd);
         }
     } else {
         F[0] = FR0; F[1] = FR1; F[2] = FR2;
@@ -223,11 +227,12 @@ __device__ __forceinline__ void face_flux(real g, real half_g, real hthr,
 {
     real uL = real(0), vL = real(0);
     if (gt_nn(HfL, hthr)) {
+        const Recip rH = recip(HfL);
         if constexpr (FAST) {
-            const real r = real(1) / HfL;
+            const real r = inverse(rH);
             uL = HufL * r; vL = HvfL * r;
         } else {
-            uL = HufL / HfL; vL = HvfL / HfL;
+            uL = quot(HufL, rH); vL = quot(HvfL, rH);
         }
     }
     real unL = uL * nx + vL * ny;
@@ -253,11 +258,12 @@ __device__ __forceinline__ void face_flux(real g, real half_g, real hthr,
     } else {
         real uR = real(0), vR = real(0);
         if (gt_nn(HfR, hthr)) {
+            const Recip rH = recip(HfR);
             if constexpr (FAST) {
-                const real r = real(1) / HfR;
+                const real r = inverse(rH);
                 uR = HufR * r; vR = HvfR * r;
             } else {
-                uR = HufR / HfR; vR = HvfR / HfR;
+                uR = quot(HufR, rH); vR = quot(HvfR, rH);
             }
         }
         unR = uR * nx + vR * ny;
@@ -483,9 +489,16 @@ __device__ __forceinline__ uint8_t rk2_final(const real x[3], real W1, real Hu1,
                                              real RHv, real dt, real z1, real hthr, real &W, real &Hu, real &Hv)
 {
     constexpr bool ETA = EtaForm<real>::value;
-    W = real(0.5) * x[0] + real(0.5) * (W1 + dt * RH);
-    Hu = real(0.5) * x[1] + real(0.5) * (Hu1 + dt * RHu);
-    Hv = real(0.5) * x[2] + real(0.5) * (Hv1 + dt * RHv);
+    if constexpr (ETA) {
+        W = real(0.5) * x[0] + real(0.5) * (W1 + dt * RH);
+        Hu = real(0.5) * x[1] + real(0.5) * (Hu1 + dt * RHu);
+        Hv = real(0.5) * x[2] + real(0.5) * (Hv1 + dt * RHv);
+    } else {
+        // x / 2 + y / 2 rounded once is (x + y) / 2 rounded once
+        W = half_of(x[0] + (W1 + dt * RH));
+        Hu = half_of(x[1] + (Hu1 + dt * RHu));
+        Hv = half_of(x[2] + (Hv1 + dt * RHv));
+    }
     const real H = ETA ? W - z1 : W;
     if (is_neg(H)) {
         W = ETA ? z1 : real(0);
@@ -505,23 +518,29 @@ __device__ __forceinline__ uint8_t rk2_final(const real x[3], real W1, real Hu1,
 // w^n = x, w1 from shared memory, and the dry fix.
 template <typename real, int STAGE, bool FAST = false>
 __device__ __forceinline__ void finish_cell(const KArgs<real> &a, int gid, const real *sWl, real aH, real aHu,
-                                            real aHv, real am, const real x[3], real area, real dt, real &my_min,
-                                            long long &my_neg, bool &bad)
+                                            real aHv, real am, const real x[3], real area, real rarea, real dt,
+                                            real &my_min, long long &my_neg, bool &bad)
 {
     constexpr bool ETA = EtaForm<real>::value;
     const int nc = (int)a.nc;
     real RH, RHu, RHv;
-    if constexpr (FAST) {
-        const real ia = real(1) / area;
-        RH = -aH * ia; RHu = -aHu * ia; RHv = -aHv * ia;
-    } else {
+    if constexpr (ETA) {
         RH = -aH / area; RHu = -aHu / area; RHv = -aHv / area;
+    } else if constexpr (FAST) {
+        RH = -aH * rarea; RHu = -aHu * rarea; RHv = -aHv * rarea;
+    } else {
+        const Recip ra = recip_given(area, rarea);
+        RH = quot(-aH, ra); RHu = quot(-aHu, ra); RHv = quot(-aHv, ra);
     }
     if (STAGE == 1) {
         a.R0[gid] = RH;
         a.R0[nc + gid] = RHu;
         a.R0[2 * nc + gid] = RHv;
-        const real bnd = is_pos(am) ? area / (real(3) * am) : real_inf<real>();
+        real bnd = real_inf<real>();
+        if (is_pos(am)) {
+            if constexpr (ETA) bnd = area / (real(3) * am);
+            else bnd = quot(area, recip(real(3) * am));
+        }
         my_min = smin(my_min, bnd);
         if constexpr (!ETA)
             if (a.bound_out) a.bound_out[gid] = bnd;
@@ -725,8 +744,8 @@ __device__ __forceinline__ void process_block(const KArgs<real> &a, const int b,
             real x[3] = {real(0), real(0), real(0)};
             if (STAGE == 2) { x[0] = a.w[gid]; x[1] = a.w[nc + gid]; x[2] = a.w[2 * nc + gid]; }
             // R = -0 / |K| = -0 for any area, so the area is not read
-            finish_cell<real, STAGE, FAST>(a, gid, sW + 4 * tid, real(0), real(0), real(0), real(0), x, real(1), dt,
-                                     my_min, my_neg, bad);
+            finish_cell<real, STAGE, FAST>(a, gid, sW + 4 * tid, real(0), real(0), real(0), real(0), x, real(1), real(1),
+                                           dt, my_min, my_neg, bad);
         }
         return;
     }
@@ -821,40 +840,44 @@ __device__ __forceinline__ void process_block(const KArgs<real> &a, const int b,
 #pragma unroll
                     for (int f = 0; f < 3; f++) D[f] = gx * fx[f] + gy * fy[f];
                 }
-                real qmax = qK[v], qmin = qK[v];
-#pragma unroll
-                for (int f = 0; f < 3; f++) {
-                    qmax = smax(qmax, qn[f][v]);
-                    qmin = smin(qmin, qn[f][v]);
-                }
                 real alpha = real(1);
                 if constexpr (ETA) {
+                    float qmax = qK[v], qmin = qK[v];
+#pragma unroll
+                    for (int f = 0; f < 3; f++) {
+                        qmax = fmaxf(qmax, qn[f][v]);
+                        qmin = fminf(qmin, qn[f][v]);
+                    }
                     // phi_f = |r_f| / |D_f| with r_f = qmax - q_K or q_K - qmin by the
                     // sign of D_f; D_f = 0 gives +inf or NaN, which fminf ignores
                     const float up = qmax - qK[v], dn = qK[v] - qmin;
 #pragma unroll
                     for (int f = 0; f < 3; f++)
                         alpha = fminf(alpha, (D[f] > 0.f ? up : dn) * rcp_approx(fabsf(D[f])));
-                } else if constexpr (FAST) {
-                    // the smallest ratio |r_f| / |D_f| below 1 (r_f = q_max - q_K or
-                    // q_K - q_min by the sign of D_f) found by cross products; one
-                    // division, none when no face limits
-                    const real up = qmax - qK[v], dn = qK[v] - qmin;
-                    real num = real(1), den = real(1);
-#pragma unroll
-                    for (int f = 0; f < 3; f++) {
-                        const real aD = vabs(D[f]);
-                        const real r = is_pos(D[f]) ? up : dn;
-                        if (gt_nn(num * aD, r * den)) { num = r; den = aD; }   // both products >= 0
-                    }
-                    if (num != den) alpha = num / den;
                 } else {
-#pragma unroll
-                    for (int f = 0; f < 3; f++) {
-                        real phi = real(1);
-                        if (is_pos(D[f])) phi = smin(real(1), (qmax - qK[v]) / D[f]);
-                        else if (is_neg(D[f])) phi = smin(real(1), (qmin - qK[v]) / D[f]);
-                        alpha = smin(alpha, phi);
+                    // alpha = min(1, min_f r_f / D_f), r_f = q_max - q_K or q_min - q_K by
+                    // the sign of D_f.  Rounding is monotone, so q_max - q_K is the
+                    // largest of the rounded differences d_j and 0, and the smallest
+                    // quotient of a sign is that of its largest |D_f|: two candidates
+                    // up / P and dn / M, compared by cross products (rounded products
+                    // that differ order the quotients), and one division, none where
+                    // neither limits.  Nine divisions per cell become at most three.
+                    real up = max0(d0), dn = max0(-d0), P = max0(D[0]), M = max0(-D[0]);
+                    if (gt_nn(d1, up)) up = d1;
+                    if (gt_nn(d2, up)) up = d2;
+                    if (gt_nn(-d1, dn)) dn = -d1;
+                    if (gt_nn(-d2, dn)) dn = -d2;
+                    if (gt_nn(D[1], P)) P = D[1];
+                    if (gt_nn(D[2], P)) P = D[2];
+                    if (gt_nn(-D[1], M)) M = -D[1];
+                    if (gt_nn(-D[2], M)) M = -D[2];
+                    const bool limP = gt_nn(P, up), limM = gt_nn(M, dn);
+                    if (limP || limM) {
+                        const real xP = up * M, xM = dn * P;
+                        const bool takeM = limM && (!limP || gt_nn(xP, xM));
+                        const real num = takeM ? dn : up, den = takeM ? M : P;
+                        alpha = quot(num, recip(den));
+                        if (limP && limM && dbits(xP) == dbits(xM)) alpha = smin(alpha, quot(dn, recip(M)));
                     }
                 }
 #pragma unroll
@@ -955,6 +978,8 @@ __device__ __forceinline__ void process_block(const KArgs<real> &a, const int b,
         real aH = real(0), aHu = real(0), aHv = real(0), am = real(0);
         real x[3];
         const real area = ETA ? geo[(size_t)gid * G32 + G32_AREA] : geo[GEO_AREA * nc + gid];
+        real rarea = real(0);
+        if constexpr (!ETA) rarea = a.rarea[gid];
 #pragma unroll
         for (int f = 0; f < 3; f++) {
             real t0, t1, t2;
@@ -975,14 +1000,14 @@ __device__ __forceinline__ void process_block(const KArgs<real> &a, const int b,
 #pragma unroll
                 for (int f = 0; f < 3; f++) {
                     const real zff = a.zf[f * nc + gid];
-                    const real sf = g * (geo[(GEO_LEN + f) * nc + gid] * (zff * (eK - real(0.5) * zff)));
+                    const real sf = g * (geo[(GEO_LEN + f) * nc + gid] * (zff * (eK - half_of(zff))));
                     aHu = aHu + sf * geo[(GEO_NX + f) * nc + gid];
                     aHv = aHv + sf * geo[(GEO_NY + f) * nc + gid];
                 }
             }
         }
         if (STAGE == 2) { x[0] = a.w[gid]; x[1] = a.w[nc + gid]; x[2] = a.w[2 * nc + gid]; }
-        finish_cell<real, STAGE, FAST>(a, gid, sW + 4 * l, aH, aHu, aHv, am, x, area, dt, my_min, my_neg, bad);
+        finish_cell<real, STAGE, FAST>(a, gid, sW + 4 * l, aH, aHu, aHv, am, x, area, rarea, dt, my_min, my_neg, bad);
     }
 }
 
@@ -1309,6 +1334,7 @@ KArgs<real> make_args(const DevPtrs &d, const StepParams &p, const void *w_in, v
     a.max_ring1 = d.max_ring1;
     a.order = p.order;
     a.geo = static_cast<const real *>(d.geo);
+    a.rarea = d.rarea;
     a.z = static_cast<const real *>(d.z);
     a.zf = static_cast<const real *>(d.zf);
     a.nbr = d.nbr;

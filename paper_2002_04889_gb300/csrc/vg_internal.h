@@ -105,6 +105,7 @@ struct DevPtrs {
     int32_t threads;        // threads per CTA of the stage kernels (>= block)
     int32_t fp64_fast;      // FP64: launch the contracted build (step_f64_fast.cu), not the literal one
     const void *geo;        // FP64: [GEO_ROWS][nc]; FP32: [nc][16] record
+    const double *rarea;    // FP64: [nc] 1 / area, correctly rounded (FP32: null)
     const void *z;          // [nc]
     const void *zf;         // face beds: FP64 [3][nc]; FP32 [nc][2] = (z_f - z_K) of faces 0
                             // and 1 (face 2: minus their sum, the face midpoints average
