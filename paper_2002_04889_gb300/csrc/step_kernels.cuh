@@ -158,6 +158,27 @@ __device__ __forceinline__ double step_dt(const DevScalars *sc, double cfl, doub
     return dt;
 }
 
+// t_end > 0 and t >= t_end: the context has reached its end time (decided on the
+// integer units: every thread of a launch asks, and on the FP64 units the two
+// compares of an SM's 48 warps take about 1500 cycles).
+__device__ __forceinline__ bool finished(double t_end, const DevScalars *sc)
+{
+    return is_pos(t_end) && okey(sc->t) >= okey(t_end);
+}
+
+// The step's dt for every thread of a CTA, formed by one of them: a dozen FP64
+// instructions in each of an SM's 48 warps were 10,700 cycles of its FP64 units
+// (two lane-operations a cycle), 5 us a launch.  Every thread must call it.
+template <typename real>
+__device__ __forceinline__ real cta_step_dt(const DevScalars *sc, double cfl, double dt_fixed, double dt_max,
+                                            double t_end)
+{
+    __shared__ real s_dt;
+    if (threadIdx.x == 0) s_dt = (real)step_dt<real>(sc, cfl, dt_fixed, dt_max, t_end);
+    __syncthreads();
+    return s_dt;
+}
+
 // HLL flux in the face normal frame (Sec. 2.2) with the dry-bed speeds when one
 // side is dry; each side is (H*, u_n, u_t).
 template <typename real, bool FAST = false>
@@ -1046,7 +1067,7 @@ __global__ void __launch_bounds__(MAXT, StageMinCtas<real, MAXT>::value) stage_k
     // as it is: stage 1 does nothing (the CFL minimum stays empty) and stage 2
     // copies w^n to the output buffer, bit for bit (computing w/2 + (w + 0 R)/2
     // would flush the smallest FP32 values to zero), as the batched kernels do
-    if (a.t_end > 0.0 && a.sc->t >= a.t_end) {
+    if (finished(a.t_end, a.sc)) {
         if (STAGE == 2) {
             const int64_t n3 = 3 * a.nc;
             for (int64_t i = blockIdx.x * (int64_t)blockDim.x + tid; i < n3; i += (int64_t)gridDim.x * blockDim.x)
@@ -1056,7 +1077,7 @@ __global__ void __launch_bounds__(MAXT, StageMinCtas<real, MAXT>::value) stage_k
     }
 
     real dt = real(0);
-    if (STAGE == 2) dt = (real)step_dt<real>(a.sc, a.cfl, a.dt_fixed, a.dt_max, a.t_end);
+    if (STAGE == 2) dt = cta_step_dt<real>(a.sc, a.cfl, a.dt_fixed, a.dt_max, a.t_end);
 
     real my_min = real_inf<real>();
     long long my_neg = 0;
@@ -1072,7 +1093,7 @@ __global__ void __launch_bounds__(MAXT, StageMinCtas<real, MAXT>::value) stage_k
     // CTA-level reductions, then one atomic per CTA
     const int lane = tid & 31, warp = tid >> 5, nwarps = (blockDim.x + 31) >> 5;
     if (STAGE == 1) {
-        for (int o = 16; o > 0; o >>= 1) my_min = vmin(my_min, __shfl_xor_sync(0xffffffffu, my_min, o));
+        for (int o = 16; o > 0; o >>= 1) my_min = smin(my_min, __shfl_xor_sync(0xffffffffu, my_min, o));
         if (lane == 0) red_min[warp] = my_min;
     }
     for (int o = 16; o > 0; o >>= 1) my_neg += __shfl_xor_sync(0xffffffffu, my_neg, o);
@@ -1083,7 +1104,7 @@ __global__ void __launch_bounds__(MAXT, StageMinCtas<real, MAXT>::value) stage_k
         real mn = real_inf<real>();
         for (int w = 0; w < nwarps; w++) {
             neg += red_neg[w];
-            if (STAGE == 1) mn = vmin(mn, red_min[w]);
+            if (STAGE == 1) mn = smin(mn, red_min[w]);
         }
         if (STAGE == 1 && a.cfl_min && mn < real_inf<real>()) atomicMin(&a.sc->dtmin_bits, min_bits(mn));
         if (neg) atomicAdd((unsigned long long *)&a.sc->neg_count, (unsigned long long)neg);
@@ -1122,8 +1143,8 @@ __device__ __forceinline__ void cta_counts(long long my_neg, bool bad, DevScalar
 template <typename real>
 __global__ void __launch_bounds__(256) rk_update1_kernel(const KArgs<real> a, real *w1)
 {
-    if (a.t_end > 0.0 && a.sc->t >= a.t_end) return;     // finished: update 2 copies w^n
-    const real dt = (real)step_dt<real>(a.sc, a.cfl, a.dt_fixed, a.dt_max, a.t_end);
+    if (finished(a.t_end, a.sc)) return;                 // update 2 copies w^n
+    const real dt = cta_step_dt<real>(a.sc, a.cfl, a.dt_fixed, a.dt_max, a.t_end);
     const int64_t nc = a.nc;
     long long my_neg = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nc; i += (int64_t)gridDim.x * blockDim.x) {
@@ -1141,12 +1162,12 @@ template <typename real>
 __global__ void __launch_bounds__(256) rk_update2_kernel(const KArgs<real> a, const real *w1, const real *R1)
 {
     const int64_t nc = a.nc;
-    if (a.t_end > 0.0 && a.sc->t >= a.t_end) {           // as the fused kernel: w^n, bit for bit
+    if (finished(a.t_end, a.sc)) {                       // as the fused kernel: w^n, bit for bit
         for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < 3 * nc; i += (int64_t)gridDim.x * blockDim.x)
             a.wout[i] = a.w[i];
         return;
     }
-    const real dt = (real)step_dt<real>(a.sc, a.cfl, a.dt_fixed, a.dt_max, a.t_end);
+    const real dt = cta_step_dt<real>(a.sc, a.cfl, a.dt_fixed, a.dt_max, a.t_end);
     long long my_neg = 0;
     bool bad = false;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nc; i += (int64_t)gridDim.x * blockDim.x) {
@@ -1214,7 +1235,7 @@ __global__ void __launch_bounds__(256, (BatchMinCtas<real>::value)) batch_stage_
         s_dt[e] = STAGE == 2 ? (real)step_dt<real>(sc_all + e, p0.cfl, p0.dt_fixed, p0.dt_max, p0.t_end) : real(0);
         // a scenario that has reached t_end takes steps of dt = 0 that leave its
         // state as it is (as a single context's do): skip its work, copy its state
-        s_done[e] = (p0.t_end > 0.0 && sc_all[e].t >= p0.t_end) ? 1 : 0;
+        s_done[e] = finished(p0.t_end, sc_all + e) ? 1 : 0;
     }
     if (tid < 2) qcount[tid] = 0;
     __syncthreads();

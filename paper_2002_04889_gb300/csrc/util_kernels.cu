@@ -85,7 +85,11 @@ __device__ __forceinline__ double bed_ramp(double t, double onset, double rise)
 template <typename real>
 __global__ void bed_update_kernel(DevPtrs d, StepParams p, real *w, int at_step_end, double t_set)
 {
-    const double t = at_step_end ? d.sc->t + step_dt<real>(d.sc, p.cfl, p.dt_fixed, p.dt_max, p.t_end) : t_set;
+    __shared__ double s_t;           // the bed's time, formed once per CTA
+    if (threadIdx.x == 0)
+        s_t = at_step_end ? d.sc->t + step_dt<real>(d.sc, p.cfl, p.dt_fixed, p.dt_max, p.t_end) : t_set;
+    __syncthreads();
+    const double t = s_t;
     real *z = static_cast<real *>(const_cast<void *>(d.z));
     void *zf = const_cast<void *>(d.zf);
     double *z64 = const_cast<double *>(d.z64);
