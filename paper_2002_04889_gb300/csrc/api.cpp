@@ -31,6 +31,7 @@ const char *kKernelNames[kKernels] = {"stage1", "stage2", "post_step", "bed_upda
 struct vg_ctx {
     int precision = 64;
     int device = 0;
+    int sms = 1;                      // multiprocessors of the device
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     std::string err;
@@ -174,16 +175,53 @@ void free_mesh(vg_ctx *c)
 
 size_t real_size(const vg_ctx *c) { return c->precision == 64 ? 8 : 4; }
 
+// Cells and threads per block where the caller leaves both to the library.  Large
+// meshes: 256 cells, one thread each (smaller blocks reconstruct more halo cells:
+// 1M triangles, FP32 76.0 us a step against 76.6 with 128 cells, FP64 1467 against
+// 1555).  Meshes of few blocks per SM are bound by the longest chain of phases, not
+// by throughput, so they take smaller blocks and, below that, two threads per cell
+// (the ring-1 cells and the faces beyond the block's cells then share the phases'
+// first pass).  Measured, us a step, basin, against 256 cells:
+//   FP64, literal (the contracted build and FP32 keep 256 cells: their rounding
+//        depends on the partition, and a batch's scenarios equal single contexts bit
+//        for bit)
+//         2,178 and 8,450: 64 cells / 128 threads 44 against 100 and 95 (128 / 256: 59, 57)
+//        20,402: 128 / 256  55 against 95 (64 / 128: 59)
+//        49,298: 160 / 160 116 against 173 (128 / 256: 138);  99,458: 224 against 256
+//        204,800: 160 / 160 412 against 415, coast basin 436 against 427: 256 from here on
+//   FP32 20,402: 128 / 256 13.7 against 16.8;  99,458: 17.9 against 19.9;
+//        204,800: 128 cells 24.0 against 23.0 (two waves): 256 from one wave on
+struct BlockShape { int cells, threads; };
+BlockShape block_shape(const vg_ctx *c, const vg_params &p, int64_t nc)
+{
+    BlockShape s{256, 256};
+    if (p.block_cells || p.block_threads) {
+        s.cells = p.block_cells ? p.block_cells : 256;
+        s.threads = p.block_threads ? p.block_threads : s.cells;
+        return s;
+    }
+    const int64_t sms = c->sms;
+    if (c->precision == 64 && !p.fp64_literal) {
+        if (nc <= 256 * sms) s.threads = 512;                // one block per SM
+    } else if (c->precision == 64) {
+        if (nc <= 64 * sms) s = {64, 128};                   // one block of 64 per SM
+        else if (nc <= 192 * sms) s = {128, 256};            // three half-blocks per two SMs
+        else if (nc <= 4 * 256 * sms) s = {160, 160};        // fewer than four blocks of 256 per SM
+    } else if (nc <= 256 * 3 * sms) {
+        s.threads = 512;                                     // one wave of three CTAs of 512 per SM
+    }
+    return s;
+}
+
 DevPtrs dev_ptrs(const vg_ctx *c)
 {
     DevPtrs d{};
     d.nc = c->hm.nc;
     d.block = c->hm.block;
     {
-        // default: one thread per block cell.  (FP64 with two threads per cell, one
-        // CTA of 512 threads per SM, was 5-8 % slower than two CTAs of 256 that
-        // take turns at the barriers.)
-        const int t = c->prm.block_threads;
+        // one thread per block cell unless asked or chosen otherwise (a block whose
+        // shared memory did not fit has been halved)
+        const int t = block_shape(c, c->prm, c->hm.nc).threads;
         d.threads = (t >= c->hm.block && t <= 2 * c->hm.block && t <= 512) ? t : c->hm.block;
     }
     d.fp64_fast = c->precision == 64 && !c->prm.fp64_literal;
@@ -683,6 +721,7 @@ int vg_create(vg_ctx **out, int precision, int device, void *cuda_stream)
     c->device = device;
     vg_default_params(&c->prm);
     DeviceGuard guard(device);
+    if (cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || c->sms < 1) c->sms = 1;
     if (cuda_stream) {
         c->stream = (cudaStream_t)cuda_stream;
     } else {
@@ -725,7 +764,7 @@ int vg_mesh_upload(vg_ctx *c, int64_t nv, const double *xy, int64_t nc, const in
     DeviceGuard guard(c->device);
     cudaStreamSynchronize(c->stream);
     free_mesh(c);
-    int block = c->prm.block_cells ? c->prm.block_cells : 256;
+    const int block = block_shape(c, c->prm, nc).cells;
     int rc = prepare_mesh(nv, xy, nc, tri, depth_v, renumber, block, c->hm, c->err);
     if (rc) return rc;
     if ((rc = fit_blocks(c))) return rc;
@@ -769,9 +808,9 @@ int vg_set_params(vg_ctx *c, const vg_params *p)
     std::string why;
     if (validate_params(p, why)) return fail(c, VG_EINVAL, why);
     DeviceGuard guard(c->device);
-    int old_block = c->prm.block_cells ? c->prm.block_cells : 256;
-    int new_block = p->block_cells ? p->block_cells : 256;
-    bool threads_changed = p->block_threads != c->prm.block_threads || p->fp64_literal != c->prm.fp64_literal;
+    const BlockShape old_shape = block_shape(c, c->prm, c->hm.nc), new_shape = block_shape(c, *p, c->hm.nc);
+    const int old_block = old_shape.cells, new_block = new_shape.cells;
+    bool threads_changed = new_shape.threads != old_shape.threads || p->fp64_literal != c->prm.fp64_literal;
     c->prm = *p;
     c->graph_dirty = true;
     if (c->has_mesh && threads_changed && new_block == old_block) {

@@ -108,6 +108,15 @@ void scalars_init(const vg_batch *b, DevScalars &s, double t)
     }
 }
 
+// The parameters of a batch's internal contexts: its meshes share one block size
+// (one launch serves them all), so the choice by mesh size is not left to them.
+vg_params mesh_params(const vg_params &p)
+{
+    vg_params q = p;
+    if (!q.block_cells) q.block_cells = 256;
+    return q;
+}
+
 int entry_of(vg_batch *b, int32_t mesh, int32_t scen, int &e)
 {
     if (mesh < 0 || mesh >= (int)b->meshes.size()) return bfail(b, VG_EINVAL, "no such mesh");
@@ -414,7 +423,8 @@ int vg_batch_set_params(vg_batch *b, const vg_params *p)
     if (!b || !p) return VG_EINVAL;
     DeviceGuard guard(b->device);
     for (auto &M : b->meshes) {
-        int rc = vg_set_params(M.ctx, p);
+        const vg_params q = mesh_params(*p);
+        int rc = vg_set_params(M.ctx, &q);
         if (rc) return bfail(b, rc, vg_last_error(M.ctx));
     }
     b->prm = *p;
@@ -432,7 +442,8 @@ int vg_batch_add_mesh(vg_batch *b, int64_t nv, const double *xy, int64_t nc, con
     vg_batch::Mesh M;
     int rc = vg_create(&M.ctx, b->precision, b->device, (void *)b->stream);
     if (rc) return bfail(b, rc, "internal context creation failed");
-    if ((rc = vg_set_params(M.ctx, &b->prm)) || (rc = vg_mesh_upload(M.ctx, nv, xy, nc, tri, depth_v, renumber))) {
+    const vg_params mp = mesh_params(b->prm);
+    if ((rc = vg_set_params(M.ctx, &mp)) || (rc = vg_mesh_upload(M.ctx, nv, xy, nc, tri, depth_v, renumber))) {
         std::string msg = vg_last_error(M.ctx);
         vg_destroy(M.ctx);
         return bfail(b, rc, msg);

@@ -38,3 +38,27 @@ def test_adjoint_reductions_and_shared_gauge_cells(n, n_gauges):
     for k in ("H0", "Hu0", "Hv0", "depth"):
         b = ad["d" + k]
         assert np.linalg.norm(g[k] - b) <= 1e-10 * np.linalg.norm(b), k
+
+
+@pytest.mark.parametrize("precision,n", [(64, 7), (64, 69), (64, 70), (64, 120), (64, 121), (64, 279), (32, 9), (32, 241), (32, 242)])
+def test_block_shape_by_mesh_size(precision, n):
+    """The block shape that the library chooses on both sides of each size at which it
+    changes: FP64 equal bit for bit to blocks of 256 (the result does not depend on
+    the partition), FP32 within its parity bound 1e-4 of FP64."""
+    m = I.thacker_mesh(n=n, half_width=0.02 * n, h0=0.002 * n, alpha=0.02 * n, r0=0.016 * n, shuffle_cells=True)
+    s = I.thacker_initial_state(m)
+    p = m.cell_points() / (0.02 * n)
+    st = (s.H, 0.1 * s.H * np.sin(3 * p[:, 0]), 0.1 * s.H * np.cos(2 * p[:, 1]))
+    out = []
+    for prec, kw in ((precision, {}), (64, dict(block_cells=256))):
+        with volna.Solver(prec) as sv:
+            sv.set_params(h_threshold=1e-5, cfl=0.9, **kw)
+            sv.upload_mesh(m)
+            sv.set_state(*st, 0.0)
+            sv.step(7)
+            out.append(sv.get_state())
+    for a, b in zip(out[0], out[1]):
+        if precision == 64:
+            np.testing.assert_array_equal(a, b)
+        else:
+            assert np.linalg.norm(a - b) <= 1e-4 * np.linalg.norm(b)
