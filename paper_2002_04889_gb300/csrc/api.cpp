@@ -243,6 +243,7 @@ DevPtrs dev_ptrs(const vg_ctx *c)
     d.bed_uplift = c->bed_uplift;
     d.bed_onset = c->bed_onset;
     d.bed_rise = c->bed_rise;
+    d.bed_rrise = c->bed_rise > 0.0 ? 1.0 / c->bed_rise : 0.0;
     d.nbr = c->nbr;
     d.nbrl = c->nbrl;
     d.halo_ptr = c->halo_ptr;
@@ -1700,8 +1701,7 @@ int vg_adj_backward(vg_ctx *c, const double *dJ_deta, double *dJ_dH0, double *dJ
             ADJ_CHECK(err);
         }
         if (bed) {
-            // the context keeps the bed of the run's last time; the gradients stay on the host
-            ADJ_CHECK(launch_bed_update(d, p, nullptr, 64, false, tn[N], st));
+            // the gradients stay on the host
             c->adj_gU.resize(nv);
             c->adj_gOn.resize(nv);
             VG_CUDA(c, cudaMemcpyAsync(c->adj_gU.data(), gU, 8 * (size_t)nv, cudaMemcpyDeviceToHost, c->stream));
@@ -1735,6 +1735,15 @@ int vg_adj_backward(vg_ctx *c, const double *dJ_deta, double *dJ_dH0, double *dJ
     }
 done:
 #undef ADJ_CHECK
+    if (bed) {
+        // the context's bed again that of its own time (a step moves only the part of
+        // the bed that differs between its two times)
+        DevScalars now;
+        int e = read_scalars(c, now);
+        if (!e && (e = launch_bed_update(d, p, nullptr, 64, false, now.t, st)))
+            e = cuda_fail(c, (cudaError_t)e, "bed update launch");
+        if (!rc) rc = e;
+    }
     cudaStreamSynchronize(c->stream);
     for (void *q : bufs) cudaFree(q);
     return rc;

@@ -139,7 +139,7 @@ struct DevPtrs {
     // (internal order) and per-vertex initial depth, uplift and onset time
     const int32_t *bed_vtx;
     const double *bed_depth0, *bed_uplift, *bed_onset;
-    double bed_rise;
+    double bed_rise, bed_rrise;   // rise time and its reciprocal
 };
 
 // Launch wrappers (defined in step_f32.cu / step_f64.cu).  w_in, w_out are

@@ -62,3 +62,26 @@ def test_block_shape_by_mesh_size(precision, n):
             np.testing.assert_array_equal(a, b)
         else:
             assert np.linalg.norm(a - b) <= 1e-4 * np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("rise,t0", [(0.0, 0.0), (1e-3, 0.0), (0.02, 0.0), (0.02, 0.013), (5.0, 0.0)])
+def test_moving_bed_touches_only_what_moves(rise, t0):
+    """Vertices before their onset, inside their rise (some crossing both ends in one
+    step, some onsets equal to a step's time), after it, and never: FP64 equal to the
+    oracle's full update bit for bit, also after the motion has ended."""
+    m, st = _moving_basin(20)
+    r = np.hypot(m.xy[:, 0], m.xy[:, 1])
+    up = 0.02 * np.exp(-(r / 0.4) ** 2) * (m.xy[:, 1] > -0.5)
+    on = np.where(m.xy[:, 0] > 0.5, 1e9, np.round(0.04 * r, 3))
+    prm = dict(h_threshold=1e-5, dt_fixed=0.002)
+    om = O.OracleMesh.from_mesh(m)
+    ref = om.run(O.params(**prm), (*st, t0), 40, bed_motion=(m.depth, up, on, rise))
+    with volna.Solver(64) as sv:
+        sv.set_params(**prm)
+        sv.upload_mesh(m)
+        sv.set_bed_motion(up, on, rise)
+        sv.set_state(*st, t0)
+        sv.step(40)
+        got = sv.get_state()
+    for a, k in zip(got, ("H", "Hu", "Hv")):
+        np.testing.assert_array_equal(a, ref[k])
