@@ -41,13 +41,14 @@ struct vg_ctx {
 
     // device memory
     void *geo = nullptr, *z = nullptr, *w[2] = {nullptr, nullptr}, *R0 = nullptr;
-    void *zf = nullptr;               // face beds (layout: DevPtrs::zf)
-    void *rk_w1 = nullptr, *rk_R1 = nullptr;   // [3][nc] each: w1 and R(w1) of the unfused RK stages
+    void *zf = nullptr;               // FP64 face beds (FP32 keeps them in geo)
+    void *geoB = nullptr, *codes = nullptr, *ring_codes = nullptr, *fr = nullptr;   // FP32 records (DevPtrs)
+    float *area32 = nullptr;
+    void *rk_w1 = nullptr, *rk_R1 = nullptr;   // state buffers: w1 and R(w1) of the unfused RK stages
     double *rarea = nullptr;          // FP64: 1 / area of every cell
     double *z64 = nullptr;
-    float *z_orig = nullptr;          // FP32: the bed in the original cell order (state import/export)
-    double *z64_orig = nullptr;
-    bool zorig_ok = false;            // the two copies match z (false once a moving bed was set)
+    double *z64_orig = nullptr;       // FP32: the FP64 bed in the original cell order (state import/export)
+    bool zorig_ok = false;            // it matches z64 (false once a moving bed was set)
     int32_t *nbr = nullptr, *halo_ptr = nullptr, *halo_n1 = nullptr, *halo_ids = nullptr, *old_of_new = nullptr;
     int32_t *new_of_old = nullptr, *fq_ptr = nullptr, *adj_faces = nullptr;
     int64_t n_adj_faces = 0;          // built by the first adjoint sweep of a mesh
@@ -155,7 +156,8 @@ void free_mesh(vg_ctx *c)
     if (c->z64 == c->z) c->z64 = nullptr;
     dfree(c->geo); dfree(c->rarea); dfree(c->z); dfree(c->zf); dfree(c->z64); dfree(c->w[0]); dfree(c->w[1]); dfree(c->R0);
     dfree(c->rk_w1); dfree(c->rk_R1);
-    dfree(c->z_orig); dfree(c->z64_orig); c->zorig_ok = false;
+    dfree(c->geoB); dfree(c->codes); dfree(c->ring_codes); dfree(c->fr); dfree(c->area32);
+    dfree(c->z64_orig); c->zorig_ok = false;
     dfree(c->nbr); dfree(c->halo_ptr); dfree(c->halo_n1); dfree(c->halo_ids); dfree(c->ring1_nbr);
     dfree(c->old_of_new); dfree(c->new_of_old); dfree(c->nbrl); dfree(c->fq_ptr); dfree(c->fq);
     dfree(c->adj_faces); c->n_adj_faces = 0;
@@ -174,6 +176,9 @@ void free_mesh(vg_ctx *c)
 }
 
 size_t real_size(const vg_ctx *c) { return c->precision == 64 ? 8 : 4; }
+
+// Bytes of a state buffer: FP64 [3][nc] doubles, FP32 [nc] float4 (eta, Hu, Hv, z).
+size_t state_bytes(const vg_ctx *c) { return (c->precision == 64 ? 24 : 16) * (size_t)c->hm.nc; }
 
 // Cells and threads per block where the caller leaves both to the library.  Large
 // meshes: 256 cells, one thread each (smaller blocks reconstruct more halo cells:
@@ -228,15 +233,20 @@ DevPtrs dev_ptrs(const vg_ctx *c)
     d.nblocks = c->hm.nblocks;
     d.max_halo = c->hm.max_halo;
     d.max_ring1 = c->hm.max_ring1;
+    d.max_faces = c->hm.max_faces;
     d.n_gauges = c->n_gauges;
     d.ring_cap = kRingCap;
     d.geo = c->geo;
     d.rarea = c->rarea;
+    d.geoB = c->geoB;
+    d.area32 = c->area32;
+    d.codes = c->codes;
+    d.ring_codes = c->ring_codes;
+    d.fr = c->fr;
     d.z = c->z;
     d.zf = c->zf;
     d.z64 = c->z64;
     const bool zo = c->zorig_ok && !c->bed_on;
-    d.z_orig = zo ? c->z_orig : nullptr;
     d.z64_orig = zo ? c->z64_orig : nullptr;
     d.bed_vtx = c->bed_vtx;
     d.bed_depth0 = c->bed_depth0;
@@ -290,45 +300,119 @@ int upload_real(vg_ctx *c, void *dst, const double *src, size_t n)
     return VG_OK;
 }
 
-// FP32: the bed (as the kernels round it, and in FP64) in the original cell
-// order, so that the state import / export kernels, one thread per original
-// cell, read it contiguously instead of at scattered internal positions.
+// FP32: the FP64 bed in the original cell order, so that the state import / export
+// kernels, one thread per original cell, read it contiguously instead of at
+// scattered internal positions.
 int upload_bed_orig(vg_ctx *c)
 {
     c->zorig_ok = false;
     if (c->precision == 64) return VG_OK;
     const HostMesh &m = c->hm;
     int rc;
-    if (!c->z_orig && (rc = dmalloc(c, (void **)&c->z_orig, 4 * m.nc))) return rc;
     if (!c->z64_orig && (rc = dmalloc(c, (void **)&c->z64_orig, 8 * m.nc))) return rc;
     std::vector<double> zo(m.nc);
-    std::vector<float> zf(m.nc);
-    for (int64_t o = 0; o < m.nc; o++) {
-        zo[o] = m.z[m.new_of_old[o]];
-        zf[o] = (float)zo[o];             // the rounding of upload_real
-    }
+    for (int64_t o = 0; o < m.nc; o++) zo[o] = m.z[m.new_of_old[o]];
     VG_CUDA(c, cudaMemcpy(c->z64_orig, zo.data(), 8 * m.nc, cudaMemcpyHostToDevice));
-    VG_CUDA(c, cudaMemcpy(c->z_orig, zf.data(), 4 * m.nc, cudaMemcpyHostToDevice));
     c->zorig_ok = true;
     return VG_OK;
 }
 
-// Face beds of the host mesh in the device layout: FP64 [3][nc] as they are;
-// FP32 [nc][2] the differences z_f - z_K of faces 0 and 1, formed in FP64.
-int upload_face_beds(vg_ctx *c)
+// FP32: the reconstruction records (recA of block_f32.cuh): rows 0 and 1 of M_fj =
+// w_j . (x_f - x_K) and the differences z_f - z_K of faces 0 and 1, formed in FP64.
+int upload_rec_a(vg_ctx *c)
 {
     const HostMesh &m = c->hm;
     const int64_t n = m.nc;
     int rc;
-    if (!c->zf && (rc = dmalloc(c, &c->zf, c->precision == 64 ? 8 * 3 * n : 8 * n))) return rc;
-    if (c->precision == 64) {
-        VG_CUDA(c, cudaMemcpy(c->zf, m.zf.data(), 8 * 3 * n, cudaMemcpyHostToDevice));
-    } else {
-        std::vector<float> d(2 * (size_t)n);
-        for (int64_t k = 0; k < n; k++)
-            for (int f = 0; f < 2; f++) d[2 * k + f] = (float)(m.zf[f * (size_t)n + k] - m.z[k]);
-        VG_CUDA(c, cudaMemcpy(c->zf, d.data(), 4 * d.size(), cudaMemcpyHostToDevice));
+    if (!c->geo && (rc = dmalloc(c, &c->geo, 32 * (size_t)n))) return rc;
+    std::vector<float> r(8 * (size_t)n);
+    for (int64_t k = 0; k < n; k++) {
+        auto G = [&](int row) { return m.geo[(size_t)row * n + k]; };
+        float *o = &r[8 * (size_t)k];
+        for (int f = 0; f < 2; f++) {
+            for (int j = 0; j < 3; j++)
+                o[3 * f + j] = (float)(G(GEO_WX + j) * G(GEO_FX + f) + G(GEO_WY + j) * G(GEO_FY + f));
+            o[6 + f] = (float)(m.zf[f * (size_t)n + k] - m.z[k]);
+        }
     }
+    VG_CUDA(c, cudaMemcpy(c->geo, r.data(), 4 * r.size(), cudaMemcpyHostToDevice));
+    return VG_OK;
+}
+
+// Face beds of the host mesh: FP64 [3][nc] as they are, FP32 in the records.
+int upload_face_beds(vg_ctx *c)
+{
+    const HostMesh &m = c->hm;
+    if (c->precision != 64) return upload_rec_a(c);
+    int rc;
+    if (!c->zf && (rc = dmalloc(c, &c->zf, 8 * 3 * m.nc))) return rc;
+    VG_CUDA(c, cudaMemcpy(c->zf, m.zf.data(), 8 * 3 * m.nc, cudaMemcpyHostToDevice));
+    return VG_OK;
+}
+
+// FP32 partition arrays: the codes of block and ring-1 cells and the face records
+// of every block (layouts: block_f32.cuh).
+int upload_partition_f32(vg_ctx *c)
+{
+    const HostMesh &m = c->hm;
+    const int64_t nc = m.nc;
+    const int B = m.block, L1 = B + m.max_ring1;
+    struct Code { uint16_t nb[3], walls; };
+    std::vector<Code> codes(nc), ring(std::max<size_t>(1, m.halo_ids.size()));
+    std::vector<float> fr(4 * std::max<size_t>(1, m.fq.size()));
+    auto code_of = [&](uint16_t nbr_code, bool packed, int own, int f, Code &o) {
+        if (nbr_code >= NBR_ABSORB) {
+            o.nb[f] = (uint16_t)own;             // a boundary face: the open ghost is the cell itself
+            if (nbr_code == NBR_WALL) o.walls |= (uint16_t)(1 << f);
+        } else {
+            o.nb[f] = packed ? nbr_code >> 2 : nbr_code;
+        }
+    };
+#pragma omp parallel for schedule(dynamic, 64)
+    for (int32_t b = 0; b < m.nblocks; b++) {
+        const int64_t c0 = (int64_t)b * B, c1 = std::min<int64_t>(c0 + B, nc);
+        for (int64_t k = c0; k < c1; k++) {
+            codes[k].walls = 0;
+            for (int f = 0; f < 3; f++) code_of(m.nbrl[f * nc + k], true, (int)(k - c0), f, codes[k]);
+        }
+        for (int32_t h = 0; h < m.halo_n1[b]; h++) {
+            const size_t i = (size_t)m.halo_ptr[b] + h;
+            ring[i].walls = 0;
+            for (int f = 0; f < 3; f++) code_of(m.ring1_nbr[3 * i + f], false, B + h, f, ring[i]);
+        }
+        // interior faces first, so that whole warps take the interior branch
+        int32_t at = m.fq_ptr[b];
+        for (int boundary = 0; boundary < 2; boundary++)
+            for (int32_t q = m.fq_ptr[b]; q < m.fq_ptr[b + 1]; q++) {
+                const int l = m.fq[q] >> 2, f = m.fq[q] & 3;
+                const int64_t k = c0 + l;
+                const uint16_t code = m.nbrl[f * nc + k];
+                if ((code >= NBR_ABSORB) != (boundary != 0)) continue;
+                uint32_t sl = (uint32_t)(f * L1 + l), sr = code;
+                int64_t kk = k;                   // the left cell and its face
+                int ff = f;
+                if (!boundary) {
+                    const int nl = code >> 2, nf = code & 3;
+                    sr = (uint32_t)(nf * L1 + nl);
+                    const int64_t j = m.nbr[f * nc + k];
+                    if (j < k) { std::swap(sl, sr); kk = j; ff = nf; }
+                }
+                float *o = &fr[4 * (size_t)at++];
+                o[0] = (float)m.geo[(size_t)(GEO_NX + ff) * nc + kk];
+                o[1] = (float)m.geo[(size_t)(GEO_NY + ff) * nc + kk];
+                o[2] = (float)m.geo[(size_t)(GEO_LEN + ff) * nc + kk];
+                const uint32_t slots = sl | (sr << 16);
+                std::memcpy(&o[3], &slots, 4);
+            }
+    }
+    dfree(c->codes); dfree(c->ring_codes); dfree(c->fr);
+    int rc;
+    if ((rc = dmalloc(c, &c->codes, 8 * (size_t)nc))) return rc;
+    if ((rc = dmalloc(c, &c->ring_codes, 8 * ring.size()))) return rc;
+    if ((rc = dmalloc(c, &c->fr, 4 * fr.size()))) return rc;
+    VG_CUDA(c, cudaMemcpy(c->codes, codes.data(), 8 * (size_t)nc, cudaMemcpyHostToDevice));
+    VG_CUDA(c, cudaMemcpy(c->ring_codes, ring.data(), 8 * ring.size(), cudaMemcpyHostToDevice));
+    VG_CUDA(c, cudaMemcpy(c->fr, fr.data(), 4 * fr.size(), cudaMemcpyHostToDevice));
     return VG_OK;
 }
 
@@ -341,21 +425,22 @@ int upload_partition(vg_ctx *c)
     int rc;
     size_t nh = std::max<size_t>(1, m.halo_ids.size());
     if ((rc = dmalloc(c, (void **)&c->fq_ptr, 4 * (m.nblocks + 1)))) return rc;
-    if ((rc = dmalloc(c, (void **)&c->fq, 2 * m.fq.size()))) return rc;
-    VG_CUDA(c, cudaMemcpy(c->fq_ptr, m.fq_ptr.data(), 4 * (m.nblocks + 1), cudaMemcpyHostToDevice));
-    VG_CUDA(c, cudaMemcpy(c->fq, m.fq.data(), 2 * m.fq.size(), cudaMemcpyHostToDevice));
-    if ((rc = dmalloc(c, (void **)&c->nbrl, 2 * 3 * m.nc))) return rc;
     if ((rc = dmalloc(c, (void **)&c->halo_ptr, 4 * (m.nblocks + 1)))) return rc;
     if ((rc = dmalloc(c, (void **)&c->halo_n1, 4 * m.nblocks))) return rc;
     if ((rc = dmalloc(c, (void **)&c->halo_ids, 4 * nh))) return rc;
-    if ((rc = dmalloc(c, (void **)&c->ring1_nbr, 2 * 3 * nh))) return rc;
-    VG_CUDA(c, cudaMemcpy(c->nbrl, m.nbrl.data(), 2 * 3 * m.nc, cudaMemcpyHostToDevice));
+    VG_CUDA(c, cudaMemcpy(c->fq_ptr, m.fq_ptr.data(), 4 * (m.nblocks + 1), cudaMemcpyHostToDevice));
     VG_CUDA(c, cudaMemcpy(c->halo_ptr, m.halo_ptr.data(), 4 * (m.nblocks + 1), cudaMemcpyHostToDevice));
     VG_CUDA(c, cudaMemcpy(c->halo_n1, m.halo_n1.data(), 4 * m.nblocks, cudaMemcpyHostToDevice));
-    if (!m.halo_ids.empty()) {
+    if (!m.halo_ids.empty())
         VG_CUDA(c, cudaMemcpy(c->halo_ids, m.halo_ids.data(), 4 * m.halo_ids.size(), cudaMemcpyHostToDevice));
+    if (c->precision != 64) return upload_partition_f32(c);
+    if ((rc = dmalloc(c, (void **)&c->fq, 2 * m.fq.size()))) return rc;
+    if ((rc = dmalloc(c, (void **)&c->nbrl, 2 * 3 * m.nc))) return rc;
+    if ((rc = dmalloc(c, (void **)&c->ring1_nbr, 2 * 3 * nh))) return rc;
+    VG_CUDA(c, cudaMemcpy(c->fq, m.fq.data(), 2 * m.fq.size(), cudaMemcpyHostToDevice));
+    VG_CUDA(c, cudaMemcpy(c->nbrl, m.nbrl.data(), 2 * 3 * m.nc, cudaMemcpyHostToDevice));
+    if (!m.halo_ids.empty())
         VG_CUDA(c, cudaMemcpy(c->ring1_nbr, m.ring1_nbr.data(), 2 * m.ring1_nbr.size(), cudaMemcpyHostToDevice));
-    }
     return VG_OK;
 }
 
@@ -364,37 +449,34 @@ int upload_mesh_arrays(vg_ctx *c)
     const HostMesh &m = c->hm;
     size_t rs = real_size(c);
     int rc;
-    if ((rc = dmalloc(c, &c->geo, c->precision == 64 ? 8 * GEO_ROWS * m.nc : 4 * 16 * m.nc))) return rc;
     if ((rc = dmalloc(c, &c->z, rs * m.nc))) return rc;
-    if ((rc = dmalloc(c, &c->w[0], rs * 3 * m.nc))) return rc;
-    if ((rc = dmalloc(c, &c->w[1], rs * 3 * m.nc))) return rc;
-    if ((rc = dmalloc(c, &c->R0, rs * 3 * m.nc))) return rc;
+    if ((rc = dmalloc(c, &c->w[0], state_bytes(c)))) return rc;
+    if ((rc = dmalloc(c, &c->w[1], state_bytes(c)))) return rc;
+    if ((rc = dmalloc(c, &c->R0, state_bytes(c)))) return rc;
     if ((rc = dmalloc(c, (void **)&c->nbr, 4 * 3 * m.nc))) return rc;
     if ((rc = dmalloc(c, (void **)&c->old_of_new, 4 * m.nc))) return rc;
     if ((rc = dmalloc(c, (void **)&c->new_of_old, 4 * m.nc))) return rc;
     if ((rc = dmalloc(c, (void **)&c->ring_t, 8 * kRingCap))) return rc;
     if (c->precision == 64) {
+        if ((rc = dmalloc(c, &c->geo, 8 * GEO_ROWS * m.nc))) return rc;
         if ((rc = upload_real(c, c->geo, m.geo.data(), m.geo.size()))) return rc;
     } else {
-        // FP32 record per cell (16 floats): rows 0 and 1 of M_fj = w_j . (x_f - x_K)
-        // formed in FP64, the area, face lengths and normals:
-        //   M00 M01 M02 M10 | M11 M12 area l0 | nx0 ny0 nx1 ny1 | nx2 ny2 l1 l2
+        // FP32: face normals times lengths of faces 0 and 1, and the areas (recA: with
+        // the face beds below)
         const int64_t n = m.nc;
-        std::vector<float> r(16 * (size_t)n, 0.0f);
+        std::vector<float> r(4 * (size_t)n), area(n);
         for (int64_t k = 0; k < n; k++) {
             auto G = [&](int row) { return m.geo[(size_t)row * n + k]; };
-            float *o = &r[16 * (size_t)k];
-            for (int f = 0; f < 2; f++)
-                for (int j = 0; j < 3; j++)
-                    o[3 * f + j] = (float)(G(GEO_WX + j) * G(GEO_FX + f) + G(GEO_WY + j) * G(GEO_FY + f));
-            o[6] = (float)G(GEO_AREA);
-            for (int f = 0; f < 3; f++) {
-                o[8 + 2 * f] = (float)G(GEO_NX + f);
-                o[9 + 2 * f] = (float)G(GEO_NY + f);
-                o[f == 0 ? 7 : 13 + f] = (float)G(GEO_LEN + f);
+            for (int f = 0; f < 2; f++) {
+                r[4 * k + 2 * f] = (float)(G(GEO_LEN + f) * G(GEO_NX + f));
+                r[4 * k + 2 * f + 1] = (float)(G(GEO_LEN + f) * G(GEO_NY + f));
             }
+            area[k] = (float)G(GEO_AREA);
         }
-        VG_CUDA(c, cudaMemcpy(c->geo, r.data(), 4 * r.size(), cudaMemcpyHostToDevice));
+        if ((rc = dmalloc(c, &c->geoB, 16 * (size_t)n))) return rc;
+        if ((rc = dmalloc(c, (void **)&c->area32, 4 * (size_t)n))) return rc;
+        VG_CUDA(c, cudaMemcpy(c->geoB, r.data(), 4 * r.size(), cudaMemcpyHostToDevice));
+        VG_CUDA(c, cudaMemcpy(c->area32, area.data(), 4 * area.size(), cudaMemcpyHostToDevice));
     }
     if (c->precision == 64) {
         std::vector<double> ra(m.nc);
@@ -417,10 +499,11 @@ int upload_mesh_arrays(vg_ctx *c)
     return upload_partition(c);
 }
 
-size_t stage_smem(const vg_ctx *c, int block, int max_halo, int max_ring1)
+size_t stage_smem(const vg_ctx *c)
 {
-    return c->precision == 64 ? stage_smem_f64(block, max_halo, max_ring1)
-                              : stage_smem_f32(block, max_halo, max_ring1);
+    const HostMesh &m = c->hm;
+    return c->precision == 64 ? stage_smem_f64(m.block, m.max_halo, m.max_ring1)
+                              : stage_smem_f32(m.block, m.max_halo, m.max_ring1, m.max_faces);
 }
 
 // Halve the block size until the stage kernels' shared memory (block + two-ring
@@ -430,7 +513,7 @@ int fit_blocks(vg_ctx *c)
 {
     int limit = 0;
     VG_CUDA(c, cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
-    while (stage_smem(c, c->hm.block, c->hm.max_halo, c->hm.max_ring1) > (size_t)limit) {
+    while (stage_smem(c) > (size_t)limit) {
         if (c->hm.block <= 32)
             return fail(c, VG_EINVAL, "mesh blocks need more shared memory than the device has; renumber the mesh");
         int rc = partition_blocks(c->hm, c->hm.block / 2, c->err);
@@ -631,7 +714,7 @@ int validate_params(const vg_params *p, std::string &why)
 int ensure_rk_buffers(vg_ctx *c)
 {
     if (!c->has_mesh || !c->prm.rk_unfused) return VG_OK;
-    const size_t bytes = 3 * (size_t)c->hm.nc * real_size(c);
+    const size_t bytes = state_bytes(c);
     int rc;
     if (!c->rk_w1 && (rc = dmalloc(c, &c->rk_w1, bytes))) return rc;
     if (!c->rk_R1 && (rc = dmalloc(c, &c->rk_R1, bytes))) return rc;
@@ -1188,6 +1271,12 @@ int vg_set_depth(vg_ctx *c, const double *depth_v)
     if ((rc = upload_face_beds(c))) return rc;
     if (c->precision != 64) VG_CUDA(c, cudaMemcpy(c->z64, m.z.data(), 8 * m.nc, cudaMemcpyHostToDevice));
     if ((rc = upload_bed_orig(c))) return rc;
+    if (c->precision != 64 && c->has_state) {
+        // the FP32 state carries its cells' beds (eta stays, as z does in FP64's H)
+        int e = launch_state_bed(dev_ptrs(c), c->w[c->cur], (void *)c->stream);
+        if (e) return cuda_fail(c, (cudaError_t)e, "state bed launch");
+        c->launches++;
+    }
     c->depth_v.assign(depth_v, depth_v + m.nv);
     c->graph_dirty = true;
     return VG_OK;
@@ -1794,10 +1883,11 @@ int vg_step_noalloc(vg_ctx *c, const void *w_in, void *w_out, double t, double *
     StepParams p = step_params(c);
     void *s = (void *)c->stream;
     if ((e = noalloc_launch_init(sc, t, c->precision, s))) return cuda_fail(c, (cudaError_t)e, "scratch init launch");
-    e = c->precision == 64 ? launch_stage1_f64(d, p, w_in, c->cfg1, s) : launch_stage1_f32(d, p, w_in, c->cfg1, s);
+    e = c->precision == 64 ? launch_stage1_f64(d, p, w_in, c->cfg1, s)
+                           : launch_stage_soa_f32(d, p, 1, w_in, w_out, c->cfg1, s);
     if (e) return cuda_fail(c, (cudaError_t)e, "stage 1 launch");
     e = c->precision == 64 ? launch_stage2_f64(d, p, w_in, w_out, c->cfg2, s)
-                           : launch_stage2_f32(d, p, w_in, w_out, c->cfg2, s);
+                           : launch_stage_soa_f32(d, p, 2, w_in, w_out, c->cfg2, s);
     if (e) return cuda_fail(c, (cudaError_t)e, "stage 2 launch");
     if ((e = launch_post_step(d, p, w_out, c->precision, s))) return cuda_fail(c, (cudaError_t)e, "post-step launch");
     c->launches += 4;

@@ -91,7 +91,8 @@ int bcuda(vg_batch *b, cudaError_t e, const char *what)
         if (e_ != cudaSuccess) return bcuda(b, e_, #call);       \
     } while (0)
 
-size_t rsize(const vg_batch *b) { return b->precision == 64 ? 8 : 4; }
+// Bytes of one cell of a state buffer: FP64 three doubles, FP32 a float4.
+size_t cell_bytes(const vg_batch *b) { return b->precision == 64 ? 24 : 16; }
 
 void scalars_init(const vg_batch *b, DevScalars &s, double t)
 {
@@ -133,7 +134,7 @@ int rebuild(vg_batch *b)
     size_t eb = b->precision == 64 ? batch_mesh_bytes_f64() : batch_mesh_bytes_f32();
     size_t nm = b->meshes.size();
     std::vector<unsigned char> host(eb * nm);
-    int block = 0, max_halo = 0, max_ring1 = 0;
+    int block = 0, max_halo = 0, max_ring1 = 0, max_faces = 0;
     for (int parity = 0; parity < 2; parity++) {
         int item = 0;
         for (size_t m = 0; m < nm; m++) {
@@ -158,6 +159,7 @@ int rebuild(vg_batch *b)
             block = d.block;
             max_halo = std::max(max_halo, (int)d.max_halo);
             max_ring1 = std::max(max_ring1, (int)d.max_ring1);
+            max_faces = std::max(max_faces, (int)d.max_faces);
         }
         b->n_items = item;
         if (b->table[parity]) cudaFree(b->table[parity]);
@@ -165,7 +167,7 @@ int rebuild(vg_batch *b)
         VB_CUDA(b, cudaMemcpy(b->table[parity], host.data(), eb * nm, cudaMemcpyHostToDevice));
     }
     int e = b->precision == 64 ? batch_config_f64(block, max_halo, max_ring1, b->grid, b->smem, !b->prm.fp64_literal)
-                               : batch_config_f32(block, max_halo, max_ring1, b->grid, b->smem);
+                               : batch_config_f32(block, max_halo, max_ring1, max_faces, b->grid, b->smem);
     if (e) return bcuda(b, (cudaError_t)e, "batched launch configuration");
     {
         int sms = 0;
@@ -329,7 +331,7 @@ int record_now(vg_batch *b, vg_batch::Mesh &M, int k)
     d.ring_t = M.ring_t + (size_t)k * kBatchRingCap;
     d.ring_eta = M.ring_eta + (size_t)k * kBatchRingCap * M.n_gauges;
     const int64_t nc = ctx_host_mesh(M.ctx).nc;
-    const void *w = static_cast<unsigned char *>(M.w[b->cur]) + rsize(b) * 3 * (size_t)nc * k;
+    const void *w = static_cast<unsigned char *>(M.w[b->cur]) + cell_bytes(b) * (size_t)nc * k;
     int err = launch_record_gauges(d, w, b->precision, (void *)b->stream);
     if (err) return bcuda(b, (cudaError_t)err, "gauge record launch");
     b->launches++;
@@ -448,7 +450,7 @@ int vg_batch_add_mesh(vg_batch *b, int64_t nv, const double *xy, int64_t nc, con
         vg_destroy(M.ctx);
         return bfail(b, rc, msg);
     }
-    size_t bytes = rsize(b) * 3 * (size_t)nc * n_scenarios;
+    size_t bytes = cell_bytes(b) * (size_t)nc * n_scenarios;
     if (cudaMalloc(&M.w[0], bytes) != cudaSuccess || cudaMalloc(&M.w[1], bytes) != cudaSuccess ||
         cudaMalloc(&M.R0, bytes) != cudaSuccess) {
         cudaGetLastError();
@@ -479,7 +481,7 @@ int vg_batch_add_mesh(vg_batch *b, int64_t nv, const double *xy, int64_t nc, con
         // keep every mesh's current state in the same buffer index
         for (size_t m = 0; m + 1 < b->meshes.size(); m++)
             VB_CUDA(b, cudaMemcpy(b->meshes[m].w[0], b->meshes[m].w[1],
-                                  rsize(b) * 3 * ctx_host_mesh(b->meshes[m].ctx).nc * b->meshes[m].n_scen,
+                                  cell_bytes(b) * ctx_host_mesh(b->meshes[m].ctx).nc * b->meshes[m].n_scen,
                                   cudaMemcpyDeviceToDevice));
         b->cur = 0;
     }
@@ -507,7 +509,7 @@ int vg_batch_set_state(vg_batch *b, int32_t mesh, int32_t scen, const double *H,
     VB_CUDA(b, cudaMemcpyAsync(b->sc_all + e, &s, sizeof(s), cudaMemcpyHostToDevice, b->stream));
     DevPtrs d = ctx_dev_ptrs(M.ctx);
     d.sc = b->sc_all + e;
-    void *dst = static_cast<unsigned char *>(M.w[b->cur]) + rsize(b) * 3 * (size_t)nc * scen;
+    void *dst = static_cast<unsigned char *>(M.w[b->cur]) + cell_bytes(b) * (size_t)nc * scen;
     int err = launch_import_state(d, ctx_old_of_new(M.ctx), st, st + nc, st + 2 * nc, 1, dst, b->precision,
                                   (void *)b->stream);
     if (err) return bcuda(b, (cudaError_t)err, "state import launch");
@@ -535,7 +537,7 @@ int vg_batch_get_state(vg_batch *b, int32_t mesh, int32_t scen, double *H, doubl
     int64_t nc = ctx_host_mesh(M.ctx).nc;
     double *st = nullptr;
     if ((rc = ctx_staging(M.ctx, &st))) return bfail(b, rc, "staging allocation failed");
-    const void *src = static_cast<unsigned char *>(M.w[b->cur]) + rsize(b) * 3 * (size_t)nc * scen;
+    const void *src = static_cast<unsigned char *>(M.w[b->cur]) + cell_bytes(b) * (size_t)nc * scen;
     int err = launch_export_state(ctx_dev_ptrs(M.ctx), ctx_old_of_new(M.ctx), src, b->precision, st, st + nc,
                                   st + 2 * nc, 1, (void *)b->stream);
     if (err) return bcuda(b, (cudaError_t)err, "state export launch");
@@ -618,7 +620,7 @@ int vg_batch_autotune(vg_batch *b, int32_t n_steps, int32_t *best_block, int32_t
     std::vector<void *> saved(b->meshes.size(), nullptr);
     void *sc_saved = nullptr;
     for (size_t m = 0; m < b->meshes.size(); m++) {
-        size_t bytes = rsize(b) * 3 * ctx_host_mesh(b->meshes[m].ctx).nc * b->meshes[m].n_scen;
+        size_t bytes = cell_bytes(b) * ctx_host_mesh(b->meshes[m].ctx).nc * b->meshes[m].n_scen;
         VB_CUDA(b, cudaMalloc(&saved[m], bytes));
         VB_CUDA(b, cudaMemcpyAsync(saved[m], b->meshes[m].w[b->cur], bytes, cudaMemcpyDeviceToDevice, b->stream));
     }
@@ -656,7 +658,7 @@ int vg_batch_autotune(vg_batch *b, int32_t n_steps, int32_t *best_block, int32_t
             cudaEventElapsedTime(&ms, e0, e1);
             if (ms < best_t) { best_t = ms; best = candidates[k]; best_c = b->ctas_per_sm; }
             for (size_t m = 0; m < b->meshes.size(); m++) {
-                size_t bytes = rsize(b) * 3 * ctx_host_mesh(b->meshes[m].ctx).nc * b->meshes[m].n_scen;
+                size_t bytes = cell_bytes(b) * ctx_host_mesh(b->meshes[m].ctx).nc * b->meshes[m].n_scen;
                 cudaMemcpyAsync(b->meshes[m].w[cur0], saved[m], bytes, cudaMemcpyDeviceToDevice, b->stream);
             }
             cudaMemcpyAsync(b->sc_all, sc_saved, sc_bytes, cudaMemcpyDeviceToDevice, b->stream);

@@ -486,6 +486,7 @@ int partition_blocks(HostMesh &m, int block, std::string &err)
             for (int f = 0; f < 3; f++) n += owned(c, c0, f);
         m.fq_ptr[b + 1] = n;
     }
+    m.max_faces = *std::max_element(m.fq_ptr.begin(), m.fq_ptr.end());
     for (int32_t b = 0; b < nb; b++) m.fq_ptr[b + 1] += m.fq_ptr[b];
     m.fq.resize(std::max<int32_t>(m.fq_ptr[nb], 1));
 #pragma omp parallel for schedule(dynamic, 256)

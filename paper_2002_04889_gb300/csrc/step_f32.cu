@@ -2,7 +2,10 @@
 #include "step_kernels.cuh"
 
 namespace vg {
-size_t stage_smem_f32(int block, int max_halo, int max_ring1) { return stage_smem_bytes<float>(block, max_halo, max_ring1); }
+size_t stage_smem_f32(int block, int max_halo, int max_ring1, int max_faces)
+{
+    return stage_smem_bytes<float>(block, max_halo, max_ring1, max_faces);
+}
 int stage_config_f32(const DevPtrs &d, int stage, LaunchCfg &cfg) { return stage_config<float>(d, stage, cfg); }
 int launch_stage1_f32(const DevPtrs &d, const StepParams &p, const void *w_in, const LaunchCfg &c, void *stream)
 {
@@ -11,6 +14,11 @@ int launch_stage1_f32(const DevPtrs &d, const StepParams &p, const void *w_in, c
 int launch_stage2_f32(const DevPtrs &d, const StepParams &p, const void *w_in, void *w_out, const LaunchCfg &c, void *stream)
 {
     return launch_stage<float>(d, p, 2, w_in, w_out, c, stream);
+}
+int launch_stage_soa_f32(const DevPtrs &d, const StepParams &p, int stage, const void *w_in, void *w_out, const LaunchCfg &c,
+                         void *stream)
+{
+    return launch_stage<float>(d, p, stage, w_in, w_out, c, stream, true);
 }
 int launch_rk_unfused_f32(const DevPtrs &d, const StepParams &p, int part, const void *w_in, void *w_out, void *w1,
                           void *R1, const LaunchCfg &c1, void *stream)
@@ -23,9 +31,9 @@ void fill_batch_mesh_f32(void *dst, const DevPtrs &d, const StepParams &p, const
 {
     fill_batch_mesh<float>(dst, d, p, w_in, w_out, n_scen, first_item, first_entry);
 }
-int batch_config_f32(int block, int max_halo, int max_ring1, int &grid, size_t &smem)
+int batch_config_f32(int block, int max_halo, int max_ring1, int max_faces, int &grid, size_t &smem)
 {
-    return batch_config<float>(block, max_halo, max_ring1, grid, smem);
+    return batch_config<float>(block, max_halo, max_ring1, max_faces, grid, smem);
 }
 int launch_batch_step_f32(const void *table, int n_mesh, int n_items, int n_entries, DevScalars *sc_all, int block,
                           int grid, size_t smem, const StepParams &p, bool gauges, void *stream)

@@ -5,7 +5,7 @@
 #include "step_kernels.cuh"
 
 namespace vg {
-size_t stage_smem_f64(int block, int max_halo, int max_ring1) { return stage_smem_bytes<double>(block, max_halo, max_ring1); }
+size_t stage_smem_f64(int block, int max_halo, int max_ring1) { return stage_smem_bytes<double>(block, max_halo, max_ring1, 0); }
 int stage_config_f64(const DevPtrs &d, int stage, LaunchCfg &cfg)
 {
     if (d.fp64_fast) return stage_config_f64_fast(d, stage, cfg);
@@ -36,7 +36,7 @@ void fill_batch_mesh_f64(void *dst, const DevPtrs &d, const StepParams &p, const
 int batch_config_f64(int block, int max_halo, int max_ring1, int &grid, size_t &smem, bool fast)
 {
     if (fast) return batch_config_f64_fast(block, max_halo, max_ring1, grid, smem);
-    return batch_config<double, false>(block, max_halo, max_ring1, grid, smem);
+    return batch_config<double, false>(block, max_halo, max_ring1, 0, grid, smem);
 }
 int launch_batch_step_f64(const void *table, int n_mesh, int n_items, int n_entries, DevScalars *sc_all, int block,
                           int grid, size_t smem, const StepParams &p, bool gauges, void *stream)

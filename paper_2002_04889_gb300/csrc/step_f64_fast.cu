@@ -22,7 +22,7 @@ int launch_rk_unfused_f64_fast(const DevPtrs &d, const StepParams &p, int part, 
 }
 int batch_config_f64_fast(int block, int max_halo, int max_ring1, int &grid, size_t &smem)
 {
-    return batch_config<double, true>(block, max_halo, max_ring1, grid, smem);
+    return batch_config<double, true>(block, max_halo, max_ring1, 0, grid, smem);
 }
 int launch_batch_step_f64_fast(const void *table, int n_mesh, int n_items, int n_entries, DevScalars *sc_all,
                                int block, int grid, size_t smem, const StepParams &p, bool gauges, void *stream)

@@ -37,25 +37,20 @@
 //    multiplies by one reciprocal where the literal form forms several correctly
 //    rounded quotients by the same value (face velocities, the HLL star flux, the
 //    residual's 1/|K|).
-//  * FP32 ("deviation"): the state is (eta, Hu, Hv) with eta = H + z, and the
-//    momentum flux through each face is carried relative to the hydrostatic
-//    pressure g (eta_K - z_{K,f})^2 / 2 of the cell's own free surface over the
-//    bed z_{K,f} under its face value.  Summed over a closed triangle these
-//    references give exactly the centred bed-slope source of a cell standing on
-//    its face beds (and zero for a cell on its flat cell bed), so the scheme is
-//    unchanged; but the large terms g H^2 / 2 (1e8 in a 4000 m ocean) never
-//    appear, only products of small differences (eta_f - eta_K, z* - z_K), so
-//    still water stays still in FP32 and eta keeps full FP32 resolution.
+//  * FP32 ("deviation"): block_f32.cuh.
 #pragma once
 
 #include <cuda_runtime.h>
 #include <math_constants.h>
+
+#include <type_traits>
 
 #include "exact_div.cuh"
 #include "vg_internal.h"
 
 namespace vg {
 
+// FP64; the FP32 arguments and phases are in block_f32.cuh.
 template <typename real>
 struct KArgs {
     int64_t nc;
@@ -63,8 +58,7 @@ struct KArgs {
     const real *geo;        // [GEO_ROWS][nc]
     const double *rarea;    // [nc] 1 / area (FP64)
     const real *z;          // [nc]
-    const real *zf;         // face beds: FP64 [3][nc]; FP32 [nc][2] z_f - z_K of faces 0, 1
-    const int32_t *nbr;     // [3][nc]
+    const real *zf;         // [3][nc] face beds
     const uint16_t *nbrl;   // [3][nc]
     const int32_t *halo_ptr;  // [nblocks + 1]
     const int32_t *halo_n1;   // [nblocks] ring-1 count
@@ -84,7 +78,21 @@ struct KArgs {
     real g, half_g, hthr;
     double cfl, dt_fixed, dt_max, t_end;
     int cfl_min;            // stage 1: 1 adds the CFL bound to the step's minimum
+    __device__ __forceinline__ void to_scenario(int s, int64_t stride, bool stage2)
+    {
+        w += s * stride;
+        R0 += s * stride;
+        if (stage2) wout += s * stride;
+        sc += s;
+    }
 };
+
+// One cell's state in a state buffer: a double of a [3][nc] array, or a float4.
+template <typename real> struct StateWord { using type = real; };
+template <> struct StateWord<float> { using type = float4; };
+
+template <typename real>
+__host__ __device__ inline size_t stage_smem_bytes(int block, int max_halo, int max_ring1, int max_faces, bool gids = false);
 
 __device__ __forceinline__ float vmax(float a, float b) { return fmaxf(a, b); }
 __device__ __forceinline__ double vmax(double a, double b) { return fmax(a, b); }
@@ -302,194 +310,46 @@ __device__ __forceinline__ void face_flux(real g, real half_g, real hthr,
     PR = half_g * (HfR * HfR - HsR * HsR);
 }
 
-// Approximate reciprocal (PTX rcp.approx.ftz.f32, max error 1 ulp); rcp(0) = +inf.
-__device__ __forceinline__ float rcp_approx(float x)
-{
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
-// Deviation form for FP32, literal form for FP64.
-template <typename real> struct EtaForm { static constexpr bool value = false; };
-template <> struct EtaForm<float> { static constexpr bool value = true; };
-
-// FP32 cell geometry record, 16 floats (four 16-byte words, 64 bytes) per cell:
-//   M00 M01 M02 M10 | M11 M12 area l0 | nx0 ny0 nx1 ny1 | nx2 ny2 l1 l2
-// with M_fj = w_j . (x_f - x_K): the increments of the reconstruction are
-// D_f = sum_j M_fj (q_j - q_K), the same quantity as grad q . (x_f - x_K) with the
-// least-squares gradient grad q = sum_j w_j (q_j - q_K).  The face midpoints
-// average to the centroid x_K, so D_2 = -(D_0 + D_1) and row 2 is not stored.
-// (FP64 keeps the rows GEO_* and evaluates gradient then dot product, in the
-// literal order.)
-constexpr int G32 = 16;
-constexpr int G32_AREA = 6;
-__device__ __forceinline__ const float4 *g32(const float *geo, int k)
-{
-    return reinterpret_cast<const float4 *>(geo + (size_t)k * G32);
-}
-__device__ __forceinline__ float2 g32_normal(const float *geo, int k, int f)
-{
-    return *reinterpret_cast<const float2 *>(geo + (size_t)k * G32 + 8 + 2 * f);
-}
-__device__ __forceinline__ float g32_len(const float *geo, int k, int f)
-{
-    return geo[(size_t)k * G32 + (f == 0 ? 7 : 13 + f)];
-}
-
-// L1 prefetch (a hint: nothing waits for it and it holds no register).
-__device__ __forceinline__ void prefetch_l1(const void *ptr)
-{
-    asm volatile("prefetch.global.L1 [%0];" :: "l"(ptr));
-}
-
-// Stored state of cell gid as seen by the stage (H or eta first, then Hu, Hv):
+// Stored state of cell gid as seen by the stage (H, Hu, Hv):
 // stage 1 reads w^n; stage 2 forms w1 = w^n + dt R0 and applies the dry fix
 // (negative depth emptied; at or below the threshold, momentum zeroed).
 // Returns true if a negative depth was met.
 template <typename real, int STAGE>
-__device__ __forceinline__ bool stage_state(const KArgs<real> &a, int gid, real dt, real zc, real &W,
-                                            real &Hu, real &Hv, real *wn = nullptr)
+__device__ __forceinline__ bool stage_state(const KArgs<real> &a, int gid, real dt, real &W, real &Hu, real &Hv)
 {
-    constexpr bool ETA = EtaForm<real>::value;
     const int nc = (int)a.nc;
     W = a.w[gid];
     Hu = a.w[nc + gid];
     Hv = a.w[2 * nc + gid];
-    if (wn) { wn[0] = W; wn[1] = Hu; wn[2] = Hv; }
     if (STAGE == 1) return false;
     W = W + dt * a.R0[gid];
     Hu = Hu + dt * a.R0[nc + gid];
     Hv = Hv + dt * a.R0[2 * nc + gid];
-    real H = ETA ? W - zc : W;
-    if (is_neg(H)) {
-        W = ETA ? zc : real(0);
-        Hu = real(0); Hv = real(0);
+    if (is_neg(W)) {
+        W = real(0); Hu = real(0); Hv = real(0);
         return true;
     }
-    if (!gt_nn(H, a.hthr)) { Hu = real(0); Hv = real(0); }
+    if (!gt_nn(W, a.hthr)) { Hu = real(0); Hv = real(0); }
     return false;
-}
-
-// Deviation-form flux (FP32).  Inputs per side: face eta_f and momenta, the bed
-// z under the face value (face bed or cell bed) and the cell's own eta; H below
-// is eta - z of that side.  Same interface depths and HLL as face_flux, with
-//   d* = H*_L - H*_R          (eta_fL - eta_fR when both sides are wet)
-//   F1 - C_e for C_e = g H*_L H*_R / 2:  L: q_L u_nL + g H*_L d* / 2,
-//                                        R: q_R u_nR - g H*_R d* / 2
-// (HLL is affine in F with weights summing to one, so F* shifts by -C_e), and
-// side terms Q_s = C_e + P_s - g H_s^2 / 2 that replace the pressure correction:
-//   Q_L = g/2 [(eta_fL - eta_L)(H_fL + H_L) - H*_L d*],
-//   Q_R = g/2 [(eta_fR - eta_R)(H_fR + H_R) + H*_R d*].
-__device__ __forceinline__ void face_flux_dev(float g, float half_g, float hthr,
-                                              float efL, float HufL, float HvfL, float zL, float eL,
-                                              float efR, float HufR, float HvfR, float zR, float eR,
-                                              float nx, float ny, int bnd,
-                                              float Phi[3], float &QL, float &QR, float &amax)
-{
-    float HfL = efL - zL;
-    float uL = 0.f, vL = 0.f;
-    if (HfL > hthr) { const float r = rcp_approx(HfL); uL = HufL * r; vL = HvfL * r; }
-    float unL = uL * nx + vL * ny;
-    float utL = -uL * ny + vL * nx;
-    float HsL, HsR, unR, utR, ds, HfR;
-    if (bnd == 3) {
-        // absorbing: the outgoing invariant u_n + 2c of the face state and the
-        // incoming u_n - 2c of the sea at rest (eta = 0) beyond the boundary
-        HsL = fmaxf(0.f, HfL);
-        const float cL = sqrtf(g * HsL), c0 = sqrtf(g * fmaxf(0.f, -zL));
-        const float Rp = unL + 2.f * cL, Rm = -2.f * c0;
-        const float cg = fmaxf(0.f, 0.25f * (Rp - Rm));
-        unR = 0.5f * (Rp + Rm);
-        HsR = cg * cg / g;
-        utR = utL;
-        ds = HsL - HsR;
-        HfR = HsR; efR = zL + HsR; eR = efR; zR = zL;
-    } else if (bnd) {
-        HsL = fmaxf(0.f, HfL);
-        HsR = HsL;
-        unR = bnd == 2 ? unL : -unL;
-        utR = utL;
-        ds = 0.f;
-        HfR = HfL; efR = efL; eR = eL; zR = zL;
-    } else {
-        HfR = efR - zR;
-        float uR = 0.f, vR = 0.f;
-        if (HfR > hthr) { const float r = rcp_approx(HfR); uR = HufR * r; vR = HvfR * r; }
-        unR = uR * nx + vR * ny;
-        utR = -uR * ny + vR * nx;
-        float zs = fmaxf(zL, zR);
-        HsL = fmaxf(0.f, efL - zs);
-        HsR = fmaxf(0.f, efR - zs);
-        ds = (HsL > 0.f && HsR > 0.f) ? efL - efR : HsL - HsR;
-    }
-    float F[3];
-    if (HsL == 0.f && HsR == 0.f) {
-        F[0] = 0.f; F[1] = 0.f; F[2] = 0.f;
-        amax = 0.f;
-    } else {
-        float cL = sqrtf(g * HsL), cR = sqrtf(g * HsR);
-        float sL, sR;
-        if (HsL == 0.f) {
-            sL = unR - 2.f * cR;
-            sR = unR + cR;
-        } else if (HsR == 0.f) {
-            sL = unL - cL;
-            sR = unL + 2.f * cL;
-        } else {
-            float us = 0.5f * (unL + unR) + (cL - cR);
-            float cs = 0.5f * (cL + cR) - 0.25f * (unR - unL);
-            sL = fminf(unL - cL, us - cs);
-            sR = fmaxf(us + cs, unR + cR);
-        }
-        float qL = HsL * unL, qR = HsR * unR;
-        float FL0 = qL, FL1 = qL * unL + half_g * HsL * ds, FL2 = qL * utL;
-        float FR0 = qR, FR1 = qR * unR - half_g * HsR * ds, FR2 = qR * utR;
-        // HLL with the speeds clamped to a <= 0 <= b, which also gives F_L when
-        // sL >= 0 and F_R when sR <= 0 (b - a > 0 unless both sides are dry)
-        const float a = fminf(sL, 0.f), b = fmaxf(sR, 0.f);
-        const float rden = rcp_approx(b - a), ab = a * b;
-        F[0] = ((b * FL0 - a * FR0) - ab * ds) * rden;
-        F[1] = ((b * FL1 - a * FR1) + ab * (qR - qL)) * rden;
-        F[2] = ((b * FL2 - a * FR2) + ab * (HsR * utR - HsL * utL)) * rden;
-        amax = fmaxf(fabsf(sL), fabsf(sR));
-    }
-    Phi[0] = F[0];
-    Phi[1] = F[1] * nx - F[2] * ny;
-    Phi[2] = F[1] * ny + F[2] * nx;
-    float HL = eL - zL, HR = eR - zR;
-    QL = half_g * ((efL - eL) * (HfL + HL) - HsL * ds);
-    QR = half_g * ((efR - eR) * (HfR + HR) + HsR * ds);
 }
 
 // An exactly dry cell: no water and no momentum.
 template <typename real>
-__device__ __forceinline__ bool exactly_dry(real W, real Hu, real Hv, real zc)
+__device__ __forceinline__ bool exactly_dry(real H, real Hu, real Hv)
 {
-    const real H = EtaForm<real>::value ? W - zc : W;
     return is_zero(H) && is_zero(Hu) && is_zero(Hv);
 }
 
 // Stored state of cell gid as seen by the stage, and its bed.
 template <typename real, int STAGE>
 __device__ __forceinline__ bool stage_cell(const KArgs<real> &a, int gid, real dt, real &W, real &Hu, real &Hv,
-                                           real &zc, real *wn = nullptr)
+                                           real &zc)
 {
     zc = a.z[gid];
-    return stage_state<real, STAGE>(a, gid, dt, zc, W, Hu, Hv, wn);
+    return stage_state<real, STAGE>(a, gid, dt, W, Hu, Hv);
 }
 
-// Four reals in shared memory, moved as one 16-byte (FP32) or two 16-byte
-// (FP64) accesses.
-__device__ __forceinline__ void ld4(const float *p, float &x, float &y, float &z, float &w)
-{
-    float4 v = *reinterpret_cast<const float4 *>(p);
-    x = v.x; y = v.y; z = v.z; w = v.w;
-}
-__device__ __forceinline__ void st4(float *p, float x, float y, float z, float w)
-{
-    *reinterpret_cast<float4 *>(p) = make_float4(x, y, z, w);
-}
+// Four reals in shared memory, moved as two 16-byte accesses.
 __device__ __forceinline__ void ld4(const double *p, double &x, double &y, double &z, double &w)
 {
     double2 a = reinterpret_cast<const double2 *>(p)[0], b = reinterpret_cast<const double2 *>(p)[1];
@@ -507,26 +367,17 @@ __device__ __forceinline__ void st4(double *p, double x, double y, double z, dou
 // threshold), 2 negative depth emptied.
 template <typename real>
 __device__ __forceinline__ uint8_t rk2_final(const real x[3], real W1, real Hu1, real Hv1, real RH, real RHu,
-                                             real RHv, real dt, real z1, real hthr, real &W, real &Hu, real &Hv)
+                                             real RHv, real dt, real hthr, real &W, real &Hu, real &Hv)
 {
-    constexpr bool ETA = EtaForm<real>::value;
-    if constexpr (ETA) {
-        W = real(0.5) * x[0] + real(0.5) * (W1 + dt * RH);
-        Hu = real(0.5) * x[1] + real(0.5) * (Hu1 + dt * RHu);
-        Hv = real(0.5) * x[2] + real(0.5) * (Hv1 + dt * RHv);
-    } else {
-        // x / 2 + y / 2 rounded once is (x + y) / 2 rounded once
-        W = half_of(x[0] + (W1 + dt * RH));
-        Hu = half_of(x[1] + (Hu1 + dt * RHu));
-        Hv = half_of(x[2] + (Hv1 + dt * RHv));
-    }
-    const real H = ETA ? W - z1 : W;
-    if (is_neg(H)) {
-        W = ETA ? z1 : real(0);
-        Hu = real(0); Hv = real(0);
+    // x / 2 + y / 2 rounded once is (x + y) / 2 rounded once
+    W = half_of(x[0] + (W1 + dt * RH));
+    Hu = half_of(x[1] + (Hu1 + dt * RHu));
+    Hv = half_of(x[2] + (Hv1 + dt * RHv));
+    if (is_neg(W)) {
+        W = real(0); Hu = real(0); Hv = real(0);
         return 2;
     }
-    if (!gt_nn(H, hthr)) {
+    if (!gt_nn(W, hthr)) {
         Hu = real(0); Hv = real(0);
         return 1;
     }
@@ -542,12 +393,9 @@ __device__ __forceinline__ void finish_cell(const KArgs<real> &a, int gid, const
                                             real aHv, real am, const real x[3], real area, real rarea, real dt,
                                             real &my_min, long long &my_neg, bool &bad)
 {
-    constexpr bool ETA = EtaForm<real>::value;
     const int nc = (int)a.nc;
     real RH, RHu, RHv;
-    if constexpr (ETA) {
-        RH = -aH / area; RHu = -aHu / area; RHv = -aHv / area;
-    } else if constexpr (FAST) {
+    if constexpr (FAST) {
         RH = -aH * rarea; RHu = -aHu * rarea; RHv = -aHv * rarea;
     } else {
         const Recip ra = recip_given(area, rarea);
@@ -558,13 +406,9 @@ __device__ __forceinline__ void finish_cell(const KArgs<real> &a, int gid, const
         a.R0[nc + gid] = RHu;
         a.R0[2 * nc + gid] = RHv;
         real bnd = real_inf<real>();
-        if (is_pos(am)) {
-            if constexpr (ETA) bnd = area / (real(3) * am);
-            else bnd = quot(area, recip(real(3) * am));
-        }
+        if (is_pos(am)) bnd = quot(area, recip(real(3) * am));
         my_min = smin(my_min, bnd);
-        if constexpr (!ETA)
-            if (a.bound_out) a.bound_out[gid] = bnd;
+        if (a.bound_out) a.bound_out[gid] = bnd;
     } else {
         if (a.r1_out) {
             a.r1_out[gid] = RH;
@@ -574,7 +418,7 @@ __device__ __forceinline__ void finish_cell(const KArgs<real> &a, int gid, const
         real W1, Hu1, Hv1, z1;
         ld4(sWl, W1, Hu1, Hv1, z1);
         real W, Hu, Hv;
-        const uint8_t branch = rk2_final(x, W1, Hu1, Hv1, RH, RHu, RHv, dt, z1, a.hthr, W, Hu, Hv);
+        const uint8_t branch = rk2_final(x, W1, Hu1, Hv1, RH, RHu, RHv, dt, a.hthr, W, Hu, Hv);
         if (branch == 2) my_neg++;
         if (a.mask2) a.mask2[gid] = branch;
         if (!isfinite(W) || !isfinite(Hu) || !isfinite(Hv)) bad = true;
@@ -585,18 +429,15 @@ __device__ __forceinline__ void finish_cell(const KArgs<real> &a, int gid, const
 }
 
 // Shared memory of one CTA: cell states [L] x 4, face slots [3][L1] x 4 (L1 =
-// block + ring 1), with gids the global ids of block and ring-1 cells [L1],
-// face codes and owned-face queue [3B] each, and for FP64 one byte per block and
-// ring-1 cell: whether it reconstructed (phase D adds its bed-slope source).  Without gids phase B reads a
-// ring-1 cell's global id again from the halo list: at 6 CTAs per SM every
-// kilobyte of shared memory is a kilobyte less of L1.  The batched kernels keep
-// the ids (their extra scenario state leaves no register for the reload).
-template <typename real>
-__host__ __device__ inline size_t stage_smem_bytes(int block, int max_halo, int max_ring1, bool gids = false)
+// block + ring 1), with gids the global ids of block and ring-1 cells [L1], face
+// codes and owned-face queue [3B] each, and one byte per block and ring-1 cell:
+// whether it reconstructed (phase D adds its bed-slope source).  Without gids phase
+// B reads a ring-1 cell's global id again from the halo list.
+template <>
+__host__ __device__ inline size_t stage_smem_bytes<double>(int block, int max_halo, int max_ring1, int, bool gids)
 {
     size_t L = (size_t)block + max_halo, L1 = (size_t)block + max_ring1;
-    return sizeof(real) * 4 * (L + 3 * L1) + (gids ? sizeof(int32_t) * L1 : 0) + sizeof(uint16_t) * 6 * (size_t)block +
-           (sizeof(real) == 8 ? L1 : 0) + 16;
+    return sizeof(double) * 4 * (L + 3 * L1) + (gids ? sizeof(int32_t) * L1 : 0) + sizeof(uint16_t) * 6 * (size_t)block + L1 + 16;
 }
 
 // One block of cells for one scenario: phases A-D (see the top of this file).
@@ -619,8 +460,7 @@ __host__ __device__ inline size_t stage_smem_bytes(int block, int max_halo, int 
 // counter is reset in phase D, which may come after other warps have started
 // the next block).
 //
-// Shared layout: sW[l] = (W, Hu, Hv, z) of local cell l (W = eta for FP32, H
-// for FP64); sF[f][l] = face values (W_f, Hu_f, Hv_f, z_f) of face f of cell l
+// Shared layout: sW[l] = (H, Hu, Hv, z) of local cell l; sF[f][l] = face values (W_f, Hu_f, Hv_f, z_f) of face f of cell l
 // after phase B, z_f the bed the face value stands on, and after phase C the
 // cell's own term (l_f Phi_0, l_f (Phi_1 + P n_x), l_f (Phi_2 + P n_y), l_f a_f).
 // Stage 2's phase D reads w^n of its cell from global memory.
@@ -640,7 +480,6 @@ __device__ __forceinline__ void process_block(const KArgs<real> &a, const int b,
     uint16_t *queue = sCode + 3 * B;                              // [3B]
     uint8_t *sRec = reinterpret_cast<uint8_t *>(queue + 3 * B);   // [L1]
 
-    constexpr bool ETA = EtaForm<real>::value;
     const int tid = threadIdx.x;
     const real g = a.g, half_g = a.half_g, hthr = a.hthr;
     const real *geo = a.geo;
@@ -678,34 +517,18 @@ __device__ __forceinline__ void process_block(const KArgs<real> &a, const int b,
             }
             real W, Hu, Hv, zc;
             bool neg = stage_cell<real, STAGE>(a, gid, dt, W, Hu, Hv, zc);
-            if constexpr (ETA) {
-                // a wet cell may reconstruct: phase B reads its geometry record and
-                // face beds right after the barrier below, so start bringing them
-                // into L1 (a dry cell reads neither)
-                if (W - zc > hthr) {
-                    prefetch_l1(g32(geo, gid));
-                    prefetch_l1(reinterpret_cast<const float2 *>(a.zf) + gid);
-                }
-            }
             if (neg) my_neg++;
             st4(sW + 4 * tid, W, Hu, Hv, zc);
             if constexpr (GIDS) sGid[tid] = gid;
-            dry = exactly_dry(W, Hu, Hv, zc);
+            dry = exactly_dry(W, Hu, Hv);
         }
         if (gh >= 0) {
             real W, Hu, Hv, zc;
             stage_cell<real, STAGE>(a, gh, dt, W, Hu, Hv, zc);
-            if constexpr (ETA) {
-                if (tid < n1 && W - zc > hthr) {     // a wet ring-1 cell: phase B reconstructs it too
-                    prefetch_l1(g32(geo, gh));
-                    prefetch_l1(reinterpret_cast<const float2 *>(a.zf) + gh);
-                    prefetch_l1(a.ring1_nbr + 3 * (h0 + tid));
-                }
-            }
             st4(sW + 4 * (B + tid), W, Hu, Hv, zc);
             if (tid < n1) {
                 if constexpr (GIDS) sGid[B + tid] = gh;
-                dry = dry && exactly_dry(W, Hu, Hv, zc);
+                dry = dry && exactly_dry(W, Hu, Hv);
             }
         }
         for (int h = tid + blockDim.x; h < nh; h += blockDim.x) {
@@ -715,7 +538,7 @@ __device__ __forceinline__ void process_block(const KArgs<real> &a, const int b,
             st4(sW + 4 * (B + h), W, Hu, Hv, zc);
             if (h < n1) {
                 if constexpr (GIDS) sGid[B + h] = gid;
-                dry = dry && exactly_dry(W, Hu, Hv, zc);
+                dry = dry && exactly_dry(W, Hu, Hv);
             }
         }
         if constexpr (!LISTED) {
@@ -745,13 +568,12 @@ __device__ __forceinline__ void process_block(const KArgs<real> &a, const int b,
     if constexpr (DRY == 0)
         __syncthreads();
     else
-        skip = __syncthreads_and(dry) && (DRY == 1 || (!a.fv_out && !a.mask2 && !a.r1_out && (ETA || !a.rec_out)));
+        skip = __syncthreads_and(dry) && (DRY == 1 || (!a.fv_out && !a.mask2 && !a.r1_out && !a.rec_out));
     if (DRY == 1 && skip) {
         if (!LISTED && tid == 0) qcount = 0;
         if (tid < ncell) {
             const int gid = c0 + tid;
-            if constexpr (!ETA)
-                if (a.rec_out) a.rec_out[gid] = 0;
+            if (a.rec_out) a.rec_out[gid] = 0;
             if (a.fv_out) {
                 real Wc, Huc, Hvc, zc;
                 ld4(sW + 4 * tid, Wc, Huc, Hvc, zc);
@@ -780,13 +602,13 @@ __device__ __forceinline__ void process_block(const KArgs<real> &a, const int b,
         if (zero_terms) {
 #pragma unroll
             for (int f = 0; f < 3; f++) st4(sF + 4 * (f * L1 + l), real(0), real(0), real(0), real(0));
-            if constexpr (!ETA) sRec[l] = 0;
+            sRec[l] = 0;
             continue;
         }
         real WK, HuK, HvK, zK;
         ld4(sW + 4 * l, WK, HuK, HvK, zK);
-        const real HK = ETA ? WK - zK : WK;
-        real qK[3] = {ETA ? WK : HK + zK, HuK, HvK};
+        const real HK = WK;
+        real qK[3] = {HK + zK, HuK, HvK};
         real qn[3][3];
         bool recon = (a.order == 2) && gt_nn(HK, hthr);
 #pragma unroll
@@ -801,10 +623,9 @@ __device__ __forceinline__ void process_block(const KArgs<real> &a, const int b,
                 nl = code;
             }
             if (code < NBR_ABSORB) {
-                real Wj, Huj, Hvj, zj;
-                ld4(sW + 4 * nl, Wj, Huj, Hvj, zj);
-                const real Hj = ETA ? Wj - zj : Wj;
-                qn[f][0] = ETA ? Wj : Hj + zj;
+                real Hj, Huj, Hvj, zj;
+                ld4(sW + 4 * nl, Hj, Huj, Hvj, zj);
+                qn[f][0] = Hj + zj;
                 qn[f][1] = Huj;
                 qn[f][2] = Hvj;
                 if (!gt_nn(Hj, hthr)) recon = false;
@@ -814,13 +635,7 @@ __device__ __forceinline__ void process_block(const KArgs<real> &a, const int b,
                 qn[f][1] = HuK;
                 qn[f][2] = HvK;
             } else {
-                real nxf, nyf;
-                if constexpr (ETA) {
-                    float2 nf = g32_normal(geo, gid, f);
-                    nxf = nf.x; nyf = nf.y;
-                } else {
-                    nxf = geo[(GEO_NX + f) * nc + gid]; nyf = geo[(GEO_NY + f) * nc + gid];
-                }
+                const real nxf = geo[(GEO_NX + f) * nc + gid], nyf = geo[(GEO_NY + f) * nc + gid];
                 real mn = HuK * nxf + HvK * nyf;
                 qn[f][0] = qK[0];
                 qn[f][1] = HuK - real(2) * mn * nxf;
@@ -831,14 +646,8 @@ __device__ __forceinline__ void process_block(const KArgs<real> &a, const int b,
         real zfK[3] = {zK, zK, zK};       // the bed under each face value
         if (recon) {
             real face[3][3];
-            real Mf[2][3];          // FP32: rows 0 and 1 of M
             real fx[3], fy[3], wx[3], wy[3];
-            if constexpr (ETA) {
-                const float4 *r = g32(geo, gid);
-                float4 a0 = r[0], a1 = r[1];
-                Mf[0][0] = a0.x; Mf[0][1] = a0.y; Mf[0][2] = a0.z;
-                Mf[1][0] = a0.w; Mf[1][1] = a1.x; Mf[1][2] = a1.y;
-            } else {
+            {
 #pragma unroll
                 for (int f = 0; f < 3; f++) {
                     fx[f] = geo[(GEO_FX + f) * nc + gid];
@@ -851,31 +660,14 @@ __device__ __forceinline__ void process_block(const KArgs<real> &a, const int b,
             for (int v = 0; v < 3; v++) {
                 real d0 = qn[0][v] - qK[v], d1 = qn[1][v] - qK[v], d2 = qn[2][v] - qK[v];
                 real D[3];
-                if constexpr (ETA) {
-                    D[0] = Mf[0][0] * d0 + Mf[0][1] * d1 + Mf[0][2] * d2;
-                    D[1] = Mf[1][0] * d0 + Mf[1][1] * d1 + Mf[1][2] * d2;
-                    D[2] = -(D[0] + D[1]);
-                } else {
+                {
                     real gx = (wx[0] * d0 + wx[1] * d1) + wx[2] * d2;
                     real gy = (wy[0] * d0 + wy[1] * d1) + wy[2] * d2;
 #pragma unroll
                     for (int f = 0; f < 3; f++) D[f] = gx * fx[f] + gy * fy[f];
                 }
                 real alpha = real(1);
-                if constexpr (ETA) {
-                    float qmax = qK[v], qmin = qK[v];
-#pragma unroll
-                    for (int f = 0; f < 3; f++) {
-                        qmax = fmaxf(qmax, qn[f][v]);
-                        qmin = fminf(qmin, qn[f][v]);
-                    }
-                    // phi_f = |r_f| / |D_f| with r_f = qmax - q_K or q_K - qmin by the
-                    // sign of D_f; D_f = 0 gives +inf or NaN, which fminf ignores
-                    const float up = qmax - qK[v], dn = qK[v] - qmin;
-#pragma unroll
-                    for (int f = 0; f < 3; f++)
-                        alpha = fminf(alpha, (D[f] > 0.f ? up : dn) * rcp_approx(fabsf(D[f])));
-                } else {
+                {
                     // alpha = min(1, min_f r_f / D_f), r_f = q_max - q_K or q_min - q_K by
                     // the sign of D_f.  Rounding is monotone, so q_max - q_K is the
                     // largest of the rounded differences d_j and 0, and the smallest
@@ -906,31 +698,22 @@ __device__ __forceinline__ void process_block(const KArgs<real> &a, const int b,
             }
             // the face values stand on the face beds z_f (the linear bed at the
             // face midpoints); the face depths must stay above the threshold
-            if constexpr (ETA) {
-                const float2 dz = reinterpret_cast<const float2 *>(a.zf)[gid];
-                zfK[0] = zK + dz.x;
-                zfK[1] = zK + dz.y;
-                zfK[2] = zK - (dz.x + dz.y);
-            } else {
 #pragma unroll
-                for (int f = 0; f < 3; f++) zfK[f] = a.zf[f * nc + gid];
-            }
+            for (int f = 0; f < 3; f++) zfK[f] = a.zf[f * nc + gid];
 #pragma unroll
             for (int f = 0; f < 3; f++) {
                 Hf[f] = face[f][0] - zfK[f];
                 if (!gt_nn(Hf[f], hthr)) recon = false;
-                if (ETA) Hf[f] = face[f][0];      // FP32 keeps eta_f
                 Huf[f] = face[f][1];
                 Hvf[f] = face[f][2];
             }
         }
         if (!recon) {
 #pragma unroll
-            for (int f = 0; f < 3; f++) { Hf[f] = ETA ? WK : HK; Huf[f] = HuK; Hvf[f] = HvK; zfK[f] = zK; }
+            for (int f = 0; f < 3; f++) { Hf[f] = HK; Huf[f] = HuK; Hvf[f] = HvK; zfK[f] = zK; }
         }
-        if constexpr (!ETA) sRec[l] = recon ? 1 : 0;
-        if constexpr (!ETA)              // (the adjoint, which reads it, is FP64 only)
-            if (a.rec_out && l < B) a.rec_out[gid] = recon ? 1 : 0;
+        sRec[l] = recon ? 1 : 0;
+        if (a.rec_out && l < B) a.rec_out[gid] = recon ? 1 : 0;
 #pragma unroll
         for (int f = 0; f < 3; f++) st4(sF + 4 * (f * L1 + l), Hf[f], Huf[f], Hvf[f], zfK[f]);
         if (a.fv_out && l < B) {
@@ -961,29 +744,14 @@ __device__ __forceinline__ void process_block(const KArgs<real> &a, const int b,
         real *pR = sF + 4 * (nf * L1 + nl);
         // zL, zR: the bed under each side's face value (its face bed where that
         // cell reconstructed, its cell bed otherwise), from the slots' 4th word
-        real WfL, HufL, HvfL, zL, WL, HuK, HvK, zKL;
-        ld4(pL, WfL, HufL, HvfL, zL);
-        ld4(sW + 4 * l, WL, HuK, HvK, zKL);
-        real WfR = real(0), HufR = real(0), HvfR = real(0), WR = real(0), zR = real(0);
-        if (!wall) {
-            real Huj, Hvj, zKR;
-            ld4(pR, WfR, HufR, HvfR, zR);
-            ld4(sW + 4 * nl, WR, Huj, Hvj, zKR);
-        }
-        real Phi[3], PL, PR, am, nx, ny, len;
-        if constexpr (ETA) {
-            float2 nv = g32_normal(geo, gid, f);
-            nx = nv.x; ny = nv.y;
-            len = g32_len(geo, gid, f);
-            face_flux_dev(g, half_g, hthr, WfL, HufL, HvfL, zL, WL,
-                          WfR, HufR, HvfR, zR, WR, nx, ny, bnd, Phi, PL, PR, am);
-        } else {
-            nx = geo[(GEO_NX + f) * nc + gid];
-            ny = geo[(GEO_NY + f) * nc + gid];
-            len = geo[(GEO_LEN + f) * nc + gid];
-            face_flux<real, FAST>(g, half_g, hthr, WfL, HufL, HvfL, zL,
-                            WfR, HufR, HvfR, zR, nx, ny, bnd, Phi, PL, PR, am);
-        }
+        real HfL, HufL, HvfL, zL;
+        ld4(pL, HfL, HufL, HvfL, zL);
+        real HfR = real(0), HufR = real(0), HvfR = real(0), zR = real(0);
+        if (!wall) ld4(pR, HfR, HufR, HvfR, zR);
+        real Phi[3], PL, PR, am;
+        const real nx = geo[(GEO_NX + f) * nc + gid], ny = geo[(GEO_NY + f) * nc + gid];
+        const real len = geo[(GEO_LEN + f) * nc + gid];
+        face_flux<real, FAST>(g, half_g, hthr, HfL, HufL, HvfL, zL, HfR, HufR, HvfR, zR, nx, ny, bnd, Phi, PL, PR, am);
         const real t0 = len * Phi[0];
         const real la = len * am;
         st4(pL, t0, len * (Phi[1] + PL * nx), len * (Phi[2] + PL * ny), la);
@@ -998,9 +766,7 @@ __device__ __forceinline__ void process_block(const KArgs<real> &a, const int b,
         const int gid = c0 + l;
         real aH = real(0), aHu = real(0), aHv = real(0), am = real(0);
         real x[3];
-        const real area = ETA ? geo[(size_t)gid * G32 + G32_AREA] : geo[GEO_AREA * nc + gid];
-        real rarea = real(0);
-        if constexpr (!ETA) rarea = a.rarea[gid];
+        const real area = geo[GEO_AREA * nc + gid], rarea = a.rarea[gid];
 #pragma unroll
         for (int f = 0; f < 3; f++) {
             real t0, t1, t2;
@@ -1010,10 +776,9 @@ __device__ __forceinline__ void process_block(const KArgs<real> &a, const int b,
             aHv = aHv + t2;
             if (STAGE == 1) am = smax(am, x[f]);
         }
-        if constexpr (!ETA) {
+        {
             // centred bed-slope source of a cell standing on its face beds:
-            // g sum_f l_f z_f (eta_K - z_f / 2) n_f, eta_K = H_K + z_K (the deviation
-            // form carries it in its per-face terms)
+            // g sum_f l_f z_f (eta_K - z_f / 2) n_f, eta_K = H_K + z_K
             if (sRec[l]) {
                 real HKs, Hus, Hvs, zKs;
                 ld4(sW + 4 * l, HKs, Hus, Hvs, zKs);
@@ -1032,29 +797,63 @@ __device__ __forceinline__ void process_block(const KArgs<real> &a, const int b,
     }
 }
 
-// Dry-land shortcut of the single-scenario kernels: leave the block early
-// (mode 1) except in the FP32 stage-2 kernel, which at its 40-register budget
-// spills with that second exit and takes mode 2.  The batched kernels use mode 2.
-template <typename real, int STAGE> struct DryMode { static constexpr int value = 1; };
-template <> struct DryMode<float, 2> { static constexpr int value = 2; };
+}  // namespace vg
 
-// Resident CTAs per SM asked of the register allocator.  The FP32 kernels are
-// latency-bound: 40 registers a thread (no spills in these kernels) and ~48 resident warps
-// beat fewer warps with more registers (6 CTAs of 256 threads: 40 registers;
-// 5: 48; unbounded: 63, 4 CTAs).  FP64 is left unbounded.
+#include "block_f32.cuh"
+
+namespace vg {
+
+// Resident CTAs per SM asked of the register allocator.  FP32 with one thread per
+// cell: five of 256 threads at 48 registers (1M basin, us a step: 68 against 79 with
+// six at 40 registers, which spill and leave less of the SM's memory to L1, and 73
+// with four); two threads per cell are for meshes of one wave, which have registers
+// to spare.  FP64 beyond 256 threads is left unbounded.
 template <typename real, int MAXT> struct StageMinCtas { static constexpr int value = 1; };
-template <> struct StageMinCtas<float, 256> { static constexpr int value = 6; };
-template <> struct StageMinCtas<float, 384> { static constexpr int value = 4; };
-template <> struct StageMinCtas<float, 512> { static constexpr int value = 3; };
+template <> struct StageMinCtas<float, 256> { static constexpr int value = 5; };
+template <> struct StageMinCtas<float, 384> { static constexpr int value = 3; };
+template <> struct StageMinCtas<float, 512> { static constexpr int value = 2; };
 // FP64 with one thread per cell: two CTAs per SM, so that one CTA's phases run
 // while the other waits at a barrier (118-122 registers, no spills)
 template <> struct StageMinCtas<double, 256> { static constexpr int value = 2; };
 // The batched kernels' own budget (their extra scenario state needs the FP64
 // registers of one CTA per SM).
 template <typename real> struct BatchMinCtas { static constexpr int value = 1; };
-template <> struct BatchMinCtas<float> { static constexpr int value = 6; };
+template <> struct BatchMinCtas<float> { static constexpr int value = 4; };
 
-template <typename real, int STAGE, int MAXT, bool FAST = false>
+// One block of a single-scenario stage (BATCH = false) or of a batch's scenario.
+// FP64: the single-scenario kernels leave a dry block early, the batched ones let
+// phase B write zero terms and keep the ids (see process_block).
+template <int STAGE, bool FAST, bool BATCH, bool SOA>
+__device__ __forceinline__ void run_block(const KArgs<double> &a, int b, double dt, unsigned char *smem, int &qcount,
+                                          double &my_min, long long &my_neg, bool &bad)
+{
+    process_block<double, STAGE, BATCH ? 2 : 1, BATCH || STAGE == 2, BATCH, FAST>(a, b, dt, smem, qcount, my_min, my_neg,
+                                                                                  bad);
+}
+template <int STAGE, bool FAST, bool BATCH, bool SOA>
+__device__ __forceinline__ void run_block(const KArgs<float> &a, int b, float dt, unsigned char *smem, int &,
+                                          float &my_min, long long &my_neg, bool &bad)
+{
+    process_block<STAGE, SOA>(a, b, dt, smem, my_min, my_neg, bad);
+}
+
+// w^{n+1} = w^n, bit for bit, by every thread of the launch.
+template <bool SOA>
+__device__ __forceinline__ void copy_state(const KArgs<double> &a, int64_t i0, int64_t stride)
+{
+    for (int64_t i = i0; i < 3 * a.nc; i += stride) a.wout[i] = a.w[i];
+}
+template <bool SOA>
+__device__ __forceinline__ void copy_state(const KArgs<float> &a, int64_t i0, int64_t stride)
+{
+    if constexpr (SOA)
+        for (int64_t i = i0; i < 3 * a.nc; i += stride) a.wout_soa[i] = a.w_soa[i];
+    else
+        for (int64_t i = i0; i < a.nc; i += stride) a.wout[i] = a.w[i];
+}
+
+// SOA (FP32): the states are the caller's [3][nc] arrays (the no-allocation step).
+template <typename real, int STAGE, int MAXT, bool FAST = false, bool SOA = false>
 __global__ void __launch_bounds__(MAXT, StageMinCtas<real, MAXT>::value) stage_kernel(const KArgs<real> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1068,11 +867,8 @@ __global__ void __launch_bounds__(MAXT, StageMinCtas<real, MAXT>::value) stage_k
     // copies w^n to the output buffer, bit for bit (computing w/2 + (w + 0 R)/2
     // would flush the smallest FP32 values to zero), as the batched kernels do
     if (finished(a.t_end, a.sc)) {
-        if (STAGE == 2) {
-            const int64_t n3 = 3 * a.nc;
-            for (int64_t i = blockIdx.x * (int64_t)blockDim.x + tid; i < n3; i += (int64_t)gridDim.x * blockDim.x)
-                a.wout[i] = a.w[i];
-        }
+        if (STAGE == 2)
+            copy_state<SOA>(a, blockIdx.x * (int64_t)blockDim.x + tid, (int64_t)gridDim.x * blockDim.x);
         return;
     }
 
@@ -1087,8 +883,7 @@ __global__ void __launch_bounds__(MAXT, StageMinCtas<real, MAXT>::value) stage_k
 
     int parity = 0;
     for (int b = blockIdx.x; b < a.nblocks; b += gridDim.x, parity ^= 1)
-        process_block<real, STAGE, DryMode<real, STAGE>::value, STAGE == 2, false, FAST>(a, b, dt, smem_raw, qcount[parity],
-                                                                                     my_min, my_neg, bad);
+        run_block<STAGE, FAST, false, SOA>(a, b, dt, smem_raw, qcount[parity], my_min, my_neg, bad);
 
     // CTA-level reductions, then one atomic per CTA
     const int lane = tid & 31, warp = tid >> 5, nwarps = (blockDim.x + 31) >> 5;
@@ -1140,48 +935,73 @@ __device__ __forceinline__ void cta_counts(long long my_neg, bool bad, DevScalar
     }
 }
 
+__device__ __forceinline__ bool cell_update1(const KArgs<double> &a, int gid, double dt, double *w1)
+{
+    const int64_t nc = a.nc;
+    double W, Hu, Hv, zc;
+    const bool neg = stage_cell<double, 2>(a, gid, dt, W, Hu, Hv, zc);
+    w1[gid] = W;
+    w1[nc + gid] = Hu;
+    w1[2 * nc + gid] = Hv;
+    return neg;
+}
+__device__ __forceinline__ bool cell_update1(const KArgs<float> &a, int gid, float dt, float4 *w1)
+{
+    float4 q;
+    const bool neg = stage_cell<2, false>(a, gid, dt, q);
+    w1[gid] = q;
+    return neg;
+}
+__device__ __forceinline__ bool cell_update2(const KArgs<double> &a, int gid, double dt, const double *w1,
+                                             const double *R1, bool &bad)
+{
+    const int64_t nc = a.nc;
+    const double x[3] = {a.w[gid], a.w[nc + gid], a.w[2 * nc + gid]};
+    double W, Hu, Hv;
+    const uint8_t branch = rk2_final(x, w1[gid], w1[nc + gid], w1[2 * nc + gid], R1[gid], R1[nc + gid], R1[2 * nc + gid],
+                                     dt, a.hthr, W, Hu, Hv);
+    if (!isfinite(W) || !isfinite(Hu) || !isfinite(Hv)) bad = true;
+    a.wout[gid] = W;
+    a.wout[nc + gid] = Hu;
+    a.wout[2 * nc + gid] = Hv;
+    return branch == 2;
+}
+__device__ __forceinline__ bool cell_update2(const KArgs<float> &a, int gid, float dt, const float4 *w1, const float4 *R1,
+                                             bool &bad)
+{
+    const float4 r = R1[gid];
+    float4 o;
+    const bool neg = rk_second(a.w[gid], w1[gid], r.x, r.y, r.z, dt, a.hthr, o);
+    if (!isfinite(o.x) || !isfinite(o.y) || !isfinite(o.z)) bad = true;
+    a.wout[gid] = o;
+    return neg;
+}
+
 template <typename real>
-__global__ void __launch_bounds__(256) rk_update1_kernel(const KArgs<real> a, real *w1)
+__global__ void __launch_bounds__(256) rk_update1_kernel(const KArgs<real> a, typename StateWord<real>::type *w1)
 {
     if (finished(a.t_end, a.sc)) return;                 // update 2 copies w^n
     const real dt = cta_step_dt<real>(a.sc, a.cfl, a.dt_fixed, a.dt_max, a.t_end);
-    const int64_t nc = a.nc;
     long long my_neg = 0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nc; i += (int64_t)gridDim.x * blockDim.x) {
-        const int gid = (int)i;
-        real W, Hu, Hv, zc;
-        if (stage_cell<real, 2>(a, gid, dt, W, Hu, Hv, zc)) my_neg++;
-        w1[gid] = W;
-        w1[nc + gid] = Hu;
-        w1[2 * nc + gid] = Hv;
-    }
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.nc; i += (int64_t)gridDim.x * blockDim.x)
+        if (cell_update1(a, (int)i, dt, w1)) my_neg++;
     cta_counts<real>(my_neg, false, a.sc);
 }
 
 template <typename real>
-__global__ void __launch_bounds__(256) rk_update2_kernel(const KArgs<real> a, const real *w1, const real *R1)
+__global__ void __launch_bounds__(256) rk_update2_kernel(const KArgs<real> a, const typename StateWord<real>::type *w1,
+                                                         const typename StateWord<real>::type *R1)
 {
-    const int64_t nc = a.nc;
+    const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
     if (finished(a.t_end, a.sc)) {                       // as the fused kernel: w^n, bit for bit
-        for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < 3 * nc; i += (int64_t)gridDim.x * blockDim.x)
-            a.wout[i] = a.w[i];
+        copy_state<false>(a, i0, stride);
         return;
     }
     const real dt = cta_step_dt<real>(a.sc, a.cfl, a.dt_fixed, a.dt_max, a.t_end);
     long long my_neg = 0;
     bool bad = false;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nc; i += (int64_t)gridDim.x * blockDim.x) {
-        const int gid = (int)i;
-        const real x[3] = {a.w[gid], a.w[nc + gid], a.w[2 * nc + gid]};
-        real W, Hu, Hv;
-        const uint8_t branch = rk2_final(x, w1[gid], w1[nc + gid], w1[2 * nc + gid], R1[gid], R1[nc + gid],
-                                         R1[2 * nc + gid], dt, a.z[gid], a.hthr, W, Hu, Hv);
-        if (branch == 2) my_neg++;
-        if (!isfinite(W) || !isfinite(Hu) || !isfinite(Hv)) bad = true;
-        a.wout[gid] = W;
-        a.wout[nc + gid] = Hu;
-        a.wout[2 * nc + gid] = Hv;
-    }
+    for (int64_t i = i0; i < a.nc; i += stride)
+        if (cell_update2(a, (int)i, dt, w1, R1, bad)) my_neg++;
     cta_counts<real>(my_neg, bad, a.sc);
 }
 
@@ -1198,7 +1018,7 @@ constexpr int kBatchMaxEntries = 512;
 template <typename real>
 struct BatchMesh {
     KArgs<real> a;         // mesh arrays; w, R0, wout, sc point at the mesh's first scenario
-    int64_t stride;        // 3 * nc: distance between scenario slices
+    int64_t stride;        // distance between scenario slices (FP64 3 nc values, FP32 nc float4)
     int n_scen;            // scenarios of this mesh
     int first_item;        // first work item (block) of this mesh in the launch
     int first_entry;       // index of its first scenario among all scenarios
@@ -1208,6 +1028,18 @@ struct BatchMesh {
     double *ring_eta;      // [n_scen][ring_cap][n_gauges] eta at the gauges
     int ring_cap, pad;
 };
+
+__device__ __forceinline__ void copy_cell(const double *wi, double *wo, int c, int nc)
+{
+    wo[c] = wi[c];
+    wo[nc + c] = wi[nc + c];
+    wo[2 * nc + c] = wi[2 * nc + c];
+}
+__device__ __forceinline__ void copy_cell(const float4 *wi, float4 *wo, int c, int) { wo[c] = wi[c]; }
+
+// The free surface of cell c.
+__device__ __forceinline__ double surface(const double *w, const double *z, int c) { return w[c] + z[c]; }
+__device__ __forceinline__ double surface(const float4 *w, const float *, int c) { return (double)w[c].x; }
 
 // Order-preserving integer image of a non-negative value, as 32 bits (FP32) or
 // 64 bits (FP64), kept in shared memory per scenario.
@@ -1251,25 +1083,17 @@ __global__ void __launch_bounds__(256, (BatchMinCtas<real>::value)) batch_stage_
             if (s_done[bm.first_entry + s]) {
                 if (STAGE == 2) {
                     // the state carries over to the other buffer of the pair
-                    const int c = b * bm.a.block + tid, nc = (int)bm.a.nc;
-                    if (tid < bm.a.block && c < nc) {
-                        const real *wi = bm.a.w + s * bm.stride;
-                        real *wo = bm.a.wout + s * bm.stride;
-                        wo[c] = wi[c];
-                        wo[nc + c] = wi[nc + c];
-                        wo[2 * nc + c] = wi[2 * nc + c];
-                    }
+                    const int c = b * bm.a.block + tid;
+                    if (tid < bm.a.block && c < (int)bm.a.nc)
+                        copy_cell(bm.a.w + s * bm.stride, bm.a.wout + s * bm.stride, c, (int)bm.a.nc);
                 }
                 continue;
             }
             KArgs<real> a = bm.a;
-            a.w += s * bm.stride;
-            a.R0 += s * bm.stride;
-            if (STAGE == 2) a.wout += s * bm.stride;
-            a.sc += s;
+            a.to_scenario(s, bm.stride, STAGE == 2);
             const int e = bm.first_entry + s;
             real mn = real_inf<real>();
-            process_block<real, STAGE, 2, true, true, FAST>(a, b, s_dt[e], smem_raw, qcount[parity], mn, my_neg, bad);
+            run_block<STAGE, FAST, true, false>(a, b, s_dt[e], smem_raw, qcount[parity], mn, my_neg, bad);
             parity ^= 1;
             if (STAGE == 1) {
                 unsigned long long bits = warp_min_bits<real>(mn);
@@ -1311,10 +1135,9 @@ __global__ void batch_gauge_kernel(const BatchMesh<real> *meshes, DevScalars *sc
     for (int k = threadIdx.x; k < bm.n_scen * G; k += blockDim.x) {
         const int s = k / G, g = k - s * G;
         if (slot[s] < 0) continue;
-        const real *w = bm.a.wout + s * bm.stride;
+        const auto *w = bm.a.wout + s * bm.stride;
         const int32_t c = bm.gauge_cells[g];
-        bm.ring_eta[((size_t)s * bm.ring_cap + slot[s]) * G + g] =
-            EtaForm<real>::value ? (double)w[c] : (double)(w[c] + z[c]);
+        bm.ring_eta[((size_t)s * bm.ring_cap + slot[s]) * G + g] = surface(w, z, c);
     }
     __syncthreads();
     for (int s = threadIdx.x; s < bm.n_scen; s += blockDim.x) {
@@ -1344,36 +1167,21 @@ __global__ void batch_post_kernel(int n_entries, DevScalars *sc_all, double cfl,
     }
 }
 
+// Kernel arguments; the fields that both precisions have.
 template <typename real>
-KArgs<real> make_args(const DevPtrs &d, const StepParams &p, const void *w_in, void *w_out)
+KArgs<real> common_args(const DevPtrs &d, const StepParams &p)
 {
-    KArgs<real> a;
+    KArgs<real> a{};
     a.nc = d.nc;
     a.block = d.block;
     a.nblocks = d.nblocks;
     a.max_halo = d.max_halo;
     a.max_ring1 = d.max_ring1;
     a.order = p.order;
-    a.geo = static_cast<const real *>(d.geo);
-    a.rarea = d.rarea;
     a.z = static_cast<const real *>(d.z);
-    a.zf = static_cast<const real *>(d.zf);
-    a.nbr = d.nbr;
-    a.nbrl = d.nbrl;
     a.halo_ptr = d.halo_ptr;
     a.halo_n1 = d.halo_n1;
     a.halo_ids = d.halo_ids;
-    a.ring1_nbr = d.ring1_nbr;
-    a.fq_ptr = d.fq_ptr;
-    a.fq = d.fq;
-    a.w = static_cast<const real *>(w_in);
-    a.R0 = static_cast<real *>(d.R0);
-    a.wout = static_cast<real *>(w_out);
-    a.mask2 = d.mask2;
-    a.fv_out = static_cast<real *>(d.fv_out);
-    a.r1_out = static_cast<real *>(d.r1_out);
-    a.rec_out = d.rec_out;
-    a.bound_out = d.bound_out;
     a.sc = d.sc;
     a.g = (real)p.g;
     a.half_g = (real)(0.5 * p.g);
@@ -1386,16 +1194,64 @@ KArgs<real> make_args(const DevPtrs &d, const StepParams &p, const void *w_in, v
     return a;
 }
 
+template <typename real>
+KArgs<real> make_args(const DevPtrs &d, const StepParams &p, const void *w_in, void *w_out, bool soa = false);
+
+template <>
+inline KArgs<double> make_args<double>(const DevPtrs &d, const StepParams &p, const void *w_in, void *w_out, bool)
+{
+    KArgs<double> a = common_args<double>(d, p);
+    a.geo = static_cast<const double *>(d.geo);
+    a.rarea = d.rarea;
+    a.zf = static_cast<const double *>(d.zf);
+    a.nbrl = d.nbrl;
+    a.ring1_nbr = d.ring1_nbr;
+    a.fq_ptr = d.fq_ptr;
+    a.fq = d.fq;
+    a.w = static_cast<const double *>(w_in);
+    a.R0 = static_cast<double *>(d.R0);
+    a.wout = static_cast<double *>(w_out);
+    a.mask2 = d.mask2;
+    a.fv_out = static_cast<double *>(d.fv_out);
+    a.r1_out = static_cast<double *>(d.r1_out);
+    a.rec_out = d.rec_out;
+    a.bound_out = d.bound_out;
+    return a;
+}
+
+template <>
+inline KArgs<float> make_args<float>(const DevPtrs &d, const StepParams &p, const void *w_in, void *w_out, bool soa)
+{
+    KArgs<float> a = common_args<float>(d, p);
+    a.recA = static_cast<const float4 *>(d.geo);
+    a.recB = static_cast<const float4 *>(d.geoB);
+    a.area = d.area32;
+    a.codes = static_cast<const uint2 *>(d.codes);
+    a.ring_codes = static_cast<const uint2 *>(d.ring_codes);
+    a.fr_ptr = d.fq_ptr;
+    a.fr = static_cast<const float4 *>(d.fr);
+    a.max_faces = d.max_faces;
+    a.R0 = static_cast<float4 *>(d.R0);
+    if (soa) {
+        a.w_soa = static_cast<const float *>(w_in);
+        a.wout_soa = static_cast<float *>(w_out);
+    } else {
+        a.w = static_cast<const float4 *>(w_in);
+        a.wout = static_cast<float4 *>(w_out);
+    }
+    return a;
+}
+
 // Kernel instance for a launch: the register budget follows the thread count
 // (launch bounds 256 or 512).
-template <typename real, bool FAST = false>
+template <typename real, bool FAST = false, bool SOA = false>
 void *stage_kernel_ptr(int stage, int threads)
 {
     if (threads <= 256)
-        return stage == 1 ? (void *)stage_kernel<real, 1, 256, FAST> : (void *)stage_kernel<real, 2, 256, FAST>;
+        return stage == 1 ? (void *)stage_kernel<real, 1, 256, FAST, SOA> : (void *)stage_kernel<real, 2, 256, FAST, SOA>;
     if (threads <= 384)
-        return stage == 1 ? (void *)stage_kernel<real, 1, 384, FAST> : (void *)stage_kernel<real, 2, 384, FAST>;
-    return stage == 1 ? (void *)stage_kernel<real, 1, 512, FAST> : (void *)stage_kernel<real, 2, 512, FAST>;
+        return stage == 1 ? (void *)stage_kernel<real, 1, 384, FAST, SOA> : (void *)stage_kernel<real, 2, 384, FAST, SOA>;
+    return stage == 1 ? (void *)stage_kernel<real, 1, 512, FAST, SOA> : (void *)stage_kernel<real, 2, 512, FAST, SOA>;
 }
 
 // The dynamic shared memory limit is an attribute of the kernel function, shared
@@ -1414,7 +1270,7 @@ inline cudaError_t raise_smem_limit(const void *kern, size_t smem)
 template <typename real, bool FAST = false>
 int stage_config(const DevPtrs &d, int stage, LaunchCfg &cfg)
 {
-    cfg.smem = stage_smem_bytes<real>(d.block, d.max_halo, d.max_ring1);
+    cfg.smem = stage_smem_bytes<real>(d.block, d.max_halo, d.max_ring1, d.max_faces);
     const void *kern = stage_kernel_ptr<real, FAST>(stage, d.threads);
     cudaError_t e = raise_smem_limit(kern, cfg.smem);
     if (e != cudaSuccess) return (int)e;
@@ -1422,6 +1278,11 @@ int stage_config(const DevPtrs &d, int stage, LaunchCfg &cfg)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, d.threads, cfg.smem);
     if (e != cudaSuccess) return (int)e;
     if (per_sm < 1) return (int)cudaErrorInvalidConfiguration;
+    if constexpr (std::is_same<real, float>::value) {
+        // the no-allocation step's kernels, loaded here so that the step loads nothing
+        e = raise_smem_limit(stage_kernel_ptr<real, FAST, true>(stage, d.threads), cfg.smem);
+        if (e != cudaSuccess) return (int)e;
+    }
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1431,19 +1292,19 @@ int stage_config(const DevPtrs &d, int stage, LaunchCfg &cfg)
     return 0;
 }
 
-template <typename real, bool FAST = false>
+template <typename real, bool FAST = false, bool SOA = false>
 int launch_stage_args(const KArgs<real> &a, int threads, int stage, const LaunchCfg &c, cudaStream_t s)
 {
     const int t = threads;
     if (t <= 256) {
-        if (stage == 1) stage_kernel<real, 1, 256, FAST><<<c.grid, t, c.smem, s>>>(a);
-        else stage_kernel<real, 2, 256, FAST><<<c.grid, t, c.smem, s>>>(a);
+        if (stage == 1) stage_kernel<real, 1, 256, FAST, SOA><<<c.grid, t, c.smem, s>>>(a);
+        else stage_kernel<real, 2, 256, FAST, SOA><<<c.grid, t, c.smem, s>>>(a);
     } else if (t <= 384) {
-        if (stage == 1) stage_kernel<real, 1, 384, FAST><<<c.grid, t, c.smem, s>>>(a);
-        else stage_kernel<real, 2, 384, FAST><<<c.grid, t, c.smem, s>>>(a);
+        if (stage == 1) stage_kernel<real, 1, 384, FAST, SOA><<<c.grid, t, c.smem, s>>>(a);
+        else stage_kernel<real, 2, 384, FAST, SOA><<<c.grid, t, c.smem, s>>>(a);
     } else {
-        if (stage == 1) stage_kernel<real, 1, 512, FAST><<<c.grid, t, c.smem, s>>>(a);
-        else stage_kernel<real, 2, 512, FAST><<<c.grid, t, c.smem, s>>>(a);
+        if (stage == 1) stage_kernel<real, 1, 512, FAST, SOA><<<c.grid, t, c.smem, s>>>(a);
+        else stage_kernel<real, 2, 512, FAST, SOA><<<c.grid, t, c.smem, s>>>(a);
     }
     return (int)cudaGetLastError();
 }
@@ -1455,11 +1316,12 @@ template <typename real, bool FAST = false>
 int launch_rk_unfused(const DevPtrs &d, const StepParams &p, int part, const void *w_in, void *w_out, void *w1,
                       void *R1, const LaunchCfg &c1, void *stream)
 {
+    using word = typename StateWord<real>::type;
     KArgs<real> a = make_args<real>(d, p, w_in, w_out);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (part == 1) {
-        a.w = static_cast<const real *>(w1);
-        a.R0 = static_cast<real *>(R1);
+        a.w = static_cast<const word *>(w1);
+        a.R0 = static_cast<word *>(R1);
         a.wout = nullptr;
         a.cfl_min = 0;
         return launch_stage_args<real, FAST>(a, d.threads, 1, c1, s);
@@ -1469,34 +1331,27 @@ int launch_rk_unfused(const DevPtrs &d, const StepParams &p, int part, const voi
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const long long want = (d.nc + 255) / 256, cap = 8LL * (sms > 0 ? sms : 1);
     const int grid = (int)(want < 1 ? 1 : want < cap ? want : cap);
-    if (part == 0) rk_update1_kernel<real><<<grid, 256, 0, s>>>(a, static_cast<real *>(w1));
-    else rk_update2_kernel<real><<<grid, 256, 0, s>>>(a, static_cast<const real *>(w1), static_cast<const real *>(R1));
+    if (part == 0) rk_update1_kernel<real><<<grid, 256, 0, s>>>(a, static_cast<word *>(w1));
+    else rk_update2_kernel<real><<<grid, 256, 0, s>>>(a, static_cast<const word *>(w1), static_cast<const word *>(R1));
     return (int)cudaGetLastError();
 }
 
+// soa: the states are [3][nc] arrays (always so in FP64).
 template <typename real, bool FAST = false>
 int launch_stage(const DevPtrs &d, const StepParams &p, int stage, const void *w_in, void *w_out,
-                 const LaunchCfg &c, void *stream)
+                 const LaunchCfg &c, void *stream, bool soa = false)
 {
-    KArgs<real> a = make_args<real>(d, p, w_in, w_out);
+    const KArgs<real> a = make_args<real>(d, p, w_in, w_out, soa);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (d.threads <= 256) {
-        if (stage == 1) stage_kernel<real, 1, 256, FAST><<<c.grid, d.threads, c.smem, s>>>(a);
-        else stage_kernel<real, 2, 256, FAST><<<c.grid, d.threads, c.smem, s>>>(a);
-    } else if (d.threads <= 384) {
-        if (stage == 1) stage_kernel<real, 1, 384, FAST><<<c.grid, d.threads, c.smem, s>>>(a);
-        else stage_kernel<real, 2, 384, FAST><<<c.grid, d.threads, c.smem, s>>>(a);
-    } else {
-        if (stage == 1) stage_kernel<real, 1, 512, FAST><<<c.grid, d.threads, c.smem, s>>>(a);
-        else stage_kernel<real, 2, 512, FAST><<<c.grid, d.threads, c.smem, s>>>(a);
-    }
-    return (int)cudaGetLastError();
+    if constexpr (std::is_same<real, float>::value)
+        if (soa) return launch_stage_args<real, FAST, true>(a, d.threads, stage, c, s);
+    return launch_stage_args<real, FAST, false>(a, d.threads, stage, c, s);
 }
 
 template <typename real, bool FAST = false>
-int batch_config(int block, int max_halo, int max_ring1, int &grid, size_t &smem)
+int batch_config(int block, int max_halo, int max_ring1, int max_faces, int &grid, size_t &smem)
 {
-    smem = stage_smem_bytes<real>(block, max_halo, max_ring1, true);
+    smem = stage_smem_bytes<real>(block, max_halo, max_ring1, max_faces, true);
     int best = 1 << 30;
     for (int stage = 1; stage <= 2; stage++) {
         auto kern = stage == 1 ? batch_stage_kernel<real, 1, FAST> : batch_stage_kernel<real, 2, FAST>;
@@ -1534,7 +1389,7 @@ void fill_batch_mesh(void *dst, const DevPtrs &d, const StepParams &p, const voi
 {
     BatchMesh<real> *bm = static_cast<BatchMesh<real> *>(dst);
     bm->a = make_args<real>(d, p, w_in, w_out);
-    bm->stride = 3 * d.nc;
+    bm->stride = std::is_same<real, float>::value ? d.nc : 3 * d.nc;
     bm->n_scen = n_scen;
     bm->first_item = first_item;
     bm->first_entry = first_entry;

@@ -7,6 +7,8 @@ namespace vg {
 
 namespace {
 
+template <typename real> using word = typename StateWord<real>::type;    // of a state buffer
+
 template <typename real>
 __device__ __forceinline__ unsigned long long inf_bits();
 template <> __device__ __forceinline__ unsigned long long inf_bits<float>() { return (unsigned long long)__float_as_uint(CUDART_INF_F); }
@@ -15,7 +17,7 @@ template <> __device__ __forceinline__ unsigned long long inf_bits<double>() { r
 // Epilogue of one step: t += dt (Sec. 2.3), gauge record (Sec. 3 virtual gauges:
 // eta = H + z of each gauge cell), reset of the CFL minimum for the next step.
 template <typename real>
-__global__ void post_step_kernel(DevPtrs d, StepParams p, const real *w)
+__global__ void post_step_kernel(DevPtrs d, StepParams p, const word<real> *w)
 {
     __shared__ long long rec;
     DevScalars *sc = d.sc;
@@ -44,13 +46,13 @@ __global__ void post_step_kernel(DevPtrs d, StepParams p, const real *w)
         const real *z = static_cast<const real *>(d.z);
         for (int g = threadIdx.x; g < d.n_gauges; g += blockDim.x) {
             int32_t c = d.gauge_cells[g];
-            d.ring_eta[rec * d.n_gauges + g] = EtaForm<real>::value ? (double)w[c] : (double)(w[c] + z[c]);
+            d.ring_eta[rec * d.n_gauges + g] = surface(w, z, c);
         }
     }
 }
 
 template <typename real>
-__global__ void record_gauges_kernel(DevPtrs d, const real *w)
+__global__ void record_gauges_kernel(DevPtrs d, const word<real> *w)
 {
     DevScalars *sc = d.sc;
     long long rec = sc->n_rec;
@@ -61,7 +63,7 @@ __global__ void record_gauges_kernel(DevPtrs d, const real *w)
     const real *z = static_cast<const real *>(d.z);
     for (int g = threadIdx.x; g < d.n_gauges; g += blockDim.x) {
         int32_t c = d.gauge_cells[g];
-        d.ring_eta[rec * d.n_gauges + g] = EtaForm<real>::value ? (double)w[c] : (double)(w[c] + z[c]);
+        d.ring_eta[rec * d.n_gauges + g] = surface(w, z, c);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -94,7 +96,7 @@ __device__ __forceinline__ int ramp_phase(double t, double onset, double rise)
 }
 
 template <typename real>
-__global__ void bed_update_kernel(DevPtrs d, StepParams p, real *w, int at_step_end, double t_set)
+__global__ void bed_update_kernel(DevPtrs d, StepParams p, word<real> *w, int at_step_end, double t_set)
 {
     __shared__ double s_t[2];        // the stored bed's time and the new one's, formed once per CTA
     if (threadIdx.x == 0) {
@@ -105,8 +107,6 @@ __global__ void bed_update_kernel(DevPtrs d, StepParams p, real *w, int at_step_
     const double t0 = s_t[0], t = s_t[1];
     const Recip by_rise = recip_given(d.bed_rise, d.bed_rrise), by_3 = recip_given(3.0, 1.0 / 3.0);
     real *z = static_cast<real *>(const_cast<void *>(d.z));
-    void *zf = const_cast<void *>(d.zf);
-    double *z64 = const_cast<double *>(d.z64);
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < d.nc; k += (int64_t)gridDim.x * blockDim.x) {
         int32_t v[3];
         double onset[3];
@@ -130,61 +130,101 @@ __global__ void bed_update_kernel(DevPtrs d, StepParams p, real *w, int at_step_
         }
         const double zn = -quot(__dadd_rn(__dadd_rn(dv[0], dv[1]), dv[2]), by_3);
         // face beds: -(mean of the face's two vertex depths); FP32 keeps z_f - z_K
-        // of faces 0 and 1
+        // of faces 0 and 1, beside its reconstruction matrix
         double zfn[3];
 #pragma unroll
         for (int f = 0; f < 3; f++) zfn[f] = -half_of(__dadd_rn(dv[f], dv[(f + 1) % 3]));
-        if (EtaForm<real>::value)
-            reinterpret_cast<float2 *>(zf)[k] = make_float2((float)(zfn[0] - zn), (float)(zfn[1] - zn));
-        else
-            for (int f = 0; f < 3; f++) reinterpret_cast<double *>(zf)[f * d.nc + k] = zfn[f];
-        if (EtaForm<real>::value) {
-            // eta form: keep H = eta - z; a dry cell (eta == z) stays exactly dry
-            const real zo = z[k], zr = (real)zn;
-            if (w && zr != zo) {
-                const real e = w[k];
-                w[k] = e - zo <= real(0) ? zr : (e - zo) + zr;
+        if constexpr (std::is_same<real, float>::value) {
+            float *recA = static_cast<float *>(const_cast<void *>(d.geo));
+            *reinterpret_cast<float2 *>(recA + 8 * k + 6) = make_float2((float)(zfn[0] - zn), (float)(zfn[1] - zn));
+            // keep H = eta - z; a dry cell (eta == z) stays exactly dry
+            const float zr = (float)zn;
+            if (w) {
+                float4 q = w[k];
+                if (zr != q.w) {
+                    q.x = q.x - q.w <= 0.f ? zr : (q.x - q.w) + zr;
+                    q.w = zr;
+                    w[k] = q;
+                }
             }
             z[k] = zr;
-            z64[k] = zn;
+            const_cast<double *>(d.z64)[k] = zn;
         } else {
-            z[k] = (real)zn;
+            double *zf = static_cast<double *>(const_cast<void *>(d.zf));
+            for (int f = 0; f < 3; f++) zf[f * d.nc + k] = zfn[f];
+            z[k] = zn;
         }
     }
 }
 
-// State in (original order, H) -> internal order, stored form (H, or eta = H + z
-// formed with the FP64 bed before rounding to FP32, so still water at a common
-// level gets exactly the same eta everywhere).
+// FP32: the bed of every cell of a state buffer, eta kept.
+__global__ void state_bed_kernel(int64_t nc, const float *z, float4 *w)
+{
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nc; k += (int64_t)gridDim.x * blockDim.x)
+        w[k].w = z[k];
+}
+
+// One cell's state (H, Hu, Hv) in a state buffer; zk the FP64 bed (FP32: eta = H + z
+// formed with it before rounding, so still water at a common level gets exactly
+// the same eta everywhere).
+template <typename src_t>
+__device__ __forceinline__ void store_cell(double *w, int64_t nc, int64_t k, src_t h, src_t hu, src_t hv, double)
+{
+    w[k] = (double)h;
+    w[nc + k] = (double)hu;
+    w[2 * nc + k] = (double)hv;
+}
+template <typename src_t>
+__device__ __forceinline__ void store_cell(float4 *w, int64_t, int64_t k, src_t h, src_t hu, src_t hv, double zk)
+{
+    w[k] = make_float4((float)((double)h + zk), (float)hu, (float)hv, (float)zk);
+}
+
+// The inverse.  FP32: a cell is dry when eta <= z in the kernels' own (rounded)
+// bed, and then H is exactly 0.
+template <typename dst_t>
+__device__ __forceinline__ void fetch_cell(const double *w, int64_t nc, int64_t k, double, dst_t &h, dst_t &hu, dst_t &hv)
+{
+    h = (dst_t)w[k];
+    hu = (dst_t)w[nc + k];
+    hv = (dst_t)w[2 * nc + k];
+}
+template <typename dst_t>
+__device__ __forceinline__ void fetch_cell(const float4 *w, int64_t, int64_t k, double zk, dst_t &h, dst_t &hu, dst_t &hv)
+{
+    const float4 q = w[k];
+    h = (dst_t)((q.x - q.w <= 0.f) ? 0.0 : fmax(0.0, (double)q.x - zk));
+    hu = (dst_t)q.y;
+    hv = (dst_t)q.z;
+}
+
+// State in (original order, H) -> internal order, stored form.
 template <typename real, typename src_t>
 __global__ void import_state_kernel(int64_t nc, const int32_t *old_of_new, const src_t *H,
-                                    const src_t *Hu, const src_t *Hv, const double *z, real *w, DevScalars *sc)
+                                    const src_t *Hu, const src_t *Hv, const double *z, word<real> *w, DevScalars *sc)
 {
     bool bad = false;
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nc; k += (int64_t)gridDim.x * blockDim.x) {
         int64_t o = old_of_new[k];
         src_t h = H[o], hu = Hu[o], hv = Hv[o];
         if (!(h >= src_t(0)) || !isfinite(h) || !isfinite(hu) || !isfinite(hv)) bad = true;
-        w[k] = EtaForm<real>::value ? (real)((double)h + (double)z[k]) : (real)h;
-        w[nc + k] = (real)hu;
-        w[2 * nc + k] = (real)hv;
+        store_cell(w, nc, k, h, hu, hv, std::is_same<real, float>::value ? z[k] : 0.0);
     }
     if (bad) atomicOr(&sc->flags, FLAG_BAD_INPUT);
 }
 
-// Internal order, stored form -> original order, H.  In the eta form a cell is
-// dry when eta <= z in the kernels' own (rounded) bed, and then H is exactly 0.
+// Internal order, stored form -> original order, H.
 template <typename real, typename dst_t>
-__global__ void export_state_kernel(int64_t nc, const int32_t *old_of_new, const real *w, const real *zr,
-                                    const double *z, dst_t *H, dst_t *Hu, dst_t *Hv)
+__global__ void export_state_kernel(int64_t nc, const int32_t *old_of_new, const word<real> *w, const double *z, dst_t *H,
+                                    dst_t *Hu, dst_t *Hv)
 {
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nc; k += (int64_t)gridDim.x * blockDim.x) {
         int64_t o = old_of_new[k];
-        double h = (double)w[k];
-        if (EtaForm<real>::value) h = (w[k] - zr[k] <= real(0)) ? 0.0 : fmax(0.0, h - z[k]);
-        H[o] = (dst_t)h;
-        Hu[o] = (dst_t)w[nc + k];
-        Hv[o] = (dst_t)w[2 * nc + k];
+        dst_t h, hu, hv;
+        fetch_cell(w, nc, k, std::is_same<real, float>::value ? z[k] : 0.0, h, hu, hv);
+        H[o] = h;
+        Hu[o] = hu;
+        Hv[o] = hv;
     }
 }
 
@@ -200,18 +240,16 @@ template <> struct Vec16<double> { using type = double2; };
 
 template <typename real, typename src_t>
 __device__ __forceinline__ void import_one(int64_t nc, int64_t k, src_t h, src_t hu, src_t hv, double zk,
-                                           real *w, bool &bad)
+                                           word<real> *w, bool &bad)
 {
     if (!(h >= src_t(0)) || !isfinite(h) || !isfinite(hu) || !isfinite(hv)) bad = true;
-    w[k] = EtaForm<real>::value ? (real)((double)h + zk) : (real)h;
-    w[nc + k] = (real)hu;
-    w[2 * nc + k] = (real)hv;
+    store_cell(w, nc, k, h, hu, hv, zk);
 }
 
 // zo: the FP64 bed in the original order (contiguous reads), or null (z[k]).
 template <typename real, typename src_t>
 __global__ void import_state_orig_kernel(int64_t nc, const int32_t *new_of_old, const src_t *H, const src_t *Hu,
-                                         const src_t *Hv, const double *z, const double *zo, real *w,
+                                         const src_t *Hv, const double *z, const double *zo, word<real> *w,
                                          DevScalars *sc, bool vec)
 {
     constexpr int V = 16 / sizeof(src_t);
@@ -228,35 +266,21 @@ __global__ void import_state_orig_kernel(int64_t nc, const int32_t *new_of_old, 
         for (int j = 0; j < V; j++) {
             const int64_t o = gi * V + j, k = new_of_old[o];
             import_one<real, src_t>(nc, k, ph[j], phu[j], phv[j],
-                                    EtaForm<real>::value ? (zo ? zo[o] : z[k]) : 0.0, w, bad);
+                                    std::is_same<real, float>::value ? (zo ? zo[o] : z[k]) : 0.0, w, bad);
         }
     }
     for (int64_t o = ng * V + tid; o < nc; o += stride) {
         const int64_t k = new_of_old[o];
-        import_one<real, src_t>(nc, k, H[o], Hu[o], Hv[o], EtaForm<real>::value ? (zo ? zo[o] : z[k]) : 0.0, w,
+        import_one<real, src_t>(nc, k, H[o], Hu[o], Hv[o], std::is_same<real, float>::value ? (zo ? zo[o] : z[k]) : 0.0, w,
                                 bad);
     }
     if (bad) atomicOr(&sc->flags, FLAG_BAD_INPUT);
 }
 
-// H of internal cell k in the destination type (the eta form is dry at eta <= z
-// in the kernels' own rounded bed, and then H is exactly 0).
+// zo: the FP64 bed in the original order, or null (z[k]).
 template <typename real, typename dst_t>
-__device__ __forceinline__ void export_one(int64_t nc, int64_t k, const real *w, real zrk, double zk, dst_t &h,
-                                           dst_t &hu, dst_t &hv)
-{
-    double x = (double)w[k];
-    if (EtaForm<real>::value) x = (w[k] - zrk <= real(0)) ? 0.0 : fmax(0.0, x - zk);
-    h = (dst_t)x;
-    hu = (dst_t)w[nc + k];
-    hv = (dst_t)w[2 * nc + k];
-}
-
-// zro / zo: the kernels' bed and the FP64 bed in the original order, or null.
-template <typename real, typename dst_t>
-__global__ void export_state_orig_kernel(int64_t nc, const int32_t *new_of_old, const real *w, const real *zr,
-                                         const double *z, const real *zro, const double *zo, dst_t *H, dst_t *Hu,
-                                         dst_t *Hv, bool vec)
+__global__ void export_state_orig_kernel(int64_t nc, const int32_t *new_of_old, const word<real> *w, const double *z,
+                                         const double *zo, dst_t *H, dst_t *Hu, dst_t *Hv, bool vec)
 {
     constexpr int V = 16 / sizeof(dst_t);
     using vt = typename Vec16<dst_t>::type;
@@ -269,10 +293,7 @@ __global__ void export_state_orig_kernel(int64_t nc, const int32_t *new_of_old, 
 #pragma unroll
         for (int j = 0; j < V; j++) {
             const int64_t o = gi * V + j, k = new_of_old[o];
-            real zrk = real(0);
-            double zk = 0.0;
-            if (EtaForm<real>::value) { zrk = zro ? zro[o] : zr[k]; zk = zo ? zo[o] : z[k]; }
-            export_one<real, dst_t>(nc, k, w, zrk, zk, ph[j], phu[j], phv[j]);
+            fetch_cell(w, nc, k, std::is_same<real, float>::value ? (zo ? zo[o] : z[k]) : 0.0, ph[j], phu[j], phv[j]);
         }
         reinterpret_cast<vt *>(H)[gi] = h;
         reinterpret_cast<vt *>(Hu)[gi] = hu;
@@ -280,10 +301,7 @@ __global__ void export_state_orig_kernel(int64_t nc, const int32_t *new_of_old, 
     }
     for (int64_t o = ng * V + tid; o < nc; o += stride) {
         const int64_t k = new_of_old[o];
-        real zrk = real(0);
-        double zk = 0.0;
-        if (EtaForm<real>::value) { zrk = zro ? zro[o] : zr[k]; zk = zo ? zo[o] : z[k]; }
-        export_one<real, dst_t>(nc, k, w, zrk, zk, H[o], Hu[o], Hv[o]);
+        fetch_cell(w, nc, k, std::is_same<real, float>::value ? (zo ? zo[o] : z[k]) : 0.0, H[o], Hu[o], Hv[o]);
     }
 }
 
@@ -291,15 +309,16 @@ constexpr int DIAG_BLOCKS = 1024;
 
 // Fixed grid, fixed reduction tree: the sums do not depend on timing.
 template <typename real>
-__global__ void diag_partial_kernel(int64_t nc, const real *w, const double *z, const real *geo, double hthr,
+__global__ void diag_partial_kernel(int64_t nc, const word<real> *w, const double *z, const real *areas, double hthr,
                                     double *part)
 {
     __shared__ double s_mass[256], s_min[256], s_dry[256];
     double mass = 0.0, mn = CUDART_INF, dry = 0.0;
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nc; k += (int64_t)gridDim.x * blockDim.x) {
-        double h = (double)w[k];
-        if (EtaForm<real>::value) h = h - z[k];
-        double area = EtaForm<real>::value ? (double)geo[(size_t)k * G32 + G32_AREA] : (double)geo[GEO_AREA * nc + k];
+        double h;
+        if constexpr (std::is_same<real, float>::value) h = (double)w[k].x - z[k];
+        else h = w[k];
+        const double area = (double)areas[k];
         mass += area * h;
         mn = fmin(mn, h);
         dry += h <= hthr ? 1.0 : 0.0;
@@ -342,7 +361,7 @@ int launch_post_step(const DevPtrs &d, const StepParams &p, const void *w, int p
 {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (precision == 64) post_step_kernel<double><<<1, 128, 0, s>>>(d, p, static_cast<const double *>(w));
-    else post_step_kernel<float><<<1, 128, 0, s>>>(d, p, static_cast<const float *>(w));
+    else post_step_kernel<float><<<1, 128, 0, s>>>(d, p, static_cast<const float4 *>(w));
     return (int)cudaGetLastError();
 }
 
@@ -354,7 +373,14 @@ int launch_bed_update(const DevPtrs &d, const StepParams &p, void *w, int precis
     if (precision == 64)
         bed_update_kernel<double><<<blocks, 256, 0, s>>>(d, p, static_cast<double *>(w), at_step_end, t_set);
     else
-        bed_update_kernel<float><<<blocks, 256, 0, s>>>(d, p, static_cast<float *>(w), at_step_end, t_set);
+        bed_update_kernel<float><<<blocks, 256, 0, s>>>(d, p, static_cast<float4 *>(w), at_step_end, t_set);
+    return (int)cudaGetLastError();
+}
+
+int launch_state_bed(const DevPtrs &d, void *w, void *stream)
+{
+    state_bed_kernel<<<grid_for(d.nc), 256, 0, static_cast<cudaStream_t>(stream)>>>(d.nc, static_cast<const float *>(d.z),
+                                                                                    static_cast<float4 *>(w));
     return (int)cudaGetLastError();
 }
 
@@ -370,7 +396,7 @@ int launch_record_gauges(const DevPtrs &d, const void *w, int precision, void *s
 {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (precision == 64) record_gauges_kernel<double><<<1, 128, 0, s>>>(d, static_cast<const double *>(w));
-    else record_gauges_kernel<float><<<1, 128, 0, s>>>(d, static_cast<const float *>(w));
+    else record_gauges_kernel<float><<<1, 128, 0, s>>>(d, static_cast<const float4 *>(w));
     return (int)cudaGetLastError();
 }
 
@@ -388,9 +414,9 @@ int launch_import_state(const DevPtrs &d, const int32_t *old_of_new, const void 
     } else {
         const double *z = d.z64;
         if (src_is_double)
-            import_state_kernel<float, double><<<grid, 256, 0, s>>>(d.nc, old_of_new, (const double *)H, (const double *)Hu, (const double *)Hv, z, (float *)w, d.sc);
+            import_state_kernel<float, double><<<grid, 256, 0, s>>>(d.nc, old_of_new, (const double *)H, (const double *)Hu, (const double *)Hv, z, (float4 *)w, d.sc);
         else
-            import_state_kernel<float, float><<<grid, 256, 0, s>>>(d.nc, old_of_new, (const float *)H, (const float *)Hu, (const float *)Hv, z, (float *)w, d.sc);
+            import_state_kernel<float, float><<<grid, 256, 0, s>>>(d.nc, old_of_new, (const float *)H, (const float *)Hu, (const float *)Hv, z, (float4 *)w, d.sc);
     }
     return (int)cudaGetLastError();
 }
@@ -414,9 +440,9 @@ int launch_import_state_orig(const DevPtrs &d, const int32_t *new_of_old, const 
             import_state_orig_kernel<double, float><<<grid, 256, 0, s>>>(d.nc, new_of_old, (const float *)H, (const float *)Hu, (const float *)Hv, z, zo, (double *)w, d.sc, vec);
     } else {
         if (src_is_double)
-            import_state_orig_kernel<float, double><<<grid, 256, 0, s>>>(d.nc, new_of_old, (const double *)H, (const double *)Hu, (const double *)Hv, z, zo, (float *)w, d.sc, vec);
+            import_state_orig_kernel<float, double><<<grid, 256, 0, s>>>(d.nc, new_of_old, (const double *)H, (const double *)Hu, (const double *)Hv, z, zo, (float4 *)w, d.sc, vec);
         else
-            import_state_orig_kernel<float, float><<<grid, 256, 0, s>>>(d.nc, new_of_old, (const float *)H, (const float *)Hu, (const float *)Hv, z, zo, (float *)w, d.sc, vec);
+            import_state_orig_kernel<float, float><<<grid, 256, 0, s>>>(d.nc, new_of_old, (const float *)H, (const float *)Hu, (const float *)Hv, z, zo, (float4 *)w, d.sc, vec);
     }
     return (int)cudaGetLastError();
 }
@@ -430,15 +456,14 @@ int launch_export_state_orig(const DevPtrs &d, const int32_t *new_of_old, const 
     const double *zo = d.z64_orig;
     if (precision == 64) {
         if (dst_is_double)
-            export_state_orig_kernel<double, double><<<grid, 256, 0, s>>>(d.nc, new_of_old, (const double *)w, (const double *)d.z, d.z64, nullptr, zo, (double *)H, (double *)Hu, (double *)Hv, vec);
+            export_state_orig_kernel<double, double><<<grid, 256, 0, s>>>(d.nc, new_of_old, (const double *)w, d.z64, zo, (double *)H, (double *)Hu, (double *)Hv, vec);
         else
-            export_state_orig_kernel<double, float><<<grid, 256, 0, s>>>(d.nc, new_of_old, (const double *)w, (const double *)d.z, d.z64, nullptr, zo, (float *)H, (float *)Hu, (float *)Hv, vec);
+            export_state_orig_kernel<double, float><<<grid, 256, 0, s>>>(d.nc, new_of_old, (const double *)w, d.z64, zo, (float *)H, (float *)Hu, (float *)Hv, vec);
     } else {
-        const float *zro = static_cast<const float *>(d.z_orig);
         if (dst_is_double)
-            export_state_orig_kernel<float, double><<<grid, 256, 0, s>>>(d.nc, new_of_old, (const float *)w, (const float *)d.z, d.z64, zro, zo, (double *)H, (double *)Hu, (double *)Hv, vec);
+            export_state_orig_kernel<float, double><<<grid, 256, 0, s>>>(d.nc, new_of_old, (const float4 *)w, d.z64, zo, (double *)H, (double *)Hu, (double *)Hv, vec);
         else
-            export_state_orig_kernel<float, float><<<grid, 256, 0, s>>>(d.nc, new_of_old, (const float *)w, (const float *)d.z, d.z64, zro, zo, (float *)H, (float *)Hu, (float *)Hv, vec);
+            export_state_orig_kernel<float, float><<<grid, 256, 0, s>>>(d.nc, new_of_old, (const float4 *)w, d.z64, zo, (float *)H, (float *)Hu, (float *)Hv, vec);
     }
     return (int)cudaGetLastError();
 }
@@ -451,15 +476,15 @@ int launch_export_state(const DevPtrs &d, const int32_t *old_of_new, const void 
     if (precision == 64) {
         const double *z = d.z64;
         if (dst_is_double)
-            export_state_kernel<double, double><<<grid, 256, 0, s>>>(d.nc, old_of_new, (const double *)w, (const double *)d.z, z, (double *)H, (double *)Hu, (double *)Hv);
+            export_state_kernel<double, double><<<grid, 256, 0, s>>>(d.nc, old_of_new, (const double *)w, z, (double *)H, (double *)Hu, (double *)Hv);
         else
-            export_state_kernel<double, float><<<grid, 256, 0, s>>>(d.nc, old_of_new, (const double *)w, (const double *)d.z, z, (float *)H, (float *)Hu, (float *)Hv);
+            export_state_kernel<double, float><<<grid, 256, 0, s>>>(d.nc, old_of_new, (const double *)w, z, (float *)H, (float *)Hu, (float *)Hv);
     } else {
         const double *z = d.z64;
         if (dst_is_double)
-            export_state_kernel<float, double><<<grid, 256, 0, s>>>(d.nc, old_of_new, (const float *)w, (const float *)d.z, z, (double *)H, (double *)Hu, (double *)Hv);
+            export_state_kernel<float, double><<<grid, 256, 0, s>>>(d.nc, old_of_new, (const float4 *)w, z, (double *)H, (double *)Hu, (double *)Hv);
         else
-            export_state_kernel<float, float><<<grid, 256, 0, s>>>(d.nc, old_of_new, (const float *)w, (const float *)d.z, z, (float *)H, (float *)Hu, (float *)Hv);
+            export_state_kernel<float, float><<<grid, 256, 0, s>>>(d.nc, old_of_new, (const float4 *)w, z, (float *)H, (float *)Hu, (float *)Hv);
     }
     return (int)cudaGetLastError();
 }
@@ -469,9 +494,9 @@ int launch_diagnostics(const DevPtrs &d, const void *w, int precision, double ht
 {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (precision == 64)
-        diag_partial_kernel<double><<<DIAG_BLOCKS, 256, 0, s>>>(d.nc, (const double *)w, d.z64, (const double *)d.geo, hthr, part);
+        diag_partial_kernel<double><<<DIAG_BLOCKS, 256, 0, s>>>(d.nc, (const double *)w, d.z64, (const double *)d.geo + GEO_AREA * d.nc, hthr, part);
     else
-        diag_partial_kernel<float><<<DIAG_BLOCKS, 256, 0, s>>>(d.nc, (const float *)w, d.z64, (const float *)d.geo, hthr, part);
+        diag_partial_kernel<float><<<DIAG_BLOCKS, 256, 0, s>>>(d.nc, (const float4 *)w, d.z64, d.area32, hthr, part);
     diag_final_kernel<<<1, 32, 0, s>>>(part, DIAG_BLOCKS, out);
     return (int)cudaGetLastError();
 }

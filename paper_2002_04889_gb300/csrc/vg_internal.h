@@ -10,8 +10,8 @@
 namespace vg {
 
 // Per-cell geometry rows, [GEO_ROWS][nc], in the order below (host, and the
-// FP64 device copy; the FP32 device copy is a 16-float record per cell, formed
-// from these rows at upload, layout beside the stage kernels).  Face f of a cell joins its local vertices f and f+1; the local order
+// FP64 device copy; the FP32 device records, formed from these rows at upload, are
+// described in block_f32.cuh).  Face f of a cell joins its local vertices f and f+1; the local order
 // is counter-clockwise from the vertex with the smallest input id.
 enum GeoRow : int {
     GEO_NX = 0,    // 3 rows: outward unit normal x of faces 0..2
@@ -38,6 +38,7 @@ struct HostMesh {
     int32_t nblocks = 0;
     int32_t max_halo = 0;                // max ring-1 + ring-2 cells of a block
     int32_t max_ring1 = 0;               // max ring-1 cells of a block
+    int32_t max_faces = 0;               // max owned faces of a block
     std::vector<int32_t> new_of_old, old_of_new;
     std::vector<int32_t> vtx;            // [nc][3] local-order vertices (original cell order)
     std::vector<double> geo;             // [GEO_ROWS][nc]  (internal order)
@@ -101,19 +102,22 @@ struct StepParams {
 // Device pointers of one context (element type = the context's real).
 struct DevPtrs {
     int64_t nc;
-    int32_t block, nblocks, max_halo, max_ring1, n_gauges, ring_cap;
+    int32_t block, nblocks, max_halo, max_ring1, max_faces, n_gauges, ring_cap;
     int32_t threads;        // threads per CTA of the stage kernels (>= block)
     int32_t fp64_fast;      // FP64: launch the contracted build (step_f64_fast.cu), not the literal one
-    const void *geo;        // FP64: [GEO_ROWS][nc]; FP32: [nc][16] record
+    const void *geo;        // FP64: [GEO_ROWS][nc]; FP32: [nc][8] reconstruction record (recA of
+                            // block_f32.cuh, with the face beds' differences z_f - z_K)
+    const void *geoB;       // FP32: [nc][4] face normals times lengths
+    const float *area32;    // FP32: [nc]
+    const void *codes;      // FP32: [nc] four uint16, neighbours' local slots and wall bits
+    const void *ring_codes; // FP32: the same beside halo_ids for ring-1 cells
+    const void *fr;         // FP32: face records of every block's owned faces (fq_ptr)
     const double *rarea;    // FP64: [nc] 1 / area, correctly rounded (FP32: null)
     const void *z;          // [nc]
-    const void *zf;         // face beds: FP64 [3][nc]; FP32 [nc][2] = (z_f - z_K) of faces 0
-                            // and 1 (face 2: minus their sum, the face midpoints average
-                            // to the centroid)
+    const void *zf;         // FP64: [3][nc] face beds
     const double *z64;      // [nc] FP64 bed (state import/export and diagnostics)
-    const void *z_orig;     // FP32: [nc] the kernels' bed in the original cell order, or null
     const double *z64_orig; // FP32: [nc] the FP64 bed in the original cell order, or null
-                            // (both current only while no moving bed has been set)
+                            // (current only while no moving bed has been set)
     const int32_t *nbr;     // [3][nc]
     const uint16_t *nbrl;   // [3][nc]
     const int32_t *halo_ptr;
@@ -124,7 +128,7 @@ struct DevPtrs {
     const uint16_t *fq;     // owned faces of each block
     const int32_t *adj_faces;   // adjoint: every face once, (cell << 2) | face (cell = lower id or the boundary cell)
     int64_t n_adj_faces;
-    void *R0;               // [3][nc] stage-1 residual (scratch)
+    void *R0;               // stage-1 residual (scratch), laid out as a state
     uint8_t *mask2;         // optional [nc]: stage-2 dry-fix branch per cell (adjoint)
     void *fv_out;           // optional [9][nc]: face values written by the stage kernels (adjoint)
     void *r1_out;           // optional [3][nc]: stage-2 residual written by the stage-2 kernel (adjoint)
@@ -142,18 +146,22 @@ struct DevPtrs {
     double bed_rise, bed_rrise;   // rise time and its reciprocal
 };
 
-// Launch wrappers (defined in step_f32.cu / step_f64.cu).  w_in, w_out are
-// [3][nc] state buffers.  Return cudaError_t as int.
+// Launch wrappers (defined in step_f32.cu / step_f64.cu).  w_in, w_out are state
+// buffers: FP64 [3][nc] (H, Hu, Hv), FP32 [nc] float4 (eta, Hu, Hv, z).  Return
+// cudaError_t as int.
 struct LaunchCfg {
     int grid;        // persistent CTAs
     size_t smem;     // dynamic shared memory per CTA
 };
-size_t stage_smem_f32(int block, int max_halo, int max_ring1);
+size_t stage_smem_f32(int block, int max_halo, int max_ring1, int max_faces);
 size_t stage_smem_f64(int block, int max_halo, int max_ring1);
 int stage_config_f32(const DevPtrs &d, int stage, LaunchCfg &cfg);
 int stage_config_f64(const DevPtrs &d, int stage, LaunchCfg &cfg);
 int launch_stage1_f32(const DevPtrs &d, const StepParams &p, const void *w_in, const LaunchCfg &c, void *stream);
 int launch_stage2_f32(const DevPtrs &d, const StepParams &p, const void *w_in, void *w_out, const LaunchCfg &c, void *stream);
+// FP32 with [3][nc] (eta, Hu, Hv) states of the caller.
+int launch_stage_soa_f32(const DevPtrs &d, const StepParams &p, int stage, const void *w_in, void *w_out, const LaunchCfg &c,
+                         void *stream);
 int launch_stage1_f64(const DevPtrs &d, const StepParams &p, const void *w_in, const LaunchCfg &c, void *stream);
 int launch_stage2_f64(const DevPtrs &d, const StepParams &p, const void *w_in, void *w_out, const LaunchCfg &c, void *stream);
 // Unfused RK stages (vg_params.rk_unfused), after stage 1: part 0 writes
@@ -187,7 +195,7 @@ void fill_batch_mesh_f32(void *dst, const DevPtrs &d, const StepParams &p, const
                          int first_item, int first_entry);
 void fill_batch_mesh_f64(void *dst, const DevPtrs &d, const StepParams &p, const void *w_in, void *w_out, int n_scen,
                          int first_item, int first_entry);
-int batch_config_f32(int block, int max_halo, int max_ring1, int &grid, size_t &smem);
+int batch_config_f32(int block, int max_halo, int max_ring1, int max_faces, int &grid, size_t &smem);
 int batch_config_f64(int block, int max_halo, int max_ring1, int &grid, size_t &smem, bool fast);
 int launch_batch_step_f32(const void *table, int n_mesh, int n_items, int n_entries, DevScalars *sc_all, int block,
                           int grid, size_t smem, const StepParams &p, bool gauges, void *stream);
@@ -246,6 +254,8 @@ int launch_record_gauges(const DevPtrs &d, const void *w, int precision, void *s
 // depth H of the state w (NULL: no state to keep).
 int launch_bed_update(const DevPtrs &d, const StepParams &p, void *w, int precision, bool at_step_end,
                       double t_set, void *stream);
+// FP32: the bed of the state w (NULL: none) set to z, eta kept (vg_set_depth).
+int launch_state_bed(const DevPtrs &d, void *w, void *stream);
 int launch_import_state(const DevPtrs &d, const int32_t *old_of_new, const void *H, const void *Hu,
                         const void *Hv, int src_is_double, void *w, int precision, void *stream);
 int launch_export_state(const DevPtrs &d, const int32_t *old_of_new, const void *w, int precision,

@@ -85,3 +85,28 @@ def test_moving_bed_touches_only_what_moves(rise, t0):
         got = sv.get_state()
     for a, k in zip(got, ("H", "Hu", "Hv")):
         np.testing.assert_array_equal(a, ref[k])
+
+
+@pytest.mark.parametrize("n,jitter", [(8, 0.0), (33, 0.0), (40, 0.2)])
+@pytest.mark.parametrize("boundary", ["wall", "open", "absorbing"])
+def test_fp32_extrema_and_boundaries(n, jitter, boundary):
+    """Single raised and lowered cells over water at rest (every neighbour on one side
+    of the cell, increments that cancel) at and away from the boundary, on a partial
+    last block: finite, and within the FP32 parity bound 1e-4 of FP64."""
+    xy, tri = I.jittered_grid(n, 1.0, seed=2, jitter=jitter)
+    m = I.Mesh(xy, tri, np.full(xy.shape[0], 1.0))
+    H = np.ones(m.nc)
+    H[::17] += 0.25
+    H[5::23] -= 0.25
+    st = (H, np.zeros(m.nc), np.zeros(m.nc))
+    out = []
+    for prec in (32, 64):
+        with volna.Solver(prec) as sv:
+            sv.set_params(h_threshold=1e-5, cfl=0.9)
+            sv.upload_mesh(m)
+            sv.set_boundary(I.boundary_edges(m, lambda p: p[:, 0] > 0.99), boundary)
+            sv.set_state(*st, 0.0)
+            sv.step(5)
+            out.append(sv.get_state())
+    for a, b in zip(*out):
+        assert np.linalg.norm(a - b) <= 1e-4 * np.linalg.norm(b)
