@@ -59,6 +59,7 @@ struct vg_batch {
     int ctas_per_sm = 0;                   // autotuned limit of resident CTAs per SM (0: as many as fit)
     int fit_per_sm = 0;                    // CTAs per SM that fit the current block size
     size_t smem = 0;
+    int scen_at = 0;                       // byte offset of the per-scenario part of the shared memory
     int cur = 0;
     bool dirty = true;
     cudaGraphExec_t graph2 = nullptr;
@@ -166,8 +167,8 @@ int rebuild(vg_batch *b)
         VB_CUDA(b, cudaMalloc(&b->table[parity], eb * nm));
         VB_CUDA(b, cudaMemcpy(b->table[parity], host.data(), eb * nm, cudaMemcpyHostToDevice));
     }
-    int e = b->precision == 64 ? batch_config_f64(block, max_halo, max_ring1, b->grid, b->smem, !b->prm.fp64_literal)
-                               : batch_config_f32(block, max_halo, max_ring1, max_faces, b->grid, b->smem);
+    int e = b->precision == 64 ? batch_config_f64(block, max_halo, max_ring1, b->n_entries, b->grid, b->smem, b->scen_at, !b->prm.fp64_literal)
+                               : batch_config_f32(block, max_halo, max_ring1, max_faces, b->n_entries, b->grid, b->smem, b->scen_at);
     if (e) return bcuda(b, (cudaError_t)e, "batched launch configuration");
     {
         int sms = 0;
@@ -203,9 +204,9 @@ int enqueue_batch_step(vg_batch *b, int parity)
     StepParams p = batch_params(b);
     int e = b->precision == 64
                 ? launch_batch_step_f64(b->table[parity], (int)b->meshes.size(), b->n_items, b->n_entries, b->sc_all,
-                                        block, b->grid, b->smem, p, b->gauges, (void *)b->stream)
+                                        block, b->grid, b->smem, b->scen_at, p, b->gauges, (void *)b->stream)
                 : launch_batch_step_f32(b->table[parity], (int)b->meshes.size(), b->n_items, b->n_entries, b->sc_all,
-                                        block, b->grid, b->smem, p, b->gauges, (void *)b->stream);
+                                        block, b->grid, b->smem, b->scen_at, p, b->gauges, (void *)b->stream);
     if (e) return bcuda(b, (cudaError_t)e, "batched step launch");
     b->launches += b->gauges ? 4 : 3;
     return VG_OK;

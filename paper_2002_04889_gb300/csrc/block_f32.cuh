@@ -60,13 +60,6 @@ struct KArgs<float> {
     float g, half_g, hthr;
     double cfl, dt_fixed, dt_max, t_end;
     int cfl_min;            // stage 1: 1 adds the CFL bound to the step's minimum
-    __device__ __forceinline__ void to_scenario(int s, int64_t stride, bool stage2)
-    {
-        w += s * stride;
-        R0 += s * stride;
-        if (stage2) wout += s * stride;
-        sc += s;
-    }
 };
 
 // Approximate reciprocal (PTX rcp.approx.ftz.f32, max error 1 ulp); rcp(0) = +inf.

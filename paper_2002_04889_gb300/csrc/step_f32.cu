@@ -31,13 +31,13 @@ void fill_batch_mesh_f32(void *dst, const DevPtrs &d, const StepParams &p, const
 {
     fill_batch_mesh<float>(dst, d, p, w_in, w_out, n_scen, first_item, first_entry);
 }
-int batch_config_f32(int block, int max_halo, int max_ring1, int max_faces, int &grid, size_t &smem)
+int batch_config_f32(int block, int max_halo, int max_ring1, int max_faces, int n_entries, int &grid, size_t &smem, int &scen_at)
 {
-    return batch_config<float>(block, max_halo, max_ring1, max_faces, grid, smem);
+    return batch_config<float>(block, max_halo, max_ring1, max_faces, n_entries, grid, smem, scen_at);
 }
 int launch_batch_step_f32(const void *table, int n_mesh, int n_items, int n_entries, DevScalars *sc_all, int block,
-                          int grid, size_t smem, const StepParams &p, bool gauges, void *stream)
+                          int grid, size_t smem, int scen_at, const StepParams &p, bool gauges, void *stream)
 {
-    return launch_batch_step<float>(table, n_mesh, n_items, n_entries, sc_all, block, grid, smem, p, gauges, stream);
+    return launch_batch_step<float>(table, n_mesh, n_items, n_entries, sc_all, block, grid, smem, scen_at, p, gauges, stream);
 }
 }  // namespace vg

@@ -33,18 +33,18 @@ void fill_batch_mesh_f64(void *dst, const DevPtrs &d, const StepParams &p, const
 {
     fill_batch_mesh<double>(dst, d, p, w_in, w_out, n_scen, first_item, first_entry);
 }
-int batch_config_f64(int block, int max_halo, int max_ring1, int &grid, size_t &smem, bool fast)
+int batch_config_f64(int block, int max_halo, int max_ring1, int n_entries, int &grid, size_t &smem, int &scen_at, bool fast)
 {
-    if (fast) return batch_config_f64_fast(block, max_halo, max_ring1, grid, smem);
-    return batch_config<double, false>(block, max_halo, max_ring1, 0, grid, smem);
+    if (fast) return batch_config_f64_fast(block, max_halo, max_ring1, n_entries, grid, smem, scen_at);
+    return batch_config<double, false>(block, max_halo, max_ring1, 0, n_entries, grid, smem, scen_at);
 }
 int launch_batch_step_f64(const void *table, int n_mesh, int n_items, int n_entries, DevScalars *sc_all, int block,
-                          int grid, size_t smem, const StepParams &p, bool gauges, void *stream)
+                          int grid, size_t smem, int scen_at, const StepParams &p, bool gauges, void *stream)
 {
     if (p.fp64_fast)
-        return launch_batch_step_f64_fast(table, n_mesh, n_items, n_entries, sc_all, block, grid, smem, p, gauges,
+        return launch_batch_step_f64_fast(table, n_mesh, n_items, n_entries, sc_all, block, grid, smem, scen_at, p, gauges,
                                           stream);
-    return launch_batch_step<double, false>(table, n_mesh, n_items, n_entries, sc_all, block, grid, smem, p, gauges,
+    return launch_batch_step<double, false>(table, n_mesh, n_items, n_entries, sc_all, block, grid, smem, scen_at, p, gauges,
                                             stream);
 }
 }  // namespace vg

@@ -20,14 +20,14 @@ int launch_rk_unfused_f64_fast(const DevPtrs &d, const StepParams &p, int part, 
 {
     return launch_rk_unfused<double, true>(d, p, part, w_in, w_out, w1, R1, c1, stream);
 }
-int batch_config_f64_fast(int block, int max_halo, int max_ring1, int &grid, size_t &smem)
+int batch_config_f64_fast(int block, int max_halo, int max_ring1, int n_entries, int &grid, size_t &smem, int &scen_at)
 {
-    return batch_config<double, true>(block, max_halo, max_ring1, 0, grid, smem);
+    return batch_config<double, true>(block, max_halo, max_ring1, 0, n_entries, grid, smem, scen_at);
 }
 int launch_batch_step_f64_fast(const void *table, int n_mesh, int n_items, int n_entries, DevScalars *sc_all,
-                               int block, int grid, size_t smem, const StepParams &p, bool gauges, void *stream)
+                               int block, int grid, size_t smem, int scen_at, const StepParams &p, bool gauges, void *stream)
 {
-    return launch_batch_step<double, true>(table, n_mesh, n_items, n_entries, sc_all, block, grid, smem, p, gauges,
+    return launch_batch_step<double, true>(table, n_mesh, n_items, n_entries, sc_all, block, grid, smem, scen_at, p, gauges,
                                            stream);
 }
 }  // namespace vg

@@ -78,13 +78,6 @@ struct KArgs {
     real g, half_g, hthr;
     double cfl, dt_fixed, dt_max, t_end;
     int cfl_min;            // stage 1: 1 adds the CFL bound to the step's minimum
-    __device__ __forceinline__ void to_scenario(int s, int64_t stride, bool stage2)
-    {
-        w += s * stride;
-        R0 += s * stride;
-        if (stage2) wout += s * stride;
-        sc += s;
-    }
 };
 
 // One cell's state in a state buffer: a double of a [3][nc] array, or a float4.
@@ -1050,16 +1043,32 @@ __device__ __forceinline__ unsigned long long warp_min_bits(real v)
     return min_bits(v);
 }
 
+// Shared memory of a batched CTA beside the stage's: per scenario of the batch its
+// CFL minimum, its dt and whether it has reached t_end.
+template <typename real>
+__host__ __device__ inline size_t batch_smem_offset(size_t stage) { return (stage + 15) / 16 * 16; }
+template <typename real>
+__host__ __device__ inline size_t batch_smem_bytes(size_t stage, int n_entries)
+{
+    return batch_smem_offset<real>(stage) + (8 + sizeof(real) + 1) * (size_t)n_entries;
+}
+
+// The block functions read a scenario's arguments from shared memory: from the
+// mesh table in global memory each use was a load, and a copy in registers spilled
+// (the arguments are two hundred bytes).  Three slots: while a CTA's slowest warp
+// may still read the last scenario's and the others the current one's, thread 0
+// fills the next one's.
 template <typename real, int STAGE, bool FAST = false>
 __global__ void __launch_bounds__(256, (BatchMinCtas<real>::value)) batch_stage_kernel(const BatchMesh<real> *meshes, int n_mesh,
-                                                          int n_items, int n_entries, DevScalars *sc_all)
+                                                          int n_items, int n_entries, DevScalars *sc_all, int scen_at)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int qcount[2];
-    __shared__ unsigned long long s_min[kBatchMaxEntries];
-    __shared__ real s_dt[kBatchMaxEntries];
-    __shared__ unsigned char s_done[kBatchMaxEntries];
+    __shared__ __align__(16) unsigned char s_args[3][sizeof(KArgs<real>)];
     __shared__ long long red_neg[32];
+    unsigned long long *s_min = reinterpret_cast<unsigned long long *>(smem_raw + scen_at);
+    real *s_dt = reinterpret_cast<real *>(s_min + n_entries);
+    unsigned char *s_done = reinterpret_cast<unsigned char *>(s_dt + n_entries);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = (blockDim.x + 31) >> 5;
     const KArgs<real> &p0 = meshes[0].a;
     for (int e = tid; e < n_entries; e += blockDim.x) {
@@ -1070,35 +1079,56 @@ __global__ void __launch_bounds__(256, (BatchMinCtas<real>::value)) batch_stage_
         s_done[e] = finished(p0.t_end, sc_all + e) ? 1 : 0;
     }
     if (tid < 2) qcount[tid] = 0;
-    __syncthreads();
     long long my_neg = 0;
-    int parity = 0;
+    int parity = 0, slot = 0, last_m = -1;
     bool bad = false;
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
         int m = 0;
         while (m + 1 < n_mesh && item >= meshes[m + 1].first_item) m++;
         const BatchMesh<real> &bm = meshes[m];
-        const int b = item - bm.first_item;
-        for (int s = 0; s < bm.n_scen; s++) {
-            if (s_done[bm.first_entry + s]) {
-                if (STAGE == 2) {
-                    // the state carries over to the other buffer of the pair
-                    const int c = b * bm.a.block + tid;
-                    if (tid < bm.a.block && c < (int)bm.a.nc)
-                        copy_cell(bm.a.w + s * bm.stride, bm.a.wout + s * bm.stride, c, (int)bm.a.nc);
-                }
-                continue;
-            }
-            KArgs<real> a = bm.a;
-            a.to_scenario(s, bm.stride, STAGE == 2);
-            const int e = bm.first_entry + s;
+        const int b = item - bm.first_item, n_scen = bm.n_scen, e0 = bm.first_entry;
+        const int64_t stride = bm.stride;
+        __syncthreads();             // every thread has done with the last item's arguments
+        if (m != last_m) {
+            const int *src = reinterpret_cast<const int *>(&bm.a);
+            for (int i = tid; i < 3 * (int)(sizeof(KArgs<real>) / 4); i += blockDim.x)
+                reinterpret_cast<int *>(s_args[0])[i] = src[i % (int)(sizeof(KArgs<real>) / 4)];
+            last_m = m;
+            __syncthreads();
+        }
+        auto next = [&](int s) {     // the first scenario from s on that still advances
+            while (s < n_scen && s_done[e0 + s]) s++;
+            return s;
+        };
+        auto fill = [&](int s, int k) {
+            KArgs<real> &a = *reinterpret_cast<KArgs<real> *>(s_args[k]);
+            a.w = bm.a.w + s * stride;
+            a.R0 = bm.a.R0 + s * stride;
+            if (STAGE == 2) a.wout = bm.a.wout + s * stride;
+        };
+        if (STAGE == 2) {
+            // a finished scenario's state carries over to the other buffer of the pair
+            const int c = b * bm.a.block + tid;
+            if (tid < bm.a.block && c < (int)bm.a.nc)
+                for (int s = 0; s < n_scen; s++)
+                    if (s_done[e0 + s]) copy_cell(bm.a.w + s * stride, bm.a.wout + s * stride, c, (int)bm.a.nc);
+        }
+        int s = next(0);
+        if (tid == 0 && s < n_scen) fill(s, slot);
+        __syncthreads();
+        while (s < n_scen) {
+            const int after = next(s + 1), slot2 = slot == 2 ? 0 : slot + 1;
+            if (tid == 0 && after < n_scen) fill(after, slot2);
+            const KArgs<real> &a = *reinterpret_cast<const KArgs<real> *>(s_args[slot]);
             real mn = real_inf<real>();
-            run_block<STAGE, FAST, true, false>(a, b, s_dt[e], smem_raw, qcount[parity], mn, my_neg, bad);
+            run_block<STAGE, FAST, true, false>(a, b, s_dt[e0 + s], smem_raw, qcount[parity], mn, my_neg, bad);
             parity ^= 1;
             if (STAGE == 1) {
                 unsigned long long bits = warp_min_bits<real>(mn);
-                if (lane == 0 && bits != min_bits(real_inf<real>())) atomicMin(&s_min[e], bits);
+                if (lane == 0 && bits != min_bits(real_inf<real>())) atomicMin(&s_min[e0 + s], bits);
             }
+            s = after;
+            slot = slot2;
         }
     }
     for (int o = 16; o > 0; o >>= 1) my_neg += __shfl_xor_sync(0xffffffffu, my_neg, o);
@@ -1349,9 +1379,11 @@ int launch_stage(const DevPtrs &d, const StepParams &p, int stage, const void *w
 }
 
 template <typename real, bool FAST = false>
-int batch_config(int block, int max_halo, int max_ring1, int max_faces, int &grid, size_t &smem)
+int batch_config(int block, int max_halo, int max_ring1, int max_faces, int n_entries, int &grid, size_t &smem, int &scen_at)
 {
-    smem = stage_smem_bytes<real>(block, max_halo, max_ring1, max_faces, true);
+    const size_t stage_bytes = stage_smem_bytes<real>(block, max_halo, max_ring1, max_faces, true);
+    scen_at = (int)batch_smem_offset<real>(stage_bytes);
+    smem = batch_smem_bytes<real>(stage_bytes, n_entries);
     int best = 1 << 30;
     for (int stage = 1; stage <= 2; stage++) {
         auto kern = stage == 1 ? batch_stage_kernel<real, 1, FAST> : batch_stage_kernel<real, 2, FAST>;
@@ -1372,12 +1404,12 @@ int batch_config(int block, int max_halo, int max_ring1, int max_faces, int &gri
 
 template <typename real, bool FAST = false>
 int launch_batch_step(const void *table, int n_mesh, int n_items, int n_entries, DevScalars *sc_all, int block,
-                      int grid, size_t smem, const StepParams &p, bool gauges, void *stream)
+                      int grid, size_t smem, int scen_at, const StepParams &p, bool gauges, void *stream)
 {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const BatchMesh<real> *t = static_cast<const BatchMesh<real> *>(table);
-    batch_stage_kernel<real, 1, FAST><<<grid, block, smem, s>>>(t, n_mesh, n_items, n_entries, sc_all);
-    batch_stage_kernel<real, 2, FAST><<<grid, block, smem, s>>>(t, n_mesh, n_items, n_entries, sc_all);
+    batch_stage_kernel<real, 1, FAST><<<grid, block, smem, s>>>(t, n_mesh, n_items, n_entries, sc_all, scen_at);
+    batch_stage_kernel<real, 2, FAST><<<grid, block, smem, s>>>(t, n_mesh, n_items, n_entries, sc_all, scen_at);
     batch_post_kernel<real><<<1, 256, 0, s>>>(n_entries, sc_all, p.cfl, p.dt_fixed, p.dt_max, p.t_end);
     if (gauges) batch_gauge_kernel<real><<<n_mesh, 256, 0, s>>>(t, sc_all, p.gauge_every);
     return (int)cudaGetLastError();
