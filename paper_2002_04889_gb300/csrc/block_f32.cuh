@@ -336,9 +336,13 @@ __device__ __forceinline__ Smem smem_of(const KArgs<float> &a, unsigned char *ra
 // Hu_f, Hv_f) of face f of cell l after phase B, z_f the bed the face value stands on,
 // and after phase C the cell's own term (three sums, l_f a_f); sS[l] = phase B's own
 // part of the momentum sums.
+//
+// loaded: the block's areas and face records are in shared memory already (a batch's
+// later scenarios of the same block; their records of cells come from L1).
 template <int STAGE, bool SOA>
 __device__ __forceinline__ void process_block(const KArgs<float> &a, const int b, const float dt,
-                                              unsigned char *smem_raw, float &my_min, long long &my_neg, bool &bad)
+                                              unsigned char *smem_raw, float &my_min, long long &my_neg, bool &bad,
+                                              bool &loaded)
 {
     const int B = a.block, tid = threadIdx.x;
     const Smem m = smem_of(a, smem_raw);
@@ -355,11 +359,14 @@ __device__ __forceinline__ void process_block(const KArgs<float> &a, const int b
         if (tid < nh) gh = a.halo_ids[h0 + tid];
         if (tid < ncell) {
             const int gid = c0 + tid;
-            const float area = a.area[gid];
+            float area = 0.f;
+            if (!loaded) area = a.area[gid];
             float4 q = load_w<SOA>(a, gid);
             if (STAGE == 2 && rk_first(q, a.R0[gid], dt, a.hthr)) my_neg++;
-            if (q.x - q.w > a.hthr) prefetch_block_cell(a, gid);
-            m.sArea[tid] = area;
+            if (!loaded) {
+                if (q.x - q.w > a.hthr) prefetch_block_cell(a, gid);
+                m.sArea[tid] = area;
+            }
             m.sW[tid] = q;
             dry = exactly_dry(q);
         }
@@ -368,7 +375,7 @@ __device__ __forceinline__ void process_block(const KArgs<float> &a, const int b
             float4 q = load_w<SOA>(a, gh);
             if (STAGE == 2) rk_first(q, a.R0[gh], dt, a.hthr);
             if (h < n1) {
-                if (q.x - q.w > a.hthr) prefetch_ring_cell(a, gh, h0 + h);
+                if (!loaded && q.x - q.w > a.hthr) prefetch_ring_cell(a, gh, h0 + h);
                 dry = dry && exactly_dry(q);
             }
             m.sW[B + h] = q;
@@ -383,7 +390,9 @@ __device__ __forceinline__ void process_block(const KArgs<float> &a, const int b
     }
     // phase C's face records, on their way into shared memory during phase B
     const int q0 = a.fr_ptr[b], nq = a.fr_ptr[b + 1] - q0;
-    for (int q = tid; q < nq; q += blockDim.x) cp16(m.sFr + q, a.fr + q0 + q);
+    if (!loaded)
+        for (int q = tid; q < nq; q += blockDim.x) cp16(m.sFr + q, a.fr + q0 + q);
+    loaded = true;
 
     // B: face values of block + ring-1 cells (Sec. 2.4, Eq. recon with the
     // Barth-Jespersen limiter); every neighbour is in shared memory

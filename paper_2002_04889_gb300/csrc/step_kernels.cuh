@@ -818,16 +818,16 @@ template <> struct BatchMinCtas<float> { static constexpr int value = 4; };
 // phase B write zero terms and keep the ids (see process_block).
 template <int STAGE, bool FAST, bool BATCH, bool SOA>
 __device__ __forceinline__ void run_block(const KArgs<double> &a, int b, double dt, unsigned char *smem, int &qcount,
-                                          double &my_min, long long &my_neg, bool &bad)
+                                          double &my_min, long long &my_neg, bool &bad, bool &)
 {
     process_block<double, STAGE, BATCH ? 2 : 1, BATCH || STAGE == 2, BATCH, FAST>(a, b, dt, smem, qcount, my_min, my_neg,
                                                                                   bad);
 }
 template <int STAGE, bool FAST, bool BATCH, bool SOA>
 __device__ __forceinline__ void run_block(const KArgs<float> &a, int b, float dt, unsigned char *smem, int &,
-                                          float &my_min, long long &my_neg, bool &bad)
+                                          float &my_min, long long &my_neg, bool &bad, bool &loaded)
 {
-    process_block<STAGE, SOA>(a, b, dt, smem, my_min, my_neg, bad);
+    process_block<STAGE, SOA>(a, b, dt, smem, my_min, my_neg, bad, loaded);
 }
 
 // w^{n+1} = w^n, bit for bit, by every thread of the launch.
@@ -875,8 +875,10 @@ __global__ void __launch_bounds__(MAXT, StageMinCtas<real, MAXT>::value) stage_k
     __syncthreads();
 
     int parity = 0;
-    for (int b = blockIdx.x; b < a.nblocks; b += gridDim.x, parity ^= 1)
-        run_block<STAGE, FAST, false, SOA>(a, b, dt, smem_raw, qcount[parity], my_min, my_neg, bad);
+    for (int b = blockIdx.x; b < a.nblocks; b += gridDim.x, parity ^= 1) {
+        bool loaded = false;
+        run_block<STAGE, FAST, false, SOA>(a, b, dt, smem_raw, qcount[parity], my_min, my_neg, bad, loaded);
+    }
 
     // CTA-level reductions, then one atomic per CTA
     const int lane = tid & 31, warp = tid >> 5, nwarps = (blockDim.x + 31) >> 5;
@@ -1113,6 +1115,7 @@ __global__ void __launch_bounds__(256, (BatchMinCtas<real>::value)) batch_stage_
                 for (int s = 0; s < n_scen; s++)
                     if (s_done[e0 + s]) copy_cell(bm.a.w + s * stride, bm.a.wout + s * stride, c, (int)bm.a.nc);
         }
+        bool loaded = false;
         int s = next(0);
         if (tid == 0 && s < n_scen) fill(s, slot);
         __syncthreads();
@@ -1121,7 +1124,7 @@ __global__ void __launch_bounds__(256, (BatchMinCtas<real>::value)) batch_stage_
             if (tid == 0 && after < n_scen) fill(after, slot2);
             const KArgs<real> &a = *reinterpret_cast<const KArgs<real> *>(s_args[slot]);
             real mn = real_inf<real>();
-            run_block<STAGE, FAST, true, false>(a, b, s_dt[e0 + s], smem_raw, qcount[parity], mn, my_neg, bad);
+            run_block<STAGE, FAST, true, false>(a, b, s_dt[e0 + s], smem_raw, qcount[parity], mn, my_neg, bad, loaded);
             parity ^= 1;
             if (STAGE == 1) {
                 unsigned long long bits = warp_min_bits<real>(mn);
