@@ -1,9 +1,11 @@
 // Hand-written discrete adjoint of the FP64 step (reverse mode), built with
 // --fmad=false like the FP64 forward kernels.
 //
-// The residual R = L(w; z) of Sec. 2 is reversed in four kernels, each thread
-// owning what it writes (no atomics, fixed summation order):
-//   adj_face_values   forward face values FV[3 vars][3 faces][nc] at w
+// The reverse of one step is seven kernels, each thread owning what it writes (no
+// atomics, fixed summation order):
+//   adj_begin         per cell: the reverse of the second stage update, w1 again from
+//                     w and R0, and parts of dt-bar and of the search for the cell
+//                     that set the CFL step
 //   adj_flux_vjp      per owned face: Phi-bar, P-bar from R-bar of both cells,
 //                     reverse of the interface (hydrostatic depths, HLL with its
 //                     branch and speed choices, velocities) -> FV-bar and the
@@ -14,11 +16,15 @@
 //                     of the centred bed-slope source -> the cell's own w-bar,
 //                     cell-bed and face-bed adjoints, and what it sends to each
 //                     face neighbour ((cell, face) slots)
-//   adj_gather        per cell: own part + the slots its neighbours sent to it
+//   adj_gather_mid    per cell: own part + the slots its neighbours sent to it, then
+//                     the reverse of the first stage update, and more of dt-bar
+//   adj_flux_vjp, adj_recon_vjp, adj_gather   the same for stage 1's residual (with
+//                     CFL steps one more CTA of adj_flux_vjp finds the face that set
+//                     dt and reverses its wave speed meanwhile)
+// and the gauges'.  The face values, reconstruction flags, dry-fix branches and CFL
+// bounds are the forward kernels' records.
 // Branches are frozen where the forward run took them; min/max ties resolve to
 // the first argument (the convention of the oracle's taping adjoint).
-// Around them, elementwise kernels reverse the SSP-RK(2,2) stage updates, the
-// dry fixes and the gauge functional.
 #include <cuda_runtime.h>
 
 #include "step_kernels.cuh"
@@ -44,9 +50,54 @@ __device__ __forceinline__ bool gt_abs(double a, double b)    // |a| > |b|
     return (dbits(a) & 0x7fffffffffffffffLL) > (dbits(b) & 0x7fffffffffffffffLL);
 }
 
+// CTA reductions with a fixed order: a warp's shuffle tree, then the warps in turn;
+// thread 0 has the result.
+constexpr int kRedThreads = 256;
+// The two heavy reverse kernels run 64-thread CTAs: what flows back from a few gauges
+// fills a connected part of the mesh, and small CTAs spread it over the SMs (backward
+// of 16 CFL steps, ms, with 128 / 64 / 32 threads: 49k triangles 10.4 / 9.4 / 9.3, 205k
+// 22.9 / 22.6 / 23.2, 1M 92.5 / 86.1 / 87.9).
+constexpr int kVjpThreads = 64;
+
+__device__ __forceinline__ bool cfl_less(double b1, int o1, double b2, int o2)
+{
+    return b1 < b2 || (b1 == b2 && o1 < o2);
+}
+
+template <int NT>
+__device__ __forceinline__ void cta_argmin(double &b, int &o, int &k)
+{
+    __shared__ double sb[NT / 32];
+    __shared__ int so[NT / 32], sk[NT / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int s = 16; s > 0; s >>= 1) {
+        const double b2 = __shfl_down_sync(0xffffffffu, b, s);
+        const int o2 = __shfl_down_sync(0xffffffffu, o, s), k2 = __shfl_down_sync(0xffffffffu, k, s);
+        if (cfl_less(b2, o2, b, o)) { b = b2; o = o2; k = k2; }
+    }
+    if (lane == 0) { sb[warp] = b; so[warp] = o; sk[warp] = k; }
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int w = 1; w < NT / 32; w++)
+            if (cfl_less(sb[w], so[w], b, o)) { b = sb[w]; o = so[w]; k = sk[w]; }
+}
+
+template <int NT>
+__device__ __forceinline__ double cta_sum(double s)
+{
+    __shared__ double sh[NT / 32];
+    for (int k = 16; k > 0; k >>= 1) s += __shfl_down_sync(0xffffffffu, s, k);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int w = 1; w < NT / 32; w++) s += sh[w];
+    return s;
+}
+
 struct AdjMesh {
     int nc, order;
     const double *geo;       // [GEO_ROWS][nc]
+    const double *rarea;     // [nc] 1 / area
     const double *z;         // [nc]
     const double *zf;        // [3][nc] face beds
     const uint8_t *rec;      // [nc] the stage's reconstruction flags (forward record)
@@ -58,6 +109,7 @@ struct AdjMesh {
 };
 
 __device__ __forceinline__ double G(const AdjMesh &m, int row, int k) { return m.geo[row * m.nc + k]; }
+__device__ __forceinline__ Recip by_area(const AdjMesh &m, int k) { return recip_given(G(m, GEO_AREA, k), m.rarea[k]); }
 
 // The bed under face value f of cell K: its face bed where K reconstructed,
 // its cell bed otherwise.
@@ -80,7 +132,7 @@ struct ReconFwd {
     double r[3];             // q_max - q_K or q_min - q_K of the active face
 };
 
-__device__ void recon_forward(const AdjMesh &m, const double *w, int K, ReconFwd &R, double Hf[3],
+__device__ __forceinline__ void recon_forward(const AdjMesh &m, const double *w, int K, ReconFwd &R, double Hf[3],
                               double Huf[3], double Hvf[3])
 {
     const int nc = m.nc;
@@ -91,6 +143,7 @@ __device__ void recon_forward(const AdjMesh &m, const double *w, int K, ReconFwd
     R.qK[1] = HuK;
     R.qK[2] = HvK;
     bool recon = (m.order == 2) && (HK > m.hthr);
+#pragma unroll
     for (int f = 0; f < 3; f++) {
         int j = m.nbr[f * nc + K];
         R.wall[f] = j < 0;
@@ -114,35 +167,57 @@ __device__ void recon_forward(const AdjMesh &m, const double *w, int K, ReconFwd
     }
     if (recon) {
         double face[3][3];
-        for (int v = 0; v < 3; v++) {
+#pragma unroll
+ #pragma unroll
+       for (int v = 0; v < 3; v++) {
             double d0 = R.qn[0][v] - R.qK[v], d1 = R.qn[1][v] - R.qK[v], d2 = R.qn[2][v] - R.qK[v];
             double gx = (G(m, GEO_WX, K) * d0 + G(m, GEO_WX + 1, K) * d1) + G(m, GEO_WX + 2, K) * d2;
             double gy = (G(m, GEO_WY, K) * d0 + G(m, GEO_WY + 1, K) * d1) + G(m, GEO_WY + 2, K) * d2;
             double qmax = R.qK[v], qmin = R.qK[v];
             int imax = -1, imin = -1;
+#pragma unroll
             for (int f = 0; f < 3; f++) {
                 if (lt_x(qmax, R.qn[f][v])) { qmax = R.qn[f][v]; imax = f; }
                 if (lt_x(R.qn[f][v], qmin)) { qmin = R.qn[f][v]; imin = f; }
             }
-            double alpha = 1.0;
-            int fa = -1;
-            double ra = 0.0;
-            for (int f = 0; f < 3; f++) {
-                double D = gx * G(m, GEO_FX + f, K) + gy * G(m, GEO_FY + f, K);
+            // the active limiter: of the faces with the largest D > 0 and the largest
+            // -D > 0 (the first of equals) the one of smaller quotient r / D, where that
+            // is below 1; two candidates and one division, as the forward kernels
+            const double up = qmax - R.qK[v], dn = R.qK[v] - qmin;
+            double P = 0.0, M = 0.0;
+            int fP = -1, fM = -1;
+#pragma unroll
+ #pragma unroll
+           for (int f = 0; f < 3; f++) {
+                const double D = gx * G(m, GEO_FX + f, K) + gy * G(m, GEO_FY + f, K);
                 R.D[v][f] = D;
-                double phi = 1.0, rr = 0.0;
-                bool lim = false;
-                if (is_pos(D)) { rr = qmax - R.qK[v]; double t = rr / D; if (lt_pos(t, 1.0)) { phi = t; lim = true; } }
-                else if (is_neg(D)) { rr = qmin - R.qK[v]; double t = rr / D; if (lt_pos(t, 1.0)) { phi = t; lim = true; } }
-                if (lt_x(phi, alpha)) { alpha = phi; fa = lim ? f : -1; ra = rr; }
+                if (is_pos(D) && gt_nn(D, P)) { P = D; fP = f; }
+                if (is_neg(D) && gt_nn(-D, M)) { M = -D; fM = f; }
+            }
+            double alpha = 1.0, ra = 0.0;
+            int fa = -1;
+            const bool limP = gt_nn(P, up), limM = gt_nn(M, dn);
+            if (limP || limM) {
+                const double xP = up * M, xM = dn * P;
+                bool takeM = limM && (!limP || gt_nn(xP, xM));
+                alpha = quot(takeM ? dn : up, recip(takeM ? M : P));
+                if (limP && limM && dbits(xP) == dbits(xM)) {
+                    const double other = quot(dn, recip(M));          // takeM is false here
+                    takeM = lt_x(other, alpha) || (other == alpha && fM < fP);
+                    if (takeM) alpha = other;
+                }
+                fa = takeM ? fM : fP;
+                ra = takeM ? -dn : up;
             }
             R.alpha[v] = alpha;
             R.fa[v] = fa;
             R.r[v] = ra;
             R.imax[v] = imax;
             R.imin[v] = imin;
+#pragma unroll
             for (int f = 0; f < 3; f++) face[f][v] = R.qK[v] + alpha * R.D[v][f];
         }
+#pragma unroll
         for (int f = 0; f < 3; f++) {
             Hf[f] = face[f][0] - m.zf[f * nc + K];
             if (!(Hf[f] > m.hthr)) recon = false;
@@ -152,37 +227,16 @@ __device__ void recon_forward(const AdjMesh &m, const double *w, int K, ReconFwd
     }
     R.recon = recon;
     if (!recon) {
+#pragma unroll
         for (int f = 0; f < 3; f++) { Hf[f] = HK; Huf[f] = HuK; Hvf[f] = HvK; }
     }
 }
 
-// Face values are needed only where a face's flux adjoint can be nonzero, i.e.
-// where the cell or a face neighbour has a nonzero residual adjoint; elsewhere
-// the flux VJP skips the face (the VJP of zero is zero).
+// The flux VJP skips a face where neither cell has a residual adjoint (the VJP of
+// zero is zero).
 __device__ __forceinline__ bool rb_nonzero(const double *Rb, int nc, int k)
 {
     return !is_zero(Rb[k]) || !is_zero(Rb[nc + k]) || !is_zero(Rb[2 * (size_t)nc + k]);
-}
-
-__global__ void adj_face_values_kernel(AdjMesh m, const double *w, const double *Rb, double *FV)
-{
-    const int nc = m.nc;
-    for (int K = blockIdx.x * blockDim.x + threadIdx.x; K < nc; K += gridDim.x * blockDim.x) {
-        bool need = rb_nonzero(Rb, nc, K);
-        for (int f = 0; f < 3 && !need; f++) {
-            int j = m.nbr[f * nc + K];
-            if (j >= 0) need = rb_nonzero(Rb, nc, j);
-        }
-        if (!need) continue;
-        ReconFwd R;
-        double Hf[3], Huf[3], Hvf[3];
-        recon_forward(m, w, K, R, Hf, Huf, Hvf);
-        for (int f = 0; f < 3; f++) {
-            FV[(0 * 3 + f) * (size_t)nc + K] = Hf[f];
-            FV[(1 * 3 + f) * (size_t)nc + K] = Huf[f];
-            FV[(2 * 3 + f) * (size_t)nc + K] = Hvf[f];
-        }
-    }
 }
 
 // Reverse of the face flux seen from L (forward: face_flux / hll_normal).
@@ -193,7 +247,7 @@ __global__ void adj_face_values_kernel(AdjMesh m, const double *w, const double 
 // on each side.  The absorbing ghost (characteristic ghost of a sea at rest at
 // eta = 0 beyond the face) depends on the face state through the outgoing
 // invariant u_n + 2c and on the bed under the face through c_0 = sqrt(g max(0, -z)).
-__device__ void flux_vjp(const AdjMesh &m, double HfL, double HufL, double HvfL, double zL, double HfR,
+__device__ __forceinline__ void flux_vjp(const AdjMesh &m, double HfL, double HufL, double HvfL, double zL, double HfR,
                          double HufR, double HvfR, double zR, double nx, double ny, bool wall,
                          const double Pb[3], double PLb, double PRb, double bL[4], double bR[4],
                          double amb = 0.0, int bnd = 1)
@@ -203,7 +257,8 @@ __device__ void flux_vjp(const AdjMesh &m, double HfL, double HufL, double HvfL,
     // ---- forward
     double uL = 0.0, vL = 0.0;
     bool velL = gt_nn(HfL, hthr);
-    if (velL) { uL = HufL / HfL; vL = HvfL / HfL; }
+    const Recip rL = recip(HfL), rR = recip(HfR);      // (used where the side has a velocity)
+    if (velL) { uL = quot(HufL, rL); vL = quot(HvfL, rL); }
     double unL = uL * nx + vL * ny;
     double utL = -uL * ny + vL * nx;
     double HsL, HsR, unR, utR, uR = 0.0, vR = 0.0, zs = 0.0;
@@ -235,7 +290,7 @@ __device__ void flux_vjp(const AdjMesh &m, double HfL, double HufL, double HvfL,
         utR = utL;
     } else {
         velR = gt_nn(HfR, hthr);
-        if (velR) { uR = HufR / HfR; vR = HvfR / HfR; }
+        if (velR) { uR = quot(HufR, rR); vR = quot(HvfR, rR); }
         unR = uR * nx + vR * ny;
         utR = -uR * ny + vR * nx;
         zR_max = lt_x(zL, zR);
@@ -290,7 +345,7 @@ __device__ void flux_vjp(const AdjMesh &m, double HfL, double HufL, double HvfL,
         if (!is_neg(sL)) {
             for (int k = 0; k < 3; k++) FLb[k] = Fb[k];
         } else if (!is_neg(sR)) {
-            double den = sR - sL, sLR = sL * sR, iden = 1.0 / den;
+            double den = sR - sL, sLR = sL * sR, iden = inverse(recip(den));
             double denb = 0.0, sLRb = 0.0;
             for (int k = 0; k < 3; k++) {
                 double N = (sR * FL[k] - sL * FR[k]) + sLR * (wR[k] - wL[k]);
@@ -351,8 +406,8 @@ __device__ void flux_vjp(const AdjMesh &m, double HfL, double HufL, double HvfL,
             unRb -= 0.25 * csb;
             unLb += 0.25 * csb;
         }
-        if (is_pos(cL)) HsLb += cLb * (0.5 / cL) * g;
-        if (is_pos(cR)) HsRb += cRb * (0.5 / cR) * g;
+        if (is_pos(cL)) HsLb += cLb * quot(0.5, recip(cL)) * g;
+        if (is_pos(cR)) HsRb += cRb * quot(0.5, recip(cR)) * g;
     }
     // ---- reverse of the interface depths and velocities
     if (wall && bnd == 3) {
@@ -377,7 +432,7 @@ __device__ void flux_vjp(const AdjMesh &m, double HfL, double HufL, double HvfL,
         if (zR_max) bR[3] += zsb; else bL[3] += zsb;
         double uRb = unRb * nx - utRb * ny, vRb = unRb * ny + utRb * nx;
         if (velR) {
-            double inv = 1.0 / HfR;
+            double inv = inverse(rR);
             bR[1] += uRb * inv;
             bR[2] += vRb * inv;
             HfRb -= (uRb * uR + vRb * vR) * inv;
@@ -385,71 +440,13 @@ __device__ void flux_vjp(const AdjMesh &m, double HfL, double HufL, double HvfL,
     }
     double uLb = unLb * nx - utLb * ny, vLb = unLb * ny + utLb * nx;
     if (velL) {
-        double inv = 1.0 / HfL;
+        double inv = inverse(rL);
         bL[1] += uLb * inv;
         bL[2] += vLb * inv;
         HfLb -= (uLb * uL + vLb * vL) * inv;
     }
     bL[0] += HfLb;
     bR[0] += HfRb;
-}
-
-// One thread per face (the face list: the lower-numbered cell owns an interior
-// face, the cell a boundary face): R-bar of both cells -> Phi-bar, P-bar ->
-// face-state adjoints.  FVb[(v*3+f)*nc + K] and zfb[f*nc + K] are the (cell,
-// face) slots; each is written exactly once per residual.
-__global__ void adj_flux_vjp_kernel(AdjMesh m, const double *FV, const double *Rb, double *FVb, double *zfb)
-{
-    const int nc = m.nc;
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < m.nfaces; q += gridDim.x * blockDim.x) {
-        {
-            const int K = m.faces[q] >> 2, f = m.faces[q] & 3;
-            int j = m.nbr[f * nc + K];
-            bool wall = j < 0;
-            int fj = wall ? 0 : (m.nbrl[f * nc + K] & 3);
-            if (!rb_nonzero(Rb, nc, K) && (wall || !rb_nonzero(Rb, nc, j))) {
-                for (int v = 0; v < 3; v++) FVb[(v * 3 + f) * (size_t)nc + K] = 0.0;
-                zfb[f * (size_t)nc + K] = 0.0;
-                if (!wall) {
-                    for (int v = 0; v < 3; v++) FVb[(v * 3 + fj) * (size_t)nc + j] = 0.0;
-                    zfb[fj * (size_t)nc + j] = 0.0;
-                }
-                continue;
-            }
-            double nx = G(m, GEO_NX + f, K), ny = G(m, GEO_NY + f, K), l = G(m, GEO_LEN + f, K);
-            double aL = G(m, GEO_AREA, K);
-            double cLf = -l / aL;
-            double Pb[3], PLb, PRb = 0.0;
-            double RLH = Rb[K], RLU = Rb[nc + K], RLV = Rb[2 * (size_t)nc + K];
-            Pb[0] = cLf * RLH;
-            Pb[1] = cLf * RLU;
-            Pb[2] = cLf * RLV;
-            PLb = cLf * (RLU * nx + RLV * ny);
-            double HfR = 0.0, HufR = 0.0, HvfR = 0.0, zR = 0.0;
-            if (!wall) {
-                double cRf = l / G(m, GEO_AREA, j);
-                double RRH = Rb[j], RRU = Rb[nc + j], RRV = Rb[2 * (size_t)nc + j];
-                Pb[0] += cRf * RRH;
-                Pb[1] += cRf * RRU;
-                Pb[2] += cRf * RRV;
-                PRb = cRf * (RRU * nx + RRV * ny);
-                HfR = FV[(0 * 3 + fj) * (size_t)nc + j];
-                HufR = FV[(1 * 3 + fj) * (size_t)nc + j];
-                HvfR = FV[(2 * 3 + fj) * (size_t)nc + j];
-                zR = bed_under(m, j, fj);
-            }
-            double bL[4], bR[4];
-            flux_vjp(m, FV[(0 * 3 + f) * (size_t)nc + K], FV[(1 * 3 + f) * (size_t)nc + K],
-                     FV[(2 * 3 + f) * (size_t)nc + K], bed_under(m, K, f), HfR, HufR, HvfR, zR, nx, ny, wall, Pb, PLb,
-                     PRb, bL, bR, 0.0, wall ? -j : 0);
-            for (int v = 0; v < 3; v++) FVb[(v * 3 + f) * (size_t)nc + K] = bL[v];
-            zfb[f * (size_t)nc + K] = bL[3];
-            if (!wall) {
-                for (int v = 0; v < 3; v++) FVb[(v * 3 + fj) * (size_t)nc + j] = bR[v];
-                zfb[fj * (size_t)nc + j] = bR[3];
-            }
-        }
-    }
 }
 
 // Per cell: reverse of the reconstruction.  own[7][nc] = (H, Hu, Hv, z_K)-bar of
@@ -461,27 +458,51 @@ __global__ void adj_flux_vjp_kernel(AdjMesh m, const double *FV, const double *R
 // n_f of its momentum residual R = -(1/|K|)(... + source): with
 // q_f = -(g/|K|) l_f (n_f . (R-bar_Hu, R-bar_Hv)), eta-bar_K += sum_f q_f z_f and
 // z_f-bar += q_f (eta_K - z_f).
-__global__ void adj_recon_vjp_kernel(AdjMesh m, const double *w, const double *Rb, const double *FVb,
-                                     const double *zfb, double *own, double *send)
+__global__ void __launch_bounds__(kVjpThreads) adj_recon_vjp_kernel(AdjMesh m, const double *w, const double *Rb, const double *FVb,
+                                     const double *zfb, double *own, double *send, const AdjCflFace *cf)
 {
     const int nc = m.nc;
     for (int K = blockIdx.x * blockDim.x + threadIdx.x; K < nc; K += gridDim.x * blockDim.x) {
         double fb[3][3];   // [v][f]
         bool any = m.rec[K] && (!is_zero(Rb[nc + K]) || !is_zero(Rb[2 * (size_t)nc + K]));
-        for (int v = 0; v < 3; v++)
-            for (int f = 0; f < 3; f++) {
-                fb[v][f] = FVb[(v * 3 + f) * (size_t)nc + K];
-                any = any || !is_zero(fb[v][f]);
-            }
+#pragma unroll
+ #pragma unroll
+       for (int v = 0; v < 3; v++)
+#pragma unroll
+ #pragma unroll
+           for (int f = 0; f < 3; f++) fb[v][f] = FVb[(v * 3 + f) * (size_t)nc + K];
         double zsl[3];
-        for (int f = 0; f < 3; f++) zsl[f] = zfb[f * (size_t)nc + K];
+#pragma unroll
+ #pragma unroll
+       for (int f = 0; f < 3; f++) zsl[f] = zfb[f * (size_t)nc + K];
+        if (cf && (cf->cell[0] == K || cf->cell[1] == K)) {
+            // the face that set the CFL step: its wave speed's adjoint on this side
+            const int side = cf->cell[0] == K ? 0 : 1;
+#pragma unroll
+ #pragma unroll
+           for (int f = 0; f < 3; f++)
+                if (f == cf->face[side]) {
+#pragma unroll
+ #pragma unroll
+                   for (int v = 0; v < 3; v++) fb[v][f] += cf->bar[side][v];
+                    zsl[f] += cf->bar[side][3];
+                }
+        }
+#pragma unroll
+ #pragma unroll
+       for (int v = 0; v < 3; v++)
+#pragma unroll
+ #pragma unroll
+           for (int f = 0; f < 3; f++) any = any || !is_zero(fb[v][f]);
         if (!any) {                      // nothing flows back through the reconstruction
             own[K] = 0.0;
             own[nc + K] = 0.0;
             own[2 * (size_t)nc + K] = 0.0;
             const bool rk = m.rec[K];
             own[3 * (size_t)nc + K] = rk ? 0.0 : (zsl[0] + zsl[1]) + zsl[2];
+#pragma unroll
             for (int f = 0; f < 3; f++) own[(4 + f) * (size_t)nc + K] = rk ? zsl[f] : 0.0;
+#pragma unroll
             for (int q = 0; q < 12; q++) send[q * (size_t)nc + K] = 0.0;
             continue;
         }
@@ -492,16 +513,19 @@ __global__ void adj_recon_vjp_kernel(AdjMesh m, const double *w, const double *R
         double qnb[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};   // [f][v]
         if (!R.recon) {
             zb = (zsl[0] + zsl[1]) + zsl[2];
+#pragma unroll
             for (int f = 0; f < 3; f++) { Hb += fb[0][f]; Hub += fb[1][f]; Hvb += fb[2][f]; }
         } else {
             double qKb[3] = {0, 0, 0};
+#pragma unroll
             for (int f = 0; f < 3; f++) zfbK[f] = zsl[f] - fb[0][f];      // H_f = eta_f - z_f
             {
                 // the centred source
-                const double c = -m.g / G(m, GEO_AREA, K);
+                const double c = quot(-m.g, by_area(m, K));
                 const double rbu = Rb[nc + K], rbv = Rb[2 * (size_t)nc + K];
                 const double eK = w[K] + m.z[K];
                 double eb = 0.0;
+#pragma unroll
                 for (int f = 0; f < 3; f++) {
                     const double zff = m.zf[f * nc + K];
                     const double q = c * (G(m, GEO_LEN + f, K) * (G(m, GEO_NX + f, K) * rbu + G(m, GEO_NY + f, K) * rbv));
@@ -511,9 +535,13 @@ __global__ void adj_recon_vjp_kernel(AdjMesh m, const double *w, const double *R
                 Hb += eb;
                 zb += eb;
             }
-            for (int v = 0; v < 3; v++) {
+#pragma unroll
+ #pragma unroll
+           for (int v = 0; v < 3; v++) {
                 double ab = 0.0, Db[3];
-                for (int f = 0; f < 3; f++) {
+#pragma unroll
+ #pragma unroll
+               for (int f = 0; f < 3; f++) {
                     qKb[v] += fb[v][f];
                     ab += fb[v][f] * R.D[v][f];
                     Db[f] = fb[v][f] * R.alpha[v];
@@ -523,30 +551,38 @@ __global__ void adj_recon_vjp_kernel(AdjMesh m, const double *w, const double *R
                     // (faces picked by compare and select, not by index: indexed
                     // arrays would live in local memory)
                     const double D = fa == 0 ? R.D[v][0] : fa == 1 ? R.D[v][1] : R.D[v][2];
-                    double iD = 1.0 / D;
+                    double iD = inverse(recip(D));
                     double rb = ab * iD;
 #pragma unroll
-                    for (int f = 0; f < 3; f++)
+ #pragma unroll
+                   for (int f = 0; f < 3; f++)
                         if (f == fa) Db[f] -= rb * R.r[v] * iD;
                     int idx = is_pos(D) ? R.imax[v] : R.imin[v];
                     if (idx < 0) qKb[v] += rb;
 #pragma unroll
-                    for (int f = 0; f < 3; f++)
+ #pragma unroll
+                   for (int f = 0; f < 3; f++)
                         if (f == idx) qnb[f][v] += rb;
                     qKb[v] -= rb;
                 }
                 double gxb = 0.0, gyb = 0.0;
-                for (int f = 0; f < 3; f++) {
+#pragma unroll
+ #pragma unroll
+               for (int f = 0; f < 3; f++) {
                     gxb += Db[f] * G(m, GEO_FX + f, K);
                     gyb += Db[f] * G(m, GEO_FY + f, K);
                 }
-                for (int f = 0; f < 3; f++) {
+#pragma unroll
+ #pragma unroll
+               for (int f = 0; f < 3; f++) {
                     double db = gxb * G(m, GEO_WX + f, K) + gyb * G(m, GEO_WY + f, K);
                     qnb[f][v] += db;
                     qKb[v] -= db;
                 }
             }
-            for (int f = 0; f < 3; f++) {
+#pragma unroll
+ #pragma unroll
+           for (int f = 0; f < 3; f++) {
                 if (!R.wall[f]) continue;
                 if (R.open[f]) {                 // ghost = the cell's own values
                     qKb[0] += qnb[f][0];
@@ -571,7 +607,9 @@ __global__ void adj_recon_vjp_kernel(AdjMesh m, const double *w, const double *R
         own[nc + K] = Hub;
         own[2 * (size_t)nc + K] = Hvb;
         own[3 * (size_t)nc + K] = zb;
+#pragma unroll
         for (int f = 0; f < 3; f++) own[(4 + f) * (size_t)nc + K] = zfbK[f];
+#pragma unroll
         for (int f = 0; f < 3; f++) {
             send[(f * 4 + 0) * (size_t)nc + K] = qnb[f][0];     // eta-bar -> H-bar and z-bar
             send[(f * 4 + 1) * (size_t)nc + K] = qnb[f][1];
@@ -581,24 +619,31 @@ __global__ void adj_recon_vjp_kernel(AdjMesh m, const double *w, const double *R
     }
 }
 
-// wb[3][nc] += own + sum over faces of what the face neighbour sent; zb[nc] (cell
-// beds) likewise; zb rows 1..3 (face beds) += the cell's own face-bed adjoints.
+// Own part + what the face neighbours sent: a = the adjoints of (H, Hu, Hv, z_K) of
+// cell K; zb[nc] (cell beds) and rows 1..3 (face beds) +=.
+__device__ __forceinline__ void gathered(const AdjMesh &m, int K, const double *own, const double *send, double *zb, double a[3])
+{
+    const int nc = m.nc;
+    double s[4] = {own[K], own[nc + K], own[2 * (size_t)nc + K], own[3 * (size_t)nc + K]};
+    for (int f = 0; f < 3; f++) {
+        const int j = m.nbr[f * nc + K];
+        if (j < 0) continue;
+        const int fj = m.nbrl[f * nc + K] & 3;
+        for (int k = 0; k < 4; k++) s[k] += send[(fj * 4 + k) * (size_t)nc + j];
+    }
+    zb[K] += s[3];
+    for (int f = 0; f < 3; f++) zb[(1 + f) * (size_t)nc + K] += own[(4 + f) * (size_t)nc + K];
+    a[0] = s[0]; a[1] = s[1]; a[2] = s[2];
+}
+
+// wb[3][nc] += the gathered adjoints.
 __global__ void adj_gather_kernel(AdjMesh m, const double *own, const double *send, double *wb, double *zb)
 {
     const int nc = m.nc;
     for (int K = blockIdx.x * blockDim.x + threadIdx.x; K < nc; K += gridDim.x * blockDim.x) {
-        double a[4] = {own[K], own[nc + K], own[2 * (size_t)nc + K], own[3 * (size_t)nc + K]};
-        for (int f = 0; f < 3; f++) {
-            int j = m.nbr[f * nc + K];
-            if (j < 0) continue;
-            int fj = m.nbrl[f * nc + K] & 3;
-            for (int k = 0; k < 4; k++) a[k] += send[(fj * 4 + k) * (size_t)nc + j];
-        }
-        wb[K] += a[0];
-        wb[nc + K] += a[1];
-        wb[2 * (size_t)nc + K] += a[2];
-        zb[K] += a[3];
-        for (int f = 0; f < 3; f++) zb[(1 + f) * (size_t)nc + K] += own[(4 + f) * (size_t)nc + K];
+        double a[3];
+        gathered(m, K, own, send, zb, a);
+        for (int k = 0; k < 3; k++) wb[k * (size_t)nc + K] += a[k];
     }
 }
 
@@ -610,55 +655,81 @@ __device__ __forceinline__ void dry_fix_mask(double Hpre, double hthr, double &H
     else if (!gt_nn(Hpre, hthr)) { Hub = 0.0; Hvb = 0.0; }
 }
 
-// w1 = fix(w + dt R0), keeping the pre-fix depth for the mask.
-__global__ void adj_stage1_kernel(int nc, double dt, double hthr, const double *w, const double *R0, double *w1,
-                                  double *H1pre)
+// The beginning of a step's reverse, per cell:
+//  * w1 = fix(w + dt R0), keeping the pre-fix depth for the mask;
+//  * the reverse of stage 2, w^{n+1} = fix(w/2 + (w1 + dt R1)/2), with the dry-fix
+//    branch recorded by the forward stage-2 kernel (0 none, 1 momentum cut, 2
+//    emptied): from wb (adjoint of w^{n+1}), wb_n = wb_1 = 1/2 wbpre, Rb = dt/2 wbpre;
+//  * with CFL steps the CTA's part of sum Rb . R1 (dt-bar) and of the search for the
+//    cell of smallest CFL bound.
+// (Three elementwise kernels and a reduction of their own moved these arrays through
+// memory twice, 18 us of launches and passes at 49k triangles.)
+__global__ void __launch_bounds__(kRedThreads) adj_begin_kernel(int nc, double dt, double hthr, const double *w, const double *R0,
+                                                                double *w1, double *H1pre, const uint8_t *mask2, const double *wb,
+                                                                double *wbn, double *wb1, double *Rb, const AdjCfl cfl)
 {
+    double sum = 0.0, bb = INFINITY;
+    int bo = 0x7fffffff, bk = -1;
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nc; k += gridDim.x * blockDim.x) {
-        double H = w[k] + dt * R0[k];
-        double Hu = w[nc + k] + dt * R0[nc + k];
-        double Hv = w[2 * (size_t)nc + k] + dt * R0[2 * (size_t)nc + k];
-        H1pre[k] = H;
-        if (is_neg(H)) { H = 0.0; Hu = 0.0; Hv = 0.0; }
-        else if (!gt_nn(H, hthr)) { Hu = 0.0; Hv = 0.0; }
-        w1[k] = H;
-        w1[nc + k] = Hu;
-        w1[2 * (size_t)nc + k] = Hv;
-    }
-}
-
-// Reverse of stage 2: w^{n+1} = fix(w/2 + (w1 + dt R1)/2), with the dry-fix
-// branch recorded by the forward stage-2 kernel (0 none, 1 momentum cut, 2
-// emptied).  From wb (adjoint of w^{n+1}): wb_n = wb_1 = 1/2 wbpre, Rb = dt/2 wbpre.
-__global__ void adj_stage2_rev_kernel(int nc, double dt, const uint8_t *mask2, const double *wb, double *wbn,
-                                      double *wb1, double *Rb)
-{
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nc; k += gridDim.x * blockDim.x) {
-        uint8_t br = mask2[k];
+        double q[3];
+        for (int c = 0; c < 3; c++) q[c] = w[c * (size_t)nc + k] + dt * R0[c * (size_t)nc + k];
+        H1pre[k] = q[0];
+        if (is_neg(q[0])) { q[0] = 0.0; q[1] = 0.0; q[2] = 0.0; }
+        else if (!gt_nn(q[0], hthr)) { q[1] = 0.0; q[2] = 0.0; }
+        const uint8_t br = mask2[k];
         double b[3] = {wb[k], wb[nc + k], wb[2 * (size_t)nc + k]};
         if (br == 2) { b[0] = 0.0; b[1] = 0.0; b[2] = 0.0; }
         else if (br == 1) { b[1] = 0.0; b[2] = 0.0; }
         for (int c = 0; c < 3; c++) {
-            wbn[c * (size_t)nc + k] = 0.5 * b[c];
-            wb1[c * (size_t)nc + k] = 0.5 * b[c];
-            Rb[c * (size_t)nc + k] = 0.5 * dt * b[c];
+            const size_t i = c * (size_t)nc + k;
+            w1[i] = q[c];
+            const double h = half_of(b[c]), r = 0.5 * dt * b[c];
+            wbn[i] = h;
+            wb1[i] = h;
+            Rb[i] = r;
+            if (cfl.dt) sum += r * cfl.R1[i];
         }
+        if (cfl.dt) {
+            const double bd = cfl.bound[k];              // +inf where nothing moves
+            if (bd <= bb && bd < INFINITY && cfl_less(bd, cfl.orig[k], bb, bo)) { bb = bd; bo = cfl.orig[k]; bk = k; }
+        }
+    }
+    if (!cfl.dt) return;
+    sum = cta_sum<kRedThreads>(sum);
+    cta_argmin<kRedThreads>(bb, bo, bk);
+    if (threadIdx.x == 0) {
+        cfl.part_s1[blockIdx.x] = sum;
+        cfl.part_b[blockIdx.x] = bb;
+        cfl.part_o[blockIdx.x] = bo;
+        cfl.part_k[blockIdx.x] = bk;
     }
 }
 
-// Reverse of stage 1: w1 = fix(w + dt R0).  wbn += wb1pre, Rb = dt wb1pre.
-__global__ void adj_stage1_rev_kernel(int nc, double dt, double hthr, const double *H1pre, const double *wb1,
-                                      double *wbn, double *Rb)
+// Between the two residuals, per cell: wb1 += what stage 2's residual gathered, then
+// the reverse of stage 1, w1 = fix(w + dt R0): wbn += wb1pre, Rb = dt wb1pre, and
+// with CFL steps the CTA's part of sum Rb . R0.
+__global__ void __launch_bounds__(kRedThreads) adj_gather_mid_kernel(AdjMesh m, const double *own, const double *send, double *zb,
+                                                                     double dt, double hthr, const double *H1pre, const double *wb1,
+                                                                     double *wbn, double *Rb, const AdjCfl cfl)
 {
+    const int nc = m.nc;
+    double sum = 0.0;
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nc; k += gridDim.x * blockDim.x) {
-        double b0 = wb1[k], b1 = wb1[nc + k], b2 = wb1[2 * (size_t)nc + k];
-        dry_fix_mask(H1pre[k], hthr, b0, b1, b2);
-        double b[3] = {b0, b1, b2};
+        double b[3];
+        gathered(m, k, own, send, zb, b);
+        for (int c = 0; c < 3; c++) b[c] = wb1[c * (size_t)nc + k] + b[c];
+        dry_fix_mask(H1pre[k], hthr, b[0], b[1], b[2]);
         for (int c = 0; c < 3; c++) {
-            wbn[c * (size_t)nc + k] += b[c];
-            Rb[c * (size_t)nc + k] = dt * b[c];
+            const size_t i = c * (size_t)nc + k;
+            const double r = dt * b[c];
+            wbn[i] += b[c];
+            Rb[i] = r;
+            if (cfl.dt) sum += r * cfl.R0[i];
         }
     }
+    if (!cfl.dt) return;
+    sum = cta_sum<kRedThreads>(sum);
+    if (threadIdx.x == 0) cfl.part_s0[blockIdx.x] = sum;
 }
 
 // Gauge functional J = sum weights * (H + z) at the gauge cells: its adjoint.
@@ -765,62 +836,34 @@ __device__ FaceIn face_in(const AdjMesh &m, const double *FV, int K, int f)
     return r;
 }
 
-__device__ __forceinline__ bool cfl_less(double b1, int o1, double b2, int o2)
-{
-    return b1 < b2 || (b1 == b2 && o1 < o2);
-}
 
-// Per CTA: the cell of smallest CFL bound |K| / (3 max_f l_f a_f) (ties: lowest
-// original id) -> part_b, part_o, part_k [gridDim].  The bounds are those that the
-// forward stage-1 kernel recorded (recomputing every face's speed here took as
-// long as the reconstruction VJP).
-constexpr int kRedThreads = 256;
-__device__ __forceinline__ void cta_argmin(double &b, int &o, int &k)
-{
-    __shared__ double sb[kRedThreads / 32];
-    __shared__ int so[kRedThreads / 32], sk[kRedThreads / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int s = 16; s > 0; s >>= 1) {
-        const double b2 = __shfl_down_sync(0xffffffffu, b, s);
-        const int o2 = __shfl_down_sync(0xffffffffu, o, s), k2 = __shfl_down_sync(0xffffffffu, k, s);
-        if (cfl_less(b2, o2, b, o)) { b = b2; o = o2; k = k2; }
-    }
-    if (lane == 0) { sb[warp] = b; so[warp] = o; sk[warp] = k; }
-    __syncthreads();
-    if (threadIdx.x == 0)
-        for (int w = 1; w < kRedThreads / 32; w++)
-            if (cfl_less(sb[w], so[w], b, o)) { b = sb[w]; o = so[w]; k = sk[w]; }
-}
-
-__global__ void __launch_bounds__(kRedThreads) adj_cfl_part_kernel(int nc, const double *bound, const int32_t *orig,
-                                                                   double *part_b, int *part_o, int *part_k)
-{
-    double bb = INFINITY;
-    int bo = 0x7fffffff, bk = -1;
-    for (int K = blockIdx.x * blockDim.x + threadIdx.x; K < nc; K += gridDim.x * blockDim.x) {
-        const double b = bound[K];                       // +inf where nothing moves
-        if (b <= bb && b < INFINITY && cfl_less(b, orig[K], bb, bo)) { bb = b; bo = orig[K]; bk = K; }
-    }
-    cta_argmin(bb, bo, bk);
-    if (threadIdx.x == 0) { part_b[blockIdx.x] = bb; part_o[blockIdx.x] = bo; part_k[blockIdx.x] = bk; }
-}
-
-// dt-bar's face: one CTA reduces the parts, three threads form the speeds of the
-// chosen cell's faces, one finds f* (the first of largest l_f a_f) and adds the
-// wave-speed adjoint's contribution to both sides' face slots.  (One thread
-// walking the parts and the faces took 99 us.)
-__global__ void __launch_bounds__(kRedThreads) adj_cfl_face_kernel(AdjMesh m, const double *FV, int nparts,
-                                    const double *part_b, const int *part_o, const int *part_k, const double *dtbar,
-                                    double cfl, double dt_max, double *FVb, double *zfb)
+// dt-bar's face (one CTA): sums the parts of dt-bar, reduces the parts of the search,
+// forms the speeds of the chosen cell's faces, finds f* (the first of largest l_f a_f)
+// and writes its wave speed's adjoint on both sides to *cfl.out, from where the
+// reconstruction VJP adds it.  (A kernel of its own between the flux and the
+// reconstruction VJP was 28 us of latency at any size.)
+__device__ __noinline__ void cfl_face_vjp(const AdjMesh &m, const double *FV, const AdjCfl &cfl)
 {
     __shared__ double s_a[3], s_la[3];
     __shared__ int s_k;
-    double bb = INFINITY;
+    AdjCflFace *out = cfl.out;
+    double s1 = 0.0, s0 = 0.0, bb = INFINITY;
     int bo = 0x7fffffff, K = -1;
-    for (int q = threadIdx.x; q < nparts; q += blockDim.x)
-        if (part_k[q] >= 0 && cfl_less(part_b[q], part_o[q], bb, bo)) { bb = part_b[q]; bo = part_o[q]; K = part_k[q]; }
-    cta_argmin(bb, bo, K);
-    if (threadIdx.x == 0) s_k = K;
+    for (int q = threadIdx.x; q < cfl.nparts; q += blockDim.x) {
+        s1 += cfl.part_s1[q];
+        s0 += cfl.part_s0[q];
+        if (cfl.part_k[q] >= 0 && cfl_less(cfl.part_b[q], cfl.part_o[q], bb, bo)) {
+            bb = cfl.part_b[q]; bo = cfl.part_o[q]; K = cfl.part_k[q];
+        }
+    }
+    s1 = cta_sum<kVjpThreads>(s1);
+    __syncthreads();
+    s0 = cta_sum<kVjpThreads>(s0);
+    cta_argmin<kVjpThreads>(bb, bo, K);
+    if (threadIdx.x == 0) {
+        s_k = K;
+        out->cell[0] = out->cell[1] = -1;
+    }
     __syncthreads();
     K = s_k;
     if (K < 0) return;                                   // nothing moves: dt = dt_max or 0
@@ -833,56 +876,88 @@ __global__ void __launch_bounds__(kRedThreads) adj_cfl_face_kernel(AdjMesh m, co
     }
     __syncthreads();
     if (threadIdx.x != 0) return;
-    const double dtc = cfl * bb;
-    if (dt_max > 0.0 && dt_max < dtc) return;            // clamped by dt_max: no dependence
+    const double dtc = cfl.cfl * bb;
+    if (cfl.dt_max > 0.0 && cfl.dt_max < dtc) return;    // clamped by dt_max: no dependence
     int f = 0;
     for (int k = 1; k < 3; k++)
         if (gt_nn(s_la[k], s_la[f])) f = k;
     const FaceIn q = face_in(m, FV, K, f);
-    const double ab = -(*dtbar) * dtc / s_a[f];
+    // dt-bar: sum w-bar_pre . R1 / 2 + sum w1-bar_pre . R0 (each Rb . R / dt), and with
+    // a moving bed every later bed through the time
+    double dtbar = (s1 + s0) / cfl.dt;
+    if (cfl.tsum) dtbar += *cfl.tsum;
+    const double ab = -dtbar * dtc / s_a[f];
     const double P0[3] = {0.0, 0.0, 0.0};
     double bL[4], bR[4];
     flux_vjp(m, q.HfL, q.HufL, q.HvfL, q.zL, q.HfR, q.HufR, q.HvfR, q.zR, q.nx, q.ny, q.wall, P0, 0.0, 0.0, bL, bR, ab,
              q.bnd);
-    const int nc = m.nc;
-    for (int v = 0; v < 3; v++) FVb[(v * 3 + f) * (size_t)nc + K] += bL[v];
-    zfb[f * (size_t)nc + K] += bL[3];
-    if (!q.wall) {
-        for (int v = 0; v < 3; v++) FVb[(v * 3 + q.fj) * (size_t)nc + q.j] += bR[v];
-        zfb[q.fj * (size_t)nc + q.j] += bR[3];
+    for (int k = 0; k < 4; k++) { out->bar[0][k] = bL[k]; out->bar[1][k] = bR[k]; }
+    out->face[0] = f;
+    out->cell[0] = K;
+    if (!q.wall) { out->face[1] = q.fj; out->cell[1] = q.j; }
+}
+
+// One thread per face (the face list: the lower-numbered cell owns an interior
+// face, the cell a boundary face): R-bar of both cells -> Phi-bar, P-bar ->
+// face-state adjoints.  FVb[(v*3+f)*nc + K] and zfb[f*nc + K] are the (cell,
+// face) slots; each is written exactly once per residual.
+// With CFL steps the launch has one more CTA, which reverses the time step meanwhile.
+__global__ void __launch_bounds__(kVjpThreads) adj_flux_vjp_kernel(AdjMesh m, const double *FV, const double *Rb, double *FVb,
+                                                                   double *zfb, const AdjCfl cfl)
+{
+    const int nc = m.nc, ctas = gridDim.x - (cfl.dt ? 1 : 0);
+    if ((int)blockIdx.x == ctas) {
+        cfl_face_vjp(m, FV, cfl);
+        return;
     }
-}
-
-// Deterministic dot product: per-CTA partial sums, then one CTA adds them, times
-// scale, into *acc (reset: replaces it).  Both sums have a fixed order: a warp's
-// shuffle tree, then the warps in turn.  (One thread adding 1024 partial sums
-// was 58 us of dependent FP64 adds.)
-__device__ __forceinline__ double cta_sum(double s)
-{
-    __shared__ double sh[kRedThreads / 32];
-    for (int k = 16; k > 0; k >>= 1) s += __shfl_down_sync(0xffffffffu, s, k);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0)
-        for (int w = 1; w < kRedThreads / 32; w++) s += sh[w];
-    return s;                                            // thread 0's is the sum
-}
-
-__global__ void __launch_bounds__(kRedThreads) adj_dot_part_kernel(int64_t n, const double *a, const double *b, double *part)
-{
-    double s = 0.0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        s += a[i] * b[i];
-    s = cta_sum(s);
-    if (threadIdx.x == 0) part[blockIdx.x] = s;
-}
-
-__global__ void __launch_bounds__(kRedThreads) adj_dot_final_kernel(int nparts, const double *part, double scale, double *acc, int reset)
-{
-    double s = 0.0;
-    for (int q = threadIdx.x; q < nparts; q += blockDim.x) s += part[q];
-    s = cta_sum(s);
-    if (threadIdx.x == 0) *acc = reset ? s * scale : *acc + s * scale;
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < m.nfaces; q += ctas * blockDim.x) {
+        {
+            const int K = m.faces[q] >> 2, f = m.faces[q] & 3;
+            int j = m.nbr[f * nc + K];
+            bool wall = j < 0;
+            int fj = wall ? 0 : (m.nbrl[f * nc + K] & 3);
+            if (!rb_nonzero(Rb, nc, K) && (wall || !rb_nonzero(Rb, nc, j))) {
+                for (int v = 0; v < 3; v++) FVb[(v * 3 + f) * (size_t)nc + K] = 0.0;
+                zfb[f * (size_t)nc + K] = 0.0;
+                if (!wall) {
+                    for (int v = 0; v < 3; v++) FVb[(v * 3 + fj) * (size_t)nc + j] = 0.0;
+                    zfb[fj * (size_t)nc + j] = 0.0;
+                }
+                continue;
+            }
+            double nx = G(m, GEO_NX + f, K), ny = G(m, GEO_NY + f, K), l = G(m, GEO_LEN + f, K);
+            double cLf = quot(-l, by_area(m, K));
+            double Pb[3], PLb, PRb = 0.0;
+            double RLH = Rb[K], RLU = Rb[nc + K], RLV = Rb[2 * (size_t)nc + K];
+            Pb[0] = cLf * RLH;
+            Pb[1] = cLf * RLU;
+            Pb[2] = cLf * RLV;
+            PLb = cLf * (RLU * nx + RLV * ny);
+            double HfR = 0.0, HufR = 0.0, HvfR = 0.0, zR = 0.0;
+            if (!wall) {
+                double cRf = quot(l, by_area(m, j));
+                double RRH = Rb[j], RRU = Rb[nc + j], RRV = Rb[2 * (size_t)nc + j];
+                Pb[0] += cRf * RRH;
+                Pb[1] += cRf * RRU;
+                Pb[2] += cRf * RRV;
+                PRb = cRf * (RRU * nx + RRV * ny);
+                HfR = FV[(0 * 3 + fj) * (size_t)nc + j];
+                HufR = FV[(1 * 3 + fj) * (size_t)nc + j];
+                HvfR = FV[(2 * 3 + fj) * (size_t)nc + j];
+                zR = bed_under(m, j, fj);
+            }
+            double bL[4], bR[4];
+            flux_vjp(m, FV[(0 * 3 + f) * (size_t)nc + K], FV[(1 * 3 + f) * (size_t)nc + K],
+                     FV[(2 * 3 + f) * (size_t)nc + K], bed_under(m, K, f), HfR, HufR, HvfR, zR, nx, ny, wall, Pb, PLb,
+                     PRb, bL, bR, 0.0, wall ? -j : 0);
+            for (int v = 0; v < 3; v++) FVb[(v * 3 + f) * (size_t)nc + K] = bL[v];
+            zfb[f * (size_t)nc + K] = bL[3];
+            if (!wall) {
+                for (int v = 0; v < 3; v++) FVb[(v * 3 + fj) * (size_t)nc + j] = bR[v];
+                zfb[fj * (size_t)nc + j] = bR[3];
+            }
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -921,19 +996,23 @@ __global__ void __launch_bounds__(kRedThreads) adj_bed_vertex_kernel(int nv, int
         gOn[v] -= q;
         tb += q;
     }
-    tb = cta_sum(tb);
+    tb = cta_sum<kRedThreads>(tb);
     if (threadIdx.x == 0) part[blockIdx.x] = tb;
+}
+
+// *acc += the sum of nparts partial sums.
+__global__ void __launch_bounds__(kRedThreads) adj_sum_parts_kernel(int nparts, const double *part, double *acc)
+{
+    double s = 0.0;
+    for (int q = threadIdx.x; q < nparts; q += blockDim.x) s += part[q];
+    s = cta_sum<kRedThreads>(s);
+    if (threadIdx.x == 0) *acc += s;
 }
 
 __global__ void adj_axpy_kernel(int64_t n, const double *x, double *y)
 {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         y[i] += x[i];
-}
-
-__global__ void adj_scalar_add_kernel(double *y, const double *x)
-{
-    if (threadIdx.x == 0 && blockIdx.x == 0) *y += *x;
 }
 
 // CTAs of a reduction over n values: at least four values a thread, at most
@@ -944,10 +1023,6 @@ int grid_red(int64_t n)
     return (int)(g < 1 ? 1 : g < kAdjCflParts ? g : kAdjCflParts);
 }
 int grid_of(int n) { return (n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096; }
-// The two heavy reverse kernels run 128-thread CTAs: at 110 / 146 registers a
-// thread that fits 4 / 3 CTAs per SM (16 / 12 warps) where 256-thread CTAs fit
-// 2 / 1.
-constexpr int kVjpThreads = 128;
 int grid_vjp(int n) { return (n + kVjpThreads - 1) / kVjpThreads < 8192 ? (n + kVjpThreads - 1) / kVjpThreads : 8192; }
 
 AdjMesh adj_mesh(const DevPtrs &d, const StepParams &p)
@@ -956,6 +1031,7 @@ AdjMesh adj_mesh(const DevPtrs &d, const StepParams &p)
     m.nc = (int)d.nc;
     m.order = p.order;
     m.geo = static_cast<const double *>(d.geo);
+    m.rarea = d.rarea;
     m.z = static_cast<const double *>(d.z);
     m.zf = static_cast<const double *>(d.zf);
     m.rec = nullptr;
@@ -971,63 +1047,28 @@ AdjMesh adj_mesh(const DevPtrs &d, const StepParams &p)
 
 }  // namespace
 
-// Adds the VJP of the residual at w: (wb, zb) += (dR/dw, dR/dz)^T Rb, zb [4][nc]
-// = (cell beds, face beds of faces 0..2).  rec: the stage's reconstruction flags.
-// Scratch: FV, FVb [9][nc], zfb [3][nc], own [7][nc], send [12][nc].
-int adjoint_residual_vjp(const DevPtrs &d, const StepParams &p, const double *w, const uint8_t *rec, const double *Rb,
-                         double *wb, double *zb, double *FV, bool fv_given, double *FVb, double *zfb, double *own,
-                         double *send, void *stream, const AdjCfl *cfl)
+// CTAs of the per-cell kernels that also reduce.
+static int grid_cells(int nc) { const int g = (nc + kRedThreads - 1) / kRedThreads; return g < kAdjCflParts ? g : kAdjCflParts; }
+
+// The reverse of one step (see the top of this file).
+int adjoint_step(const DevPtrs &d, const StepParams &p, const AdjStep &a, void *stream)
 {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     AdjMesh m = adj_mesh(d, p);
-    m.rec = rec;
-    if (!rec) return (int)cudaErrorInvalidValue;
-    int grid = grid_of(m.nc);
-    if (!fv_given) adj_face_values_kernel<<<grid, 256, 0, s>>>(m, w, Rb, FV);
     if (!m.faces) return (int)cudaErrorInvalidValue;     // the face list is built by vg_adj_backward
-    adj_flux_vjp_kernel<<<grid_vjp(m.nfaces), kVjpThreads, 0, s>>>(m, FV, Rb, FVb, zfb);
-    if (cfl) {
-        const int parts = grid_red(m.nc);
-        adj_cfl_part_kernel<<<parts, kRedThreads, 0, s>>>(m.nc, cfl->bound, cfl->orig, cfl->part_b, cfl->part_o,
-                                                          cfl->part_k);
-        adj_cfl_face_kernel<<<1, kRedThreads, 0, s>>>(m, FV, parts, cfl->part_b, cfl->part_o, cfl->part_k, cfl->dtbar,
-                                             cfl->cfl, cfl->dt_max, FVb, zfb);
-    }
-    adj_recon_vjp_kernel<<<grid_vjp(m.nc), kVjpThreads, 0, s>>>(m, w, Rb, FVb, zfb, own, send);
-    adj_gather_kernel<<<grid, 256, 0, s>>>(m, own, send, wb, zb);
-    return (int)cudaGetLastError();
-}
-
-int adjoint_stage1(int nc, double dt, double hthr, const double *w, const double *R0, double *w1, double *H1pre,
-                   void *stream)
-{
-    adj_stage1_kernel<<<grid_of(nc), 256, 0, static_cast<cudaStream_t>(stream)>>>(nc, dt, hthr, w, R0, w1, H1pre);
-    return (int)cudaGetLastError();
-}
-
-int adjoint_stage2_rev(int nc, double dt, const uint8_t *mask2, const double *wb, double *wbn, double *wb1,
-                       double *Rb, void *stream)
-{
-    adj_stage2_rev_kernel<<<grid_of(nc), 256, 0, static_cast<cudaStream_t>(stream)>>>(nc, dt, mask2, wb, wbn, wb1,
-                                                                                       Rb);
-    return (int)cudaGetLastError();
-}
-
-int adjoint_stage1_rev(int nc, double dt, double hthr, const double *H1pre, const double *wb1, double *wbn,
-                       double *Rb, void *stream)
-{
-    adj_stage1_rev_kernel<<<grid_of(nc), 256, 0, static_cast<cudaStream_t>(stream)>>>(nc, dt, hthr, H1pre, wb1, wbn,
-                                                                                       Rb);
-    return (int)cudaGetLastError();
-}
-
-int adjoint_dot(int64_t n, const double *a, const double *b, double scale, double *acc, bool reset, double *part,
-                void *stream)
-{
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const int parts = grid_red(n);
-    adj_dot_part_kernel<<<parts, kRedThreads, 0, s>>>(n, a, b, part);
-    adj_dot_final_kernel<<<1, kRedThreads, 0, s>>>(parts, part, scale, acc, reset ? 1 : 0);
+    const int nc = m.nc, cells = grid_cells(nc), vjp_cells = grid_vjp(nc), vjp_faces = grid_vjp(m.nfaces);
+    AdjCfl cfl = a.cfl, none{};
+    cfl.nparts = cells;
+    adj_begin_kernel<<<cells, kRedThreads, 0, s>>>(nc, a.dt, p.hthr, a.w, a.R0, a.w1, a.H1pre, a.mask2, a.wb, a.wbn, a.wb1, a.Rb,
+                                                   cfl);
+    m.rec = a.rec1;
+    adj_flux_vjp_kernel<<<vjp_faces, kVjpThreads, 0, s>>>(m, a.FV1, a.Rb, a.FVb, a.zfb, none);
+    adj_recon_vjp_kernel<<<vjp_cells, kVjpThreads, 0, s>>>(m, a.w1, a.Rb, a.FVb, a.zfb, a.own, a.send, nullptr);
+    adj_gather_mid_kernel<<<cells, kRedThreads, 0, s>>>(m, a.own, a.send, a.zb, a.dt, p.hthr, a.H1pre, a.wb1, a.wbn, a.Rb, cfl);
+    m.rec = a.rec0;
+    adj_flux_vjp_kernel<<<vjp_faces + (cfl.dt ? 1 : 0), kVjpThreads, 0, s>>>(m, a.FV0, a.Rb, a.FVb, a.zfb, cfl);
+    adj_recon_vjp_kernel<<<vjp_cells, kVjpThreads, 0, s>>>(m, a.w, a.Rb, a.FVb, a.zfb, a.own, a.send, cfl.dt ? cfl.out : nullptr);
+    adj_gather_kernel<<<grid_of(nc), 256, 0, s>>>(m, a.own, a.send, a.wbn, a.zb);
     return (int)cudaGetLastError();
 }
 
@@ -1038,14 +1079,8 @@ int adjoint_bed_flush(int nc, int nv, const int32_t *vptr, const int32_t *vcell,
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int parts = grid_red(nv);
     adj_bed_vertex_kernel<<<parts, kRedThreads, 0, s>>>(nv, nc, vptr, vcell, zs, uplift, onset, rise, t, gU, gOn, part);
-    adj_dot_final_kernel<<<1, kRedThreads, 0, s>>>(parts, part, 1.0, tsum, 0);
+    adj_sum_parts_kernel<<<1, kRedThreads, 0, s>>>(parts, part, tsum);
     adj_axpy_kernel<<<grid_of(4 * nc), 256, 0, s>>>(4 * (int64_t)nc, zs, zb_total);
-    return (int)cudaGetLastError();
-}
-
-int adjoint_scalar_add(double *y, const double *x, void *stream)
-{
-    adj_scalar_add_kernel<<<1, 32, 0, static_cast<cudaStream_t>(stream)>>>(y, x);
     return (int)cudaGetLastError();
 }
 

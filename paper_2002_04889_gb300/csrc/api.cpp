@@ -1546,7 +1546,7 @@ int vg_adj_backward(vg_ctx *c, const double *dJ_deta, double *dJ_dH0, double *dJ
         (rc = alloc(w3 * (size_t)RC, &R0seg)) || (rc = alloc(((size_t)nc * RC + 7) / 8, &m2raw)) ||
         (rc = alloc((2 * (size_t)nc * RC + 7) / 8, &recraw)) ||
         (adaptive && ((rc = alloc(w3 * (size_t)RC, &R1seg)) || (rc = alloc((size_t)nc * RC, &bndseg)) ||
-                      (rc = alloc(8 + 3 * (size_t)kAdjCflParts, &cflscr))))) {
+                      (rc = alloc(16 + 4 * (size_t)kAdjCflParts, &cflscr))))) {
         for (void *q : bufs) cudaFree(q);
         return rc;
     }
@@ -1594,15 +1594,15 @@ int vg_adj_backward(vg_ctx *c, const double *dJ_deta, double *dJ_dH0, double *dJ
     double *tsum = bed ? bedscr : nullptr, *bedpart = bed ? bedscr + 8 : nullptr;
     double *zacc;                          // where the bed adjoint goes: per step (moving bed) or total
     AdjCfl cfl{};
-    double *dtbar = nullptr, *dotpart = nullptr;
     if (adaptive) {
-        dtbar = cflscr;
-        dotpart = cflscr + 8;
         cfl.orig = c->old_of_new;
-        cfl.dtbar = dtbar;
+        cfl.tsum = tsum;
         cfl.cfl = c->adj_cfl;
         cfl.dt_max = c->adj_dt_max;
-        cfl.part_b = cflscr + 8 + kAdjCflParts;
+        cfl.out = reinterpret_cast<AdjCflFace *>(cflscr);
+        cfl.part_s1 = cflscr + 16;
+        cfl.part_s0 = cfl.part_s1 + kAdjCflParts;
+        cfl.part_b = cfl.part_s0 + kAdjCflParts;
         cfl.part_o = reinterpret_cast<int *>(cfl.part_b + kAdjCflParts);
         cfl.part_k = cfl.part_o + kAdjCflParts;
     }
@@ -1620,7 +1620,6 @@ int vg_adj_backward(vg_ctx *c, const double *dJ_deta, double *dJ_dH0, double *dJ
     p.dt_fixed = c->adj_dt;
     p.t_end = 0.0;
     p.dt_max = 0.0;
-    const double hthr = p.hthr;
     void *st = (void *)c->stream;
     DevPtrs d = dev_ptrs(c);
     d.sc = asc;
@@ -1689,30 +1688,31 @@ int vg_adj_backward(vg_ctx *c, const double *dJ_deta, double *dJ_dH0, double *dJ
                 if ((e = launch_bed_update(d, p, nullptr, 64, false, tn[n], st))) return e;     // bed of step n
                 if ((e = (int)cudaMemsetAsync(zstep, 0, 8 * 4 * (size_t)nc, c->stream))) return e;
             }
-            if ((e = adjoint_stage1(nc, dtn, hthr, w, R0, w1, H1pre, st))) return e;
-            if ((e = adjoint_stage2_rev(nc, dtn, m2seg + (size_t)r * nc, wb, wbn, wb1, Rb, st))) return e;
-            // dt-bar, stage 2: sum w-bar_pre . R1 / 2 = sum Rb . R1 / dt
-            if (adaptive && (e = adjoint_dot((int64_t)w3, Rb, R1seg + (size_t)r * w3, 1.0 / dtn, dtbar, true,
-                                             dotpart, st)))
-                return e;
-            double *FV0 = FVseg + (size_t)r * 18 * nc, *FV1 = FV0 + 9 * (size_t)nc;
-            const uint8_t *rec0 = recseg + (size_t)r * 2 * nc, *rec1 = rec0 + nc;
-            if ((e = adjoint_residual_vjp(d, p, w1, rec1, Rb, wb1, zacc, FV1, true, FVb, zfb, own, send, st))) return e;
-            if ((e = adjoint_stage1_rev(nc, dtn, hthr, H1pre, wb1, wbn, Rb, st))) return e;
-            // dt-bar, stage 1: sum w1-bar_pre . R0 = sum Rb . R0 / dt
-            if (adaptive && (e = adjoint_dot((int64_t)w3, Rb, R0, 1.0 / dtn, dtbar, false, dotpart, st))) return e;
-            // a moving bed: every later bed depends on this dt through the time
-            if (adaptive && bed && (e = adjoint_scalar_add(dtbar, tsum, st))) return e;
-            cfl.bound = adaptive ? bndseg + (size_t)r * nc : nullptr;
-            if ((e = adjoint_residual_vjp(d, p, w, rec0, Rb, wbn, zacc, FV0, true, FVb, zfb, own, send, st,
-                                          adaptive ? &cfl : nullptr)))
-                return e;
+            AdjStep a{};
+            a.dt = dtn;
+            a.w = w;
+            a.R0 = R0;
+            a.FV0 = FVseg + (size_t)r * 18 * nc;
+            a.FV1 = a.FV0 + 9 * (size_t)nc;
+            a.mask2 = m2seg + (size_t)r * nc;
+            a.rec0 = recseg + (size_t)r * 2 * nc;
+            a.rec1 = a.rec0 + nc;
+            a.wb = wb; a.wbn = wbn; a.wb1 = wb1; a.zb = zacc; a.Rb = Rb; a.w1 = w1; a.H1pre = H1pre;
+            a.FVb = FVb; a.zfb = zfb; a.own = own; a.send = send;
+            if (adaptive) {
+                a.cfl = cfl;
+                a.cfl.dt = dtn;
+                a.cfl.R1 = R1seg + (size_t)r * w3;
+                a.cfl.R0 = R0;
+                a.cfl.bound = bndseg + (size_t)r * nc;
+            }
+            if ((e = adjoint_step(d, p, a, st))) return e;
             if ((e = adjoint_gauge(G, c->gauge_cells, W + (size_t)n * G, wbn, zacc, st))) return e;
             if (bed && (e = adjoint_bed_flush(nc, nv, vptr, vcell, zstep, c->bed_uplift, c->bed_onset, c->bed_rise,
                                               tn[n], gU, gOn, zb, tsum, bedpart, st)))
                 return e;
             std::swap(wb, wbn);
-            c->launches += (adaptive ? 17 : 11) + (bed ? 6 : 0);
+            c->launches += 8 + (bed ? 5 : 0);
             return 0;
         };
         if (!binomial) {

@@ -203,32 +203,41 @@ int launch_batch_step_f64(const void *table, int n_mesh, int n_items, int n_entr
                           int grid, size_t smem, int scen_at, const StepParams &p, bool gauges, void *stream);
 
 // Discrete adjoint (adjoint_f64.cu, FP64 contexts).
-// The CFL time step's dependence on the state (adaptive steps): orig = original
-// cell ids [nc] (argmin ties), bound = the CFL bound of every cell [nc] recorded by
-// the forward stage-1 kernel, *dtbar = the step's dt adjoint, cfl / dt_max as in the
-// forward run, part_* scratch of kAdjCflParts entries.
 constexpr int kAdjCflParts = 1024;
-struct AdjCfl {
-    const int32_t *orig;
-    const double *bound;
-    const double *dtbar;
-    double cfl, dt_max;
-    double *part_b;
-    int *part_o, *part_k;
+// The face that set a CFL step, and its wave speed's adjoint of (H, Hu, Hv)_f and the
+// bed on both sides (cell -1: none).
+struct AdjCflFace {
+    double bar[2][4];
+    int cell[2], face[2];
 };
-// FV: the face values at w, precomputed by the forward stage kernel (fv_out)
-// or, if fv_given is false, computed here into FV.  cfl (may be NULL): also
-// the adjoint of the stage-1 CFL time step through the wave speed of the face
-// that set it.
-// rec: the reconstruction flags [nc] of the stage (recorded by the forward kernel
-// with rec_out).  zb [4][nc] receives the bed adjoints: row 0 the cell beds z_K,
-// rows 1..3 the face beds z_f of faces 0..2.
-int adjoint_residual_vjp(const DevPtrs &d, const StepParams &p, const double *w, const uint8_t *rec, const double *Rb,
-                         double *wb, double *zb, double *FV, bool fv_given, double *FVb, double *zfb, double *own,
-                         double *send, void *stream, const AdjCfl *cfl = nullptr);
-// *acc (= or +=) scale * sum_i a[i] b[i], deterministic; part: kAdjCflParts doubles.
-int adjoint_dot(int64_t n, const double *a, const double *b, double scale, double *acc, bool reset, double *part,
-                void *stream);
+// The CFL time step's dependence on the state (adaptive steps; dt = 0: none): dt the
+// step taken, R1 / R0 the stages' residuals, orig = original cell ids [nc] (argmin
+// ties), bound = the CFL bound of every cell [nc] recorded by the forward stage-1
+// kernel, tsum (may be null) the adjoint of time, cfl / dt_max as in the forward run,
+// part_* scratch of kAdjCflParts entries, out scratch.
+struct AdjCfl {
+    double dt, cfl, dt_max;
+    const double *R1, *R0, *bound, *tsum;
+    const int32_t *orig;
+    double *part_s1, *part_s0, *part_b;
+    int *part_o, *part_k;
+    int nparts;
+    AdjCflFace *out;
+};
+// The reverse of one step of size dt from w: wb (adjoint of w^{n+1}, read) -> wbn
+// (adjoint of w^n, written), zb [4][nc] += the bed adjoints (row 0 the cell beds z_K,
+// rows 1..3 the face beds z_f of faces 0..2).  Records of the forward run: R0, the
+// stage-2 dry-fix branches mask2, the stages' reconstruction flags rec0, rec1 and face
+// values FV0, FV1.  Scratch: w1, wb1, Rb [3][nc], H1pre [nc], FVb [9][nc], zfb [3][nc],
+// own [7][nc], send [12][nc].
+struct AdjStep {
+    double dt;
+    const double *w, *R0, *FV0, *FV1, *wb;
+    const uint8_t *mask2, *rec0, *rec1;
+    double *wbn, *zb, *w1, *H1pre, *wb1, *Rb, *FVb, *zfb, *own, *send;
+    AdjCfl cfl;
+};
+int adjoint_step(const DevPtrs &d, const StepParams &p, const AdjStep &a, void *stream);
 // Moving bed: one step's bed adjoint zs [4][nc] (cell beds, then the face beds of
 // faces 0..2) at time t -> uplift / onset gradients gU, gOn [nv] (+=), zb_total
 // [4][nc] (+= zs), *tsum (+= the adjoint of t); vptr [nv+1], vcell: the cells
@@ -236,14 +245,6 @@ int adjoint_dot(int64_t n, const double *a, const double *b, double scale, doubl
 int adjoint_bed_flush(int nc, int nv, const int32_t *vptr, const int32_t *vcell, double *zs, const double *uplift,
                       const double *onset, double rise, double t, double *gU, double *gOn, double *zb_total,
                       double *tsum, double *part, void *stream);
-// *y += *x on the device.
-int adjoint_scalar_add(double *y, const double *x, void *stream);
-int adjoint_stage1(int nc, double dt, double hthr, const double *w, const double *R0, double *w1, double *H1pre,
-                   void *stream);
-int adjoint_stage2_rev(int nc, double dt, const uint8_t *mask2, const double *wb, double *wbn, double *wb1,
-                       double *Rb, void *stream);
-int adjoint_stage1_rev(int nc, double dt, double hthr, const double *H1pre, const double *wb1, double *wbn,
-                       double *Rb, void *stream);
 int adjoint_gauge(int n_gauges, const int32_t *cells, const double *weights, double *wb, double *zb, void *stream);
 
 // Utility kernels (util_kernels.cu).
