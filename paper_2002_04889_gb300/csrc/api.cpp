@@ -350,6 +350,36 @@ int upload_face_beds(vg_ctx *c)
     return VG_OK;
 }
 
+// Orders a block's faces so that the eight lanes that one shared-memory cycle serves
+// find their 16-byte slots in different banks (slot mod 8), on the left side and on the
+// right: greedily, from the fullest pair of bank groups that is still free.  In mesh
+// order about 2.5 lanes shared a group (4M triangles, us a step: 231.8 -> 228.2).
+template <typename Face>
+void order_for_banks(std::vector<Face> &v)
+{
+    std::vector<Face> pool[64], out;
+    for (const Face &x : v) pool[(x.slots & 7) * 8 + ((x.slots >> 16) & 7)].push_back(x);
+    out.reserve(v.size());
+    while (out.size() < v.size()) {
+        unsigned left = 0, right = 0;                 // groups taken in this cycle
+        for (int lane = 0; lane < 8 && out.size() < v.size(); lane++) {
+            int best = -1;
+            size_t most = 0;
+            int score = -1;                           // 2: both sides free, 1: one, 0: none
+            for (int g = 0; g < 64; g++) {
+                if (pool[g].empty()) continue;
+                const int s = !((left >> (g >> 3)) & 1) + !((right >> (g & 7)) & 1);
+                if (s > score || (s == score && pool[g].size() > most)) { best = g; most = pool[g].size(); score = s; }
+            }
+            out.push_back(pool[best].back());
+            pool[best].pop_back();
+            left |= 1u << (best >> 3);
+            right |= 1u << (best & 7);
+        }
+    }
+    v.swap(out);
+}
+
 // FP32 partition arrays: the codes of block and ring-1 cells and the face records
 // of every block (layouts: block_f32.cuh).
 int upload_partition_f32(vg_ctx *c)
@@ -381,29 +411,33 @@ int upload_partition_f32(vg_ctx *c)
             for (int f = 0; f < 3; f++) code_of(m.ring1_nbr[3 * i + f], false, B + h, f, ring[i]);
         }
         // interior faces first, so that whole warps take the interior branch
-        int32_t at = m.fq_ptr[b];
-        for (int boundary = 0; boundary < 2; boundary++)
-            for (int32_t q = m.fq_ptr[b]; q < m.fq_ptr[b + 1]; q++) {
-                const int l = m.fq[q] >> 2, f = m.fq[q] & 3;
-                const int64_t k = c0 + l;
-                const uint16_t code = m.nbrl[f * nc + k];
-                if ((code >= NBR_ABSORB) != (boundary != 0)) continue;
-                uint32_t sl = (uint32_t)(f * L1 + l), sr = code;
-                int64_t kk = k;                   // the left cell and its face
-                int ff = f;
-                if (!boundary) {
-                    const int nl = code >> 2, nf = code & 3;
-                    sr = (uint32_t)(nf * L1 + nl);
-                    const int64_t j = m.nbr[f * nc + k];
-                    if (j < k) { std::swap(sl, sr); kk = j; ff = nf; }
-                }
-                float *o = &fr[4 * (size_t)at++];
-                o[0] = (float)m.geo[(size_t)(GEO_NX + ff) * nc + kk];
-                o[1] = (float)m.geo[(size_t)(GEO_NY + ff) * nc + kk];
-                o[2] = (float)m.geo[(size_t)(GEO_LEN + ff) * nc + kk];
-                const uint32_t slots = sl | (sr << 16);
-                std::memcpy(&o[3], &slots, 4);
+        struct Face { uint32_t slots; int64_t cell; int f; };
+        std::vector<Face> inner, edge;
+        for (int32_t q = m.fq_ptr[b]; q < m.fq_ptr[b + 1]; q++) {
+            const int l = m.fq[q] >> 2, f = m.fq[q] & 3;
+            const int64_t k = c0 + l;
+            const uint16_t code = m.nbrl[f * nc + k];
+            const uint32_t sl = (uint32_t)(f * L1 + l);
+            if (code >= NBR_ABSORB) {
+                edge.push_back({sl | ((uint32_t)code << 16), k, f});
+                continue;
             }
+            const int nl = code >> 2, nf = code & 3;
+            const uint32_t sr = (uint32_t)(nf * L1 + nl);
+            const int64_t j = m.nbr[f * nc + k];
+            if (j < k) inner.push_back({sr | (sl << 16), j, nf});     // the left cell: the lower internal id
+            else inner.push_back({sl | (sr << 16), k, f});
+        }
+        order_for_banks(inner);
+        inner.insert(inner.end(), edge.begin(), edge.end());
+        int32_t at = m.fq_ptr[b];
+        for (const Face &x : inner) {
+            float *o = &fr[4 * (size_t)at++];
+            o[0] = (float)m.geo[(size_t)(GEO_NX + x.f) * nc + x.cell];
+            o[1] = (float)m.geo[(size_t)(GEO_NY + x.f) * nc + x.cell];
+            o[2] = (float)m.geo[(size_t)(GEO_LEN + x.f) * nc + x.cell];
+            std::memcpy(&o[3], &x.slots, 4);
+        }
     }
     dfree(c->codes); dfree(c->ring_codes); dfree(c->fr);
     int rc;
