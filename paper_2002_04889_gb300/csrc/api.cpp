@@ -22,6 +22,7 @@ namespace {
 
 constexpr int kRingCap = 2048;       // gauge records held on the device between drains
 constexpr int kDiagBlocks = 1024;
+constexpr size_t kPinned = 256 << 10;   // pinned host memory of a context
 constexpr int kKernels = 7;
 const char *kKernelNames[kKernels] = {"stage1", "stage2", "post_step", "bed_update",
                                       "rk_update1", "residual_w1", "rk_update2"};
@@ -54,6 +55,13 @@ struct vg_ctx {
     int64_t n_adj_faces = 0;          // built by the first adjoint sweep of a mesh
     uint16_t *nbrl = nullptr, *ring1_nbr = nullptr, *fq = nullptr;
     DevScalars *sc = nullptr;
+    // the device scalars as last read (mirror_ok: nothing has changed them since),
+    // t_end as the device has it, and pinned memory for reads that one wait completes:
+    // scalars, then gauge records
+    DevScalars mirror{};
+    bool mirror_ok = false;
+    double dev_t_end = 0.0;
+    unsigned char *pinned = nullptr;
     int32_t *gauge_cells = nullptr;
     double *ring_t = nullptr, *ring_eta = nullptr;
     double *diag_part = nullptr, *diag_out = nullptr;
@@ -280,7 +288,6 @@ StepParams step_params(const vg_ctx *c)
     p.hthr = c->prm.h_threshold;
     p.dt_fixed = c->prm.dt_fixed;
     p.dt_max = c->prm.dt_max;
-    p.t_end = c->prm.t_end;
     p.order = c->prm.order;
     p.gauge_every = c->prm.gauge_every;
     p.fp64_fast = c->precision == 64 && !c->prm.fp64_literal;
@@ -687,27 +694,76 @@ int build_graph(vg_ctx *c)
 
 int read_scalars(vg_ctx *c, DevScalars &s)
 {
-    VG_CUDA(c, cudaMemcpyAsync(&s, c->sc, sizeof(DevScalars), cudaMemcpyDeviceToHost, c->stream));
-    VG_CUDA(c, cudaStreamSynchronize(c->stream));
+    if (!c->mirror_ok) {
+        VG_CUDA(c, cudaMemcpyAsync(c->pinned, c->sc, sizeof(DevScalars), cudaMemcpyDeviceToHost, c->stream));
+        VG_CUDA(c, cudaStreamSynchronize(c->stream));
+        std::memcpy(&c->mirror, c->pinned, sizeof(DevScalars));
+        c->mirror_ok = true;
+    }
+    s = c->mirror;
+    return VG_OK;
+}
+
+// Gives the device the context's t_end (the step kernels read it there).
+int push_t_end(vg_ctx *c)
+{
+    if (c->dev_t_end == c->prm.t_end) return VG_OK;
+    VG_CUDA(c, cudaMemcpyAsync(&c->sc->t_end, &c->prm.t_end, sizeof(double), cudaMemcpyHostToDevice, c->stream));
+    c->dev_t_end = c->prm.t_end;
+    c->mirror.t_end = c->prm.t_end;
+    return VG_OK;
+}
+
+// The device ring holds no records any more (the stream orders the store before the
+// next step).
+int empty_ring(vg_ctx *c, DevScalars &s)
+{
+    static const long long zero = 0;
+    VG_CUDA(c, cudaMemcpyAsync(&c->sc->n_rec, &zero, sizeof(zero), cudaMemcpyHostToDevice, c->stream));
+    s.n_rec = 0;
+    c->mirror.n_rec = 0;
     return VG_OK;
 }
 
 // Move the device gauge records to the host and empty the device ring.
 int drain_gauges(vg_ctx *c, DevScalars &s)
 {
-    if (c->n_gauges > 0 && s.n_rec > 0) {
+    if (s.n_rec == 0) return VG_OK;
+    if (c->n_gauges > 0) {
         size_t n = (size_t)s.n_rec, G = (size_t)c->n_gauges;
         size_t t0 = c->rec_t.size();
         c->rec_t.resize(t0 + n);
         c->rec_eta.resize((t0 + n) * G);
         VG_CUDA(c, cudaMemcpyAsync(c->rec_t.data() + t0, c->ring_t, n * 8, cudaMemcpyDeviceToHost, c->stream));
         VG_CUDA(c, cudaMemcpyAsync(c->rec_eta.data() + t0 * G, c->ring_eta, n * G * 8, cudaMemcpyDeviceToHost, c->stream));
+        VG_CUDA(c, cudaStreamSynchronize(c->stream));
     }
-    static const long long zero = 0;
-    VG_CUDA(c, cudaMemcpyAsync(&c->sc->n_rec, &zero, sizeof(zero), cudaMemcpyHostToDevice, c->stream));
+    return empty_ring(c, s);
+}
+
+// After queued steps: the scalars and at most n_max gauge records, whose number only
+// the scalars tell, with one wait where the records fit the pinned memory.
+int read_and_drain(vg_ctx *c, DevScalars &s, int64_t n_max)
+{
+    const size_t G = (size_t)c->n_gauges, n = (size_t)std::min<int64_t>(n_max, kRingCap);
+    const size_t at_t = 128, at_eta = at_t + 8 * n;
+    if (G == 0 || at_eta + 8 * n * G > kPinned) {
+        int rc = read_scalars(c, s);
+        return rc ? rc : drain_gauges(c, s);
+    }
+    VG_CUDA(c, cudaMemcpyAsync(c->pinned, c->sc, sizeof(DevScalars), cudaMemcpyDeviceToHost, c->stream));
+    VG_CUDA(c, cudaMemcpyAsync(c->pinned + at_t, c->ring_t, 8 * n, cudaMemcpyDeviceToHost, c->stream));
+    VG_CUDA(c, cudaMemcpyAsync(c->pinned + at_eta, c->ring_eta, 8 * n * G, cudaMemcpyDeviceToHost, c->stream));
     VG_CUDA(c, cudaStreamSynchronize(c->stream));
-    s.n_rec = 0;
-    return VG_OK;
+    std::memcpy(&c->mirror, c->pinned, sizeof(DevScalars));
+    c->mirror_ok = true;
+    s = c->mirror;
+    const size_t got = (size_t)s.n_rec;
+    if (got > n) return drain_gauges(c, s);          // (more than foreseen: read them all)
+    const double *t = reinterpret_cast<const double *>(c->pinned + at_t), *e = reinterpret_cast<const double *>(c->pinned + at_eta);
+    c->rec_t.insert(c->rec_t.end(), t, t + got);
+    c->rec_eta.insert(c->rec_eta.end(), e, e + got * G);
+    return got ? empty_ring(c, s) : VG_OK;
 }
 
 int check_flags(vg_ctx *c, const DevScalars &s, int64_t neg_before)
@@ -761,6 +817,8 @@ int record_now(vg_ctx *c)
     int e = launch_record_gauges(dev_ptrs(c), c->w[c->cur], c->precision, (void *)c->stream);
     if (e) return cuda_fail(c, (cudaError_t)e, "gauge record launch");
     c->launches++;
+    if (c->mirror.n_rec < kRingCap) c->mirror.n_rec++;       // as the kernel counts
+    else c->mirror_ok = false;
     return VG_OK;
 }
 
@@ -848,7 +906,8 @@ int vg_create(vg_ctx **out, int precision, int device, void *cuda_stream)
     }
     if (cudaMalloc((void **)&c->sc, sizeof(DevScalars)) != cudaSuccess ||
         cudaMalloc((void **)&c->diag_part, 8 * 3 * kDiagBlocks) != cudaSuccess ||
-        cudaMalloc((void **)&c->diag_out, 8 * 4) != cudaSuccess) {
+        cudaMalloc((void **)&c->diag_out, 8 * 4) != cudaSuccess ||
+        cudaHostAlloc((void **)&c->pinned, kPinned, cudaHostAllocDefault) != cudaSuccess) {
         vg_destroy(c);
         return VG_ENOMEM;
     }
@@ -868,6 +927,7 @@ void vg_destroy(vg_ctx *c)
     dfree(c->sc);
     dfree(c->diag_part);
     dfree(c->diag_out);
+    if (c->pinned) cudaFreeHost(c->pinned);
     for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
     delete c;
@@ -974,6 +1034,8 @@ static int set_state_impl(vg_ctx *c, const void *H, const void *Hu, const void *
 {
     DevScalars s;
     reset_scalars_host(c, s, t);
+    s.t_end = c->dev_t_end = c->prm.t_end;
+    c->mirror_ok = false;
     VG_CUDA(c, cudaMemcpyAsync(c->sc, &s, sizeof(s), cudaMemcpyHostToDevice, c->stream));
     c->cur = 0;
     if (c->bed_on) {
@@ -1062,8 +1124,9 @@ static int get_state_host(vg_ctx *c, void *H, void *Hu, void *Hv, bool dbl, doub
                                          (void *)c->stream);
         if (e) return cuda_fail(c, (cudaError_t)e, "state export launch");
         c->launches++;
+        VG_CUDA(c, cudaStreamSynchronize(c->stream));
         DevScalars s;
-        if ((rc = read_scalars(c, s))) return rc;     // synchronises the stream
+        if ((rc = read_scalars(c, s))) return rc;
         if (t) *t = s.t;
         return VG_OK;
     }
@@ -1076,6 +1139,7 @@ static int get_state_host(vg_ctx *c, void *H, void *Hu, void *Hv, bool dbl, doub
     VG_CUDA(c, cudaMemcpyAsync(H, st, bytes, cudaMemcpyDeviceToHost, c->stream));
     VG_CUDA(c, cudaMemcpyAsync(Hu, st + bytes, bytes, cudaMemcpyDeviceToHost, c->stream));
     VG_CUDA(c, cudaMemcpyAsync(Hv, st + 2 * bytes, bytes, cudaMemcpyDeviceToHost, c->stream));
+    VG_CUDA(c, cudaStreamSynchronize(c->stream));
     DevScalars s;
     if ((rc = read_scalars(c, s))) return rc;
     if (t) *t = s.t;
@@ -1130,8 +1194,7 @@ int vg_set_gauges(vg_ctx *c, int32_t n, const double *xy)
     if ((rc = dmalloc(c, (void **)&c->ring_eta, 8 * (size_t)n * kRingCap))) return rc;
     VG_CUDA(c, cudaMemcpy(c->gauge_cells, internal.data(), 4 * n, cudaMemcpyHostToDevice));
     c->n_gauges = n;
-    static const long long zero = 0;
-    VG_CUDA(c, cudaMemcpyAsync(&c->sc->n_rec, &zero, sizeof(zero), cudaMemcpyHostToDevice, c->stream));
+    if ((rc = empty_ring(c, c->mirror))) return rc;
     return record_now(c);
 }
 
@@ -1150,12 +1213,17 @@ int vg_step(vg_ctx *c, int64_t n_steps)
     DevScalars s;
     int rc = read_scalars(c, s);
     if (rc) return rc;
-    if ((rc = drain_gauges(c, s))) return rc;
+    if ((rc = push_t_end(c))) return rc;
     int64_t neg_before = s.neg_count;
-    int64_t chunk_max = c->n_gauges > 0 ? (int64_t)(kRingCap - 1) * c->prm.gauge_every : n_steps;
-    if (chunk_max < 1) chunk_max = 1;
     while (n_steps > 0) {
-        int64_t chunk = std::min(n_steps, chunk_max);
+        // with gauges, as many steps as the ring surely takes beside what it holds
+        int64_t chunk = n_steps;
+        if (c->n_gauges > 0) {
+            if (s.n_rec >= kRingCap - 1 && (rc = drain_gauges(c, s))) return rc;
+            chunk = std::min(n_steps, (int64_t)(kRingCap - 1 - s.n_rec) * c->prm.gauge_every);
+        }
+        const int64_t records = s.n_rec + (chunk + c->prm.gauge_every - 1) / c->prm.gauge_every;
+        c->mirror_ok = false;
         n_steps -= chunk;
         int64_t left = chunk;
         if (c->profile) {
@@ -1184,9 +1252,8 @@ int vg_step(vg_ctx *c, int64_t n_steps)
                 c->launches += step_kernels(c);
             }
         }
-        if ((rc = read_scalars(c, s))) return rc;
+        if ((rc = read_and_drain(c, s, records))) return rc;
         if ((rc = ev_collect(c))) return rc;
-        if ((rc = drain_gauges(c, s))) return rc;
         if ((rc = check_flags(c, s, neg_before))) return rc;
     }
     cudaError_t e = cudaGetLastError();
@@ -1201,8 +1268,7 @@ int vg_advance_to(vg_ctx *c, double t_target)
     vg_params saved = c->prm;
     vg_params p = saved;
     if (!(p.t_end > 0) || p.t_end > t_target) p.t_end = t_target;
-    c->prm = p;
-    c->graph_dirty = true;
+    c->prm = p;                  // t_end is read from the device: the graph stays
     int rc = VG_OK;
     for (int iter = 0; iter < 1000000; iter++) {
         DevScalars s;
@@ -1214,7 +1280,6 @@ int vg_advance_to(vg_ctx *c, double t_target)
         if (s.t <= t_before) { rc = fail(c, VG_ESTATE, "time does not advance (zero time step)"); break; }
     }
     c->prm = saved;
-    c->graph_dirty = true;
     return rc;
 }
 
@@ -1250,6 +1315,7 @@ int vg_get_diagnostics(vg_ctx *c, vg_diag *d)
     c->launches += 2;
     double out[3];
     VG_CUDA(c, cudaMemcpyAsync(out, c->diag_out, 8 * 3, cudaMemcpyDeviceToHost, c->stream));
+    VG_CUDA(c, cudaStreamSynchronize(c->stream));
     DevScalars s;
     int rc = read_scalars(c, s);
     if (rc) return rc;
@@ -1461,12 +1527,14 @@ int vg_adj_forward(vg_ctx *c, int64_t n_steps, double dt, int64_t checkpoint_eve
     // restart the gauge record at the current state
     DevScalars s;
     int rc = read_scalars(c, s);
+    if (!rc) rc = push_t_end(c);
     const double t0 = s.t;
     if (!rc) rc = drain_gauges(c, s);
     c->rec_t.clear();
     c->rec_eta.clear();
     if (!rc) rc = record_now(c);
     for (int64_t n = 0; n < n_steps && !rc; n++) {
+        c->mirror_ok = false;
         if (n % C == 0) {
             cudaError_t e = cudaMemcpyAsync(c->ckpt[n / C], c->w[c->cur], bytes, cudaMemcpyDeviceToDevice, c->stream);
             if (e != cudaSuccess) { rc = cuda_fail(c, e, "checkpoint copy"); break; }
@@ -1652,7 +1720,6 @@ int vg_adj_backward(vg_ctx *c, const double *dJ_deta, double *dJ_dH0, double *dJ
     reset_scalars_host(c, s0, 0.0);
     StepParams p = step_params(c);
     p.dt_fixed = c->adj_dt;
-    p.t_end = 0.0;
     p.dt_max = 0.0;
     void *st = (void *)c->stream;
     DevPtrs d = dev_ptrs(c);
@@ -1916,7 +1983,7 @@ int vg_step_noalloc(vg_ctx *c, const void *w_in, void *w_out, double t, double *
     d.ring_eta = nullptr;
     StepParams p = step_params(c);
     void *s = (void *)c->stream;
-    if ((e = noalloc_launch_init(sc, t, c->precision, s))) return cuda_fail(c, (cudaError_t)e, "scratch init launch");
+    if ((e = noalloc_launch_init(sc, t, c->prm.t_end, c->precision, s))) return cuda_fail(c, (cudaError_t)e, "scratch init launch");
     e = c->precision == 64 ? launch_stage1_f64(d, p, w_in, c->cfg1, s)
                            : launch_stage_soa_f32(d, p, 1, w_in, w_out, c->cfg1, s);
     if (e) return cuda_fail(c, (cudaError_t)e, "stage 1 launch");
@@ -1926,8 +1993,9 @@ int vg_step_noalloc(vg_ctx *c, const void *w_in, void *w_out, double t, double *
     if ((e = launch_post_step(d, p, w_out, c->precision, s))) return cuda_fail(c, (cudaError_t)e, "post-step launch");
     c->launches += 4;
     DevScalars r;
-    VG_CUDA(c, cudaMemcpyAsync(&r, sc, sizeof(DevScalars), cudaMemcpyDeviceToHost, c->stream));
+    VG_CUDA(c, cudaMemcpyAsync(c->pinned, sc, sizeof(DevScalars), cudaMemcpyDeviceToHost, c->stream));
     VG_CUDA(c, cudaStreamSynchronize(c->stream));
+    std::memcpy(&r, c->pinned, sizeof(DevScalars));
     if (dt_out) *dt_out = r.dt;
     if (r.flags & FLAG_NONFINITE_STATE) return fail(c, VG_ENONFINITE, "a non-finite value appeared in the state");
     if (r.flags & FLAG_NONFINITE_DT) return fail(c, VG_ENONFINITE, "the time step is not finite");

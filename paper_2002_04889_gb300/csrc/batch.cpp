@@ -53,6 +53,7 @@ struct vg_batch {
     std::vector<char> has_state;           // per scenario
     DevScalars *sc_all = nullptr;          // [n_entries + 1]
     int n_entries = 0;
+    double dev_t_end = 0.0;                // t_end in the batch-wide device record
     void *table[2] = {nullptr, nullptr};   // device BatchMesh arrays for both step parities
     int n_items = 0;
     int grid = 0;
@@ -191,7 +192,6 @@ StepParams batch_params(const vg_batch *b)
     p.hthr = b->prm.h_threshold;
     p.dt_fixed = b->prm.dt_fixed;
     p.dt_max = b->prm.dt_max;
-    p.t_end = b->prm.t_end;
     p.order = b->prm.order;
     p.gauge_every = b->prm.gauge_every > 0 ? b->prm.gauge_every : 1;
     p.fp64_fast = b->precision == 64 && !b->prm.fp64_literal;
@@ -238,6 +238,11 @@ int ready(vg_batch *b)
     if (b->dirty) {
         int rc = rebuild(b);
         if (rc) return rc;
+    }
+    if (b->dev_t_end != b->prm.t_end) {
+        VB_CUDA(b, cudaMemcpyAsync(&b->sc_all[b->n_entries].t_end, &b->prm.t_end, sizeof(double), cudaMemcpyHostToDevice,
+                                   b->stream));
+        b->dev_t_end = b->prm.t_end;
     }
     if (!b->graph2) {
         int rc = build_batch_graph(b);
@@ -475,6 +480,7 @@ int vg_batch_add_mesh(vg_batch *b, int64_t nv, const double *xy, int64_t nc, con
     VB_CUDA(b, cudaMemcpy(sc, host.data(), sizeof(DevScalars) * (n_new + 1), cudaMemcpyHostToDevice));
     cudaFree(b->sc_all);
     b->sc_all = sc;
+    b->dev_t_end = 0.0;
     b->n_entries = n_new;
     b->has_state.resize(n_new, 0);
     b->meshes.push_back(M);
@@ -578,13 +584,8 @@ int vg_batch_run(vg_batch *b, double t_end, int64_t max_steps, int64_t *steps_ta
 {
     if (!b || !(t_end > 0) || max_steps < 0) return VG_EINVAL;
     DeviceGuard guard(b->device);
-    vg_params saved = b->prm;
-    if (b->prm.t_end != t_end) {
-        vg_params p = b->prm;
-        p.t_end = t_end;
-        int rc = vg_batch_set_params(b, &p);
-        if (rc) return rc;
-    }
+    const double saved = b->prm.t_end;
+    b->prm.t_end = t_end;            // read from the device: tables and graph stay
     int rc = ready(b);
     int64_t taken = 0;
     std::vector<DevScalars> s;
@@ -599,10 +600,7 @@ int vg_batch_run(vg_batch *b, double t_end, int64_t max_steps, int64_t *steps_ta
         if (done) break;
     }
     if (steps_taken) *steps_taken = taken;
-    if (saved.t_end != t_end) {
-        int rc2 = vg_batch_set_params(b, &saved);
-        if (!rc) rc = rc2;
-    }
+    b->prm.t_end = saved;
     return rc;
 }
 

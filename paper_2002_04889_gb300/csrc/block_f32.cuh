@@ -58,7 +58,7 @@ struct KArgs<float> {
     float4 *wout;           // w^{n+1} [nc] (stage 2)
     DevScalars *sc;
     float g, half_g, hthr;
-    double cfl, dt_fixed, dt_max, t_end;
+    double cfl, dt_fixed, dt_max;
     int cfl_min;            // stage 1: 1 adds the CFL bound to the step's minimum
 };
 

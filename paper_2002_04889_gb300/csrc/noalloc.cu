@@ -46,10 +46,11 @@ void *g_addr[kMaxDevices] = {};
 
 // Clear the step scalars at the start of every call: time t, empty CFL minimum
 // (+inf in the context's precision), no flags, no records.
-__global__ void noalloc_init_kernel(DevScalars *sc, double t, int precision)
+__global__ void noalloc_init_kernel(DevScalars *sc, double t, double t_end, int precision)
 {
     if (threadIdx.x == 0 && blockIdx.x == 0) {
         sc->t = t;
+        sc->t_end = t_end;
         sc->dt = 0.0;
         if (precision == 64) {
             sc->dtmin_bits = (unsigned long long)__double_as_longlong(CUDART_INF);
@@ -100,9 +101,9 @@ int noalloc_prepare(int device)
     return (int)cudaFuncGetAttributes(&fa, (const void *)noalloc_init_kernel);
 }
 
-int noalloc_launch_init(void *scalars, double t, int precision, void *stream)
+int noalloc_launch_init(void *scalars, double t, double t_end, int precision, void *stream)
 {
-    noalloc_init_kernel<<<1, 32, 0, static_cast<cudaStream_t>(stream)>>>(static_cast<DevScalars *>(scalars), t,
+    noalloc_init_kernel<<<1, 32, 0, static_cast<cudaStream_t>(stream)>>>(static_cast<DevScalars *>(scalars), t, t_end,
                                                                          precision);
     return (int)cudaGetLastError();
 }

@@ -76,7 +76,7 @@ struct KArgs {
     double *bound_out;      // optional [nc]: the stage-1 CFL bound of each cell, +inf where nothing moves (FP64)
     DevScalars *sc;
     real g, half_g, hthr;
-    double cfl, dt_fixed, dt_max, t_end;
+    double cfl, dt_fixed, dt_max;
     int cfl_min;            // stage 1: 1 adds the CFL bound to the step's minimum
 };
 
@@ -199,11 +199,10 @@ __device__ __forceinline__ bool finished(double t_end, const DevScalars *sc)
 // instructions in each of an SM's 48 warps were 10,700 cycles of its FP64 units
 // (two lane-operations a cycle), 5 us a launch.  Every thread must call it.
 template <typename real>
-__device__ __forceinline__ real cta_step_dt(const DevScalars *sc, double cfl, double dt_fixed, double dt_max,
-                                            double t_end)
+__device__ __forceinline__ real cta_step_dt(const DevScalars *sc, double cfl, double dt_fixed, double dt_max)
 {
     __shared__ real s_dt;
-    if (threadIdx.x == 0) s_dt = (real)step_dt<real>(sc, cfl, dt_fixed, dt_max, t_end);
+    if (threadIdx.x == 0) s_dt = (real)step_dt<real>(sc, cfl, dt_fixed, dt_max, sc->t_end);
     __syncthreads();
     return s_dt;
 }
@@ -889,14 +888,14 @@ __global__ void __launch_bounds__(MAXT, StageMinCtas<real, MAXT>::value) stage_k
     // as it is: stage 1 does nothing (the CFL minimum stays empty) and stage 2
     // copies w^n to the output buffer, bit for bit (computing w/2 + (w + 0 R)/2
     // would flush the smallest FP32 values to zero), as the batched kernels do
-    if (finished(a.t_end, a.sc)) {
+    if (finished(a.sc->t_end, a.sc)) {
         if (STAGE == 2)
             copy_state<SOA>(a, blockIdx.x * (int64_t)blockDim.x + tid, (int64_t)gridDim.x * blockDim.x);
         return;
     }
 
     real dt = real(0);
-    if (STAGE == 2) dt = cta_step_dt<real>(a.sc, a.cfl, a.dt_fixed, a.dt_max, a.t_end);
+    if (STAGE == 2) dt = cta_step_dt<real>(a.sc, a.cfl, a.dt_fixed, a.dt_max);
 
     real my_min = real_inf<real>();
     long long my_neg = 0;
@@ -1005,8 +1004,8 @@ __device__ __forceinline__ bool cell_update2(const KArgs<float> &a, int gid, flo
 template <typename real>
 __global__ void __launch_bounds__(256) rk_update1_kernel(const KArgs<real> a, typename StateWord<real>::type *w1)
 {
-    if (finished(a.t_end, a.sc)) return;                 // update 2 copies w^n
-    const real dt = cta_step_dt<real>(a.sc, a.cfl, a.dt_fixed, a.dt_max, a.t_end);
+    if (finished(a.sc->t_end, a.sc)) return;                 // update 2 copies w^n
+    const real dt = cta_step_dt<real>(a.sc, a.cfl, a.dt_fixed, a.dt_max);
     long long my_neg = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.nc; i += (int64_t)gridDim.x * blockDim.x)
         if (cell_update1(a, (int)i, dt, w1)) my_neg++;
@@ -1018,11 +1017,11 @@ __global__ void __launch_bounds__(256) rk_update2_kernel(const KArgs<real> a, co
                                                          const typename StateWord<real>::type *R1)
 {
     const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
-    if (finished(a.t_end, a.sc)) {                       // as the fused kernel: w^n, bit for bit
+    if (finished(a.sc->t_end, a.sc)) {                       // as the fused kernel: w^n, bit for bit
         copy_state<false>(a, i0, stride);
         return;
     }
-    const real dt = cta_step_dt<real>(a.sc, a.cfl, a.dt_fixed, a.dt_max, a.t_end);
+    const real dt = cta_step_dt<real>(a.sc, a.cfl, a.dt_fixed, a.dt_max);
     long long my_neg = 0;
     bool bad = false;
     for (int64_t i = i0; i < a.nc; i += stride)
@@ -1105,12 +1104,13 @@ __global__ void __launch_bounds__(256, (BatchMinCtas<real>::value)) batch_stage_
     const KArgs<real> &p0 = meshes[0].a;
     if (STAGE == 2) chain_next();
     chain_wait();
+    const double t_end = sc_all[n_entries].t_end;
     for (int e = tid; e < n_entries; e += blockDim.x) {
         s_min[e] = min_bits(real_inf<real>());
-        s_dt[e] = STAGE == 2 ? (real)step_dt<real>(sc_all + e, p0.cfl, p0.dt_fixed, p0.dt_max, p0.t_end) : real(0);
+        s_dt[e] = STAGE == 2 ? (real)step_dt<real>(sc_all + e, p0.cfl, p0.dt_fixed, p0.dt_max, t_end) : real(0);
         // a scenario that has reached t_end takes steps of dt = 0 that leave its
         // state as it is (as a single context's do): skip its work, copy its state
-        s_done[e] = finished(p0.t_end, sc_all + e) ? 1 : 0;
+        s_done[e] = finished(t_end, sc_all + e) ? 1 : 0;
     }
     if (tid < 2) qcount[tid] = 0;
     long long my_neg = 0;
@@ -1216,11 +1216,11 @@ __global__ void batch_gauge_kernel(const BatchMesh<real> *meshes, DevScalars *sc
 // Epilogue of one batched step: per scenario t += dt (dt = 0 once it reached
 // t_end), and reset of its CFL minimum.
 template <typename real>
-__global__ void batch_post_kernel(int n_entries, DevScalars *sc_all, double cfl, double dt_fixed, double dt_max,
-                                  double t_end)
+__global__ void batch_post_kernel(int n_entries, DevScalars *sc_all, double cfl, double dt_fixed, double dt_max)
 {
     chain_wait();
     chain_next();
+    const double t_end = sc_all[n_entries].t_end;
     for (int e = threadIdx.x; e < n_entries; e += blockDim.x) {
         DevScalars *sc = sc_all + e;
         double dt = step_dt<real>(sc, cfl, dt_fixed, dt_max, t_end);
@@ -1256,7 +1256,6 @@ KArgs<real> common_args(const DevPtrs &d, const StepParams &p)
     a.cfl = p.cfl;
     a.dt_fixed = p.dt_fixed;
     a.dt_max = p.dt_max;
-    a.t_end = p.t_end;
     a.cfl_min = 1;
     return a;
 }
@@ -1442,7 +1441,7 @@ int launch_batch_step(const void *table, int n_mesh, int n_items, int n_entries,
     if (e == cudaSuccess)
         e = launch_after(batch_stage_kernel<real, 2, FAST>, grid, block, smem, s, t, n_mesh, n_items, n_entries, sc_all, scen_at);
     if (e == cudaSuccess)
-        e = launch_after(batch_post_kernel<real>, 1, 256, 0, s, n_entries, sc_all, p.cfl, p.dt_fixed, p.dt_max, p.t_end);
+        e = launch_after(batch_post_kernel<real>, 1, 256, 0, s, n_entries, sc_all, p.cfl, p.dt_fixed, p.dt_max);
     if (e != cudaSuccess) return (int)e;
     if (gauges) batch_gauge_kernel<real><<<n_mesh, 256, 0, s>>>(t, sc_all, p.gauge_every);
     return (int)cudaGetLastError();

@@ -32,7 +32,7 @@ __global__ void post_step_kernel(DevPtrs d, StepParams p, const word<real> *w)
     if (mine) eta = surface(w, z, d.gauge_cells[threadIdx.x]);
     if (threadIdx.x == 0) {
         const DevScalars v = *sc;
-        const double dt = step_dt<real>(&v, p.cfl, p.dt_fixed, p.dt_max, p.t_end);
+        const double dt = step_dt<real>(&v, p.cfl, p.dt_fixed, p.dt_max, v.t_end);
         sc->dt = dt;
         long long r = -1;
         if (!isfinite(dt)) sc->flags = v.flags | FLAG_NONFINITE_DT;
@@ -112,7 +112,7 @@ __global__ void bed_update_kernel(DevPtrs d, StepParams p, word<real> *w, int at
     __shared__ double s_t[2];        // the stored bed's time and the new one's, formed once per CTA
     if (threadIdx.x == 0) {
         s_t[0] = d.sc->t;
-        s_t[1] = at_step_end ? d.sc->t + step_dt<real>(d.sc, p.cfl, p.dt_fixed, p.dt_max, p.t_end) : t_set;
+        s_t[1] = at_step_end ? d.sc->t + step_dt<real>(d.sc, p.cfl, p.dt_fixed, p.dt_max, d.sc->t_end) : t_set;
     }
     __syncthreads();
     const double t0 = s_t[0], t = s_t[1];

@@ -76,6 +76,8 @@ void locate_points(const HostMesh &m, int32_t n, const double *pts, int32_t *cel
 // Device scalars shared by the step kernels of one context.
 struct DevScalars {
     double t;             // simulated time
+    double t_end;         // > 0: steps end here (in device memory, so that a run to another time
+                          // replays the same graph); of a batch: in its batch-wide record
     double dt;            // time step of the current step
     unsigned long long dtmin_bits;  // running min of the stage-1 CFL bound (bits of a
                                     // non-negative real: integer order = value order)
@@ -94,7 +96,7 @@ enum : unsigned int {
 };
 
 struct StepParams {
-    double g, cfl, hthr, dt_fixed, dt_max, t_end;
+    double g, cfl, hthr, dt_fixed, dt_max;
     int order, gauge_every;
     int fp64_fast;          // FP64: the contracted build of the stage kernels (step_f64_fast.cu)
 };
@@ -271,7 +273,7 @@ int launch_export_state_orig(const DevPtrs &d, const int32_t *new_of_old, const 
 // No-allocation step scratch (noalloc.cu): the device address and size of the
 // file-scope scratch array on `device`, and the kernel that clears its scalars.
 int noalloc_scratch(int device, void **addr, size_t *bytes);
-int noalloc_launch_init(void *scalars, double t, int precision, void *stream);
+int noalloc_launch_init(void *scalars, double t, double t_end, int precision, void *stream);
 // Set-up at mesh upload: resolves the scratch address on `device` and loads the
 // no-allocation kernels (no launch), so that a later step loads nothing.
 int noalloc_prepare(int device);

@@ -110,3 +110,54 @@ def test_fp32_extrema_and_boundaries(n, jitter, boundary):
             out.append(sv.get_state())
     for a, b in zip(*out):
         assert np.linalg.norm(a - b) <= 1e-4 * np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("every,calls", [(1, (0, 1, 2046, 3, 2047)), (3, (1, 2, 6140, 7)), (1, (5000,))])
+def test_gauge_ring_over_many_calls(every, calls):
+    """Records over calls of any length beside the device ring's 2048: one initial record
+    and one every `every` steps, the same as a run in calls of 50 steps."""
+    m, st = _moving_basin(6)
+    out = []
+    for parts in (calls, None):
+        with volna.Solver(64) as sv:
+            sv.set_params(h_threshold=1e-5, cfl=0.5, gauge_every=every)
+            sv.upload_mesh(m)
+            sv.set_gauges(np.array([[0.0, 0.0], [0.2, 0.1]]))
+            sv.set_state(*st, 0.0)
+            left = sum(calls)
+            for n in parts if parts else [50] * (left // 50) + [left % 50]:
+                sv.step(n)
+            out.append(sv.gauges())
+    assert len(out[0][0]) == 1 + sum(calls) // every
+    np.testing.assert_array_equal(out[0][0], out[1][0])
+    np.testing.assert_array_equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("precision", [32, 64])
+def test_run_to_several_end_times(precision):
+    """t_end lives on the device: advance, plain steps past it, another end time, a new
+    state and a parameter t_end, against a fresh context each time."""
+    m, st = _moving_basin(12)
+    def fresh(ends):
+        with volna.Solver(precision) as sv:
+            sv.set_params(h_threshold=1e-5, cfl=0.5)
+            sv.upload_mesh(m)
+            sv.set_state(*st, 0.0)
+            for e in ends:
+                sv.advance_to(e) if isinstance(e, float) else sv.step(e)
+            return sv.get_state()
+    with volna.Solver(precision) as sv:
+        sv.set_params(h_threshold=1e-5, cfl=0.5)
+        sv.upload_mesh(m)
+        for ends in ([0.03], [0.05, 3], [4, 0.04, 0.06]):
+            sv.set_state(*st, 0.0)
+            for e in ends:
+                sv.advance_to(e) if isinstance(e, float) else sv.step(e)
+            for a, b in zip(sv.get_state(), fresh(ends)):
+                np.testing.assert_array_equal(a, b)
+        sv.set_params(t_end=0.02)
+        sv.set_state(*st, 0.0)
+        sv.step(200)
+        assert sv.get_state()[3] == 0.02
+        for a, b in zip(sv.get_state(), fresh([0.02])):
+            np.testing.assert_array_equal(a, b)
