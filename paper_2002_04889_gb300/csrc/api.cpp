@@ -47,6 +47,7 @@ struct vg_ctx {
     float *area32 = nullptr;
     void *rk_w1 = nullptr, *rk_R1 = nullptr;   // state buffers: w1 and R(w1) of the unfused RK stages
     double *rarea = nullptr;          // FP64: 1 / area of every cell
+    double *M64 = nullptr;            // FP64: the contracted build's increment matrices, once asked for
     double *z64 = nullptr;
     double *z64_orig = nullptr;       // FP32: the FP64 bed in the original cell order (state import/export)
     bool zorig_ok = false;            // it matches z64 (false once a moving bed was set)
@@ -162,7 +163,7 @@ void free_mesh(vg_ctx *c)
     free_adjoint(c);
     if (c->graph2) { cudaGraphExecDestroy(c->graph2); c->graph2 = nullptr; }
     if (c->z64 == c->z) c->z64 = nullptr;
-    dfree(c->geo); dfree(c->rarea); dfree(c->z); dfree(c->zf); dfree(c->z64); dfree(c->w[0]); dfree(c->w[1]); dfree(c->R0);
+    dfree(c->geo); dfree(c->rarea); dfree(c->M64); dfree(c->z); dfree(c->zf); dfree(c->z64); dfree(c->w[0]); dfree(c->w[1]); dfree(c->R0);
     dfree(c->rk_w1); dfree(c->rk_R1);
     dfree(c->geoB); dfree(c->codes); dfree(c->ring_codes); dfree(c->fr); dfree(c->area32);
     dfree(c->z64_orig); c->zorig_ok = false;
@@ -237,7 +238,7 @@ DevPtrs dev_ptrs(const vg_ctx *c)
         const int t = block_shape(c, c->prm, c->hm.nc).threads;
         d.threads = (t >= c->hm.block && t <= 2 * c->hm.block && t <= 512) ? t : c->hm.block;
     }
-    d.fp64_fast = c->precision == 64 && !c->prm.fp64_literal;
+    d.fp64_fast = c->precision == 64 && !c->prm.fp64_literal && c->M64;
     d.nblocks = c->hm.nblocks;
     d.max_halo = c->hm.max_halo;
     d.max_ring1 = c->hm.max_ring1;
@@ -246,6 +247,7 @@ DevPtrs dev_ptrs(const vg_ctx *c)
     d.ring_cap = kRingCap;
     d.geo = c->geo;
     d.rarea = c->rarea;
+    d.M64 = c->M64;
     d.geoB = c->geoB;
     d.area32 = c->area32;
     d.codes = c->codes;
@@ -290,7 +292,7 @@ StepParams step_params(const vg_ctx *c)
     p.dt_max = c->prm.dt_max;
     p.order = c->prm.order;
     p.gauge_every = c->prm.gauge_every;
-    p.fp64_fast = c->precision == 64 && !c->prm.fp64_literal;
+    p.fp64_fast = c->precision == 64 && !c->prm.fp64_literal && c->M64;
     return p;
 }
 
@@ -811,6 +813,34 @@ int ensure_rk_buffers(vg_ctx *c)
     return VG_OK;
 }
 
+// The contracted FP64 build's increment matrices M_fj = w_j . (x_f - x_K), once a
+// context with a mesh asks for that build (before its launches are configured: without
+// the matrices dev_ptrs keeps the literal build).
+int ensure_fast_matrix(vg_ctx *c)
+{
+    if (c->precision != 64 || c->prm.fp64_literal || c->M64) return VG_OK;
+    const HostMesh &m = c->hm;
+    const size_t n = (size_t)m.nc;
+    std::vector<double> M(9 * n);
+#pragma omp parallel for
+    for (int64_t k = 0; k < m.nc; k++)
+        for (int f = 0; f < 3; f++)
+            for (int j = 0; j < 3; j++)
+                M[(3 * f + j) * n + k] = m.geo[(GEO_WX + j) * n + k] * m.geo[(GEO_FX + f) * n + k] +
+                                         m.geo[(GEO_WY + j) * n + k] * m.geo[(GEO_FY + f) * n + k];
+    double *dev = nullptr;
+    int rc = dmalloc(c, (void **)&dev, 8 * M.size());
+    if (rc) return rc;
+    cudaError_t e = cudaMemcpy(dev, M.data(), 8 * M.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) {
+        c->dev_bytes -= (int64_t)(8 * M.size());
+        dfree(dev);
+        return cuda_fail(c, e, "increment matrix upload");
+    }
+    c->M64 = dev;                     // kept only once complete
+    return VG_OK;
+}
+
 int record_now(vg_ctx *c)
 {
     if (c->n_gauges <= 0 || !c->has_state) return VG_OK;
@@ -947,6 +977,7 @@ int vg_mesh_upload(vg_ctx *c, int64_t nv, const double *xy, int64_t nc, const in
     if (rc) return rc;
     if ((rc = fit_blocks(c))) return rc;
     if ((rc = upload_mesh_arrays(c))) { free_mesh(c); return rc; }
+    if ((rc = ensure_fast_matrix(c))) { free_mesh(c); return rc; }
     if ((rc = configure_launch(c))) { free_mesh(c); return rc; }
     {
         // the no-allocation step's scratch and kernels are resolved here, so that
@@ -989,7 +1020,12 @@ int vg_set_params(vg_ctx *c, const vg_params *p)
     const BlockShape old_shape = block_shape(c, c->prm, c->hm.nc), new_shape = block_shape(c, *p, c->hm.nc);
     const int old_block = old_shape.cells, new_block = new_shape.cells;
     bool threads_changed = new_shape.threads != old_shape.threads || p->fp64_literal != c->prm.fp64_literal;
+    const vg_params old_prm = c->prm;
     c->prm = *p;
+    if (c->has_mesh) {
+        int rc = ensure_fast_matrix(c);
+        if (rc) { c->prm = old_prm; return rc; }
+    }
     c->graph_dirty = true;
     if (c->has_mesh && threads_changed && new_block == old_block) {
         cudaStreamSynchronize(c->stream);

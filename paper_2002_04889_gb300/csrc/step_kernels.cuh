@@ -36,7 +36,7 @@
 //    scheme; the fast one (FAST = true, step_f64_fast.cu, contraction allowed)
 //    multiplies by one reciprocal where the literal form forms several correctly
 //    rounded quotients by the same value (face velocities, the HLL star flux, the
-//    residual's 1/|K|).
+//    residual's 1/|K|) and forms a cell's increments with one precomputed matrix.
 //  * FP32 ("deviation"): block_f32.cuh.
 #pragma once
 
@@ -57,6 +57,7 @@ struct KArgs {
     int block, nblocks, max_halo, max_ring1, order;
     const real *geo;        // [GEO_ROWS][nc]
     const double *rarea;    // [nc] 1 / area (FP64)
+    const double *M;        // [9][nc] M_fj = w_j . (x_f - x_K), contracted build only
     const real *z;          // [nc]
     const real *zf;         // [3][nc] face beds
     const uint16_t *nbrl;   // [3][nc]
@@ -126,6 +127,8 @@ __device__ __forceinline__ float smin(float a, float b) { return fminf(a, b); }
 __device__ __forceinline__ double smin(double a, double b) { return okey(b) < okey(a) ? b : a; }
 __device__ __forceinline__ float max0(float x) { return fmaxf(0.f, x); }
 __device__ __forceinline__ double max0(double x) { return dbits(x) > 0 ? x : 0.0; }
+// isfinite on the integer units.
+__device__ __forceinline__ bool finite(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
 
 // Programmatic dependent launch: a step's kernels are launched while their
 // predecessor in the stream still runs (launch_after), wait in chain_wait for it to
@@ -441,7 +444,7 @@ __device__ __forceinline__ void finish_cell(const KArgs<real> &a, int gid, const
         const uint8_t branch = rk2_final(x, W1, Hu1, Hv1, RH, RHu, RHv, dt, a.hthr, W, Hu, Hv);
         if (branch == 2) my_neg++;
         if (a.mask2) a.mask2[gid] = branch;
-        if (!isfinite(W) || !isfinite(Hu) || !isfinite(Hv)) bad = true;
+        if (!finite(W) || !finite(Hu) || !finite(Hv)) bad = true;
         a.wout[gid] = W;
         a.wout[nc + gid] = Hu;
         a.wout[2 * nc + gid] = Hv;
@@ -450,14 +453,15 @@ __device__ __forceinline__ void finish_cell(const KArgs<real> &a, int gid, const
 
 // Shared memory of one CTA: cell states [L] x 4, face slots [3][L1] x 4 (L1 =
 // block + ring 1), with gids the global ids of block and ring-1 cells [L1], face
-// codes and owned-face queue [3B] each, and one byte per block and ring-1 cell:
-// whether it reconstructed (phase D adds its bed-slope source).  Without gids phase
+// codes and owned-face queue [3B] each, one byte per block and ring-1 cell: whether it
+// reconstructed (phase D adds its bed-slope source), and the cells' free surfaces [L]
+// (formed once; four neighbours and the source read each).  Without gids phase
 // B reads a ring-1 cell's global id again from the halo list.
 template <>
 __host__ __device__ inline size_t stage_smem_bytes<double>(int block, int max_halo, int max_ring1, int, bool gids)
 {
     size_t L = (size_t)block + max_halo, L1 = (size_t)block + max_ring1;
-    return sizeof(double) * 4 * (L + 3 * L1) + (gids ? sizeof(int32_t) * L1 : 0) + sizeof(uint16_t) * 6 * (size_t)block + L1 + 16;
+    return sizeof(double) * (5 * L + 12 * L1) + (gids ? sizeof(int32_t) * L1 : 0) + sizeof(uint16_t) * 6 * (size_t)block + L1 + 16;
 }
 
 // One block of cells for one scenario: phases A-D (see the top of this file).
@@ -495,7 +499,8 @@ __device__ __forceinline__ void process_block(const KArgs<real> &a, const int b,
     const int nc = (int)a.nc;    // per-cell arrays hold < 2^31 entries (checked at upload)
     real *sW = reinterpret_cast<real *>(smem_raw);          // [L][4]
     real *sF = sW + 4 * L;                                   // [3][L1][4]
-    int32_t *sGid = reinterpret_cast<int32_t *>(sF + 12 * L1);   // [L1] (GIDS)
+    real *sE = sF + 12 * L1;                                 // [L] H + z
+    int32_t *sGid = reinterpret_cast<int32_t *>(sE + L);     // [L1] (GIDS)
     uint16_t *sCode = reinterpret_cast<uint16_t *>(GIDS ? sGid + L1 : sGid);   // [3][B]
     uint16_t *queue = sCode + 3 * B;                              // [3B]
     uint8_t *sRec = reinterpret_cast<uint8_t *>(queue + 3 * B);   // [L1]
@@ -539,6 +544,7 @@ __device__ __forceinline__ void process_block(const KArgs<real> &a, const int b,
             bool neg = stage_cell<real, STAGE>(a, gid, dt, W, Hu, Hv, zc);
             if (neg) my_neg++;
             st4(sW + 4 * tid, W, Hu, Hv, zc);
+            sE[tid] = W + zc;
             if constexpr (GIDS) sGid[tid] = gid;
             dry = exactly_dry(W, Hu, Hv);
         }
@@ -546,6 +552,7 @@ __device__ __forceinline__ void process_block(const KArgs<real> &a, const int b,
             real W, Hu, Hv, zc;
             stage_cell<real, STAGE>(a, gh, dt, W, Hu, Hv, zc);
             st4(sW + 4 * (B + tid), W, Hu, Hv, zc);
+            sE[B + tid] = W + zc;
             if (tid < n1) {
                 if constexpr (GIDS) sGid[B + tid] = gh;
                 dry = dry && exactly_dry(W, Hu, Hv);
@@ -556,6 +563,7 @@ __device__ __forceinline__ void process_block(const KArgs<real> &a, const int b,
             real W, Hu, Hv, zc;
             stage_cell<real, STAGE>(a, gid, dt, W, Hu, Hv, zc);
             st4(sW + 4 * (B + h), W, Hu, Hv, zc);
+            sE[B + h] = W + zc;
             if (h < n1) {
                 if constexpr (GIDS) sGid[B + h] = gid;
                 dry = dry && exactly_dry(W, Hu, Hv);
@@ -628,7 +636,7 @@ __device__ __forceinline__ void process_block(const KArgs<real> &a, const int b,
         real WK, HuK, HvK, zK;
         ld4(sW + 4 * l, WK, HuK, HvK, zK);
         const real HK = WK;
-        real qK[3] = {HK + zK, HuK, HvK};
+        real qK[3] = {sE[l], HuK, HvK};
         real qn[3][3];
         bool recon = (a.order == 2) && gt_nn(HK, hthr);
 #pragma unroll
@@ -645,7 +653,7 @@ __device__ __forceinline__ void process_block(const KArgs<real> &a, const int b,
             if (code < NBR_ABSORB) {
                 real Hj, Huj, Hvj, zj;
                 ld4(sW + 4 * nl, Hj, Huj, Hvj, zj);
-                qn[f][0] = Hj + zj;
+                qn[f][0] = sE[nl];
                 qn[f][1] = Huj;
                 qn[f][2] = Hvj;
                 if (!gt_nn(Hj, hthr)) recon = false;
@@ -666,10 +674,14 @@ __device__ __forceinline__ void process_block(const KArgs<real> &a, const int b,
         real zfK[3] = {zK, zK, zK};       // the bed under each face value
         if (recon) {
             real face[3][3];
-            real fx[3], fy[3], wx[3], wy[3];
-            {
+            real fx[3], fy[3], wx[3], wy[3];       // literal: gradient, then its dot products
+            real Mf[3][3];                         // contracted: the increments' matrix, 9 instead of 12
 #pragma unroll
-                for (int f = 0; f < 3; f++) {
+            for (int f = 0; f < 3; f++) {
+                if constexpr (FAST) {
+#pragma unroll
+                    for (int j = 0; j < 3; j++) Mf[f][j] = a.M[(3 * f + j) * (size_t)nc + gid];
+                } else {
                     fx[f] = geo[(GEO_FX + f) * nc + gid];
                     fy[f] = geo[(GEO_FY + f) * nc + gid];
                     wx[f] = geo[(GEO_WX + f) * nc + gid];
@@ -680,7 +692,10 @@ __device__ __forceinline__ void process_block(const KArgs<real> &a, const int b,
             for (int v = 0; v < 3; v++) {
                 real d0 = qn[0][v] - qK[v], d1 = qn[1][v] - qK[v], d2 = qn[2][v] - qK[v];
                 real D[3];
-                {
+                if constexpr (FAST) {
+#pragma unroll
+                    for (int f = 0; f < 3; f++) D[f] = Mf[f][0] * d0 + Mf[f][1] * d1 + Mf[f][2] * d2;
+                } else {
                     real gx = (wx[0] * d0 + wx[1] * d1) + wx[2] * d2;
                     real gy = (wy[0] * d0 + wy[1] * d1) + wy[2] * d2;
 #pragma unroll
@@ -800,9 +815,7 @@ __device__ __forceinline__ void process_block(const KArgs<real> &a, const int b,
             // centred bed-slope source of a cell standing on its face beds:
             // g sum_f l_f z_f (eta_K - z_f / 2) n_f, eta_K = H_K + z_K
             if (sRec[l]) {
-                real HKs, Hus, Hvs, zKs;
-                ld4(sW + 4 * l, HKs, Hus, Hvs, zKs);
-                const real eK = HKs + zKs;
+                const real eK = sE[l];
 #pragma unroll
                 for (int f = 0; f < 3; f++) {
                     const real zff = a.zf[f * nc + gid];
@@ -984,7 +997,7 @@ __device__ __forceinline__ bool cell_update2(const KArgs<double> &a, int gid, do
     double W, Hu, Hv;
     const uint8_t branch = rk2_final(x, w1[gid], w1[nc + gid], w1[2 * nc + gid], R1[gid], R1[nc + gid], R1[2 * nc + gid],
                                      dt, a.hthr, W, Hu, Hv);
-    if (!isfinite(W) || !isfinite(Hu) || !isfinite(Hv)) bad = true;
+    if (!finite(W) || !finite(Hu) || !finite(Hv)) bad = true;
     a.wout[gid] = W;
     a.wout[nc + gid] = Hu;
     a.wout[2 * nc + gid] = Hv;
@@ -1269,6 +1282,7 @@ inline KArgs<double> make_args<double>(const DevPtrs &d, const StepParams &p, co
     KArgs<double> a = common_args<double>(d, p);
     a.geo = static_cast<const double *>(d.geo);
     a.rarea = d.rarea;
+    a.M = d.M64;
     a.zf = static_cast<const double *>(d.zf);
     a.nbrl = d.nbrl;
     a.ring1_nbr = d.ring1_nbr;

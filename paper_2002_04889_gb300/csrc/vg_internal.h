@@ -115,6 +115,7 @@ struct DevPtrs {
     const void *ring_codes; // FP32: the same beside halo_ids for ring-1 cells
     const void *fr;         // FP32: face records of every block's owned faces (fq_ptr)
     const double *rarea;    // FP64: [nc] 1 / area, correctly rounded (FP32: null)
+    const double *M64;      // FP64, contracted build: [9][nc] M_fj = w_j . (x_f - x_K) (else null)
     const void *z;          // [nc]
     const void *zf;         // FP64: [3][nc] face beds
     const double *z64;      // [nc] FP64 bed (state import/export and diagnostics)
