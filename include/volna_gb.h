@@ -114,7 +114,8 @@ typedef struct vg_diag {
     int64_t steps;         /* steps taken with dt > 0                              */
     int64_t neg_count;     /* negative depths met (and emptied) so far             */
     int64_t dry_count;     /* cells with H <= H_threshold                          */
-    int64_t launches;      /* kernels launched by the library so far               */
+    int64_t launches;      /* kernels launched by the library so far; a launch that
+                              runs n steps counts as the n steps' kernels        */
     int64_t n_records;     /* gauge records available to vg_get_gauges             */
 } vg_diag;
 

@@ -83,7 +83,7 @@ struct vg_ctx {
     double *bed_depth0 = nullptr, *bed_uplift = nullptr, *bed_onset = nullptr;
     double bed_rise = 0.0;
 
-    LaunchCfg cfg1{}, cfg2{};
+    LaunchCfg cfg1{}, cfg2{}, cfgn{};   // stages 1 and 2, and the multi-step kernel (grid 0: none)
     cudaGraphExec_t graph2 = nullptr;
     bool graph_dirty = true;
     int64_t launches = 0;
@@ -196,15 +196,16 @@ size_t state_bytes(const vg_ctx *c) { return (c->precision == 64 ? 24 : 16) * (s
 // by throughput, so they take smaller blocks and, below that, two threads per cell
 // (the ring-1 cells and the faces beyond the block's cells then share the phases'
 // first pass).  Measured, us a step, basin, against 256 cells:
-//   FP64, literal (the contracted build and FP32 keep 256 cells: their rounding
-//        depends on the partition, and a batch's scenarios equal single contexts bit
-//        for bit)
+//   FP64, literal (the contracted build keeps 256 cells: its rounding depends on the
+//        partition, and a batch's scenarios equal single contexts bit for bit)
 //         2,178 and 8,450: 64 cells / 128 threads 44 against 100 and 95 (128 / 256: 59, 57)
 //        20,402: 128 / 256  55 against 95 (64 / 128: 59)
 //        49,298: 160 / 160 116 against 173 (128 / 256: 138);  99,458: 224 against 256
 //        204,800: 160 / 160 412 against 415, coast basin 436 against 427: 256 from here on
-//   FP32 20,402: 128 / 256 13.7 against 16.8;  99,458: 17.9 against 19.9;
-//        204,800: 128 cells 24.0 against 23.0 (two waves): 256 from one wave on
+//   FP32, many steps in a launch (steps_config_f32)
+//         8,712: 64 / 128 9.6 against 12.1 (128 / 256: 9.8);  20,402: 128 / 256 9.9 against
+//        12.1 (64 / 128: 10.3);  49,298: 128 / 256 11.5 against 13.0 (256 / 512: 11.7)
+//        69,938: 256 / 512 12.1 against 13.4 (128 / 256: 12.5);  99,458: 17.0 against 14.5
 struct BlockShape { int cells, threads; };
 BlockShape block_shape(const vg_ctx *c, const vg_params &p, int64_t nc)
 {
@@ -221,8 +222,10 @@ BlockShape block_shape(const vg_ctx *c, const vg_params &p, int64_t nc)
         if (nc <= 64 * sms) s = {64, 128};                   // one block of 64 per SM
         else if (nc <= 192 * sms) s = {128, 256};            // three half-blocks per two SMs
         else if (nc <= 4 * 256 * sms) s = {160, 160};        // fewer than four blocks of 256 per SM
-    } else if (nc <= 256 * 3 * sms) {
-        s.threads = 512;                                     // one wave of three CTAs of 512 per SM
+    } else {
+        if (nc <= 64 * sms) s = {64, 128};                   // one block of 64 per SM
+        else if (nc <= 3 * 128 * sms) s = {128, 256};        // three of 128 per SM
+        else if (nc <= 2 * 256 * sms) s = {256, 512};        // two of 256 per SM
     }
     return s;
 }
@@ -572,6 +575,7 @@ int configure_launch(vg_ctx *c)
     if (e) return cuda_fail(c, (cudaError_t)e, "stage 1 launch configuration");
     e = c->precision == 64 ? stage_config_f64(d, 2, c->cfg2) : stage_config_f32(d, 2, c->cfg2);
     if (e) return cuda_fail(c, (cudaError_t)e, "stage 2 launch configuration");
+    if (c->precision == 32 && (e = steps_config_f32(d, c->cfgn))) return cuda_fail(c, (cudaError_t)e, "multi-step launch configuration");
     return VG_OK;
 }
 
@@ -588,6 +592,7 @@ void reset_scalars_host(vg_ctx *c, DevScalars &s, double t)
         std::memcpy(&b, &inf, 4);
         s.dtmin_bits = b;
     }
+    for (int k = 0; k < 3; k++) s.dtmin3[k] = s.dtmin_bits;
 }
 
 int ev_begin(vg_ctx *c, int kernel)
@@ -768,8 +773,18 @@ int read_and_drain(vg_ctx *c, DevScalars &s, int64_t n_max)
     return got ? empty_ring(c, s) : VG_OK;
 }
 
+// Whether vg_step runs n steps in cooperative launches of many: FP32 meshes of a few
+// waves of blocks (steps_config_f32 has the figures), the plain step only.  The FP64
+// kernels gained nothing from it: their step is 40 us and more, and the joined kernel's
+// registers leave one CTA per SM (20,402 cells 66 us against 54; 8,712: 39 against 42).
+bool use_multi_step(const vg_ctx *c, int64_t n)
+{
+    return n >= 2 && c->cfgn.grid > 0 && !c->bed_on && !c->prm.rk_unfused;
+}
+
 int check_flags(vg_ctx *c, const DevScalars &s, int64_t neg_before)
 {
+    if (s.flags & FLAG_TIMEOUT) return fail(c, VG_ETIMEOUT, "a grid barrier of the step kernel was not reached by all CTAs");
     if (s.flags & FLAG_NONFINITE_STATE) return fail(c, VG_ENONFINITE, "a non-finite value appeared in the state");
     if (s.flags & FLAG_NONFINITE_DT) return fail(c, VG_ENONFINITE, "the time step is not finite");
     if (s.flags & FLAG_RING_FULL) return fail(c, VG_ESTATE, "gauge ring overflow");
@@ -934,7 +949,7 @@ int vg_create(vg_ctx **out, int precision, int device, void *cuda_stream)
         if (cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking) != cudaSuccess) { delete c; return VG_ECUDA; }
         c->own_stream = true;
     }
-    if (cudaMalloc((void **)&c->sc, sizeof(DevScalars)) != cudaSuccess ||
+    if (cudaMalloc((void **)&c->sc, kScalarAlloc) != cudaSuccess ||
         cudaMalloc((void **)&c->diag_part, 8 * 3 * kDiagBlocks) != cudaSuccess ||
         cudaMalloc((void **)&c->diag_out, 8 * 4) != cudaSuccess ||
         cudaHostAlloc((void **)&c->pinned, kPinned, cudaHostAllocDefault) != cudaSuccess) {
@@ -943,7 +958,7 @@ int vg_create(vg_ctx **out, int precision, int device, void *cuda_stream)
     }
     DevScalars s;
     reset_scalars_host(c, s, 0.0);
-    if (cudaMemcpy(c->sc, &s, sizeof(s), cudaMemcpyHostToDevice) != cudaSuccess) { vg_destroy(c); return VG_ECUDA; }
+    if (cudaMemset(c->sc, 0, kScalarAlloc) != cudaSuccess || cudaMemcpy(c->sc, &s, sizeof(s), cudaMemcpyHostToDevice) != cudaSuccess) { vg_destroy(c); return VG_ECUDA; }
     *out = c;
     return VG_OK;
 }
@@ -1270,7 +1285,20 @@ int vg_step(vg_ctx *c, int64_t n_steps)
                 left--;
             }
         } else {
-            if (c->graph_dirty && (rc = build_graph(c))) return rc;
+            while (use_multi_step(c, left)) {
+                const int n = (int)std::min<int64_t>(left, 4096);     // tens of ms: others get their turn on the GPU
+                int e = launch_steps_f32(dev_ptrs(c), step_params(c), c->w[c->cur], c->w[1 - c->cur], n, c->cfgn, (void *)c->stream);
+                if (e == (int)cudaErrorCooperativeLaunchTooLarge) {   // a part of the GPU only (MPS): the graph
+                    cudaGetLastError();
+                    c->cfgn.grid = 0;
+                    break;
+                }
+                if (e) return cuda_fail(c, (cudaError_t)e, "multi-step launch");
+                c->launches += (int64_t)n * step_kernels(c);
+                if (n & 1) c->cur = 1 - c->cur;
+                left -= n;
+            }
+            if (left >= 2 && c->graph_dirty && (rc = build_graph(c))) return rc;
             if (c->cur == 1 && left > 0) {
                 if ((rc = enqueue_step(c, 1))) return rc;
                 c->cur = 0;

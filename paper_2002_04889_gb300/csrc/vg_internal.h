@@ -86,13 +86,22 @@ struct DevScalars {
     long long neg_count;  // negative depths met
     unsigned int flags;   // FLAG_* bits
     int pad;
+    unsigned long long dtmin3[3];   // the multi-step kernel's CFL minima of three consecutive steps
 };
+
+// CTAs that have arrived at the multi-step kernel's barriers and that have left it (zero
+// between launches): kBarrierAt bytes behind a context's DevScalars, on a line of its own.
+struct StepsBarrier {
+    unsigned int arrived, left;
+};
+constexpr int kBarrierAt = 256, kScalarAlloc = kBarrierAt + 128;
 
 enum : unsigned int {
     FLAG_NONFINITE_STATE = 1u,
     FLAG_NONFINITE_DT = 2u,
     FLAG_RING_FULL = 4u,
     FLAG_BAD_INPUT = 8u,
+    FLAG_TIMEOUT = 16u,
 };
 
 struct StepParams {
@@ -155,6 +164,7 @@ struct DevPtrs {
 struct LaunchCfg {
     int grid;        // persistent CTAs
     size_t smem;     // dynamic shared memory per CTA
+    int ctas;        // multi-step kernel: the variant, CTAs of 256 threads per SM
 };
 size_t stage_smem_f32(int block, int max_halo, int max_ring1, int max_faces);
 size_t stage_smem_f64(int block, int max_halo, int max_ring1);
@@ -177,6 +187,11 @@ int launch_rk_unfused_f64(const DevPtrs &d, const StepParams &p, int part, const
                           void *R1, const LaunchCfg &c1, void *stream);
 int launch_rk_unfused_f64_fast(const DevPtrs &d, const StepParams &p, int part, const void *w_in, void *w_out,
                                void *w1, void *R1, const LaunchCfg &c1, void *stream);
+
+// n steps in one cooperative launch from w_in, for n odd to w_out (the other buffer of
+// the pair).  steps_config: grid 0 where the thread count has no such kernel.
+int steps_config_f32(const DevPtrs &d, LaunchCfg &cfg);
+int launch_steps_f32(const DevPtrs &d, const StepParams &p, const void *w_in, void *w_out, int n, const LaunchCfg &c, void *stream);
 
 // The contracted FP64 build (step_f64_fast.cu); the *_f64 entry points above
 // dispatch to it when DevPtrs::fp64_fast / StepParams::fp64_fast is set.

@@ -161,3 +161,26 @@ def test_run_to_several_end_times(precision):
         assert sv.get_state()[3] == 0.02
         for a, b in zip(sv.get_state(), fresh([0.02])):
             np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("precision,literal", [(32, 1), (64, 1), (64, 0)])
+@pytest.mark.parametrize("n,steps,t_end", [(1, 2, 0.0), (9, 7, 0.0), (33, 8, 0.0), (33, 23, 0.012), (110, 9, 0.0), (290, 5, 0.0), (330, 4, 0.0), (420, 5, 0.0)])
+def test_many_steps_in_one_launch(precision, literal, n, steps, t_end):
+    """A call of many steps against as many calls of one step, bit for bit: state, time,
+    counts and gauge records; odd and even step counts, an end time between them, meshes
+    of one block and of more than one block per CTA."""
+    m, st = _moving_basin(n)
+    out = []
+    for parts in ([steps], [1] * steps, [1, 2, steps - 3] if steps > 3 else [0, steps]):
+        with volna.Solver(precision) as sv:
+            sv.set_params(h_threshold=1e-5, cfl=0.9, fp64_literal=literal, t_end=t_end, gauge_every=2)
+            sv.upload_mesh(m)
+            sv.set_gauges(np.array([[0.01, 0.005], [0.2, 0.1], [-0.11, 0.2]]))
+            sv.set_state(*st, 0.0)
+            for k in parts:
+                sv.step(k)
+            d = sv.diagnostics()
+            out.append(list(sv.get_state()) + list(sv.gauges()) + [d[k] for k in ("t", "last_dt", "steps", "neg_count", "launches")])
+    for other in out[1:]:
+        for a, b in zip(out[0], other):
+            np.testing.assert_array_equal(a, b)
