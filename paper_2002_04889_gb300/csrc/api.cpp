@@ -338,6 +338,7 @@ int upload_rec_a(vg_ctx *c)
     int rc;
     if (!c->geo && (rc = dmalloc(c, &c->geo, 32 * (size_t)n))) return rc;
     std::vector<float> r(8 * (size_t)n);
+#pragma omp parallel for
     for (int64_t k = 0; k < n; k++) {
         auto G = [&](int row) { return m.geo[(size_t)row * n + k]; };
         float *o = &r[8 * (size_t)k];
@@ -369,22 +370,26 @@ int upload_face_beds(vg_ctx *c)
 template <typename Face>
 void order_for_banks(std::vector<Face> &v)
 {
-    std::vector<Face> pool[64], out;
-    for (const Face &x : v) pool[(x.slots & 7) * 8 + ((x.slots >> 16) & 7)].push_back(x);
-    out.reserve(v.size());
-    while (out.size() < v.size()) {
+    auto group = [](const Face &x) { return (x.slots & 7) * 8 + ((x.slots >> 16) & 7); };
+    const int n = (int)v.size();
+    int first[64] = {}, left_in[64] = {};             // of each pair of groups, in `pool`
+    for (const Face &x : v) left_in[group(x)]++;
+    for (int g = 1; g < 64; g++) first[g] = first[g - 1] + left_in[g - 1];
+    std::vector<Face> pool(n), out;
+    int put[64];
+    std::memcpy(put, first, sizeof(put));
+    for (const Face &x : v) pool[put[group(x)]++] = x;
+    out.reserve(n);
+    while ((int)out.size() < n) {
         unsigned left = 0, right = 0;                 // groups taken in this cycle
-        for (int lane = 0; lane < 8 && out.size() < v.size(); lane++) {
-            int best = -1;
-            size_t most = 0;
-            int score = -1;                           // 2: both sides free, 1: one, 0: none
+        for (int lane = 0; lane < 8 && (int)out.size() < n; lane++) {
+            int best = -1, most = 0;                  // both sides free before one before none, then the fullest
             for (int g = 0; g < 64; g++) {
-                if (pool[g].empty()) continue;
-                const int s = !((left >> (g >> 3)) & 1) + !((right >> (g & 7)) & 1);
-                if (s > score || (s == score && pool[g].size() > most)) { best = g; most = pool[g].size(); score = s; }
+                const int free = !((left >> (g >> 3)) & 1) + !((right >> (g & 7)) & 1);
+                const int rank = left_in[g] ? (free << 20) + left_in[g] : -1;
+                if (rank > most) { best = g; most = rank; }
             }
-            out.push_back(pool[best].back());
-            pool[best].pop_back();
+            out.push_back(pool[first[best] + --left_in[best]]);
             left |= 1u << (best >> 3);
             right |= 1u << (best & 7);
         }
@@ -410,7 +415,7 @@ int upload_partition_f32(vg_ctx *c)
             o.nb[f] = packed ? nbr_code >> 2 : nbr_code;
         }
     };
-#pragma omp parallel for schedule(dynamic, 64)
+#pragma omp parallel for schedule(dynamic, 4)
     for (int32_t b = 0; b < m.nblocks; b++) {
         const int64_t c0 = (int64_t)b * B, c1 = std::min<int64_t>(c0 + B, nc);
         for (int64_t k = c0; k < c1; k++) {
@@ -511,6 +516,7 @@ int upload_mesh_arrays(vg_ctx *c)
         // the face beds below)
         const int64_t n = m.nc;
         std::vector<float> r(4 * (size_t)n), area(n);
+#pragma omp parallel for
         for (int64_t k = 0; k < n; k++) {
             auto G = [&](int row) { return m.geo[(size_t)row * n + k]; };
             for (int f = 0; f < 2; f++) {
@@ -526,6 +532,7 @@ int upload_mesh_arrays(vg_ctx *c)
     }
     if (c->precision == 64) {
         std::vector<double> ra(m.nc);
+#pragma omp parallel for
         for (int64_t k = 0; k < m.nc; k++) ra[k] = 1.0 / m.geo[(size_t)GEO_AREA * m.nc + k];
         if ((rc = dmalloc(c, (void **)&c->rarea, 8 * m.nc))) return rc;
         VG_CUDA(c, cudaMemcpy(c->rarea, ra.data(), 8 * m.nc, cudaMemcpyHostToDevice));

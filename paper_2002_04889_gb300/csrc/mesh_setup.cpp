@@ -399,7 +399,7 @@ int partition_blocks(HostMesh &m, int block, std::string &err)
     m.block = block;
     m.nblocks = nb;
     std::vector<std::vector<int32_t>> r1(nb), r2(nb);
-#pragma omp parallel for schedule(dynamic, 64)
+#pragma omp parallel for schedule(dynamic, 4)
     for (int32_t b = 0; b < nb; b++) {
         int64_t c0 = (int64_t)b * block, c1 = std::min<int64_t>(c0 + block, nc);
         std::vector<int32_t> &h = r1[b];
@@ -435,7 +435,7 @@ int partition_blocks(HostMesh &m, int block, std::string &err)
     m.halo_ids.resize(m.halo_ptr[nb]);
     m.ring1_nbr.assign(3 * (size_t)m.halo_ptr[nb], NBR_WALL);
     std::vector<uint16_t> nbrl(3 * nc, NBR_WALL);
-#pragma omp parallel for schedule(dynamic, 64)
+#pragma omp parallel for schedule(dynamic, 4)
     for (int32_t b = 0; b < nb; b++) {
         int64_t c0 = (int64_t)b * block, c1 = std::min<int64_t>(c0 + block, nc);
         const std::vector<int32_t> &h = r1[b], &h2 = r2[b];
