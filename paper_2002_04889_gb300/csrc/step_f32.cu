@@ -255,9 +255,9 @@ int batch_config_f32(int block, int max_halo, int max_ring1, int max_faces, int 
 {
     return batch_config<float>(block, max_halo, max_ring1, max_faces, n_entries, grid, smem, scen_at);
 }
-int launch_batch_step_f32(const void *table, int n_mesh, int n_items, int n_entries, DevScalars *sc_all, int block,
+int launch_batch_step_f32(const void *table, int n_mesh, int n_items, int groups, int n_entries, DevScalars *sc_all, int block,
                           int grid, size_t smem, int scen_at, const StepParams &p, bool gauges, void *stream)
 {
-    return launch_batch_step<float>(table, n_mesh, n_items, n_entries, sc_all, block, grid, smem, scen_at, p, gauges, stream);
+    return launch_batch_step<float>(table, n_mesh, n_items, groups, n_entries, sc_all, block, grid, smem, scen_at, p, gauges, stream);
 }
 }  // namespace vg

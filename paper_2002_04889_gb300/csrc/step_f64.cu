@@ -38,13 +38,13 @@ int batch_config_f64(int block, int max_halo, int max_ring1, int n_entries, int 
     if (fast) return batch_config_f64_fast(block, max_halo, max_ring1, n_entries, grid, smem, scen_at);
     return batch_config<double, false>(block, max_halo, max_ring1, 0, n_entries, grid, smem, scen_at);
 }
-int launch_batch_step_f64(const void *table, int n_mesh, int n_items, int n_entries, DevScalars *sc_all, int block,
+int launch_batch_step_f64(const void *table, int n_mesh, int n_items, int groups, int n_entries, DevScalars *sc_all, int block,
                           int grid, size_t smem, int scen_at, const StepParams &p, bool gauges, void *stream)
 {
     if (p.fp64_fast)
-        return launch_batch_step_f64_fast(table, n_mesh, n_items, n_entries, sc_all, block, grid, smem, scen_at, p, gauges,
+        return launch_batch_step_f64_fast(table, n_mesh, n_items, groups, n_entries, sc_all, block, grid, smem, scen_at, p, gauges,
                                           stream);
-    return launch_batch_step<double, false>(table, n_mesh, n_items, n_entries, sc_all, block, grid, smem, scen_at, p, gauges,
+    return launch_batch_step<double, false>(table, n_mesh, n_items, groups, n_entries, sc_all, block, grid, smem, scen_at, p, gauges,
                                             stream);
 }
 }  // namespace vg

@@ -24,10 +24,10 @@ int batch_config_f64_fast(int block, int max_halo, int max_ring1, int n_entries,
 {
     return batch_config<double, true>(block, max_halo, max_ring1, 0, n_entries, grid, smem, scen_at);
 }
-int launch_batch_step_f64_fast(const void *table, int n_mesh, int n_items, int n_entries, DevScalars *sc_all,
+int launch_batch_step_f64_fast(const void *table, int n_mesh, int n_items, int groups, int n_entries, DevScalars *sc_all,
                                int block, int grid, size_t smem, int scen_at, const StepParams &p, bool gauges, void *stream)
 {
-    return launch_batch_step<double, true>(table, n_mesh, n_items, n_entries, sc_all, block, grid, smem, scen_at, p, gauges,
+    return launch_batch_step<double, true>(table, n_mesh, n_items, groups, n_entries, sc_all, block, grid, smem, scen_at, p, gauges,
                                            stream);
 }
 }  // namespace vg

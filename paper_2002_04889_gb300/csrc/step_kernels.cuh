@@ -1044,9 +1044,9 @@ __global__ void __launch_bounds__(256) rk_update2_kernel(const KArgs<real> a, co
 
 // ---------------------------------------------------------------------------
 // Batched ensembles: many scenarios on several meshes in one persistent launch
-// per stage.  A work item is one block of one mesh; the CTA runs that block for
-// every scenario of the mesh in turn, so the block's mesh data stays in L1/L2
-// across scenarios.  Scenario e (meshes' scenarios numbered consecutively) has
+// per stage.  A work item is one block of one mesh and one of `groups` groups of its
+// scenarios; the CTA runs that block for every scenario of the group in turn, so the
+// block's mesh data stays in L1/L2 across scenarios.  Scenario e (meshes' scenarios numbered consecutively) has
 // its own state slice, its own device scalars sc[e] and its own time step.
 // ---------------------------------------------------------------------------
 
@@ -1104,7 +1104,7 @@ __host__ __device__ inline size_t batch_smem_bytes(size_t stage, int n_entries)
 // fills the next one's.
 template <typename real, int STAGE, bool FAST = false>
 __global__ void __launch_bounds__(256, (BatchMinCtas<real>::value)) batch_stage_kernel(const BatchMesh<real> *meshes, int n_mesh,
-                                                          int n_items, int n_entries, DevScalars *sc_all, int scen_at)
+                                                          int n_items, int groups, int n_entries, DevScalars *sc_all, int scen_at)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int qcount[2];
@@ -1130,10 +1130,13 @@ __global__ void __launch_bounds__(256, (BatchMinCtas<real>::value)) batch_stage_
     int parity = 0, slot = 0, last_m = -1;
     bool bad = false;
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+        const int blk = item / groups, group = item - blk * groups;
         int m = 0;
-        while (m + 1 < n_mesh && item >= meshes[m + 1].first_item) m++;
+        while (m + 1 < n_mesh && blk >= meshes[m + 1].first_item) m++;
         const BatchMesh<real> &bm = meshes[m];
-        const int b = item - bm.first_item, n_scen = bm.n_scen, e0 = bm.first_entry;
+        const int b = blk - bm.first_item, e0 = bm.first_entry;
+        const int per_group = (bm.n_scen + groups - 1) / groups;
+        const int s0 = group * per_group, n_scen = min(s0 + per_group, bm.n_scen);
         const int64_t stride = bm.stride;
         __syncthreads();             // every thread has done with the last item's arguments
         if (m != last_m) {
@@ -1157,11 +1160,11 @@ __global__ void __launch_bounds__(256, (BatchMinCtas<real>::value)) batch_stage_
             // a finished scenario's state carries over to the other buffer of the pair
             const int c = b * bm.a.block + tid;
             if (tid < bm.a.block && c < (int)bm.a.nc)
-                for (int s = 0; s < n_scen; s++)
+                for (int s = s0; s < n_scen; s++)
                     if (s_done[e0 + s]) copy_cell(bm.a.w + s * stride, bm.a.wout + s * stride, c, (int)bm.a.nc);
         }
         bool loaded = false;
-        int s = next(0);
+        int s = next(s0);
         if (tid == 0 && s < n_scen) fill(s, slot);
         __syncthreads();
         while (s < n_scen) {
@@ -1446,14 +1449,14 @@ int batch_config(int block, int max_halo, int max_ring1, int max_faces, int n_en
 }
 
 template <typename real, bool FAST = false>
-int launch_batch_step(const void *table, int n_mesh, int n_items, int n_entries, DevScalars *sc_all, int block,
+int launch_batch_step(const void *table, int n_mesh, int n_items, int groups, int n_entries, DevScalars *sc_all, int block,
                       int grid, size_t smem, int scen_at, const StepParams &p, bool gauges, void *stream)
 {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const BatchMesh<real> *t = static_cast<const BatchMesh<real> *>(table);
-    cudaError_t e = launch_after(batch_stage_kernel<real, 1, FAST>, grid, block, smem, s, t, n_mesh, n_items, n_entries, sc_all, scen_at);
+    cudaError_t e = launch_after(batch_stage_kernel<real, 1, FAST>, grid, block, smem, s, t, n_mesh, n_items, groups, n_entries, sc_all, scen_at);
     if (e == cudaSuccess)
-        e = launch_after(batch_stage_kernel<real, 2, FAST>, grid, block, smem, s, t, n_mesh, n_items, n_entries, sc_all, scen_at);
+        e = launch_after(batch_stage_kernel<real, 2, FAST>, grid, block, smem, s, t, n_mesh, n_items, groups, n_entries, sc_all, scen_at);
     if (e == cudaSuccess)
         e = launch_after(batch_post_kernel<real>, 1, 256, 0, s, n_entries, sc_all, p.cfl, p.dt_fixed, p.dt_max);
     if (e != cudaSuccess) return (int)e;

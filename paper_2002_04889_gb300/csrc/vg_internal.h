@@ -200,7 +200,7 @@ int launch_stage1_f64_fast(const DevPtrs &d, const StepParams &p, const void *w_
 int launch_stage2_f64_fast(const DevPtrs &d, const StepParams &p, const void *w_in, void *w_out, const LaunchCfg &c,
                            void *stream);
 int batch_config_f64_fast(int block, int max_halo, int max_ring1, int n_entries, int &grid, size_t &smem, int &scen_at);
-int launch_batch_step_f64_fast(const void *table, int n_mesh, int n_items, int n_entries, DevScalars *sc_all,
+int launch_batch_step_f64_fast(const void *table, int n_mesh, int n_items, int groups, int n_entries, DevScalars *sc_all,
                                int block, int grid, size_t smem, int scen_at, const StepParams &p, bool gauges, void *stream);
 
 // Batched ensembles (step_f32.cu / step_f64.cu): the device table entry of one
@@ -215,9 +215,9 @@ void fill_batch_mesh_f64(void *dst, const DevPtrs &d, const StepParams &p, const
                          int first_item, int first_entry);
 int batch_config_f32(int block, int max_halo, int max_ring1, int max_faces, int n_entries, int &grid, size_t &smem, int &scen_at);
 int batch_config_f64(int block, int max_halo, int max_ring1, int n_entries, int &grid, size_t &smem, int &scen_at, bool fast);
-int launch_batch_step_f32(const void *table, int n_mesh, int n_items, int n_entries, DevScalars *sc_all, int block,
+int launch_batch_step_f32(const void *table, int n_mesh, int n_items, int groups, int n_entries, DevScalars *sc_all, int block,
                           int grid, size_t smem, int scen_at, const StepParams &p, bool gauges, void *stream);
-int launch_batch_step_f64(const void *table, int n_mesh, int n_items, int n_entries, DevScalars *sc_all, int block,
+int launch_batch_step_f64(const void *table, int n_mesh, int n_items, int groups, int n_entries, DevScalars *sc_all, int block,
                           int grid, size_t smem, int scen_at, const StepParams &p, bool gauges, void *stream);
 
 // Discrete adjoint (adjoint_f64.cu, FP64 contexts).

@@ -184,3 +184,28 @@ def test_many_steps_in_one_launch(precision, literal, n, steps, t_end):
     for other in out[1:]:
         for a, b in zip(out[0], other):
             np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("precision,n,scenarios", [(32, (9, 40), (1, 5)), (32, (250, 12), (3, 8)), (64, (33, 101), (7, 2))])
+def test_batch_scenario_groups(precision, n, scenarios):
+    """Scenarios of a batch in groups: uneven counts (groups without a scenario), few and
+    many blocks per CTA, an end time that some scenarios reach earlier; bit for bit the
+    single contexts."""
+    cases = [_moving_basin(k) for k in n]
+    with volna.Batch(precision) as b:
+        b.set_params(h_threshold=1e-5, cfl=0.9)
+        for (m, st), k in zip(cases, scenarios):
+            mid = b.add_mesh(m, k)
+            for j in range(k):
+                b.set_state(mid, j, st[0], st[1] * (1 + j), st[2], 0.0)
+        b.run(0.02)
+        for mid, ((m, st), k) in enumerate(zip(cases, scenarios)):
+            for j in sorted({0, k - 1}):
+                with volna.Solver(precision) as sv:
+                    sv.set_params(h_threshold=1e-5, cfl=0.9)
+                    sv.upload_mesh(m)
+                    sv.set_state(st[0], st[1] * (1 + j), st[2], 0.0)
+                    sv.advance_to(0.02)
+                    ref = sv.get_state()
+                for a, r in zip(b.get_state(mid, j)[:4], ref):
+                    np.testing.assert_array_equal(a, r)
