@@ -55,9 +55,16 @@ struct Gauges {
     double *ring_t, *ring_eta;
 };
 
-template <int MAXT, int MINCTAS>
+// SOA: one step of the caller's states from its time (CallerStep); the context's own
+// scalars keep their values, and the last CTA writes the outcome to host memory.
+struct CallerStep {
+    double t, t_end;
+    StepOutcome *out;
+};
+
+template <int MAXT, int MINCTAS, bool SOA>
 __global__ void __launch_bounds__(MAXT, MINCTAS) steps_kernel(const KArgs<float> args, StepsBarrier *bar, const Gauges gauges,
-                                                             int n_steps)
+                                                             int n_steps, const CallerStep caller)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ float red_min[32], s_dt;
@@ -67,14 +74,14 @@ __global__ void __launch_bounds__(MAXT, MINCTAS) steps_kernel(const KArgs<float>
     const bool scribe = blockIdx.x == gridDim.x - 1;
     KArgs<float> a = args;
     DevScalars *sc = args.sc;
-    const double t_end = sc->t_end;
+    const double t_end = SOA ? caller.t_end : sc->t_end;
     double dt_last = 0.0;                    // dt_last ... target: thread 0 only
     long long steps = 0, n_rec = 0;
     unsigned flags = 0, target = 0;
     if (tid == 0) {
-        s_t = sc->t;
-        steps = sc->steps;
-        n_rec = sc->n_rec;
+        s_t = SOA ? caller.t : sc->t;
+        steps = SOA ? 0 : sc->steps;
+        n_rec = SOA ? 0 : sc->n_rec;
     }
     __syncthreads();
     long long my_neg = 0;
@@ -86,7 +93,7 @@ __global__ void __launch_bounds__(MAXT, MINCTAS) steps_kernel(const KArgs<float>
         float my_min = real_inf<float>();
         for (int b = blockIdx.x; b < a.nblocks; b += gridDim.x) {
             bool loaded = false;
-            process_block<1, false>(a, b, 0.f, smem_raw, my_min, my_neg, bad, loaded);
+            process_block<1, SOA>(a, b, 0.f, smem_raw, my_min, my_neg, bad, loaded);
         }
         for (int o = 16; o > 0; o >>= 1) my_min = smin(my_min, __shfl_xor_sync(0xffffffffu, my_min, o));
         if (lane == 0) red_min[warp] = my_min;
@@ -109,7 +116,7 @@ __global__ void __launch_bounds__(MAXT, MINCTAS) steps_kernel(const KArgs<float>
         const float dt = s_dt;
         for (int b = blockIdx.x; b < a.nblocks; b += gridDim.x) {
             bool loaded = false;
-            process_block<2, false>(a, b, dt, smem_raw, my_min, my_neg, bad, loaded);
+            process_block<2, SOA>(a, b, dt, smem_raw, my_min, my_neg, bad, loaded);
         }
         if (!(ok = grid_barrier(bar, target))) break;
         if (tid == 0) {
@@ -130,36 +137,48 @@ __global__ void __launch_bounds__(MAXT, MINCTAS) steps_kernel(const KArgs<float>
             s_rec = rec;
         }
         __syncthreads();
-        if (scribe && s_rec >= 0)
-            for (int g = tid; g < gauges.n; g += blockDim.x)
-                gauges.ring_eta[s_rec * gauges.n + g] = surface(a.wout, a.z, gauges.cells[g]);
-        float4 *w_new = a.wout;                // the state buffers change roles
-        a.wout = const_cast<float4 *>(a.w);
-        a.w = w_new;
+        if constexpr (!SOA) {
+            if (scribe && s_rec >= 0)
+                for (int g = tid; g < gauges.n; g += blockDim.x)
+                    gauges.ring_eta[s_rec * gauges.n + g] = surface(a.wout, a.z, gauges.cells[g]);
+            float4 *w_new = a.wout;            // the state buffers change roles
+            a.wout = const_cast<float4 *>(a.w);
+            a.w = w_new;
+        }
     }
     // steps past t_end leave the state as it is; an odd number of them leaves it in
     // the other buffer
     if (ok && ((n_steps - i) & 1))
-        copy_state<false>(a, blockIdx.x * (int64_t)blockDim.x + tid, (int64_t)gridDim.x * blockDim.x);
+        copy_state<SOA>(a, blockIdx.x * (int64_t)blockDim.x + tid, (int64_t)gridDim.x * blockDim.x);
     for (int o = 16; o > 0; o >>= 1) my_neg += __shfl_xor_sync(0xffffffffu, my_neg, o);
     if (lane == 0) red_neg[warp] = my_neg;
     bad = __syncthreads_or(bad);
     if (tid == 0) {
         long long neg = 0;
         for (int w = 0; w < nwarps; w++) neg += red_neg[w];
-        if (neg) atomicAdd((unsigned long long *)&sc->neg_count, (unsigned long long)neg);
         if (!ok) flags |= FLAG_TIMEOUT;
         if (bad) flags |= FLAG_NONFINITE_STATE;
-        if (flags) atomicOr(&sc->flags, flags);
+        if (neg) atomicAdd((unsigned long long *)(SOA ? &bar->neg_count : &sc->neg_count), (unsigned long long)neg);
+        if (flags) atomicOr(SOA ? &bar->flags : &sc->flags, flags);
         if (scribe) {
-            sc->t = s_t;
-            sc->dt = i < n_steps ? 0.0 : dt_last;
-            sc->steps = steps;
-            sc->n_rec = n_rec;
+            if constexpr (!SOA) {
+                sc->t = s_t;
+                sc->dt = i < n_steps ? 0.0 : dt_last;
+                sc->steps = steps;
+                sc->n_rec = n_rec;
+            }
             for (int k = 0; k < 3; k++) sc->dtmin3[k] = min_bits(real_inf<float>());
         }
         __threadfence();
         if (atomicAdd(&bar->left, 1u) == gridDim.x - 1) {    // the last CTA to leave
+            if constexpr (SOA) {
+                __threadfence();
+                StepOutcome o;
+                o.dt = i < n_steps ? 0.0 : dt_last;
+                o.neg_count = (long long)atomicExch((unsigned long long *)&bar->neg_count, 0ull);
+                o.flags = atomicExch(&bar->flags, 0u);
+                *caller.out = o;
+            }
             bar->left = 0;
             bar->arrived = 0;
         }
@@ -167,10 +186,11 @@ __global__ void __launch_bounds__(MAXT, MINCTAS) steps_kernel(const KArgs<float>
 }
 
 // The kernel for a thread count with `ctas` CTAs of 256 threads per SM (null: none).
+template <bool SOA>
 static const void *steps_kernel_ptr(int threads, int ctas)
 {
-    if (threads <= 256) return ctas > 4 ? (const void *)steps_kernel<256, 5> : (const void *)steps_kernel<256, 4>;
-    return threads > 384 ? (const void *)steps_kernel<512, 2> : nullptr;
+    if (threads <= 256) return ctas > 4 ? (const void *)steps_kernel<256, 5, SOA> : (const void *)steps_kernel<256, 4, SOA>;
+    return threads > 384 ? (const void *)steps_kernel<512, 2, SOA> : nullptr;
 }
 
 // Rounds of blocks that a launch of `kern` takes (grid: its resident CTAs, at most one
@@ -201,25 +221,40 @@ int steps_config_f32(const DevPtrs &d, LaunchCfg &cfg)
 {
     cfg.grid = 0;
     cfg.smem = stage_smem_bytes<float>(d.block, d.max_halo, d.max_ring1, d.max_faces);
-    const void *k4 = steps_kernel_ptr(d.threads, 4), *k5 = steps_kernel_ptr(d.threads, 5);
+    const void *k4 = steps_kernel_ptr<false>(d.threads, 4), *k5 = steps_kernel_ptr<false>(d.threads, 5);
     if (!k4) return 0;
     int g4 = 0, r4 = 0, g5 = 0, r5 = 0;
     cudaError_t e = steps_rounds(k4, d, cfg.smem, g4, r4);
     if (e == cudaSuccess) e = steps_rounds(k5, d, cfg.smem, g5, r5);
     if (e != cudaSuccess) return (int)e;
     cfg.ctas = r5 < r4 ? 5 : 4;
-    if (std::min(r4, r5) <= 3) cfg.grid = cfg.ctas == 5 ? g5 : g4;
-    return 0;
+    if (std::min(r4, r5) > 3) return 0;
+    // the same grid has to fit with the caller's states
+    int g = 0, r = 0;
+    e = steps_rounds(steps_kernel_ptr<true>(d.threads, cfg.ctas), d, cfg.smem, g, r);
+    if (e == cudaSuccess) cfg.grid = std::min(g, cfg.ctas == 5 ? g5 : g4);
+    return (int)e;
+}
+
+static int launch_steps(const void *kern, const DevPtrs &d, KArgs<float> a, Gauges gauges, int n, CallerStep caller,
+                        const LaunchCfg &c, void *stream)
+{
+    StepsBarrier *bar = reinterpret_cast<StepsBarrier *>(reinterpret_cast<char *>(d.sc) + kBarrierAt);
+    void *args[] = {&a, &bar, &gauges, &n, &caller};
+    return (int)cudaLaunchCooperativeKernel(kern, dim3(c.grid), dim3(d.threads), args, c.smem, static_cast<cudaStream_t>(stream));
 }
 
 int launch_steps_f32(const DevPtrs &d, const StepParams &p, const void *w_in, void *w_out, int n, const LaunchCfg &c, void *stream)
 {
-    KArgs<float> a = make_args<float>(d, p, w_in, w_out);
-    StepsBarrier *bar = reinterpret_cast<StepsBarrier *>(reinterpret_cast<char *>(d.sc) + kBarrierAt);
-    Gauges g{d.n_gauges, d.ring_cap, p.gauge_every, d.gauge_cells, d.ring_t, d.ring_eta};
-    void *args[] = {&a, &bar, &g, &n};
-    return (int)cudaLaunchCooperativeKernel(steps_kernel_ptr(d.threads, c.ctas), dim3(c.grid), dim3(d.threads), args, c.smem,
-                                            static_cast<cudaStream_t>(stream));
+    return launch_steps(steps_kernel_ptr<false>(d.threads, c.ctas), d, make_args<float>(d, p, w_in, w_out),
+                        {d.n_gauges, d.ring_cap, p.gauge_every, d.gauge_cells, d.ring_t, d.ring_eta}, n, {}, c, stream);
+}
+
+int launch_caller_step_f32(const DevPtrs &d, const StepParams &p, const void *w_in, void *w_out, double t, double t_end,
+                           StepOutcome *out, const LaunchCfg &c, void *stream)
+{
+    return launch_steps(steps_kernel_ptr<true>(d.threads, c.ctas), d, make_args<float>(d, p, w_in, w_out, true), {}, 1,
+                        {t, t_end, out}, c, stream);
 }
 
 size_t stage_smem_f32(int block, int max_halo, int max_ring1, int max_faces)

@@ -89,10 +89,19 @@ struct DevScalars {
     unsigned long long dtmin3[3];   // the multi-step kernel's CFL minima of three consecutive steps
 };
 
-// CTAs that have arrived at the multi-step kernel's barriers and that have left it (zero
-// between launches): kBarrierAt bytes behind a context's DevScalars, on a line of its own.
+// CTAs that have arrived at the multi-step kernel's barriers and that have left it, and a
+// step of a caller's states' flags and negative depths (all zero between launches):
+// kBarrierAt bytes behind a context's DevScalars, on a line of its own.
 struct StepsBarrier {
-    unsigned int arrived, left;
+    unsigned int arrived, left, flags, pad;
+    long long neg_count;
+};
+
+// What a step of a caller's states reports.
+struct StepOutcome {
+    double dt;
+    long long neg_count;
+    unsigned int flags, pad;
 };
 constexpr int kBarrierAt = 256, kScalarAlloc = kBarrierAt + 128;
 
@@ -192,6 +201,11 @@ int launch_rk_unfused_f64_fast(const DevPtrs &d, const StepParams &p, int part, 
 // the pair).  steps_config: grid 0 where the thread count has no such kernel.
 int steps_config_f32(const DevPtrs &d, LaunchCfg &cfg);
 int launch_steps_f32(const DevPtrs &d, const StepParams &p, const void *w_in, void *w_out, int n, const LaunchCfg &c, void *stream);
+
+// One step of a caller's [3][nc] states from time t, in one cooperative launch; the
+// outcome goes to `out` (host memory that the device can write).
+int launch_caller_step_f32(const DevPtrs &d, const StepParams &p, const void *w_in, void *w_out, double t, double t_end,
+                           StepOutcome *out, const LaunchCfg &c, void *stream);
 
 // The contracted FP64 build (step_f64_fast.cu); the *_f64 entry points above
 // dispatch to it when DevPtrs::fp64_fast / StepParams::fp64_fast is set.

@@ -166,18 +166,20 @@ def test_run_to_several_end_times(precision):
 @pytest.mark.parametrize("precision,literal", [(32, 1), (64, 1), (64, 0)])
 @pytest.mark.parametrize("n,steps,t_end", [(1, 2, 0.0), (9, 7, 0.0), (33, 8, 0.0), (33, 23, 0.012), (110, 9, 0.0), (290, 5, 0.0), (330, 4, 0.0), (420, 5, 0.0)])
 def test_many_steps_in_one_launch(precision, literal, n, steps, t_end):
-    """A call of many steps against as many calls of one step, bit for bit: state, time,
-    counts and gauge records; odd and even step counts, an end time between them, meshes
-    of one block and of more than one block per CTA."""
+    """Steps in one launch against the step kernels one by one (which a profile asks for)
+    and against a split into calls, bit for bit: state, time, counts and gauge records;
+    odd and even step counts, an end time between them, meshes of one block and of more
+    than one block per CTA."""
     m, st = _moving_basin(n)
     out = []
-    for parts in ([steps], [1] * steps, [1, 2, steps - 3] if steps > 3 else [0, steps]):
+    for parts in ([steps], "profile", [1, 2, steps - 3] if steps > 3 else [0, steps]):
         with volna.Solver(precision) as sv:
             sv.set_params(h_threshold=1e-5, cfl=0.9, fp64_literal=literal, t_end=t_end, gauge_every=2)
             sv.upload_mesh(m)
             sv.set_gauges(np.array([[0.01, 0.005], [0.2, 0.1], [-0.11, 0.2]]))
             sv.set_state(*st, 0.0)
-            for k in parts:
+            sv.profile(parts == "profile")
+            for k in [steps] if parts == "profile" else parts:
                 sv.step(k)
             d = sv.diagnostics()
             out.append(list(sv.get_state()) + list(sv.gauges()) + [d[k] for k in ("t", "last_dt", "steps", "neg_count", "launches")])
@@ -209,3 +211,40 @@ def test_batch_scenario_groups(precision, n, scenarios):
                     ref = sv.get_state()
                 for a, r in zip(b.get_state(mid, j)[:4], ref):
                     np.testing.assert_array_equal(a, r)
+
+
+@pytest.mark.parametrize("n,t_end", [(1, 0.0), (9, 0.0), (66, 0.0), (110, 1e-3), (300, 0.0), (360, 0.0)])
+def test_caller_step_in_one_launch(n, t_end):
+    """The step of caller-owned states in one launch against the separate kernels (which
+    a shape of 384 threads keeps), bit for bit: states, dt, past t_end, and a context of
+    its own that is not disturbed; a non-finite state is reported and leaves nothing
+    behind."""
+    import torch
+    m, st = _moving_basin(n)
+    w0 = torch.from_numpy(np.stack([st[0] - m.vertex_mean(m.depth), st[1], st[2]])).float().cuda()
+    out = []
+    for kw in ({}, dict(block_cells=192, block_threads=384)):
+        with volna.Solver(32) as sv:
+            sv.set_params(h_threshold=1e-5, cfl=0.9, t_end=t_end, **kw)
+            sv.upload_mesh(m)
+            sv.set_state(*st, 0.0)
+            sv.step(2)
+            before = sv.get_state()
+            w = torch.empty_like(w0)
+            w[:, torch.from_numpy(sv.permutation().astype(np.int64)).cuda()] = w0
+            bufs, t, res = [torch.empty_like(w) for _ in range(2)], 0.0, []
+            for k in range(4):
+                dt = volna.vg_step_noalloc(sv.ctx, w.data_ptr(), bufs[k & 1].data_ptr(), t)
+                t, w = t + dt, bufs[k & 1]
+                res += [dt, w.cpu().numpy()]
+            broken = w.clone()
+            broken[1, 0] = float("nan")
+            broken[0, 0] += 10.0
+            with pytest.raises(volna.VolnaError):
+                volna.vg_step_noalloc(sv.ctx, broken.data_ptr(), bufs[0].data_ptr(), 0.0)
+            res += [volna.vg_step_noalloc(sv.ctx, w.data_ptr(), bufs[0].data_ptr(), 0.0)]
+            for a, b in zip(before, sv.get_state()):
+                np.testing.assert_array_equal(a, b)
+            out.append(res)
+    for a, b in zip(*out):
+        np.testing.assert_array_equal(a, b)
