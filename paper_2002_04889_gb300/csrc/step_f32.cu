@@ -10,11 +10,12 @@ namespace vg {
 //
 // A step of three kernels from a graph pays for two ends of a kernel and starts of the
 // next, and for the one-CTA epilogue: 12.4 us on 20k triangles, of which the blocks'
-// chains of phases take about 7.  The barriers cost about 1.3 us each: 9.9 us (steps_
-// config_f32 has the other sizes).  A barrier is bound by the arrivals at one address
-// (2400 CTAs of 64 threads: 10 us), so the waiting CTAs poll with pauses (99k: 14.8 ->
-// 14.5); arrivals spread over eight addresses, all of which every CTA then polls, and a
-// flag written by the last to arrive were both slower (14.7, 16.5).
+// chains of phases take about 7.  The barriers cost about 1.3 us each: 9.9 us, and 9.3
+// where a CTA keeps its one block's mesh data in shared memory (steps_config_f32 has the
+// other sizes).  A barrier is bound by the arrivals at one address (2400 CTAs of 64
+// threads: 10 us), so the waiting CTAs poll with pauses (99k: 14.8 -> 14.5); arrivals
+// spread over eight addresses, all of which every CTA then polls, and a flag written by
+// the last to arrive were both slower (14.7, 16.5).
 //
 // Every CTA keeps the time and forms dt for itself, from the same bits.  The last CTA
 // (it has no more blocks than another) also keeps the counts and records the gauges,
@@ -86,14 +87,16 @@ __global__ void __launch_bounds__(MAXT, MINCTAS) steps_kernel(const KArgs<float>
     __syncthreads();
     long long my_neg = 0;
     bool bad = false, ok = true;
+    const bool one_block = a.nblocks <= (int)gridDim.x;       // its mesh data stay in shared memory
+    bool loaded = false;
     int i = 0;
     for (; i < n_steps; i++) {
         if (is_pos(t_end) && okey(s_t) >= okey(t_end)) break;      // the same in every CTA
         // stage 1 and the CTA's CFL bound
         float my_min = real_inf<float>();
         for (int b = blockIdx.x; b < a.nblocks; b += gridDim.x) {
-            bool loaded = false;
-            process_block<1, SOA>(a, b, 0.f, smem_raw, my_min, my_neg, bad, loaded);
+            if (!one_block) loaded = false;
+            process_block<1, SOA, KEEP_STEPS>(a, b, 0.f, smem_raw, my_min, my_neg, bad, loaded);
         }
         for (int o = 16; o > 0; o >>= 1) my_min = smin(my_min, __shfl_xor_sync(0xffffffffu, my_min, o));
         if (lane == 0) red_min[warp] = my_min;
@@ -115,8 +118,8 @@ __global__ void __launch_bounds__(MAXT, MINCTAS) steps_kernel(const KArgs<float>
         __syncthreads();
         const float dt = s_dt;
         for (int b = blockIdx.x; b < a.nblocks; b += gridDim.x) {
-            bool loaded = false;
-            process_block<2, SOA>(a, b, dt, smem_raw, my_min, my_neg, bad, loaded);
+            if (!one_block) loaded = false;
+            process_block<2, SOA, KEEP_STEPS>(a, b, dt, smem_raw, my_min, my_neg, bad, loaded);
         }
         if (!(ok = grid_barrier(bar, target))) break;
         if (tid == 0) {
@@ -210,7 +213,8 @@ static cudaError_t steps_rounds(const void *kern, const DevPtrs &d, size_t smem,
 
 // Four CTAs of 256 threads per SM have registers enough; five spill a little and are
 // taken where they save a round of blocks.  Figures: us a step, four / five CTAs / the
-// three kernels in a graph (basin, 256 cells):
+// three kernels in a graph (basin, 256 cells; before a CTA with one block kept its mesh
+// data, which took another us off one round):
 //   99,458 (389 blocks): 14.5 / 15.7 / 17.6;  151,250 (591): 16.3 / 17.3 / 18.9
 //   186,050 (727): 21.6 / 19.1 / 19.6;  245,000 (958): 23.2 / 24.8 / 25.8
 //   320,000 (1250): 25.0 / 26.3 / 28.8;  500,000 (1954): 34.5 / 35.7 / 36.9

@@ -867,7 +867,7 @@ template <int STAGE, bool FAST, bool BATCH, bool SOA>
 __device__ __forceinline__ void run_block(const KArgs<float> &a, int b, float dt, unsigned char *smem, int &,
                                           float &my_min, long long &my_neg, bool &bad, bool &loaded)
 {
-    process_block<STAGE, SOA>(a, b, dt, smem, my_min, my_neg, bad, loaded);
+    process_block<STAGE, SOA, BATCH ? KEEP_SCENARIOS : KEEP_NOTHING>(a, b, dt, smem, my_min, my_neg, bad, loaded);
 }
 
 // w^{n+1} = w^n, bit for bit, by every thread of the launch.
