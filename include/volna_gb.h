@@ -322,10 +322,16 @@ int vg_set_depth(vg_ctx *ctx, const double *depth_v);
  * every checkpoint_every-th step is kept on the device, and vg_adj_backward
  * recomputes each segment of checkpoint_every steps once, recording it (about
  * r = 192 bytes per cell and step with a fixed dt, 224 with CFL steps, against
- * 24 per checkpoint).  0 picks the segment length that minimises device memory,
- * round(sqrt(24 n_steps / r)): recordings and checkpoints then take about equal
- * shares, 2 sqrt(24 r n_steps) bytes per cell in all (about 6.1 KB per cell for
- * 2000 steps).  The context's state advances to step n_steps.  dt < 0 or
+ * 24 per checkpoint).  0 leaves the choice to the library: where the recordings of
+ * all steps take at most 1/32 of the device's memory and a quarter of what is
+ * free, the bed is static and the run is not profiled, the forward run records
+ * every step and the sweep recomputes none; the recordings are held until the
+ * next forward run, a new mesh, or a call that changes the parameters, the depth,
+ * the boundaries or the bed motion (the sweep then recomputes from the
+ * checkpoints).  Otherwise it picks the segment length that minimises device
+ * memory, round(sqrt(24 n_steps / r)): recordings and checkpoints then take about
+ * equal shares, 2 sqrt(24 r n_steps) bytes per cell in all (about 6.1 KB per cell
+ * for 2000 steps).  The context's state advances to step n_steps.  dt < 0 or
  * non-finite: VG_EINVAL.
  */
 int vg_adj_forward(vg_ctx *ctx, int64_t n_steps, double dt, int64_t checkpoint_every);

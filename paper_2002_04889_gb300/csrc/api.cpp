@@ -29,6 +29,16 @@ const char *kKernelNames[kKernels] = {"stage1", "stage2", "post_step", "bed_upda
 
 }  // namespace
 
+// What the reversal of every step of a forward run needs, in one allocation: states,
+// stage-1 residuals, face values of both stages, with CFL steps the stage-2 residuals and
+// the cells' bounds, the dry-fix branches and the reconstruction flags.
+struct AdjRecordings {
+    void *base = nullptr;
+    int64_t bytes = 0;
+    double *w = nullptr, *R0 = nullptr, *FV = nullptr, *R1 = nullptr, *bound = nullptr;
+    uint8_t *mask2 = nullptr, *flags = nullptr;
+};
+
 struct vg_ctx {
     int precision = 64;
     int device = 0;
@@ -88,8 +98,10 @@ struct vg_ctx {
     bool graph_dirty = true;
     int64_t launches = 0;
 
-    // discrete adjoint: checkpoints of the last vg_adj_forward run
+    // discrete adjoint: checkpoints of the last vg_adj_forward run, and the recordings of
+    // all its steps where they were kept (AdjRecordings)
     std::vector<void *> ckpt;
+    AdjRecordings rec;
     int64_t adj_n = 0, adj_every = 0;
     double adj_dt = 0.0;                // > 0 fixed step; 0: the CFL steps below
     double adj_cfl = 0.0, adj_dt_max = 0.0;
@@ -151,8 +163,16 @@ void dfree(T *&p)
     p = nullptr;
 }
 
+void drop_recordings(vg_ctx *c)
+{
+    if (c->rec.base) cudaFree(c->rec.base);
+    c->dev_bytes -= c->rec.bytes;
+    c->rec = AdjRecordings{};
+}
+
 void free_adjoint(vg_ctx *c)
 {
+    drop_recordings(c);
     for (void *p : c->ckpt) cudaFree(p);
     c->ckpt.clear();
     c->adj_n = 0;
@@ -1043,6 +1063,7 @@ int vg_set_params(vg_ctx *c, const vg_params *p)
     const int old_block = old_shape.cells, new_block = new_shape.cells;
     bool threads_changed = new_shape.threads != old_shape.threads || p->fp64_literal != c->prm.fp64_literal;
     const vg_params old_prm = c->prm;
+    drop_recordings(c);                  // of the old parameters; the checkpoints serve any
     c->prm = *p;
     if (c->has_mesh) {
         int rc = ensure_fast_matrix(c);
@@ -1434,6 +1455,7 @@ int vg_set_depth(vg_ctx *c, const double *depth_v)
     HostMesh &m = c->hm;
     for (int64_t v = 0; v < m.nv; v++)
         if (!std::isfinite(depth_v[v])) return fail(c, VG_EINVAL, "non-finite depth");
+    drop_recordings(c);
     std::string err;
     if (bed_arrays(m, depth_v, err)) return fail(c, VG_EINVAL, err);
     cudaStreamSynchronize(c->stream);
@@ -1466,6 +1488,7 @@ int vg_set_boundary(vg_ctx *c, int64_t n, const int32_t *edges, const int32_t *k
             return fail(c, VG_EINVAL, "boundary kind " + std::to_string(kinds[e]) + " of edge " + std::to_string(e));
     if (!c->has_mesh) return fail(c, VG_ESTATE, "no mesh");
     DeviceGuard guard(c->device);
+    drop_recordings(c);
     HostMesh &m = c->hm;
     const int64_t nc = m.nc;
     // boundary faces by their (sorted) original vertex pair
@@ -1512,6 +1535,7 @@ int vg_set_bed_motion(vg_ctx *c, const double *uplift_v, const double *onset_v, 
     if (uplift_v && (!onset_v || !(rise >= 0.0) || !std::isfinite(rise)))
         return fail(c, VG_EINVAL, "onset times and a finite rise time >= 0 are required");
     DeviceGuard guard(c->device);
+    drop_recordings(c);
     const HostMesh &m = c->hm;
     const int64_t nv = m.nv, nc = m.nc;
     if (uplift_v)
@@ -1558,6 +1582,69 @@ int vg_set_bed_motion(vg_ctx *c, const double *uplift_v, const double *onset_v, 
     return VG_OK;
 }
 
+// Room for the recordings of n steps, where that is at most 1/32 of the device's memory
+// and a quarter of what is free; without it the backward pass recomputes the steps.
+static void keep_recordings(vg_ctx *c, int64_t n, bool adaptive)
+{
+    const size_t nc = (size_t)c->hm.nc, steps = (size_t)n;
+    const double want = (double)steps * nc * (8.0 * (24 + (adaptive ? 4 : 0)) + 3.0);
+    size_t free_bytes = 0, total = 0;
+    if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess || want > total / 32.0 || want > free_bytes / 4.0) {
+        cudaGetLastError();
+        return;
+    }
+    AdjRecordings r;
+    r.bytes = (int64_t)(steps * nc * (8 * (24 + (adaptive ? 4 : 0)) + 3));
+    if (cudaMalloc(&r.base, (size_t)r.bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    r.w = static_cast<double *>(r.base);
+    r.R0 = r.w + 3 * steps * nc;
+    r.FV = r.R0 + 3 * steps * nc;
+    double *end = r.FV + 18 * steps * nc;
+    if (adaptive) {
+        r.R1 = end;
+        r.bound = r.R1 + 3 * steps * nc;
+        end = r.bound + steps * nc;
+    }
+    r.mask2 = reinterpret_cast<uint8_t *>(end);
+    r.flags = r.mask2 + steps * nc;
+    c->dev_bytes += r.bytes;
+    c->rec = r;
+}
+
+// Kernel arguments that record step r of a run: stage 1, then (second) stage 2.
+static DevPtrs recording_ptrs(DevPtrs d, size_t nc, size_t r, bool second, double *R0, double *FV, uint8_t *mask2, uint8_t *flags,
+                              double *R1, double *bound)
+{
+    d.R0 = R0 + r * 3 * nc;
+    d.mask2 = mask2 + r * nc;
+    d.fv_out = FV + (r * 18 + (second ? 9 : 0)) * nc;
+    d.rec_out = flags + (r * 2 + (second ? 1 : 0)) * nc;
+    if (bound) d.bound_out = bound + r * nc;
+    if (second && R1) d.r1_out = R1 + r * 3 * nc;
+    return d;
+}
+
+// Step n of a forward run into its recordings; the last one ends in the context's state.
+static int recorded_step(vg_ctx *c, int64_t n, int64_t n_steps)
+{
+    const AdjRecordings &a = c->rec;
+    const size_t nc = (size_t)c->hm.nc;
+    const DevPtrs d = dev_ptrs(c);
+    const StepParams p = step_params(c);
+    void *s = (void *)c->stream;
+    const double *win = a.w + (size_t)n * 3 * nc;
+    void *wout = n + 1 < n_steps ? (void *)(win + 3 * nc) : c->w[c->cur];
+    int e = launch_stage1_f64(recording_ptrs(d, nc, n, false, a.R0, a.FV, a.mask2, a.flags, a.R1, a.bound), p, win, c->cfg1, s);
+    if (e) return cuda_fail(c, (cudaError_t)e, "stage 1 launch");
+    e = launch_stage2_f64(recording_ptrs(d, nc, n, true, a.R0, a.FV, a.mask2, a.flags, a.R1, a.bound), p, win, wout, c->cfg2, s);
+    if (e) return cuda_fail(c, (cudaError_t)e, "stage 2 launch");
+    if ((e = launch_post_step(d, p, wout, 64, s))) return cuda_fail(c, (cudaError_t)e, "post-step launch");
+    return VG_OK;
+}
+
 int vg_adj_forward(vg_ctx *c, int64_t n_steps, double dt, int64_t checkpoint_every)
 {
     if (!c || n_steps < 1 || !(dt >= 0) || !std::isfinite(dt) || checkpoint_every < 0) return VG_EINVAL;
@@ -1583,6 +1670,11 @@ int vg_adj_forward(vg_ctx *c, int64_t n_steps, double dt, int64_t checkpoint_eve
     }
     double *dts_dev = nullptr;
     if (dmalloc(c, (void **)&dts_dev, 8 * (size_t)n_steps)) { free_adjoint(c); return VG_ENOMEM; }
+    // With the segment length left to the library a run records its steps at once where
+    // they fit (50k triangles, 40 CFL steps, 0.45 GB: 16.8 ms forward and back against 22.0
+    // with the steps recomputed; recording costs a step 5 us of 120); a moving
+    // bed's and a profiled run recompute them.
+    if (!checkpoint_every && !c->bed_on && !c->profile) keep_recordings(c, n_steps, !(dt > 0.0));
     vg_params saved = c->prm;
     const LaunchCfg saved_cfg1 = c->cfg1, saved_cfg2 = c->cfg2;
     c->prm.dt_fixed = dt;               // 0: the CFL rule of every step
@@ -1604,18 +1696,24 @@ int vg_adj_forward(vg_ctx *c, int64_t n_steps, double dt, int64_t checkpoint_eve
     c->rec_t.clear();
     c->rec_eta.clear();
     if (!rc) rc = record_now(c);
+    const bool keep = c->rec.base != nullptr;
+    if (!rc && keep) {
+        cudaError_t e = cudaMemcpyAsync(c->rec.w, c->w[c->cur], bytes, cudaMemcpyDeviceToDevice, c->stream);
+        if (e != cudaSuccess) rc = cuda_fail(c, e, "first state copy");
+    }
     for (int64_t n = 0; n < n_steps && !rc; n++) {
         c->mirror_ok = false;
         if (n % C == 0) {
-            cudaError_t e = cudaMemcpyAsync(c->ckpt[n / C], c->w[c->cur], bytes, cudaMemcpyDeviceToDevice, c->stream);
+            const void *w = keep ? (const void *)(c->rec.w + (size_t)n * 3 * (size_t)c->hm.nc) : c->w[c->cur];
+            cudaError_t e = cudaMemcpyAsync(c->ckpt[n / C], w, bytes, cudaMemcpyDeviceToDevice, c->stream);
             if (e != cudaSuccess) { rc = cuda_fail(c, e, "checkpoint copy"); break; }
         }
-        if ((rc = enqueue_step(c, c->cur))) break;
+        if ((rc = keep ? recorded_step(c, n, n_steps) : enqueue_step(c, c->cur))) break;
         {
             cudaError_t e = cudaMemcpyAsync(dts_dev + n, &c->sc->dt, 8, cudaMemcpyDeviceToDevice, c->stream);
             if (e != cudaSuccess) { rc = cuda_fail(c, e, "time-step record"); break; }
         }
-        c->cur = 1 - c->cur;
+        if (!keep) c->cur = 1 - c->cur;
         c->launches += step_kernels(c);
         if ((n + 1) % 1024 == 0) {
             if ((rc = read_scalars(c, s))) break;
@@ -1692,6 +1790,7 @@ int vg_adj_backward(vg_ctx *c, const double *dJ_deta, double *dJ_dH0, double *dJ
     const int nc = (int)c->hm.nc, G = c->n_gauges;
     const size_t w3 = 3 * (size_t)nc;
     const bool binomial = c->adj_slots > 0;
+    const bool kept = c->rec.base != nullptr && !binomial;   // the forward run's own recordings
     const int64_t RC = binomial ? 1 : C;    // steps whose recordings are held at once
     // scratch (freed at the end)
     std::vector<void *> bufs;
@@ -1701,24 +1800,27 @@ int vg_adj_backward(vg_ctx *c, const double *dJ_deta, double *dJ_dH0, double *dJ
         if (!rc) { bufs.push_back(q); *p = static_cast<double *>(q); }
         return rc;
     };
+    auto alloc_seg = [&](size_t n_doubles, double **p) { return kept ? 0 : alloc(n_doubles, p); };
     // seg: the segment's states, R0seg: their stage-1 residuals, m2seg: stage-2
     // dry-fix branches (all recorded by one forward recompute of the segment)
-    double *W, *wb, *wbn, *wb1, *zb, *Rb, *w1, *H1pre, *FVb, *zfb, *own, *send, *seg, *R0seg, *wlast, *m2raw;
-    double *recraw;  // reconstruction flags of both stages of every recorded step [RC][2][nc] (bytes)
-    double *FVseg;   // face values of both stages of every step of the segment [C][2][9][nc]
+    double *W, *wb, *wbn, *wb1, *zb, *Rb, *w1, *H1pre, *FVb, *zfb, *own, *send, *wlast;
+    double *seg = c->rec.w, *R0seg = c->rec.R0, *m2raw = reinterpret_cast<double *>(c->rec.mask2);
+    double *recraw = reinterpret_cast<double *>(c->rec.flags);   // reconstruction flags of both stages of every recorded
+                                                                 // step [RC][2][nc] (bytes)
+    double *FVseg = c->rec.FV;   // face values of both stages of every step of the segment [C][2][9][nc]
     const bool adaptive = !(c->adj_dt > 0.0);
-    double *R1seg = nullptr, *cflscr = nullptr, *bndseg = nullptr;   // adaptive steps: stage-2 residuals; dt-bar and
+    double *R1seg = c->rec.R1, *cflscr = nullptr, *bndseg = c->rec.bound;   // adaptive steps: stage-2 residuals; dt-bar and
                                                                      // reduction scratch; the cells' CFL bounds
     int rc = 0;
     if ((rc = alloc((size_t)(N + 1) * G, &W)) || (rc = alloc(w3, &wb)) || (rc = alloc(w3, &wbn)) ||
         (rc = alloc(w3, &wb1)) || (rc = alloc(4 * (size_t)nc, &zb)) || (rc = alloc(w3, &Rb)) || (rc = alloc(w3, &wlast)) ||
-        (rc = alloc(w3, &w1)) || (rc = alloc(nc, &H1pre)) || (rc = alloc(18 * (size_t)nc * RC, &FVseg)) ||
+        (rc = alloc(w3, &w1)) || (rc = alloc(nc, &H1pre)) || (rc = alloc_seg(18 * (size_t)nc * RC, &FVseg)) ||
         (rc = alloc(9 * (size_t)nc, &FVb)) || (rc = alloc(3 * (size_t)nc, &zfb)) || (rc = alloc(7 * (size_t)nc, &own)) ||
         (rc = alloc(12 * (size_t)nc, &send)) ||
-        (rc = alloc(w3 * (size_t)(binomial ? 2 + c->adj_slots : C), &seg)) ||
-        (rc = alloc(w3 * (size_t)RC, &R0seg)) || (rc = alloc(((size_t)nc * RC + 7) / 8, &m2raw)) ||
-        (rc = alloc((2 * (size_t)nc * RC + 7) / 8, &recraw)) ||
-        (adaptive && ((rc = alloc(w3 * (size_t)RC, &R1seg)) || (rc = alloc((size_t)nc * RC, &bndseg)) ||
+        (rc = alloc_seg(w3 * (size_t)(binomial ? 2 + c->adj_slots : C), &seg)) ||
+        (rc = alloc_seg(w3 * (size_t)RC, &R0seg)) || (rc = alloc_seg(((size_t)nc * RC + 7) / 8, &m2raw)) ||
+        (rc = alloc_seg((2 * (size_t)nc * RC + 7) / 8, &recraw)) ||
+        (adaptive && ((rc = alloc_seg(w3 * (size_t)RC, &R1seg)) || (rc = alloc_seg((size_t)nc * RC, &bndseg)) ||
                       (rc = alloc(16 + 4 * (size_t)kAdjCflParts, &cflscr))))) {
         for (void *q : bufs) cudaFree(q);
         return rc;
@@ -1823,21 +1925,15 @@ int vg_adj_backward(vg_ctx *c, const double *dJ_deta, double *dJ_dH0, double *dJ
         // its reversal needs (stage-1 residual, face values of both stages, the
         // stage-2 dry-fix branches, with CFL steps the stage-2 residual)
         auto record_step = [&](int64_t n, const double *win, double *wout, int64_t r) -> int {
-            DevPtrs dd = d;
-            dd.R0 = R0seg + (size_t)r * w3;
-            dd.mask2 = m2seg + (size_t)r * nc;
-            dd.fv_out = FVseg + (size_t)r * 18 * nc;
-            dd.rec_out = recseg + (size_t)r * 2 * nc;
+            auto ptrs = [&](bool second) {
+                return recording_ptrs(d, nc, r, second, R0seg, FVseg, m2seg, recseg, R1seg, bndseg);
+            };
             StepParams pn = p;
             pn.dt_fixed = c->adj_dts[n];        // the step the forward run took
             int e;
             if (bed && (e = launch_bed_update(d, p, nullptr, 64, false, tn[n], st))) return e;   // bed of step n
-            if (adaptive) dd.bound_out = bndseg + (size_t)r * nc;
-            if ((e = launch_stage1_f64(dd, pn, win, lc1, st))) return e;
-            dd.fv_out = FVseg + ((size_t)r * 18 + 9) * nc;
-            dd.rec_out = recseg + ((size_t)r * 2 + 1) * nc;
-            if (adaptive) dd.r1_out = R1seg + (size_t)r * w3;
-            return launch_stage2_f64(dd, pn, win, wout, lc2, st);
+            if ((e = launch_stage1_f64(ptrs(false), pn, win, lc1, st))) return e;
+            return launch_stage2_f64(ptrs(true), pn, win, wout, lc2, st);
         };
         // one forward step without recordings (binomial schedule)
         auto advance_step = [&](int64_t n, const double *win, double *wout) -> int {
@@ -1887,7 +1983,9 @@ int vg_adj_backward(vg_ctx *c, const double *dJ_deta, double *dJ_dH0, double *dJ
             c->launches += 8 + (bed ? 5 : 0);
             return 0;
         };
-        if (!binomial) {
+        if (kept) {
+            for (int64_t n = N - 1; n >= 0; n--) ADJ_CHECK(reverse_step(n, seg + (size_t)n * w3, n));
+        } else if (!binomial) {
             // sqrt(N) segments: recompute each segment once from its checkpoint,
             // recording every step, then reverse it
             int64_t nseg = (N + C - 1) / C;

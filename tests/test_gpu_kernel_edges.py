@@ -248,3 +248,32 @@ def test_caller_step_in_one_launch(n, t_end):
             out.append(res)
     for a, b in zip(*out):
         np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("dt", [0.0, 1e-3])
+def test_adjoint_with_kept_recordings(dt):
+    """Gradients from the forward run's own recordings (the default where they fit), from
+    segments that are recomputed, and after a call that drops the recordings: bit for bit
+    the same, twice in a row, and the state that the forward run leaves too."""
+    m, st = _moving_basin(33)
+    pts = np.array([[0.0, 0.0], [0.31, -0.12]])
+    W = np.random.default_rng(5).normal(size=(12, 2))
+    out = []
+    with volna.Solver(64) as sv:
+        sv.set_params(h_threshold=1e-5, cfl=0.9)
+        sv.upload_mesh(m)
+        sv.set_gauges(pts)
+        for every, drop in ((0, False), (3, False), (0, True)):
+            sv.set_state(*st, 0.0)
+            _, eta = sv.adj_forward(11, dt, every)
+            if drop:
+                sv.set_params(h_threshold=1e-5, cfl=0.9)
+            state = sv.get_state()
+            sv.step(2)
+            g, again = sv.adj_backward(W, m.nv), sv.adj_backward(W, m.nv)
+            for k in g:
+                np.testing.assert_array_equal(g[k], again[k])
+            out.append([eta, *state] + [g[k] for k in sorted(g)])
+    for other in out[1:]:
+        for a, b in zip(out[0], other):
+            np.testing.assert_array_equal(a, b)
