@@ -88,7 +88,7 @@ typedef struct vg_params {
                               the scheme (the oracle's order) bit for bit; 0 lets
                               the compiler contract multiply-adds and divides
                               once where the literal form divides several times
-                              by the same value: about 1.8x faster, rounding
+                              by the same value: 1.2 to 1.5x faster, rounding
                               differences only, but over long runs with moving
                               shorelines those decide discontinuous switches
                               (a thin film's velocity, hence the CFL step)
@@ -325,10 +325,10 @@ int vg_set_depth(vg_ctx *ctx, const double *depth_v);
  * 24 per checkpoint).  0 leaves the choice to the library: where the recordings of
  * all steps take at most 1/32 of the device's memory and a quarter of what is
  * free, the bed is static and the run is not profiled, the forward run records
- * every step and the sweep recomputes none; the recordings are held until the
- * next forward run, a new mesh, or a call that changes the parameters, the depth,
- * the boundaries or the bed motion (the sweep then recomputes from the
- * checkpoints).  Otherwise it picks the segment length that minimises device
+ * every step and the sweep recomputes none (but from the checkpoints after a call
+ * that changes the parameters, the depth, the boundaries or the bed motion).  The
+ * context holds this memory until a forward run of another shape or a new mesh.
+ * Otherwise it picks the segment length that minimises device
  * memory, round(sqrt(24 n_steps / r)): recordings and checkpoints then take about
  * equal shares, 2 sqrt(24 r n_steps) bytes per cell in all (about 6.1 KB per cell
  * for 2000 steps).  The context's state advances to step n_steps.  dt < 0 or

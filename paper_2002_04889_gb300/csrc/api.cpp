@@ -35,6 +35,7 @@ const char *kKernelNames[kKernels] = {"stage1", "stage2", "post_step", "bed_upda
 struct AdjRecordings {
     void *base = nullptr;
     int64_t bytes = 0;
+    bool valid = false;                 // they are those of the last forward run and of the present parameters
     double *w = nullptr, *R0 = nullptr, *FV = nullptr, *R1 = nullptr, *bound = nullptr;
     uint8_t *mask2 = nullptr, *flags = nullptr;
 };
@@ -1063,7 +1064,7 @@ int vg_set_params(vg_ctx *c, const vg_params *p)
     const int old_block = old_shape.cells, new_block = new_shape.cells;
     bool threads_changed = new_shape.threads != old_shape.threads || p->fp64_literal != c->prm.fp64_literal;
     const vg_params old_prm = c->prm;
-    drop_recordings(c);                  // of the old parameters; the checkpoints serve any
+    c->rec.valid = false;                // of the old parameters; the checkpoints serve any
     c->prm = *p;
     if (c->has_mesh) {
         int rc = ensure_fast_matrix(c);
@@ -1455,7 +1456,7 @@ int vg_set_depth(vg_ctx *c, const double *depth_v)
     HostMesh &m = c->hm;
     for (int64_t v = 0; v < m.nv; v++)
         if (!std::isfinite(depth_v[v])) return fail(c, VG_EINVAL, "non-finite depth");
-    drop_recordings(c);
+    c->rec.valid = false;
     std::string err;
     if (bed_arrays(m, depth_v, err)) return fail(c, VG_EINVAL, err);
     cudaStreamSynchronize(c->stream);
@@ -1488,7 +1489,7 @@ int vg_set_boundary(vg_ctx *c, int64_t n, const int32_t *edges, const int32_t *k
             return fail(c, VG_EINVAL, "boundary kind " + std::to_string(kinds[e]) + " of edge " + std::to_string(e));
     if (!c->has_mesh) return fail(c, VG_ESTATE, "no mesh");
     DeviceGuard guard(c->device);
-    drop_recordings(c);
+    c->rec.valid = false;
     HostMesh &m = c->hm;
     const int64_t nc = m.nc;
     // boundary faces by their (sorted) original vertex pair
@@ -1535,7 +1536,7 @@ int vg_set_bed_motion(vg_ctx *c, const double *uplift_v, const double *onset_v, 
     if (uplift_v && (!onset_v || !(rise >= 0.0) || !std::isfinite(rise)))
         return fail(c, VG_EINVAL, "onset times and a finite rise time >= 0 are required");
     DeviceGuard guard(c->device);
-    drop_recordings(c);
+    c->rec.valid = false;
     const HostMesh &m = c->hm;
     const int64_t nv = m.nv, nc = m.nc;
     if (uplift_v)
@@ -1611,6 +1612,7 @@ static void keep_recordings(vg_ctx *c, int64_t n, bool adaptive)
     r.mask2 = reinterpret_cast<uint8_t *>(end);
     r.flags = r.mask2 + steps * nc;
     c->dev_bytes += r.bytes;
+    r.valid = true;
     c->rec = r;
 }
 
@@ -1652,7 +1654,6 @@ int vg_adj_forward(vg_ctx *c, int64_t n_steps, double dt, int64_t checkpoint_eve
     if (!c->has_mesh || !c->has_state) return fail(c, VG_ESTATE, "mesh and state must be set");
     if (c->n_gauges < 1) return fail(c, VG_ESTATE, "the adjoint differentiates gauge records: set gauges first");
     DeviceGuard guard(c->device);
-    free_adjoint(c);
     // default segment length: the one that minimises device memory, C checkpoints'
     // worth of recordings (per cell: face values of both stages, the segment state,
     // R0, R1 with CFL steps, flag bits) plus n_steps / C checkpoints of 24 bytes
@@ -1662,7 +1663,13 @@ int vg_adj_forward(vg_ctx *c, int64_t n_steps, double dt, int64_t checkpoint_eve
                                  : std::max<int64_t>(1, std::llround(std::sqrt((double)n_steps * ckpt_bytes / rec_bytes)));
     int64_t nck = (n_steps + C - 1) / C;
     size_t bytes = 8 * 3 * (size_t)c->hm.nc;
-    for (int64_t k = 0; k < nck; k++) {
+    // a run of the last one's shape takes over its checkpoints and its room for recordings
+    // (allocating and freeing 0.45 GB and 20 checkpoints took 1.3 of a 40-step run's 6.3 ms)
+    const bool same = c->adj_n == n_steps && c->adj_every == C && (c->adj_dt > 0.0) == (dt > 0.0) &&
+                      (int64_t)c->ckpt.size() == nck && !checkpoint_every == (c->rec.base != nullptr);
+    if (!same) free_adjoint(c);
+    c->adj_n = 0;
+    for (int64_t k = 0; !same && k < nck; k++) {
         void *p = nullptr;
         int rc = dmalloc(c, &p, bytes);
         if (rc) { free_adjoint(c); return rc; }
@@ -1671,10 +1678,14 @@ int vg_adj_forward(vg_ctx *c, int64_t n_steps, double dt, int64_t checkpoint_eve
     double *dts_dev = nullptr;
     if (dmalloc(c, (void **)&dts_dev, 8 * (size_t)n_steps)) { free_adjoint(c); return VG_ENOMEM; }
     // With the segment length left to the library a run records its steps at once where
-    // they fit (50k triangles, 40 CFL steps, 0.45 GB: 16.8 ms forward and back against 22.0
+    // they fit (50k triangles, 40 CFL steps, 0.45 GB: 15.8 ms forward and back against 20.7
     // with the steps recomputed; recording costs a step 5 us of 120); a moving
     // bed's and a profiled run recompute them.
-    if (!checkpoint_every && !c->bed_on && !c->profile) keep_recordings(c, n_steps, !(dt > 0.0));
+    c->rec.valid = false;
+    if (!checkpoint_every && !c->bed_on && !c->profile) {
+        if (c->rec.base) c->rec.valid = true;
+        else keep_recordings(c, n_steps, !(dt > 0.0));
+    }
     vg_params saved = c->prm;
     const LaunchCfg saved_cfg1 = c->cfg1, saved_cfg2 = c->cfg2;
     c->prm.dt_fixed = dt;               // 0: the CFL rule of every step
@@ -1696,7 +1707,7 @@ int vg_adj_forward(vg_ctx *c, int64_t n_steps, double dt, int64_t checkpoint_eve
     c->rec_t.clear();
     c->rec_eta.clear();
     if (!rc) rc = record_now(c);
-    const bool keep = c->rec.base != nullptr;
+    const bool keep = c->rec.valid;
     if (!rc && keep) {
         cudaError_t e = cudaMemcpyAsync(c->rec.w, c->w[c->cur], bytes, cudaMemcpyDeviceToDevice, c->stream);
         if (e != cudaSuccess) rc = cuda_fail(c, e, "first state copy");
@@ -1790,7 +1801,7 @@ int vg_adj_backward(vg_ctx *c, const double *dJ_deta, double *dJ_dH0, double *dJ
     const int nc = (int)c->hm.nc, G = c->n_gauges;
     const size_t w3 = 3 * (size_t)nc;
     const bool binomial = c->adj_slots > 0;
-    const bool kept = c->rec.base != nullptr && !binomial;   // the forward run's own recordings
+    const bool kept = c->rec.valid && !binomial;   // the forward run's own recordings
     const int64_t RC = binomial ? 1 : C;    // steps whose recordings are held at once
     // scratch (freed at the end)
     std::vector<void *> bufs;
