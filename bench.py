@@ -224,7 +224,7 @@ def code_digest(texts) -> str:
 
 def kernel_source_sha() -> str:
     texts = []
-    for f in ("step_kernels.cuh", "step_f32.cu", "step_f64.cu", "step_f64_fast.cu"):
+    for f in ("step_kernels.cuh", "block_f32.cuh", "exact_div.cuh", "step_f32.cu", "step_f64.cu", "step_f64_fast.cu"):
         with open(os.path.join(ROOT, "paper_2002_04889_gb300", "csrc", f)) as fh:
             texts.append(fh.read())
     return code_digest(texts)
