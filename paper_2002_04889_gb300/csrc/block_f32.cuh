@@ -185,13 +185,13 @@ __device__ __forceinline__ void face_terms(float g, float half_g, float hthr, fl
 {
     const float HfL = sub_(L.x, L.y);
     const float rL = HfL > hthr ? rcp_approx(HfL) : 0.f;
-    const float unL = mul_(fma_(L.z, nx, mul_(L.w, ny)), rL);
+    const float unL = mul_(fma_(L.w, ny, mul_(L.z, nx)), rL);
     const float utL = mul_(fma_(L.w, nx, -mul_(L.z, ny)), rL);
     float HsL, HsR, unR, utR, ds;
     if (bnd == 0) {
         const float HfR = sub_(R.x, R.y);
         const float rR = HfR > hthr ? rcp_approx(HfR) : 0.f;
-        unR = mul_(fma_(R.z, nx, mul_(R.w, ny)), rR);
+        unR = mul_(fma_(R.w, ny, mul_(R.z, nx)), rR);
         utR = mul_(fma_(R.w, nx, -mul_(R.z, ny)), rR);
         const float zs = fmaxf(L.y, R.y);
         HsL = fmaxf(0.f, sub_(L.x, zs));
@@ -258,8 +258,8 @@ __device__ __forceinline__ void face_terms(float g, float half_g, float hthr, fl
 __device__ __forceinline__ void limited(const float4 m0, const float4 m1, float q, float q0, float q1, float q2, float D[3])
 {
     const float d0 = sub_(q0, q), d1 = sub_(q1, q), d2 = sub_(q2, q);
-    D[0] = fma_(m0.z, d2, fma_(m0.y, d1, mul_(m0.x, d0)));
-    D[1] = fma_(m1.y, d2, fma_(m1.x, d1, mul_(m0.w, d0)));
+    D[0] = fma_(m0.x, d0, fma_(m0.y, d1, mul_(m0.z, d2)));
+    D[1] = fma_(m0.w, d0, fma_(m1.x, d1, mul_(m1.y, d2)));
     D[2] = -add_(D[0], D[1]);
     const float up = fmaxf(fmaxf(d0, d1), fmaxf(d2, 0.f)), dn = -fminf(fminf(d0, d1), fminf(d2, 0.f));
     const float P = fabsf(fmaxf(fmaxf(D[0], D[1]), D[2])), M = fabsf(fminf(fminf(D[0], D[1]), D[2]));   // never -0
@@ -509,8 +509,8 @@ __device__ __forceinline__ void process_block(const KArgs<float> &a, const int b
         const float2 own = m.sS[tid];
         const float area = m.sArea[tid];
         const float aH = add_(add_(t0.x, t1.x), t2.x);
-        const float aHu = add_(add_(add_(t0.y, t1.y), t2.y), own.x);
-        const float aHv = add_(add_(add_(t0.z, t1.z), t2.z), own.y);
+        const float aHu = add_(add_(add_(own.x, t0.y), t1.y), t2.y);
+        const float aHv = add_(add_(add_(own.y, t0.z), t1.z), t2.z);
         const float am = STAGE == 1 ? fmaxf(fmaxf(t0.w, t1.w), t2.w) : 0.f;
         const float ra = -rcp_approx(area);
         finish_cell<STAGE, SOA>(a, c0 + tid, m.sW + tid, mul_(aH, ra), mul_(aHu, ra), mul_(aHv, ra), am, area, dt,
