@@ -221,8 +221,10 @@ int vg_get_gauge_cells(vg_ctx *ctx, int32_t *cells);
  * each comes from the CFL rule on the stage-1 wave speeds,
  *   dt = cfl * min_K |K| / (3 max_f l_f a_f),
  * unless params.dt_fixed > 0, clamped by dt_max and t_end.  The whole loop
- * stays on the device (CUDA-graph replays); the call synchronises once at the
- * end and returns VG_ENONFINITE / VG_ENEGDEPTH if a step went wrong.
+ * stays on the device (many steps per launch on small and medium FP32 meshes,
+ * CUDA-graph replays otherwise); the call synchronises once at the end and
+ * returns VG_ENONFINITE / VG_ENEGDEPTH if a step went wrong, VG_ETIMEOUT if a
+ * launch's thread blocks lost one another (the state is then undefined).
  */
 int vg_step(vg_ctx *ctx, int64_t n_steps);
 

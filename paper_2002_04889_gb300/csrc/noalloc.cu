@@ -19,6 +19,8 @@
 //  * all calls share the array, which keeps the last call's contents; each call
 //    clears what must start fresh (the step scalars) before its kernels run, and
 //    calls that overlap on the GPU (other streams, other threads) race on it;
+//  * FP32 meshes of a few rounds of blocks take their step in one launch
+//    (steps_kernel, step_f32.cu), which uses the array for R0 only;
 //  * the device address of the array is looked up once per device (with that
 //    device current) at that set-up and cached, so a step loads nothing.
 #include <cuda_runtime.h>
