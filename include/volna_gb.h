@@ -225,6 +225,8 @@ int vg_get_gauge_cells(vg_ctx *ctx, int32_t *cells);
  * CUDA-graph replays otherwise); the call synchronises once at the end and
  * returns VG_ENONFINITE / VG_ENEGDEPTH if a step went wrong, VG_ETIMEOUT if a
  * launch's thread blocks lost one another (the state is then undefined).
+ * A launch of many steps starts when the GPU has room for all of its thread
+ * blocks at once (kernels of other streams that are running finish first).
  */
 int vg_step(vg_ctx *ctx, int64_t n_steps);
 
