@@ -89,10 +89,12 @@ struct vg_ctx {
     // moving bed (vg_set_bed_motion): device copies while it is on
     std::vector<double> depth_v;
     bool bed_on = false;
+    bool moving = false;                // FP32: the bed still moves, so the stages take that form (set_moving)
+    void *normals = nullptr;            // FP32, while moving: the faces' unit normals
     int64_t n_open = 0;                 // open or absorbing boundary faces (vg_set_boundary)
     int32_t *bed_vtx = nullptr;
     double *bed_depth0 = nullptr, *bed_uplift = nullptr, *bed_onset = nullptr;
-    double bed_rise = 0.0;
+    double bed_rise = 0.0, bed_last = -INFINITY;   // the rise time, and the last onset of a vertex with an uplift
 
     LaunchCfg cfg1{}, cfg2{}, cfgn{};   // stages 1 and 2, and the multi-step kernel (grid 0: none)
     cudaGraphExec_t graph2 = nullptr;
@@ -193,7 +195,8 @@ void free_mesh(vg_ctx *c)
     dfree(c->adj_faces); c->n_adj_faces = 0;
     dfree(c->gauge_cells); dfree(c->ring_t); dfree(c->ring_eta); dfree(c->staging);
     dfree(c->bed_vtx); dfree(c->bed_depth0); dfree(c->bed_uplift); dfree(c->bed_onset);
-    c->bed_on = false;
+    c->bed_on = c->moving = false;
+    dfree(c->normals);
     c->n_open = 0;
     c->depth_v.clear();
     c->dev_bytes = 0;
@@ -237,7 +240,9 @@ BlockShape block_shape(const vg_ctx *c, const vg_params &p, int64_t nc)
         return s;
     }
     const int64_t sms = c->sms;
-    if (c->precision == 64 && !p.fp64_literal) {
+    if (c->moving) {                                         // its rounding depends on the partition too
+        if (nc <= 2 * 256 * sms) s.threads = 512;
+    } else if (c->precision == 64 && !p.fp64_literal) {
         if (nc <= 256 * sms) s.threads = 512;                // one block per SM
     } else if (c->precision == 64) {
         if (nc <= 64 * sms) s = {64, 128};                   // one block of 64 per SM
@@ -277,6 +282,8 @@ DevPtrs dev_ptrs(const vg_ctx *c)
     d.codes = c->codes;
     d.ring_codes = c->ring_codes;
     d.fr = c->fr;
+    d.normals = c->normals;
+    d.moving = c->moving;
     d.z = c->z;
     d.zf = c->zf;
     d.z64 = c->z64;
@@ -463,7 +470,8 @@ int upload_partition_f32(vg_ctx *c)
             const int nl = code >> 2, nf = code & 3;
             const uint32_t sr = (uint32_t)(nf * L1 + nl);
             const int64_t j = m.nbr[f * nc + k];
-            if (j < k) inner.push_back({sr | (sl << 16), j, nf});     // the left cell: the lower internal id
+            // the left cell: the lower internal id; on a moving bed the owned one
+            if (j < k && !c->moving) inner.push_back({sr | (sl << 16), j, nf});
             else inner.push_back({sl | (sr << 16), k, f});
         }
         order_for_banks(inner);
@@ -571,6 +579,24 @@ int upload_mesh_arrays(vg_ctx *c)
     VG_CUDA(c, cudaMemcpy(c->old_of_new, m.old_of_new.data(), 4 * m.nc, cudaMemcpyHostToDevice));
     VG_CUDA(c, cudaMemcpy(c->new_of_old, m.new_of_old.data(), 4 * m.nc, cudaMemcpyHostToDevice));
     return upload_partition(c);
+}
+
+// FP32: the unit normals of every cell's faces (a moving bed's wall ghosts).
+int upload_normals_f32(vg_ctx *c)
+{
+    const HostMesh &m = c->hm;
+    const size_t n = (size_t)m.nc;
+    std::vector<float> v(6 * n);
+#pragma omp parallel for
+    for (int64_t k = 0; k < m.nc; k++)
+        for (int f = 0; f < 3; f++) {
+            v[2 * (f * n + k)] = (float)m.geo[(GEO_NX + f) * n + k];
+            v[2 * (f * n + k) + 1] = (float)m.geo[(GEO_NY + f) * n + k];
+        }
+    int rc;
+    if (!c->normals && (rc = dmalloc(c, &c->normals, 4 * v.size()))) return rc;
+    VG_CUDA(c, cudaMemcpy(c->normals, v.data(), 4 * v.size(), cudaMemcpyHostToDevice));
+    return VG_OK;
 }
 
 size_t stage_smem(const vg_ctx *c)
@@ -1106,12 +1132,42 @@ static const void *mapped_view(const void *p)
     return a.type == cudaMemoryTypeHost ? a.devicePointer : nullptr;
 }
 
+// FP32: a context whose bed still moves from time t on takes the stage kernels' form of
+// a moving bed, with the partition and face records that go with it (block_f32.cuh); a
+// bed that has come to rest is a static one.
+static int set_moving(vg_ctx *c, double t)
+{
+    const bool rests = c->bed_rise > 0.0 ? t - c->bed_last >= c->bed_rise : t >= c->bed_last;
+    const bool on = c->precision == 32 && c->bed_on && !rests;
+    if (on == c->moving) return VG_OK;
+    VG_CUDA(c, cudaStreamSynchronize(c->stream));
+    c->moving = on;
+    c->graph_dirty = true;
+    int rc;
+    if (on && (rc = upload_normals_f32(c))) { c->moving = false; return rc; }
+    const int block = block_shape(c, c->prm, c->hm.nc).cells;
+    if (block != c->hm.block) {
+        if ((rc = partition_blocks(c->hm, block, c->err))) return rc;
+        if ((rc = fit_blocks(c))) return rc;
+    }
+    if ((rc = upload_partition(c))) return rc;
+    if (!on) {
+        dfree(c->normals);
+        c->dev_bytes -= 24 * c->hm.nc;
+    }
+    return configure_launch(c);
+}
+
 // Stores a state given in the original cell order.  host_order: one thread per
 // original cell, so the source may be pinned host memory read in place over the
 // CPU-GPU link; otherwise one thread per internal cell gathers from device arrays.
 static int set_state_impl(vg_ctx *c, const void *H, const void *Hu, const void *Hv, bool src_double, bool host_order,
                           double t)
 {
+    if (c->bed_on) {
+        int rc = set_moving(c, t);
+        if (rc) return rc;
+    }
     DevScalars s;
     reset_scalars_host(c, s, t);
     s.t_end = c->dev_t_end = c->prm.t_end;
@@ -1562,6 +1618,9 @@ int vg_set_bed_motion(vg_ctx *c, const double *uplift_v, const double *onset_v, 
         VG_CUDA(c, cudaMemcpy(c->bed_uplift, uplift_v, 8 * nv, cudaMemcpyHostToDevice));
         VG_CUDA(c, cudaMemcpy(c->bed_onset, onset_v, 8 * nv, cudaMemcpyHostToDevice));
         c->bed_rise = rise;
+        c->bed_last = -INFINITY;
+        for (int64_t v = 0; v < nv; v++)
+            if (uplift_v[v] != 0.0) c->bed_last = std::max(c->bed_last, onset_v[v]);
     } else {
         // back to the static bed: zero uplift evaluated once, then the motion is off
         VG_CUDA(c, cudaMemset(c->bed_uplift, 0, 8 * nv));
@@ -1580,7 +1639,7 @@ int vg_set_bed_motion(vg_ctx *c, const double *uplift_v, const double *onset_v, 
         dfree(c->bed_vtx); dfree(c->bed_depth0); dfree(c->bed_uplift); dfree(c->bed_onset);
     }
     c->graph_dirty = true;
-    return VG_OK;
+    return set_moving(c, sc.t);
 }
 
 // Room for the recordings of n steps, where that is at most 1/32 of the device's memory

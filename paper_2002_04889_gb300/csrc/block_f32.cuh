@@ -28,6 +28,7 @@
 //   fr      float4 per owned face of a block: unit normal, length, and the face's two
 //           shared-memory slots; the face's left cell is the one of lower internal
 //           id whatever block computes it, so results do not depend on the partition
+//           (on a moving bed, face_terms_by_side, they do)
 // with M_fj = w_j . (x_f - x_K) in FP64 on the host: D_f = sum_j M_fj (q_j - q_K) is
 // grad q . (x_f - x_K) for the least-squares gradient, and since the face midpoints
 // average to the centroid D_2 = -(D_0 + D_1), dz_2 = -(dz_0 + dz_1).
@@ -49,6 +50,7 @@ struct KArgs<float> {
     const uint2 *ring_codes;  // beside halo_ids: codes of the ring-1 cells
     const int32_t *fr_ptr;  // [nblocks + 1] into fr
     const float4 *fr;       // owned faces of each block, interior faces first
+    const float2 *normals;  // moving bed: [3][nc] unit normals of every cell's faces
     int max_faces;          // owned faces of a block at most
     const float *w_soa;     // SOA kernels: w^n [3][nc] and w^{n+1} [3][nc] of the caller, the bed [nc]
     float *wout_soa;
@@ -269,6 +271,119 @@ __device__ __forceinline__ void limited(const float4 m0, const float4 m1, float 
     D[2] = fma_(alpha, D[2], q);
 }
 
+// ---------------------------------------------------------------------------
+// The form of a moving bed: pressure terms per face side, the limiter's ratios one by
+// one, a face's left cell the one whose block computes it.  The same scheme; only the
+// roundings differ.  A moving bed keeps them because its update is no continuous
+// function of the state: the free surface of a moving cell is rounded to the bed's grid
+// (2.4e-4 m over 4000 m of water) in every step, so that one ulp of dt, which another
+// order of these sums changes now and then, decides many of those roundings: momenta
+// off by 3e-5 of their norm and 2e-3 at most (298k cells, 40 steps; 2 of 24 sources).
+// With this form a run repeats those of the kernels before the 16-byte states bit for
+// bit, as static beds, which have no such switch, need not.  The expressions are left
+// to the compiler's contraction, as they were there.  Not slower: 298k cells, 40 steps
+// 1.76 ms, 1.79 to 1.81 with the form of a static bed (its two kernels spill a little,
+// these do not).
+// ---------------------------------------------------------------------------
+
+// Limited face values of one variable from the cell's value q and the neighbours' qn.
+__device__ __forceinline__ void limited_by_face(const float4 m0, const float4 m1, float q, float qn0, float qn1, float qn2,
+                                                float face[3])
+{
+    const float d0 = qn0 - q, d1 = qn1 - q, d2 = qn2 - q;
+    float D[3];
+    D[0] = m0.x * d0 + m0.y * d1 + m0.z * d2;
+    D[1] = m0.w * d0 + m1.x * d1 + m1.y * d2;
+    D[2] = -(D[0] + D[1]);
+    const float up = fmaxf(fmaxf(fmaxf(q, qn0), qn1), qn2) - q, dn = q - fminf(fminf(fminf(q, qn0), qn1), qn2);
+    float alpha = 1.f;
+#pragma unroll
+    for (int f = 0; f < 3; f++) alpha = fminf(alpha, (D[f] > 0.f ? up : dn) * rcp_approx(fabsf(D[f])));
+#pragma unroll
+    for (int f = 0; f < 3; f++) face[f] = q + alpha * D[f];
+}
+
+// Flux and side terms of one face, arguments as face_terms and the cells' own eta:
+//   Q_L = g/2 [(eta_fL - eta_L)(H_fL + H_L) - H*_L d*],
+//   Q_R = g/2 [(eta_fR - eta_R)(H_fR + H_R) + H*_R d*].
+__device__ __forceinline__ void face_terms_by_side(float g, float half_g, float hthr, float4 L, float eL, float4 R, float eR,
+                                                   float nx, float ny, float len, int bnd, float4 &tL, float4 &tR)
+{
+    const float efL = L.x, zL = L.y, HufL = L.z, HvfL = L.w;
+    float efR = R.x, zR = R.y;
+    const float HufR = R.z, HvfR = R.w;
+    float HfL = efL - zL;
+    float uL = 0.f, vL = 0.f;
+    if (HfL > hthr) { const float r = rcp_approx(HfL); uL = HufL * r; vL = HvfL * r; }
+    float unL = uL * nx + vL * ny;
+    float utL = -uL * ny + vL * nx;
+    float HsL, HsR, unR, utR, ds, HfR;
+    if (bnd == 3) {
+        HsL = fmaxf(0.f, HfL);
+        const float cL = sqrtf(g * HsL), c0 = sqrtf(g * fmaxf(0.f, -zL));
+        const float Rp = unL + 2.f * cL, Rm = -2.f * c0;
+        const float cg = fmaxf(0.f, 0.25f * (Rp - Rm));
+        unR = 0.5f * (Rp + Rm);
+        HsR = cg * cg / g;
+        utR = utL;
+        ds = HsL - HsR;
+        HfR = HsR; efR = zL + HsR; eR = efR; zR = zL;
+    } else if (bnd) {
+        HsL = fmaxf(0.f, HfL);
+        HsR = HsL;
+        unR = bnd == 2 ? unL : -unL;
+        utR = utL;
+        ds = 0.f;
+        HfR = HfL; efR = efL; eR = eL; zR = zL;
+    } else {
+        HfR = efR - zR;
+        float uR = 0.f, vR = 0.f;
+        if (HfR > hthr) { const float r = rcp_approx(HfR); uR = HufR * r; vR = HvfR * r; }
+        unR = uR * nx + vR * ny;
+        utR = -uR * ny + vR * nx;
+        float zs = fmaxf(zL, zR);
+        HsL = fmaxf(0.f, efL - zs);
+        HsR = fmaxf(0.f, efR - zs);
+        ds = (HsL > 0.f && HsR > 0.f) ? efL - efR : HsL - HsR;
+    }
+    float F[3], amax;
+    if (HsL == 0.f && HsR == 0.f) {
+        F[0] = 0.f; F[1] = 0.f; F[2] = 0.f;
+        amax = 0.f;
+    } else {
+        float cL = sqrtf(g * HsL), cR = sqrtf(g * HsR);
+        float sL, sR;
+        if (HsL == 0.f) {
+            sL = unR - 2.f * cR;
+            sR = unR + cR;
+        } else if (HsR == 0.f) {
+            sL = unL - cL;
+            sR = unL + 2.f * cL;
+        } else {
+            float us = 0.5f * (unL + unR) + (cL - cR);
+            float cs = 0.5f * (cL + cR) - 0.25f * (unR - unL);
+            sL = fminf(unL - cL, us - cs);
+            sR = fmaxf(us + cs, unR + cR);
+        }
+        float qL = HsL * unL, qR = HsR * unR;
+        float FL0 = qL, FL1 = qL * unL + half_g * HsL * ds, FL2 = qL * utL;
+        float FR0 = qR, FR1 = qR * unR - half_g * HsR * ds, FR2 = qR * utR;
+        const float a = fminf(sL, 0.f), b = fmaxf(sR, 0.f);
+        const float rden = rcp_approx(b - a), ab = a * b;
+        F[0] = ((b * FL0 - a * FR0) - ab * ds) * rden;
+        F[1] = ((b * FL1 - a * FR1) + ab * (qR - qL)) * rden;
+        F[2] = ((b * FL2 - a * FR2) + ab * (HsR * utR - HsL * utL)) * rden;
+        amax = fmaxf(fabsf(sL), fabsf(sR));
+    }
+    const float P0 = F[0], P1 = F[1] * nx - F[2] * ny, P2 = F[1] * ny + F[2] * nx;
+    float HL = eL - zL, HR = eR - zR;
+    const float QL = half_g * ((efL - eL) * (HfL + HL) - HsL * ds);
+    const float QR = half_g * ((efR - eR) * (HfR + HR) + HsR * ds);
+    const float t0 = len * P0, la = len * amax;
+    tL = make_float4(t0, len * (P1 + QL * nx), len * (P2 + QL * ny), la);
+    tR = make_float4(-t0, -(len * (P1 + QR * nx)), -(len * (P2 + QR * ny)), la);
+}
+
 // The wall ghost's momentum for a wall face of normal N (any length): m - 2 (m.n) n.
 __device__ __forceinline__ void wall_ghost(float4 &q, float Nx, float Ny)
 {
@@ -349,7 +464,7 @@ __device__ __forceinline__ Smem smem_of(const KArgs<float> &a, unsigned char *ra
 // three in a row (8.7k cells 9.8 -> 9.0 us a step, 99k 14.5 -> 13.5; 32 coast
 // scenarios 215 -> 210).
 enum { KEEP_NOTHING, KEEP_SCENARIOS, KEEP_STEPS };
-template <int STAGE, bool SOA, int KEEP>
+template <int STAGE, bool SOA, int KEEP, bool MOVING = false>
 __device__ __forceinline__ void process_block(const KArgs<float> &a, const int b, const float dt,
                                               unsigned char *smem_raw, float &my_min, long long &my_neg, bool &bad,
                                               bool &loaded)
@@ -432,7 +547,38 @@ __device__ __forceinline__ void process_block(const KArgs<float> &a, const int b
         // the slots' first and second halves, stored as they come: (eta_f, z_f), (Hu_f, Hv_f)
         float2 *f0 = reinterpret_cast<float2 *>(m.sF + l), *f1 = f0 + 2 * m.L1, *f2 = f1 + 2 * m.L1;
         bool recon = false;
-        if (a.order == 2 && q.x - q.w > a.hthr) {
+        if (MOVING && a.order == 2 && q.x - q.w > a.hthr) {
+            const int gid = l < B ? c0 + l : a.halo_ids[h0 + (l - B)];
+            const uint2 c = l < B ? a.codes[gid] : a.ring_codes[h0 + (l - B)];
+            const float4 m0 = a.recA[2 * gid], m1 = a.recA[2 * gid + 1];
+            const float4 qn[3] = {m.sW[c.x & 0xffffu], m.sW[c.x >> 16], m.sW[c.y & 0xffffu]};
+            recon = qn[0].x - qn[0].w > a.hthr && qn[1].x - qn[1].w > a.hthr && qn[2].x - qn[2].w > a.hthr;
+            if (recon) {
+                float un[3], vn[3], e[3], u[3], v[3];
+#pragma unroll
+                for (int f = 0; f < 3; f++) {
+                    un[f] = qn[f].y;
+                    vn[f] = qn[f].z;
+                    if ((c.y >> (16 + f)) & 1) {
+                        const float2 n = a.normals[f * (size_t)a.nc + gid];
+                        const float mn = q.y * n.x + q.z * n.y;
+                        un[f] = q.y - 2.f * mn * n.x;
+                        vn[f] = q.z - 2.f * mn * n.y;
+                    }
+                }
+                limited_by_face(m0, m1, q.x, qn[0].x, qn[1].x, qn[2].x, e);
+                limited_by_face(m0, m1, q.y, un[0], un[1], un[2], u);
+                limited_by_face(m0, m1, q.z, vn[0], vn[1], vn[2], v);
+                const float z0 = q.w + m1.z, z1 = q.w + m1.w, z2 = q.w - (m1.z + m1.w);
+                recon = e[0] - z0 > a.hthr && e[1] - z1 > a.hthr && e[2] - z2 > a.hthr;
+                if (recon) {
+                    f0[0] = make_float2(e[0], z0); f0[1] = make_float2(u[0], v[0]);
+                    f1[0] = make_float2(e[1], z1); f1[1] = make_float2(u[1], v[1]);
+                    f2[0] = make_float2(e[2], z2); f2[1] = make_float2(u[2], v[2]);
+                }
+            }
+        }
+        if (!MOVING && a.order == 2 && q.x - q.w > a.hthr) {
             const int gid = l < B ? c0 + l : KEEP ? m.sHid[l - B] : a.halo_ids[h0 + (l - B)];
             const uint2 c = l < B ? a.codes[gid] : a.ring_codes[h0 + (l - B)];
             // the records in flight together, before the neighbours' states decide on them
@@ -481,7 +627,7 @@ __device__ __forceinline__ void process_block(const KArgs<float> &a, const int b
             m.sF[l] = v;
             m.sF[m.L1 + l] = v;
             m.sF[2 * m.L1 + l] = v;
-            if (l < B) m.sS[l] = make_float2(0.f, 0.f);
+            if (!MOVING && l < B) m.sS[l] = make_float2(0.f, 0.f);
         }
     }
     cp_wait();
@@ -497,7 +643,12 @@ __device__ __forceinline__ void process_block(const KArgs<float> &a, const int b
         const float4 L = m.sF[sl];
         const float4 R = bnd ? L : m.sF[sr];
         float4 tL, tR;
-        face_terms(a.g, a.half_g, a.hthr, L, R, r.x, r.y, r.z, bnd, tL, tR);
+        if constexpr (MOVING) {
+            auto own_eta = [&](unsigned slot) { return m.sW[slot >= 2 * m.L1 ? slot - 2 * m.L1 : slot >= m.L1 ? slot - m.L1 : slot].x; };
+            const float eL = own_eta(sl), eR = bnd ? eL : own_eta(sr);
+            face_terms_by_side(a.g, a.half_g, a.hthr, L, eL, R, eR, r.x, r.y, r.z, bnd, tL, tR);
+        } else
+            face_terms(a.g, a.half_g, a.hthr, L, R, r.x, r.y, r.z, bnd, tL, tR);
         m.sF[sl] = tL;
         if (!bnd) m.sF[sr] = tR;
     }
@@ -506,8 +657,15 @@ __device__ __forceinline__ void process_block(const KArgs<float> &a, const int b
     // D: residual R_K = -(1/|K|) sum_f (side terms), faces in local order
     if (tid < ncell) {
         const float4 t0 = m.sF[tid], t1 = m.sF[m.L1 + tid], t2 = m.sF[2 * m.L1 + tid];
-        const float2 own = m.sS[tid];
         const float area = m.sArea[tid];
+        if constexpr (MOVING) {
+            const float aH = t0.x + t1.x + t2.x, aHu = t0.y + t1.y + t2.y, aHv = t0.z + t1.z + t2.z;
+            const float am = STAGE == 1 ? fmaxf(fmaxf(t0.w, t1.w), t2.w) : 0.f;
+            finish_cell<STAGE, SOA>(a, c0 + tid, m.sW + tid, -aH / area, -aHu / area, -aHv / area, am, area, dt, my_min, my_neg,
+                                    bad);
+            return;
+        }
+        const float2 own = m.sS[tid];
         const float aH = add_(add_(t0.x, t1.x), t2.x);
         const float aHu = add_(add_(add_(own.x, t0.y), t1.y), t2.y);
         const float aHv = add_(add_(add_(own.y, t0.z), t1.z), t2.z);

@@ -853,21 +853,26 @@ template <> struct StageMinCtas<double, 256> { static constexpr int value = 2; }
 template <typename real> struct BatchMinCtas { static constexpr int value = 1; };
 template <> struct BatchMinCtas<float> { static constexpr int value = 4; };
 
+// FP32 instances: the context's states, the caller's [3][nc] arrays (the no-allocation
+// step), or the context's on a moving bed (block_f32.cuh has that form's arithmetic).
+enum { OWN, CALLERS, ON_MOVING_BED };
+
 // One block of a single-scenario stage (BATCH = false) or of a batch's scenario.
 // FP64: the single-scenario kernels leave a dry block early, the batched ones let
 // phase B write zero terms and keep the ids (see process_block).
-template <int STAGE, bool FAST, bool BATCH, bool SOA>
+template <int STAGE, bool FAST, bool BATCH, int STATE>
 __device__ __forceinline__ void run_block(const KArgs<double> &a, int b, double dt, unsigned char *smem, int &qcount,
                                           double &my_min, long long &my_neg, bool &bad, bool &)
 {
     process_block<double, STAGE, BATCH ? 2 : 1, BATCH || STAGE == 2, BATCH, FAST>(a, b, dt, smem, qcount, my_min, my_neg,
                                                                                   bad);
 }
-template <int STAGE, bool FAST, bool BATCH, bool SOA>
+template <int STAGE, bool FAST, bool BATCH, int STATE>
 __device__ __forceinline__ void run_block(const KArgs<float> &a, int b, float dt, unsigned char *smem, int &,
                                           float &my_min, long long &my_neg, bool &bad, bool &loaded)
 {
-    process_block<STAGE, SOA, BATCH ? KEEP_SCENARIOS : KEEP_NOTHING>(a, b, dt, smem, my_min, my_neg, bad, loaded);
+    process_block<STAGE, STATE == CALLERS, BATCH ? KEEP_SCENARIOS : KEEP_NOTHING, STATE == ON_MOVING_BED>(a, b, dt, smem, my_min,
+                                                                                                        my_neg, bad, loaded);
 }
 
 // w^{n+1} = w^n, bit for bit, by every thread of the launch.
@@ -885,8 +890,7 @@ __device__ __forceinline__ void copy_state(const KArgs<float> &a, int64_t i0, in
         for (int64_t i = i0; i < a.nc; i += stride) a.wout[i] = a.w[i];
 }
 
-// SOA (FP32): the states are the caller's [3][nc] arrays (the no-allocation step).
-template <typename real, int STAGE, int MAXT, bool FAST = false, bool SOA = false>
+template <typename real, int STAGE, int MAXT, bool FAST = false, int STATE = OWN>
 __global__ void __launch_bounds__(MAXT, StageMinCtas<real, MAXT>::value) stage_kernel(const KArgs<real> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -903,7 +907,7 @@ __global__ void __launch_bounds__(MAXT, StageMinCtas<real, MAXT>::value) stage_k
     // would flush the smallest FP32 values to zero), as the batched kernels do
     if (finished(a.sc->t_end, a.sc)) {
         if (STAGE == 2)
-            copy_state<SOA>(a, blockIdx.x * (int64_t)blockDim.x + tid, (int64_t)gridDim.x * blockDim.x);
+            copy_state<STATE == CALLERS>(a, blockIdx.x * (int64_t)blockDim.x + tid, (int64_t)gridDim.x * blockDim.x);
         return;
     }
 
@@ -919,7 +923,7 @@ __global__ void __launch_bounds__(MAXT, StageMinCtas<real, MAXT>::value) stage_k
     int parity = 0;
     for (int b = blockIdx.x; b < a.nblocks; b += gridDim.x, parity ^= 1) {
         bool loaded = false;
-        run_block<STAGE, FAST, false, SOA>(a, b, dt, smem_raw, qcount[parity], my_min, my_neg, bad, loaded);
+        run_block<STAGE, FAST, false, STATE>(a, b, dt, smem_raw, qcount[parity], my_min, my_neg, bad, loaded);
     }
 
     // CTA-level reductions, then one atomic per CTA
@@ -1172,7 +1176,7 @@ __global__ void __launch_bounds__(256, (BatchMinCtas<real>::value)) batch_stage_
             if (tid == 0 && after < n_scen) fill(after, slot2);
             const KArgs<real> &a = *reinterpret_cast<const KArgs<real> *>(s_args[slot]);
             real mn = real_inf<real>();
-            run_block<STAGE, FAST, true, false>(a, b, s_dt[e0 + s], smem_raw, qcount[parity], mn, my_neg, bad, loaded);
+            run_block<STAGE, FAST, true, OWN>(a, b, s_dt[e0 + s], smem_raw, qcount[parity], mn, my_neg, bad, loaded);
             parity ^= 1;
             if (STAGE == 1) {
                 unsigned long long bits = warp_min_bits<real>(mn);
@@ -1313,6 +1317,7 @@ inline KArgs<float> make_args<float>(const DevPtrs &d, const StepParams &p, cons
     a.ring_codes = static_cast<const uint2 *>(d.ring_codes);
     a.fr_ptr = d.fq_ptr;
     a.fr = static_cast<const float4 *>(d.fr);
+    a.normals = static_cast<const float2 *>(d.normals);
     a.max_faces = d.max_faces;
     a.R0 = static_cast<float4 *>(d.R0);
     if (soa) {
@@ -1327,14 +1332,14 @@ inline KArgs<float> make_args<float>(const DevPtrs &d, const StepParams &p, cons
 
 // Kernel instance for a launch: the register budget follows the thread count
 // (launch bounds 256 or 512).
-template <typename real, bool FAST = false, bool SOA = false>
+template <typename real, bool FAST = false, int STATE = OWN>
 void *stage_kernel_ptr(int stage, int threads)
 {
     if (threads <= 256)
-        return stage == 1 ? (void *)stage_kernel<real, 1, 256, FAST, SOA> : (void *)stage_kernel<real, 2, 256, FAST, SOA>;
+        return stage == 1 ? (void *)stage_kernel<real, 1, 256, FAST, STATE> : (void *)stage_kernel<real, 2, 256, FAST, STATE>;
     if (threads <= 384)
-        return stage == 1 ? (void *)stage_kernel<real, 1, 384, FAST, SOA> : (void *)stage_kernel<real, 2, 384, FAST, SOA>;
-    return stage == 1 ? (void *)stage_kernel<real, 1, 512, FAST, SOA> : (void *)stage_kernel<real, 2, 512, FAST, SOA>;
+        return stage == 1 ? (void *)stage_kernel<real, 1, 384, FAST, STATE> : (void *)stage_kernel<real, 2, 384, FAST, STATE>;
+    return stage == 1 ? (void *)stage_kernel<real, 1, 512, FAST, STATE> : (void *)stage_kernel<real, 2, 512, FAST, STATE>;
 }
 
 // The dynamic shared memory limit is an attribute of the kernel function, shared
@@ -1355,6 +1360,8 @@ int stage_config(const DevPtrs &d, int stage, LaunchCfg &cfg)
 {
     cfg.smem = stage_smem_bytes<real>(d.block, d.max_halo, d.max_ring1, d.max_faces);
     const void *kern = stage_kernel_ptr<real, FAST>(stage, d.threads);
+    if constexpr (std::is_same<real, float>::value)
+        if (d.moving) kern = stage_kernel_ptr<real, FAST, ON_MOVING_BED>(stage, d.threads);
     cudaError_t e = raise_smem_limit(kern, cfg.smem);
     if (e != cudaSuccess) return (int)e;
     int per_sm = 0;
@@ -1363,7 +1370,7 @@ int stage_config(const DevPtrs &d, int stage, LaunchCfg &cfg)
     if (per_sm < 1) return (int)cudaErrorInvalidConfiguration;
     if constexpr (std::is_same<real, float>::value) {
         // the no-allocation step's kernels, loaded here so that the step loads nothing
-        e = raise_smem_limit(stage_kernel_ptr<real, FAST, true>(stage, d.threads), cfg.smem);
+        e = raise_smem_limit(stage_kernel_ptr<real, FAST, CALLERS>(stage, d.threads), cfg.smem);
         if (e != cudaSuccess) return (int)e;
     }
     int dev = 0, sms = 0;
@@ -1375,13 +1382,13 @@ int stage_config(const DevPtrs &d, int stage, LaunchCfg &cfg)
     return 0;
 }
 
-template <typename real, bool FAST = false, bool SOA = false>
+template <typename real, bool FAST = false, int STATE = OWN>
 int launch_stage_args(const KArgs<real> &a, int threads, int stage, const LaunchCfg &c, cudaStream_t s)
 {
     void (*k)(const KArgs<real>);
-    if (threads <= 256) k = stage == 1 ? stage_kernel<real, 1, 256, FAST, SOA> : stage_kernel<real, 2, 256, FAST, SOA>;
-    else if (threads <= 384) k = stage == 1 ? stage_kernel<real, 1, 384, FAST, SOA> : stage_kernel<real, 2, 384, FAST, SOA>;
-    else k = stage == 1 ? stage_kernel<real, 1, 512, FAST, SOA> : stage_kernel<real, 2, 512, FAST, SOA>;
+    if (threads <= 256) k = stage == 1 ? stage_kernel<real, 1, 256, FAST, STATE> : stage_kernel<real, 2, 256, FAST, STATE>;
+    else if (threads <= 384) k = stage == 1 ? stage_kernel<real, 1, 384, FAST, STATE> : stage_kernel<real, 2, 384, FAST, STATE>;
+    else k = stage == 1 ? stage_kernel<real, 1, 512, FAST, STATE> : stage_kernel<real, 2, 512, FAST, STATE>;
     return (int)launch_after(k, c.grid, threads, c.smem, s, a);
 }
 
@@ -1400,6 +1407,8 @@ int launch_rk_unfused(const DevPtrs &d, const StepParams &p, int part, const voi
         a.R0 = static_cast<word *>(R1);
         a.wout = nullptr;
         a.cfl_min = 0;
+        if constexpr (std::is_same<real, float>::value)
+            if (d.moving) return launch_stage_args<real, FAST, ON_MOVING_BED>(a, d.threads, 1, c1, s);
         return launch_stage_args<real, FAST>(a, d.threads, 1, c1, s);
     }
     int dev = 0, sms = 0;
@@ -1419,9 +1428,11 @@ int launch_stage(const DevPtrs &d, const StepParams &p, int stage, const void *w
 {
     const KArgs<real> a = make_args<real>(d, p, w_in, w_out, soa);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if constexpr (std::is_same<real, float>::value)
-        if (soa) return launch_stage_args<real, FAST, true>(a, d.threads, stage, c, s);
-    return launch_stage_args<real, FAST, false>(a, d.threads, stage, c, s);
+    if constexpr (std::is_same<real, float>::value) {
+        if (soa) return launch_stage_args<real, FAST, CALLERS>(a, d.threads, stage, c, s);
+        if (d.moving) return launch_stage_args<real, FAST, ON_MOVING_BED>(a, d.threads, stage, c, s);
+    }
+    return launch_stage_args<real, FAST>(a, d.threads, stage, c, s);
 }
 
 template <typename real, bool FAST = false>

@@ -132,6 +132,8 @@ struct DevPtrs {
     const void *codes;      // FP32: [nc] four uint16, neighbours' local slots and wall bits
     const void *ring_codes; // FP32: the same beside halo_ids for ring-1 cells
     const void *fr;         // FP32: face records of every block's owned faces (fq_ptr)
+    const void *normals;    // FP32, moving bed: [3][nc] two floats, unit normals (else null)
+    int32_t moving;         // FP32: the bed still moves (block_f32.cuh: the form of a moving bed)
     const double *rarea;    // FP64: [nc] 1 / area, correctly rounded (FP32: null)
     const double *M64;      // FP64, contracted build: [9][nc] M_fj = w_j . (x_f - x_K) (else null)
     const void *z;          // [nc]
