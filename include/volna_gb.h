@@ -290,7 +290,10 @@ int vg_device_bytes(vg_ctx *ctx, int64_t *bytes);
  * the scratch array and leave the last call's contents in it; each call clears
  * the scalars it needs before its kernels run, but calls that overlap on the
  * GPU (other streams or host threads) race on the array.  Returns
- * VG_ENONFINITE or VG_ENEGDEPTH (with params.strict_positivity) like vg_step.
+ * VG_ENONFINITE or VG_ENEGDEPTH (with params.strict_positivity) like vg_step,
+ * and VG_ETIMEOUT if the thread blocks of a step in one launch (small and medium
+ * FP32 meshes) lost one another: w_out is then undefined, the context and later
+ * calls are not affected.
  */
 #define VG_NOALLOC_MAX_CELLS 262144
 int vg_step_noalloc(vg_ctx *ctx, const void *w_in, void *w_out, double t, double *dt_out);

@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 #include <functional>
 #include <new>
@@ -1373,6 +1374,7 @@ int vg_step(vg_ctx *c, int64_t n_steps)
             while (use_multi_step(c, left)) {
                 const int n = (int)std::min<int64_t>(left, 4096);     // tens of ms: others get their turn on the GPU
                 int e = launch_steps_f32(dev_ptrs(c), step_params(c), c->w[c->cur], c->w[1 - c->cur], n, c->cfgn, (void *)c->stream);
+                c->cfgn.max_polls = LaunchCfg{}.max_polls;
                 if (e == (int)cudaErrorCooperativeLaunchTooLarge) {   // a part of the GPU only (MPS): the graph
                     cudaGetLastError();
                     c->cfgn.grid = 0;
@@ -2228,6 +2230,7 @@ int vg_step_noalloc(vg_ctx *c, const void *w_in, void *w_out, double t, double *
         // cells: 23.0 us a call; four launches and a copy: 29.6)
         StepOutcome *out = reinterpret_cast<StepOutcome *>(c->pinned);
         e = launch_caller_step_f32(d, p, w_in, w_out, t, c->prm.t_end, out, c->cfgn, s);
+        c->cfgn.max_polls = LaunchCfg{}.max_polls;
         if (e == (int)cudaErrorCooperativeLaunchTooLarge) {
             cudaGetLastError();
             c->cfgn.grid = 0;
@@ -2262,6 +2265,22 @@ int vg_step_noalloc(vg_ctx *c, const void *w_in, void *w_out, double t, double *
     if (r.flags & FLAG_NONFINITE_DT) return fail(c, VG_ENONFINITE, "the time step is not finite");
     if (c->prm.strict_positivity && r.neg_count > 0)
         return fail(c, VG_ENEGDEPTH, "a stage produced a negative depth (" + std::to_string(r.neg_count) + " cells)");
+    return VG_OK;
+}
+
+// For tests (not in the public header): the next launch of many steps, or of a caller's
+// step, finds its barrier one arrival short and gives up after max_polls polls; later
+// launches find it as it was.  VG_ESTATE where the context has no such launch.
+int vg_debug_lose_arrival(vg_ctx *c, uint32_t max_polls)
+{
+    if (!c || max_polls < 1) return VG_EINVAL;
+    if (!c->has_mesh || c->cfgn.grid < 1) return fail(c, VG_ESTATE, "no launch of many steps");
+    DeviceGuard guard(c->device);
+    const unsigned one_short = ~0u;
+    VG_CUDA(c, cudaMemcpyAsync(reinterpret_cast<char *>(c->sc) + kBarrierAt + offsetof(StepsBarrier, arrived), &one_short,
+                               sizeof(one_short), cudaMemcpyHostToDevice, c->stream));
+    VG_CUDA(c, cudaStreamSynchronize(c->stream));
+    c->cfgn.max_polls = max_polls;
     return VG_OK;
 }
 

@@ -21,13 +21,15 @@ namespace vg {
 // (it has no more blocks than another) also keeps the counts and records the gauges,
 // while the others begin the next step: the state that it reads is next written behind
 // two more barriers.  dtmin3[i % 3] is step i's CFL minimum; the last CTA empties the
-// next step's between the two barriers of a step, when nobody uses it.
+// next step's between the two barriers of a step, when nobody uses it.  The last CTA to
+// leave empties all three and the barrier's counts, also when CTAs have given up (the
+// others may then still be in stage 1): a launch leaves nothing behind for the next.
 // ---------------------------------------------------------------------------
 
 // What a CTA wrote before it every CTA sees behind it.  Every thread must call it.
 // False when the others have not arrived after about a second: the launch is
 // cooperative, all its CTAs are resident, so this says that one of them has stopped.
-__device__ __forceinline__ bool grid_barrier(StepsBarrier *bar, unsigned &target)
+__device__ __forceinline__ bool grid_barrier(StepsBarrier *bar, unsigned &target, unsigned max_polls)
 {
     __shared__ int arrived;
     __syncthreads();
@@ -36,7 +38,7 @@ __device__ __forceinline__ bool grid_barrier(StepsBarrier *bar, unsigned &target
         atomicAdd(&bar->arrived, 1u);
         target += gridDim.x;
         int ok = 0;
-        for (unsigned polls = 0; polls < (1u << 20); polls++) {
+        for (unsigned polls = 0; polls < max_polls; polls++) {
             unsigned v;
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&bar->arrived) : "memory");
             if ((ok = (int)(v - target) >= 0)) break;
@@ -65,7 +67,7 @@ struct CallerStep {
 
 template <int MAXT, int MINCTAS, bool SOA>
 __global__ void __launch_bounds__(MAXT, MINCTAS) steps_kernel(const KArgs<float> args, StepsBarrier *bar, const Gauges gauges,
-                                                             int n_steps, const CallerStep caller)
+                                                             int n_steps, const CallerStep caller, unsigned max_polls)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ float red_min[32], s_dt;
@@ -106,7 +108,7 @@ __global__ void __launch_bounds__(MAXT, MINCTAS) steps_kernel(const KArgs<float>
             for (int w = 0; w < nwarps; w++) mn = smin(mn, red_min[w]);
             if (mn < real_inf<float>()) atomicMin(&sc->dtmin3[i % 3], min_bits(mn));
         }
-        if (!(ok = grid_barrier(bar, target))) break;
+        if (!(ok = grid_barrier(bar, target, max_polls))) break;
         if (tid == 0) {
             DevScalars v;
             v.t = s_t;
@@ -121,7 +123,7 @@ __global__ void __launch_bounds__(MAXT, MINCTAS) steps_kernel(const KArgs<float>
             if (!one_block) loaded = false;
             process_block<2, SOA, KEEP_STEPS>(a, b, dt, smem_raw, my_min, my_neg, bad, loaded);
         }
-        if (!(ok = grid_barrier(bar, target))) break;
+        if (!(ok = grid_barrier(bar, target, max_polls))) break;
         if (tid == 0) {
             if (!isfinite(dt_last)) flags |= FLAG_NONFINITE_DT;
             long long rec = -1;
@@ -163,19 +165,17 @@ __global__ void __launch_bounds__(MAXT, MINCTAS) steps_kernel(const KArgs<float>
         if (bad) flags |= FLAG_NONFINITE_STATE;
         if (neg) atomicAdd((unsigned long long *)(SOA ? &bar->neg_count : &sc->neg_count), (unsigned long long)neg);
         if (flags) atomicOr(SOA ? &bar->flags : &sc->flags, flags);
-        if (scribe) {
-            if constexpr (!SOA) {
-                sc->t = s_t;
-                sc->dt = i < n_steps ? 0.0 : dt_last;
-                sc->steps = steps;
-                sc->n_rec = n_rec;
-            }
-            for (int k = 0; k < 3; k++) sc->dtmin3[k] = min_bits(real_inf<float>());
+        if (!SOA && scribe) {
+            sc->t = s_t;
+            sc->dt = i < n_steps ? 0.0 : dt_last;
+            sc->steps = steps;
+            sc->n_rec = n_rec;
         }
         __threadfence();
         if (atomicAdd(&bar->left, 1u) == gridDim.x - 1) {    // the last CTA to leave
+            __threadfence();
+            for (int k = 0; k < 3; k++) sc->dtmin3[k] = min_bits(real_inf<float>());
             if constexpr (SOA) {
-                __threadfence();
                 StepOutcome o;
                 o.dt = i < n_steps ? 0.0 : dt_last;
                 o.neg_count = (long long)atomicExch((unsigned long long *)&bar->neg_count, 0ull);
@@ -241,10 +241,10 @@ int steps_config_f32(const DevPtrs &d, LaunchCfg &cfg)
 }
 
 static int launch_steps(const void *kern, const DevPtrs &d, KArgs<float> a, Gauges gauges, int n, CallerStep caller,
-                        const LaunchCfg &c, void *stream)
+                        LaunchCfg c, void *stream)
 {
     StepsBarrier *bar = reinterpret_cast<StepsBarrier *>(reinterpret_cast<char *>(d.sc) + kBarrierAt);
-    void *args[] = {&a, &bar, &gauges, &n, &caller};
+    void *args[] = {&a, &bar, &gauges, &n, &caller, &c.max_polls};
     return (int)cudaLaunchCooperativeKernel(kern, dim3(c.grid), dim3(d.threads), args, c.smem, static_cast<cudaStream_t>(stream));
 }
 

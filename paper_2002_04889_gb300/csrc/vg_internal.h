@@ -176,6 +176,7 @@ struct LaunchCfg {
     int grid;        // persistent CTAs
     size_t smem;     // dynamic shared memory per CTA
     int ctas;        // multi-step kernel: the variant, CTAs of 256 threads per SM
+    unsigned max_polls = 1u << 20;   // multi-step kernel: polls of a barrier before a CTA gives up (about a second)
 };
 size_t stage_smem_f32(int block, int max_halo, int max_ring1, int max_faces);
 size_t stage_smem_f64(int block, int max_halo, int max_ring1);
