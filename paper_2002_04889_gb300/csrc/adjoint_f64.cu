@@ -180,19 +180,20 @@ __device__ __forceinline__ void recon_forward(const AdjMesh &m, const double *w,
                 if (lt_x(qmax, R.qn[f][v])) { qmax = R.qn[f][v]; imax = f; }
                 if (lt_x(R.qn[f][v], qmin)) { qmin = R.qn[f][v]; imin = f; }
             }
-            // the active limiter: of the faces with the largest D > 0 and the largest
-            // -D > 0 (the first of equals) the one of smaller quotient r / D, where that
-            // is below 1; two candidates and one division, as the forward kernels
+            // The active limiter: the first face of smallest quotient r / D below 1.  The
+            // smallest quotient is that of the largest D > 0 or of the largest -D > 0, so
+            // two candidates and one division serve, as in the forward kernels; but a face
+            // whose D is a few ulps smaller may have the same rounded quotient, and so may
+            // the two candidates where their cross products differ in the last bits.  Only
+            // such faces are divided for.
             const double up = qmax - R.qK[v], dn = R.qK[v] - qmin;
             double P = 0.0, M = 0.0;
-            int fP = -1, fM = -1;
 #pragma unroll
- #pragma unroll
-           for (int f = 0; f < 3; f++) {
+            for (int f = 0; f < 3; f++) {
                 const double D = gx * G(m, GEO_FX + f, K) + gy * G(m, GEO_FY + f, K);
                 R.D[v][f] = D;
-                if (is_pos(D) && gt_nn(D, P)) { P = D; fP = f; }
-                if (is_neg(D) && gt_nn(-D, M)) { M = -D; fM = f; }
+                if (is_pos(D) && gt_nn(D, P)) P = D;
+                if (is_neg(D) && gt_nn(-D, M)) M = -D;
             }
             double alpha = 1.0, ra = 0.0;
             int fa = -1;
@@ -201,13 +202,26 @@ __device__ __forceinline__ void recon_forward(const AdjMesh &m, const double *w,
                 const double xP = up * M, xM = dn * P;
                 bool takeM = limM && (!limP || gt_nn(xP, xM));
                 alpha = quot(takeM ? dn : up, recip(takeM ? M : P));
-                if (limP && limM && dbits(xP) == dbits(xM)) {
-                    const double other = quot(dn, recip(M));          // takeM is false here
-                    takeM = lt_x(other, alpha) || (other == alpha && fM < fP);
-                    if (takeM) alpha = other;
+                const long long apart = dbits(xP) - dbits(xM);
+                const bool both = limP && limM && apart <= 8 && apart >= -8;
+                if (both) {
+                    const double other = quot(takeM ? up : dn, recip(takeM ? P : M));
+                    if (lt_x(other, alpha)) { alpha = other; takeM = !takeM; }
                 }
-                fa = takeM ? fM : fP;
-                ra = takeM ? -dn : up;
+                // (two D of one sign have one rounded quotient at most four steps apart,
+                // but for quotients near the subnormal numbers)
+                const bool tiny = dbits(alpha) < (64LL << 52);
+#pragma unroll
+                for (int f = 0; f < 3; f++) {
+                    const double D = R.D[v][f];
+                    const bool neg = is_neg(D);
+                    const long long below = dbits(neg ? M : P) - dbits(neg ? -D : D);
+                    if (fa >= 0 || is_zero(D) || (neg != takeM && !both) || (below > 4 && !tiny)) continue;
+                    if ((below == 0 && neg == takeM) || quot(neg ? dn : up, recip(neg ? -D : D)) == alpha) {
+                        fa = f;
+                        ra = neg ? -dn : up;
+                    }
+                }
             }
             R.alpha[v] = alpha;
             R.fa[v] = fa;
