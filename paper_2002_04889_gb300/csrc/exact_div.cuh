@@ -90,4 +90,16 @@ __device__ __forceinline__ double half_of(double x)
     return (((unsigned)hi << 1) | (unsigned)lo) == 0u ? x : 0.5 * x;
 }
 
+// x / 2 + y / 2, each rounded once: (x + y) / 2 except where a half is not exact or the
+// sum overflows, that is for sums below 2^-959 (a subnormal half may then decide a
+// rounding) and at the top of the range.
+__device__ __forceinline__ double half_sum(double x, double y)
+{
+    const double s = x + y;
+    const int hi = __double2hiint(s), lo = __double2loint(s);
+    const unsigned e = ((unsigned)hi >> 20) & 0x7ffu;
+    if (e - 64u < 1983u) return __hiloint2double(hi - 0x100000, lo);
+    return (((unsigned)hi << 1) | (unsigned)lo) == 0u ? s : 0.5 * x + 0.5 * y;
+}
+
 }  // namespace vg

@@ -392,10 +392,9 @@ template <typename real>
 __device__ __forceinline__ uint8_t rk2_final(const real x[3], real W1, real Hu1, real Hv1, real RH, real RHu,
                                              real RHv, real dt, real hthr, real &W, real &Hu, real &Hv)
 {
-    // x / 2 + y / 2 rounded once is (x + y) / 2 rounded once
-    W = half_of(x[0] + (W1 + dt * RH));
-    Hu = half_of(x[1] + (Hu1 + dt * RHu));
-    Hv = half_of(x[2] + (Hv1 + dt * RHv));
+    W = half_sum(x[0], W1 + dt * RH);
+    Hu = half_sum(x[1], Hu1 + dt * RHu);
+    Hv = half_sum(x[2], Hv1 + dt * RHv);
     if (is_neg(W)) {
         W = real(0); Hu = real(0); Hv = real(0);
         return 2;
