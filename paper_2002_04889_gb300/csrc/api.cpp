@@ -101,6 +101,7 @@ struct vg_ctx {
     cudaGraphExec_t graph2 = nullptr;
     bool graph_dirty = true;
     int64_t launches = 0;
+    int64_t joined_launches = 0;      // of them, launches of many steps or of a caller's whole step
 
     // discrete adjoint: checkpoints of the last vg_adj_forward run, and the recordings of
     // all its steps where they were kept (AdjRecordings)
@@ -1382,6 +1383,7 @@ int vg_step(vg_ctx *c, int64_t n_steps)
                 }
                 if (e) return cuda_fail(c, (cudaError_t)e, "multi-step launch");
                 c->launches += (int64_t)n * step_kernels(c);
+                c->joined_launches++;
                 if (n & 1) c->cur = 1 - c->cur;
                 left -= n;
             }
@@ -2240,6 +2242,7 @@ int vg_step_noalloc(vg_ctx *c, const void *w_in, void *w_out, double t, double *
             VG_CUDA(c, cudaStreamSynchronize(c->stream));
             r = *out;
             done = true;
+            c->joined_launches++;
         }
     }
     if (!done) {
@@ -2281,6 +2284,18 @@ int vg_debug_lose_arrival(vg_ctx *c, uint32_t max_polls)
                                sizeof(one_short), cudaMemcpyHostToDevice, c->stream));
     VG_CUDA(c, cudaStreamSynchronize(c->stream));
     c->cfgn.max_polls = max_polls;
+    return VG_OK;
+}
+
+// For tests: thread blocks of a launch of many steps (0: the context has none), its
+// variant (CTAs of 256 threads per SM) and how many such launches, a caller's step in one
+// launch included, the context has made.
+int vg_debug_joined(vg_ctx *c, int32_t *grid, int32_t *ctas, int64_t *launches)
+{
+    if (!c || !grid || !ctas || !launches) return VG_EINVAL;
+    *grid = c->cfgn.grid;
+    *ctas = c->cfgn.ctas;
+    *launches = c->joined_launches;
     return VG_OK;
 }
 
