@@ -72,16 +72,20 @@ typedef struct vg_params {
                               and counted): 0                                      */
     int32_t block_cells;   /* cells per thread block of the step kernels
                               (32..512, multiple of 32, at most 256 in a batch;
-                              0 = chosen by the library: 256, in literal FP64 on
-                              meshes of few blocks per SM 64 to 160 (256 too in
-                              a batch or with block_threads given);
+                              0 = chosen by the library: 256, on meshes of few
+                              blocks per SM 64 to 160 in literal FP64 and 64 or
+                              128 in FP32 (256 too in a batch, with
+                              block_threads given and in FP32 while a bed moves);
                               halved automatically while the block and its
                               two-ring halo exceed shared memory)                 */
     int32_t block_threads; /* threads per thread block of the step kernels: a
                               multiple of 32 from block_cells to 2 x block_cells
                               and at most 512 (the extra threads share the halo
-                              and face work); 0 = block_cells, or chosen with
-                              block_cells = 0                                  */
+                              and face work); 0 = block_cells, or with
+                              block_cells = 0 chosen by the library: two threads
+                              a cell on small meshes (FP32 up to two blocks of
+                              256 cells per SM, contracted FP64 up to one,
+                              literal FP64 up to 192 cells per SM)             */
     int32_t fp64_literal;  /* FP64 contexts and batches: 1 evaluates every formula
                               as written, without multiply-add contraction, so
                               the result equals a plain FP64 implementation of

@@ -168,8 +168,7 @@ __device__ __forceinline__ void recon_forward(const AdjMesh &m, const double *w,
     if (recon) {
         double face[3][3];
 #pragma unroll
- #pragma unroll
-       for (int v = 0; v < 3; v++) {
+        for (int v = 0; v < 3; v++) {
             double d0 = R.qn[0][v] - R.qK[v], d1 = R.qn[1][v] - R.qK[v], d2 = R.qn[2][v] - R.qK[v];
             double gx = (G(m, GEO_WX, K) * d0 + G(m, GEO_WX + 1, K) * d1) + G(m, GEO_WX + 2, K) * d2;
             double gy = (G(m, GEO_WY, K) * d0 + G(m, GEO_WY + 1, K) * d1) + G(m, GEO_WY + 2, K) * d2;
@@ -480,34 +479,27 @@ __global__ void __launch_bounds__(kVjpThreads) adj_recon_vjp_kernel(AdjMesh m, c
         double fb[3][3];   // [v][f]
         bool any = m.rec[K] && (!is_zero(Rb[nc + K]) || !is_zero(Rb[2 * (size_t)nc + K]));
 #pragma unroll
- #pragma unroll
-       for (int v = 0; v < 3; v++)
+        for (int v = 0; v < 3; v++)
 #pragma unroll
- #pragma unroll
-           for (int f = 0; f < 3; f++) fb[v][f] = FVb[(v * 3 + f) * (size_t)nc + K];
+            for (int f = 0; f < 3; f++) fb[v][f] = FVb[(v * 3 + f) * (size_t)nc + K];
         double zsl[3];
 #pragma unroll
- #pragma unroll
-       for (int f = 0; f < 3; f++) zsl[f] = zfb[f * (size_t)nc + K];
+        for (int f = 0; f < 3; f++) zsl[f] = zfb[f * (size_t)nc + K];
         if (cf && (cf->cell[0] == K || cf->cell[1] == K)) {
             // the face that set the CFL step: its wave speed's adjoint on this side
             const int side = cf->cell[0] == K ? 0 : 1;
 #pragma unroll
- #pragma unroll
-           for (int f = 0; f < 3; f++)
+            for (int f = 0; f < 3; f++)
                 if (f == cf->face[side]) {
 #pragma unroll
- #pragma unroll
-                   for (int v = 0; v < 3; v++) fb[v][f] += cf->bar[side][v];
+                    for (int v = 0; v < 3; v++) fb[v][f] += cf->bar[side][v];
                     zsl[f] += cf->bar[side][3];
                 }
         }
 #pragma unroll
- #pragma unroll
-       for (int v = 0; v < 3; v++)
+        for (int v = 0; v < 3; v++)
 #pragma unroll
- #pragma unroll
-           for (int f = 0; f < 3; f++) any = any || !is_zero(fb[v][f]);
+            for (int f = 0; f < 3; f++) any = any || !is_zero(fb[v][f]);
         if (!any) {                      // nothing flows back through the reconstruction
             own[K] = 0.0;
             own[nc + K] = 0.0;
@@ -550,12 +542,10 @@ __global__ void __launch_bounds__(kVjpThreads) adj_recon_vjp_kernel(AdjMesh m, c
                 zb += eb;
             }
 #pragma unroll
- #pragma unroll
-           for (int v = 0; v < 3; v++) {
+            for (int v = 0; v < 3; v++) {
                 double ab = 0.0, Db[3];
 #pragma unroll
- #pragma unroll
-               for (int f = 0; f < 3; f++) {
+                for (int f = 0; f < 3; f++) {
                     qKb[v] += fb[v][f];
                     ab += fb[v][f] * R.D[v][f];
                     Db[f] = fb[v][f] * R.alpha[v];
@@ -568,35 +558,30 @@ __global__ void __launch_bounds__(kVjpThreads) adj_recon_vjp_kernel(AdjMesh m, c
                     double iD = inverse(recip(D));
                     double rb = ab * iD;
 #pragma unroll
- #pragma unroll
-                   for (int f = 0; f < 3; f++)
+                    for (int f = 0; f < 3; f++)
                         if (f == fa) Db[f] -= rb * R.r[v] * iD;
                     int idx = is_pos(D) ? R.imax[v] : R.imin[v];
                     if (idx < 0) qKb[v] += rb;
 #pragma unroll
- #pragma unroll
-                   for (int f = 0; f < 3; f++)
+                    for (int f = 0; f < 3; f++)
                         if (f == idx) qnb[f][v] += rb;
                     qKb[v] -= rb;
                 }
                 double gxb = 0.0, gyb = 0.0;
 #pragma unroll
- #pragma unroll
-               for (int f = 0; f < 3; f++) {
+                for (int f = 0; f < 3; f++) {
                     gxb += Db[f] * G(m, GEO_FX + f, K);
                     gyb += Db[f] * G(m, GEO_FY + f, K);
                 }
 #pragma unroll
- #pragma unroll
-               for (int f = 0; f < 3; f++) {
+                for (int f = 0; f < 3; f++) {
                     double db = gxb * G(m, GEO_WX + f, K) + gyb * G(m, GEO_WY + f, K);
                     qnb[f][v] += db;
                     qKb[v] -= db;
                 }
             }
 #pragma unroll
- #pragma unroll
-           for (int f = 0; f < 3; f++) {
+            for (int f = 0; f < 3; f++) {
                 if (!R.wall[f]) continue;
                 if (R.open[f]) {                 // ghost = the cell's own values
                     qKb[0] += qnb[f][0];

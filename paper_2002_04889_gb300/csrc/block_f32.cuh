@@ -11,9 +11,11 @@
 // ocean) never appear, only products of small differences (eta_f - eta_K, z* - z_K),
 // so still water stays still in FP32 and eta keeps full FP32 resolution.
 //
-// What bounds it: the kernels are issue-bound (58-62 % of issue slots busy at 44
-// resident warps per SM, DRAM below half its rate), so the layout is the one with
-// the fewest instructions and shared or global accesses per cell:
+// What bounds it: latency.  4M triangles: 50 % of issue slots busy at 37 resident warps
+// per SM, DRAM at 44 %; warps wait for halo states and records (7.5 cycles an issue) and
+// at the barriers between the phases (4.6).  The layout is the one with the fewest
+// instructions and shared or global accesses per cell (the former one, separate arrays,
+// was at 58-60 % of the issue slots with 40 % more instructions):
 //   state   float4 per cell (eta, Hu, Hv, z): one 16-byte load per block or halo
 //           cell and one 16-byte shared slot, where separate arrays took four loads
 //           with an address each and touched four sectors per halo cell

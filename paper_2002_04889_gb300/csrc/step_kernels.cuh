@@ -88,22 +88,15 @@ template <> struct StateWord<float> { using type = float4; };
 template <typename real>
 __host__ __device__ inline size_t stage_smem_bytes(int block, int max_halo, int max_ring1, int max_faces, bool gids = false);
 
-__device__ __forceinline__ float vmax(float a, float b) { return fmaxf(a, b); }
-__device__ __forceinline__ double vmax(double a, double b) { return fmax(a, b); }
 __device__ __forceinline__ float vmin(float a, float b) { return fminf(a, b); }
 __device__ __forceinline__ double vmin(double a, double b) { return fmin(a, b); }
-__device__ __forceinline__ float vabs(float a) { return fabsf(a); }
-__device__ __forceinline__ double vabs(double a) { return fabs(a); }
-__device__ __forceinline__ float vsqrt(float a) { return sqrtf(a); }
-__device__ __forceinline__ double vsqrt(double a) { return sqrt(a); }
 
 // Compare and select.  GB300 runs FP64 compares and min/max on its FP64 units,
 // which issue two lane-operations per SM and cycle, while its integer units are
 // idle in the FP64 kernels; so the FP64 forms below work on the IEEE bit patterns
 // with integer instructions.  For the non-NaN values of the step they decide and
 // select exactly as the FP64 instructions do (a zero result may carry the other
-// sign, which no later operation of the step distinguishes).  The FP32 forms are
-// the plain FP32 instructions.
+// sign, which no later operation of the step distinguishes).
 //   gt_nn(x, y): x > y for y >= +0;  is_zero(x): x == 0;  is_neg(x): x < 0;
 //   is_pos(x): x > 0;  smax / smin: max / min;  max0(x): max(0, x).
 __device__ __forceinline__ long long dbits(double x) { return __double_as_longlong(x); }
@@ -113,19 +106,13 @@ __device__ __forceinline__ long long okey(double x)   // order-preserving for ev
     const long long b = dbits(x);
     return b < 0 ? b ^ 0x7fffffffffffffffLL : b;
 }
-__device__ __forceinline__ bool gt_nn(float x, float y) { return x > y; }
 __device__ __forceinline__ bool gt_nn(double x, double y) { return dbits(x) > dbits(y); }
-__device__ __forceinline__ bool is_zero(float x) { return x == 0.f; }
 __device__ __forceinline__ bool is_zero(double x) { return (ubits(x) << 1) == 0; }
-__device__ __forceinline__ bool is_neg(float x) { return x < 0.f; }
 __device__ __forceinline__ bool is_neg(double x) { return dbits(x) < 0 && (ubits(x) << 1) != 0; }
-__device__ __forceinline__ bool is_pos(float x) { return x > 0.f; }
 __device__ __forceinline__ bool is_pos(double x) { return dbits(x) > 0; }
-__device__ __forceinline__ float smax(float a, float b) { return fmaxf(a, b); }
 __device__ __forceinline__ double smax(double a, double b) { return okey(a) < okey(b) ? b : a; }
 __device__ __forceinline__ float smin(float a, float b) { return fminf(a, b); }
 __device__ __forceinline__ double smin(double a, double b) { return okey(b) < okey(a) ? b : a; }
-__device__ __forceinline__ float max0(float x) { return fmaxf(0.f, x); }
 __device__ __forceinline__ double max0(double x) { return dbits(x) > 0 ? x : 0.0; }
 // isfinite on the integer units.
 __device__ __forceinline__ bool finite(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
@@ -192,14 +179,14 @@ __device__ __forceinline__ double step_dt(const DevScalars *sc, double cfl, doub
 
 // t_end > 0 and t >= t_end: the context has reached its end time (decided on the
 // integer units: every thread of a launch asks, and on the FP64 units the two
-// compares of an SM's 48 warps take about 1500 cycles).
+// compares of an SM's 40 warps take about 1300 cycles).
 __device__ __forceinline__ bool finished(double t_end, const DevScalars *sc)
 {
     return is_pos(t_end) && okey(sc->t) >= okey(t_end);
 }
 
 // The step's dt for every thread of a CTA, formed by one of them: a dozen FP64
-// instructions in each of an SM's 48 warps were 10,700 cycles of its FP64 units
+// instructions in each of the 48 warps that an SM then held were 10,700 cycles of its FP64 units
 // (two lane-operations a cycle), 5 us a launch.  Every thread must call it.
 template <typename real>
 __device__ __forceinline__ real cta_step_dt(const DevScalars *sc, double cfl, double dt_fixed, double dt_max)
@@ -221,8 +208,8 @@ __device__ __forceinline__ void hll_normal(real g, real half_g, real HL, real un
         amax = real(0);
         return;
     }
-    real cL = vsqrt(g * HL);
-    real cR = vsqrt(g * HR);
+    real cL = sqrt(g * HL);
+    real cR = sqrt(g * HR);
     real sL, sR;
     if (is_zero(HL)) {
         sL = unR - real(2) * cR;
@@ -259,7 +246,7 @@ __device__ __forceinline__ void hll_normal(real g, real half_g, real HL, real un
     } else {
         F[0] = FR0; F[1] = FR1; F[2] = FR2;
     }
-    amax = smax(vabs(sL), vabs(sR));
+    amax = smax(fabs(sL), fabs(sR));
 }
 
 // Flux through a face seen from its left cell: face velocities, hydrostatic
@@ -294,7 +281,7 @@ __device__ __forceinline__ void face_flux(real g, real half_g, real hthr,
         // absorbing: the characteristic ghost of a sea at rest (eta = 0) beyond
         // the boundary, on the same bed (the oracle's order of operations)
         HsL = max0((HfL + zL) - zL);
-        const real cL = vsqrt(g * HsL), c0 = vsqrt(g * max0(real(0) - zL));
+        const real cL = sqrt(g * HsL), c0 = sqrt(g * max0(real(0) - zL));
         const real Rp = unL + real(2) * cL, Rm = real(0) - real(2) * c0;
         unR = real(0.5) * (Rp + Rm);
         const real cg = max0(real(0.25) * (Rp - Rm));
@@ -591,11 +578,7 @@ __device__ __forceinline__ void process_block(const KArgs<real> &a, const int b,
     // 2) and phase C no faces, which costs a few instructions more but no
     // register spills where mode 1 would spill (runs with recordings take every
     // phase there).
-    bool skip = false;
-    if constexpr (DRY == 0)
-        __syncthreads();
-    else
-        skip = __syncthreads_and(dry) && (DRY == 1 || (!a.fv_out && !a.mask2 && !a.r1_out && !a.rec_out));
+    const bool skip = __syncthreads_and(dry) && (DRY == 1 || (!a.fv_out && !a.mask2 && !a.r1_out && !a.rec_out));
     if (DRY == 1 && skip) {
         if (!LISTED && tid == 0) qcount = 0;
         if (tid < ncell) {
