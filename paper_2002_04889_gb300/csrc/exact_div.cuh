@@ -98,8 +98,9 @@ __device__ __forceinline__ double half_sum(double x, double y)
     const double s = x + y;
     const int hi = __double2hiint(s), lo = __double2loint(s);
     const unsigned e = ((unsigned)hi >> 20) & 0x7ffu;
-    if (e - 64u < 1983u) return __hiloint2double(hi - 0x100000, lo);
-    return (((unsigned)hi << 1) | (unsigned)lo) == 0u ? s : 0.5 * x + 0.5 * y;
+    const bool zero = (((unsigned)hi << 1) | (unsigned)lo) == 0u;
+    if (__builtin_expect(e - 64u < 1983u || zero, 1)) return __hiloint2double(zero ? hi : hi - 0x100000, lo);
+    return 0.5 * x + 0.5 * y;
 }
 
 }  // namespace vg

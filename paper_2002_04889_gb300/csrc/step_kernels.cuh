@@ -375,13 +375,16 @@ __device__ __forceinline__ void st4(double *p, double x, double y, double z, dou
 // from w^n = x, w1 = (W1, Hu1, Hv1) and R(w1) = (RH, RHu, RHv), then the dry fix.
 // Returns the fix's branch: 0 none, 1 momentum cut (depth at or below the
 // threshold), 2 negative depth emptied.
-template <typename real>
+// (FAST, the contracted build: half of the sum, which is the same number but at the
+// ends of the range.)
+template <typename real, bool FAST = false>
 __device__ __forceinline__ uint8_t rk2_final(const real x[3], real W1, real Hu1, real Hv1, real RH, real RHu,
                                              real RHv, real dt, real hthr, real &W, real &Hu, real &Hv)
 {
-    W = half_sum(x[0], W1 + dt * RH);
-    Hu = half_sum(x[1], Hu1 + dt * RHu);
-    Hv = half_sum(x[2], Hv1 + dt * RHv);
+    const real yW = W1 + dt * RH, yHu = Hu1 + dt * RHu, yHv = Hv1 + dt * RHv;
+    W = FAST ? half_of(x[0] + yW) : half_sum(x[0], yW);
+    Hu = FAST ? half_of(x[1] + yHu) : half_sum(x[1], yHu);
+    Hv = FAST ? half_of(x[2] + yHv) : half_sum(x[2], yHv);
     if (is_neg(W)) {
         W = real(0); Hu = real(0); Hv = real(0);
         return 2;
@@ -427,7 +430,7 @@ __device__ __forceinline__ void finish_cell(const KArgs<real> &a, int gid, const
         real W1, Hu1, Hv1, z1;
         ld4(sWl, W1, Hu1, Hv1, z1);
         real W, Hu, Hv;
-        const uint8_t branch = rk2_final(x, W1, Hu1, Hv1, RH, RHu, RHv, dt, a.hthr, W, Hu, Hv);
+        const uint8_t branch = rk2_final<real, FAST>(x, W1, Hu1, Hv1, RH, RHu, RHv, dt, a.hthr, W, Hu, Hv);
         if (branch == 2) my_neg++;
         if (a.mask2) a.mask2[gid] = branch;
         if (!finite(W) || !finite(Hu) || !finite(Hv)) bad = true;
