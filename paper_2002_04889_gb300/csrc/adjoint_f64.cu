@@ -183,42 +183,48 @@ __device__ __forceinline__ void recon_forward(const AdjMesh &m, const double *w,
             // smallest quotient is that of the largest D > 0 or of the largest -D > 0, so
             // two candidates and one division serve, as in the forward kernels; but a face
             // whose D is a few ulps smaller may have the same rounded quotient, and so may
-            // the two candidates where their cross products differ in the last bits.  Only
-            // such faces are divided for.
+            // the two candidates where their cross products differ in the last bits.  Where
+            // the high words leave that open (or the quotient is near the subnormal
+            // numbers) the quotients of all three faces are formed and compared.
             const double up = qmax - R.qK[v], dn = R.qK[v] - qmin;
             double P = 0.0, M = 0.0;
+            int fP = -1, fM = -1;
 #pragma unroll
             for (int f = 0; f < 3; f++) {
                 const double D = gx * G(m, GEO_FX + f, K) + gy * G(m, GEO_FY + f, K);
                 R.D[v][f] = D;
-                if (is_pos(D) && gt_nn(D, P)) P = D;
-                if (is_neg(D) && gt_nn(-D, M)) M = -D;
+                if (is_pos(D) && gt_nn(D, P)) { P = D; fP = f; }
+                if (is_neg(D) && gt_nn(-D, M)) { M = -D; fM = f; }
             }
             double alpha = 1.0, ra = 0.0;
             int fa = -1;
             const bool limP = gt_nn(P, up), limM = gt_nn(M, dn);
             if (limP || limM) {
                 const double xP = up * M, xM = dn * P;
-                bool takeM = limM && (!limP || gt_nn(xP, xM));
-                alpha = quot(takeM ? dn : up, recip(takeM ? M : P));
-                const long long apart = dbits(xP) - dbits(xM);
-                const bool both = limP && limM && apart <= 8 && apart >= -8;
-                if (both) {
-                    const double other = quot(takeM ? up : dn, recip(takeM ? P : M));
-                    if (lt_x(other, alpha)) { alpha = other; takeM = !takeM; }
-                }
-                // (two D of one sign have one rounded quotient at most four steps apart,
-                // but for quotients near the subnormal numbers)
-                const bool tiny = dbits(alpha) < (64LL << 52);
+                const bool takeM = limM && (!limP || gt_nn(xP, xM));
+                const double num = takeM ? dn : up, den = takeM ? M : P;
+                alpha = quot(num, recip(den));
+                fa = takeM ? fM : fP;
+                ra = takeM ? -dn : up;
+                // integer differences of high words: <= 1 for neighbours at most 2^32 steps apart
+                const int hx = __double2hiint(xP) - __double2hiint(xM), hd = __double2hiint(den);
+                bool open = (limP && limM && hx <= 1 && hx >= -1) || (__double2hiint(alpha) < (64 << 20) && !is_zero(num));
 #pragma unroll
-                for (int f = 0; f < 3; f++) {
-                    const double D = R.D[v][f];
-                    const bool neg = is_neg(D);
-                    const long long below = dbits(neg ? M : P) - dbits(neg ? -D : D);
-                    if (fa >= 0 || is_zero(D) || (neg != takeM && !both) || (below > 4 && !tiny)) continue;
-                    if ((below == 0 && neg == takeM) || quot(neg ? dn : up, recip(neg ? -D : D)) == alpha) {
-                        fa = f;
-                        ra = neg ? -dn : up;
+                for (int f = 2; f >= 0; f--) {
+                    const int h = __double2hiint(R.D[v][f]) ^ (takeM ? (int)0x80000000 : 0);    // |D| if of the taken sign, else < 0
+                    const bool same = h >= 0 && !is_zero(R.D[v][f]);
+                    if (same && is_zero(num)) fa = f;                // every quotient of this sign is 0
+                    open = open || (same && f < fa && hd - h <= 1 && !is_zero(num));
+                }
+                if (open) {
+                    alpha = 1.0;
+#pragma unroll
+                    for (int f = 0; f < 3; f++) {
+                        const double D = R.D[v][f];
+                        if (is_zero(D)) continue;
+                        const bool neg = is_neg(D);
+                        const double t = quot(neg ? dn : up, recip(neg ? -D : D));
+                        if (lt_pos(t, alpha)) { alpha = t; fa = f; ra = neg ? -dn : up; }
                     }
                 }
             }
